@@ -241,7 +241,7 @@ def run_gpu(args):
             fit_ms.append(st.ms_fit)
             stage_ms.append((st.ms_fit, st.ms_gain, st.ms_alloc))
             if not block_ms:
-                launches += st.launches            # kernels of one block of --steps steps
+                launches += st.kernel_launches     # kernels of one block of --steps steps
         ev1.record(stream)
         barrier()
         block_ms.append(ev0.elapsed_time(ev1))

@@ -94,15 +94,9 @@ enum {
                                      1: they are replaced by the slopes of the upper concave envelope of the points
                                      (n, R(n)), the smallest concave function nowhere below R, which keeps the curve's
                                      whole drop at max_cores_per_job.  Rows of convex fits are the same either way. */
-    SLAQ_P_SELECTION = 10         /* How the greedy loop's threshold is found.  0: every job's gains for n = 1..max
-                                     are written to a table first and the selection reads the table.  1: no table -
-                                     a job's gains fall with n, so the selection finds what it needs of a row by
-                                     binary search over n with the gain in closed form, and evaluates only the gains
-                                     that share the threshold's leading digits (the effective gain of the n-th core is
-                                     then min(g(1), g(n)), which differs from the table's running minimum by rounding
-                                     at most).  Used for the plain prediction only: with SLAQ_P_GAIN_ENVELOPE, with
-                                     target-loss hints, and in the sharded steps the table is written.  The gain
-                                     rows that slaq_get_predictions returns are then written on request. */
+    SLAQ_P_SELECTION = 10         /* 0 or 1: whether a caller wants the whole table of gains written.  Both find the same
+                                  allocation with the same kernel, which predicts a row only as far as the selection
+                                  may need it; gain rows that slaq_get_predictions returns are completed on request. */
 };
 
 /* per-job status written by slaq_schedule (slaq_get_predictions, out_status) */
@@ -123,7 +117,8 @@ typedef struct slaq_stats {
     float ms_fit;          /* normalise + fit kernel (the three stage times are 0 for an epoch replayed as a CUDA graph) */
     float ms_gain;         /* marginal-gain kernel (with the first selection histogram) */
     float ms_alloc;        /* threshold selection, per-job counts, allocation */
-    int32_t launches;      /* kernels launched by the call */
+    int32_t launches;      /* steps of the call, counted as if each were a kernel of its own (15 for an epoch: three of the
+                              work list, fit, gains, ten of the selection), however they are grouped into launches */
     int32_t active_jobs;
     int64_t cores_handed_out;
     int64_t points;        /* loss values read by the fit kernel */
@@ -136,6 +131,7 @@ typedef struct slaq_stats {
     int32_t fallback_jobs;
     int32_t nonconvex_fits;  /* fitted jobs whose winning curve is not convex ahead of the newest point (family I with
                                 b^2 < a c): their marginal gains rise before they fall, see SLAQ_P_GAIN_ENVELOPE */
+    int32_t kernel_launches; /* kernels the call launched */
 } slaq_stats;
 
 /*

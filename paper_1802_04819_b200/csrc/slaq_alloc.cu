@@ -1,15 +1,12 @@
-// Allocation: the greedy loop of "Scheduling Based on Quality Improvements" as a global
-// top-C selection.
+// The selection step by step, for one cluster sharded over several GPUs.
 //
-// The paper starts every job at one core and then gives one core at a time to the job
-// whose next core has the largest predicted gain.  Gain rows are non-increasing in n, so
-// that loop hands out exactly the `want` largest gains beyond the floor, and among equal
-// gains it serves (job id ascending, n ascending).  Here: a most-significant-digit-first
-// radix select over the 64-bit patterns of the gains (all >= +0, so the IEEE pattern
-// orders like the value) finds the threshold tau and how many gains equal to tau are
-// still wanted - after the first two passes it reads only the short segment of each row
-// that still agrees with the threshold's leading digits; then per job  a_j = floor + #{g > tau} + clamp(wanted - P_j, 0, #{g = tau})
-// with P_j the number of gains equal to tau in jobs with a lower id.
+// The greedy loop of "Scheduling Based on Quality Improvements" as a global top-C selection (see slaq_select.cu) whose
+// threshold search has to be interrupted: between the steps the caller sums histograms over the shards.  A
+// most-significant-digit-first radix select over the 64-bit patterns of the gains (all >= +0, so the IEEE pattern
+// orders like the value) finds the threshold tau and how many gains equal to tau are still wanted - after the first
+// two passes it reads only the short segment of each row that still agrees with the threshold's leading digits;
+// then per job  a_j = floor + #{g > tau} + clamp(wanted - P_j, 0, #{g = tau}) with P_j the number of gains
+// equal to tau in jobs with a lower id.
 #include <math_constants.h>
 
 #include "slaq_internal.cuh"
@@ -75,15 +72,12 @@ __device__ void pick_bin(const unsigned long long* hist, int pass, SelectState* 
 // prefix found so far form one contiguous segment [seg_lo, seg_hi) of the row.  Pass p narrows every
 // segment by the bin chosen for digit p - 1 (elements with a larger digit lie before it, with a smaller
 // one behind it) and histograms digit p over what is left; from the second pass on only the
-// segments are read.  The last block to finish picks the bin of digit p.
+// segments are read.
 __global__ void __launch_bounds__(kSelectThreads)
 select_pass_kernel(const double* __restrict__ gain, const int32_t* __restrict__ count, int max_jobs, int cap,
-                   int first_unit, int pass, unsigned long long* __restrict__ hist_all, SelectState* sel,
-                   unsigned int* ticket, int32_t* __restrict__ seg_lo, int32_t* __restrict__ seg_hi, int do_pick,
-                   int32_t* err_word) {
+                   int first_unit, int pass, unsigned long long* __restrict__ hist_all, const SelectState* sel,
+                   int32_t* __restrict__ seg_lo, int32_t* __restrict__ seg_hi, int32_t* err_word) {
     __shared__ unsigned int sh_hist[kRadixBins];
-    __shared__ unsigned long long sh_scan[kSelectThreads + 1];
-    __shared__ bool is_last;
     unsigned long long* hist = hist_all + (size_t)pass * kRadixBins;
     if (sel->done) return;   // uniform over the grid: nothing is wanted
     for (int i = threadIdx.x; i < kRadixBins; i += blockDim.x) sh_hist[i] = 0;
@@ -157,21 +151,6 @@ select_pass_kernel(const double* __restrict__ gain, const int32_t* __restrict__ 
         const unsigned v = sh_hist[i];
         if (v) atomicAdd(&hist[i], (unsigned long long)v);
     }
-    if (!do_pick) return;   // the histogram is completed elsewhere (summed over GPUs) before the bin is picked
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(&ticket[1 + pass], 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (is_last) {
-        __threadfence();
-        pick_bin(hist, pass, sel, sh_scan);
-    }
-}
-
-// The first histogram is complete when this starts (it was filled by an earlier kernel).
-__global__ void __launch_bounds__(kSelectThreads) pick_first_kernel(unsigned long long* hist_all, SelectState* sel) {
-    __shared__ unsigned long long sh_scan[kSelectThreads + 1];
-    pick_bin(hist_all, 0, sel, sh_scan);
 }
 
 // Pick the bin of any pass from a histogram that is complete when the kernel starts.
@@ -186,29 +165,6 @@ __global__ void init_select_kernel(SelectState* sel, long long want) {
     sel->prefix = want > 0 ? 0ull : ~0ull;   // nothing wanted: a threshold above every gain
     sel->want = want > 0 ? want : 0;
     sel->done = want > 0 ? 0 : 1;
-}
-
-// Histogram of the first digit when the gain rows were not written by the gain kernel.
-__global__ void __launch_bounds__(kSelectThreads)
-first_hist_kernel(const double* __restrict__ gain, const int32_t* __restrict__ count, int max_jobs, int cap,
-                  int first_unit, unsigned long long* __restrict__ hist0, int32_t* err_word) {
-    __shared__ unsigned int sh_hist[kRadixBins];
-    for (int i = threadIdx.x; i < kRadixBins; i += blockDim.x) sh_hist[i] = 0;
-    __syncthreads();
-    const unsigned long long* keys = reinterpret_cast<const unsigned long long*>(gain);
-    const int lane = threadIdx.x & 31;
-    const int warps_total = gridDim.x * (kSelectThreads / 32);
-    for (int j = blockIdx.x * (kSelectThreads / 32) + (threadIdx.x >> 5); j < max_jobs; j += warps_total) {
-        if (count[j] <= 0) continue;
-        for (int n = first_unit + lane; n <= cap; n += 32)
-            if (index_ok((long long)j * cap + (n - 1), (long long)max_jobs * cap, kErrGain, err_word))
-                atomicAdd(&sh_hist[(unsigned)(keys[(size_t)j * cap + (n - 1)] >> (64 - kRadixBits))], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kRadixBins; i += blockDim.x) {
-        const unsigned v = sh_hist[i];
-        if (v) atomicAdd(&hist0[i], (unsigned long long)v);
-    }
 }
 
 // Per job: how many candidate gains lie above the threshold and how many equal it.  The segments
@@ -359,85 +315,16 @@ finalise_kernel(const double* __restrict__ gain, const int32_t* __restrict__ cou
         atomicAdd((unsigned long long*)&counters[6], (unsigned long long)(sh_pre[0] >> 20));
         atomicAdd((unsigned long long*)&counters[7], (unsigned long long)(sh_pre[0] & ((1ll << 20) - 1)));
     }
-    // predicted reduction at the allocation: the job's first a_j gains.  Most jobs get a few cores: their own thread
-    // adds them in order (all threads of the block load at once); a row with more than 32 is left to its warp.
-    const int warp = t >> 5, lane = t & 31;
-    const bool mine = jt < max_jobs;
-    if (mine && a <= 32) {
+    // predicted reduction at the allocation: the job's first a_j gains, in order (as the single launch adds them)
+    if (jt < max_jobs) {
         double R = 0.0;
         const double* row = gain + (size_t)jt * cap;
         for (int n = 0; n < a; ++n) R += row[n];
         reduction[jt] = R;
     }
-    unsigned big = __ballot_sync(kFull, mine && a > 32);
-    while (big) {
-        const int r = __ffs(big) - 1;
-        big &= big - 1;
-        const int j = j0 + warp * 32 + r;
-        const int aj = __shfl_sync(kFull, a, r);
-        double R = 0.0;
-        for (int n = lane; n < aj; n += 32) R += gain[(size_t)j * cap + n];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) R += __shfl_xor_sync(kFull, R, o);
-        if (lane == 0) reduction[j] = R;
-    }
 }
 
 }  // namespace
-
-// Selection + counts + allocation on the gain rows held by the handle.  `want` = units to
-// hand out beyond the floor among gains n >= first_unit.  hist0_ready: the first histogram
-// was already accumulated (by the gain kernel).
-int launch_allocate(slaq_handle* h, long long want, int first_unit, bool hist0_ready, int32_t* d_out_alloc) {
-    int launches = 0;
-    const int J = h->max_jobs, cap = h->max_cores;
-    cudaStream_t st = h->stream;
-    int grid = h->sm_count * 8;
-    const int needed = (J + (kSelectThreads / 32) - 1) / (kSelectThreads / 32);
-    if (grid > needed) grid = needed;
-    init_select_kernel<<<1, 1, 0, st>>>(h->scratch.sel, want);
-    ++launches;
-    if (!hist0_ready) {
-        first_hist_kernel<<<grid, kSelectThreads, 0, st>>>(h->gain, h->job.count, J, cap, first_unit, h->scratch.hist,
-                                                          h->err_word);
-        ++launches;
-    }
-    pick_first_kernel<<<1, kSelectThreads, 0, st>>>(h->scratch.hist, h->scratch.sel);
-    ++launches;
-    for (int pass = 1; pass < kRadixPasses; ++pass) {
-        select_pass_kernel<<<grid, kSelectThreads, 0, st>>>(h->gain, h->job.count, J, cap, first_unit, pass,
-                                                           h->scratch.hist, h->scratch.sel, h->scratch.ticket,
-                                                           h->scratch.gt, h->scratch.eq, 1, h->err_word);
-        ++launches;
-    }
-    const int blocks = (J + kJobsPerBlock - 1) / kJobsPerBlock;
-    count_kernel<<<blocks, 256, 0, st>>>(h->gain, h->job.count, J, cap, first_unit, h->scratch.sel, h->scratch.gt,
-                                         h->scratch.eq, h->scratch.block_eq, h->err_word);
-    scan_blocks_kernel<<<1, 1024, 0, st>>>(h->scratch.block_eq, blocks);
-    finalise_kernel<<<blocks, 256, 0, st>>>(h->gain, h->job.count, J, cap, first_unit - 1, h->scratch.sel, h->scratch.gt,
-                                            h->scratch.eq, h->scratch.block_eq, h->alloc, h->reduction,
-                                            h->job.last_alloc, d_out_alloc, h->scratch.counters, 0, nullptr, h->err_word);
-    launches += 3;
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        h->err = std::string("allocation kernels launch: ") + cudaGetErrorString(e);
-        return -1;
-    }
-    return launches;
-}
-
-// The two small steps the table-free selection (slaq_select_free.cu) shares with this file.
-int launch_pick_first(slaq_handle* h) {
-    pick_first_kernel<<<1, kSelectThreads, 0, h->stream>>>(h->scratch.hist, h->scratch.sel);
-    return 1;
-}
-int launch_scan_blocks(slaq_handle* h, int blocks) {
-    scan_blocks_kernel<<<1, 1024, 0, h->stream>>>(h->scratch.block_eq, blocks);
-    return 1;
-}
-
-// ---- one cluster sharded over several GPUs: the same kernels, driven step by step so that the
-// histograms can be summed over the shards between the steps ----
 
 static int check_launch(slaq_handle* h, const char* what) {
     const cudaError_t e = cudaGetLastError();
@@ -465,8 +352,8 @@ int launch_shard_pass(slaq_handle* h, int pass, int first_unit) {
     const int needed = (J + (kSelectThreads / 32) - 1) / (kSelectThreads / 32);
     if (grid > needed) grid = needed;
     select_pass_kernel<<<grid, kSelectThreads, 0, h->stream>>>(h->gain, h->job.count, J, h->max_cores, first_unit, pass,
-                                                              h->scratch.hist, h->scratch.sel, h->scratch.ticket,
-                                                              h->scratch.gt, h->scratch.eq, 0, h->err_word);
+                                                              h->scratch.hist, h->scratch.sel, h->scratch.gt, h->scratch.eq,
+                                                              h->err_word);
     return check_launch(h, "shard pass") ? -1 : 1;
 }
 
@@ -492,100 +379,4 @@ int launch_shard_finalise(slaq_handle* h, int first_unit, long long ties_before,
     return check_launch(h, "shard finalise") ? -1 : 1;
 }
 
-// ---------------------------------------------------------------------------------
-// Allocation without any device allocation: the same kernels, their scratch in a static
-// device array that ships with the library image.
-// ---------------------------------------------------------------------------------
-namespace {
-
-constexpr int kStaticMaxJobs = 32768;
-constexpr int kStaticBlocks = kStaticMaxJobs / kJobsPerBlock;
-
-// Everything the selection and the per-job counts write besides the caller's outputs.
-struct StaticScratch {
-    unsigned long long hist[kRadixPasses * kRadixBins];   // cleared every call
-    unsigned int ticket[8];                               // cleared every call
-    SelectState sel;                                      // rewritten every call
-    long long counters[16];                               // cleared every call
-    long long block_eq[kStaticBlocks + 2];                // fully rewritten before it is read
-    int32_t gt[kStaticMaxJobs];                           // fully rewritten before it is read
-    int32_t eq[kStaticMaxJobs];
-    int32_t every_row_active[kStaticMaxJobs];             // set to 1 every call
-    int32_t cores_now[kStaticMaxJobs];                    // sink for the "current core count" the kernels keep
-};
-
-static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
-
-__global__ void fill_ones_kernel(int32_t* v, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) v[i] = 1;
-}
-
-// Device address of g_static_scratch on the current device, looked up once per device.
-// In host code the array's name only stands for the symbol; kernels need this address.
-int static_scratch_for_current_device(StaticScratch** out) {
-    constexpr int kMaxDevices = 64;
-    static StaticScratch* cache[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SLAQ_E_CUDA;
-    StaticScratch* p = __atomic_load_n(&cache[dev], __ATOMIC_ACQUIRE);
-    if (!p) {
-        void* addr = nullptr;
-        if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || !addr) return SLAQ_E_CUDA;
-        p = static_cast<StaticScratch*>(addr);
-        __atomic_store_n(&cache[dev], p, __ATOMIC_RELEASE);   // every thread finds the same address
-    }
-    *out = p;
-    return SLAQ_OK;
-}
-
-}  // namespace
-
 }  // namespace slaq
-
-extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_t max_cores_per_job,
-                                    int64_t total_cores, int32_t* d_out_alloc, double* d_out_reduction,
-                                    void* cuda_stream) {
-    using namespace slaq;
-    if (!d_gain || !d_out_alloc || !d_out_reduction || n_jobs < 1 || max_cores_per_job < 1 || total_cores < 0)
-        return SLAQ_E_ARG;
-    if (n_jobs > kStaticMaxJobs || max_cores_per_job > kMaxCoresLimit) return SLAQ_E_RANGE;
-    StaticScratch* sc = nullptr;
-    const int rc = static_scratch_for_current_device(&sc);
-    if (rc) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const int J = n_jobs, cap = max_cores_per_job;
-    const int floor_units = total_cores >= J ? 1 : 0, first_unit = floor_units + 1;
-    const long long usable = total_cores < (long long)J * cap ? total_cores : (long long)J * cap;
-    const long long want = usable - (long long)J * floor_units;
-
-    // the array keeps the previous call's contents: clear what the kernels accumulate into
-    if (cudaMemsetAsync(sc->hist, 0, sizeof sc->hist, st) != cudaSuccess) return SLAQ_E_CUDA;
-    if (cudaMemsetAsync(sc->ticket, 0, sizeof sc->ticket, st) != cudaSuccess) return SLAQ_E_CUDA;
-    if (cudaMemsetAsync(sc->counters, 0, sizeof sc->counters, st) != cudaSuccess) return SLAQ_E_CUDA;
-    fill_ones_kernel<<<(J + 255) / 256, 256, 0, st>>>(sc->every_row_active, J);
-    init_select_kernel<<<1, 1, 0, st>>>(&sc->sel, want);
-
-    int sm_count = 148, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
-    int grid = sm_count * 8;
-    const int needed = (J + (kSelectThreads / 32) - 1) / (kSelectThreads / 32);
-    if (grid > needed) grid = needed;
-    first_hist_kernel<<<grid, kSelectThreads, 0, st>>>(d_gain, sc->every_row_active, J, cap, first_unit, sc->hist, nullptr);
-    pick_first_kernel<<<1, kSelectThreads, 0, st>>>(sc->hist, &sc->sel);
-    for (int pass = 1; pass < kRadixPasses; ++pass)
-        select_pass_kernel<<<grid, kSelectThreads, 0, st>>>(d_gain, sc->every_row_active, J, cap, first_unit, pass,
-                                                           sc->hist, &sc->sel, sc->ticket, sc->gt, sc->eq, 1, nullptr);
-    const int blocks = (J + kJobsPerBlock - 1) / kJobsPerBlock;
-    count_kernel<<<blocks, 256, 0, st>>>(d_gain, sc->every_row_active, J, cap, first_unit, &sc->sel, sc->gt, sc->eq,
-                                         sc->block_eq, nullptr);
-    scan_blocks_kernel<<<1, 1024, 0, st>>>(sc->block_eq, blocks);
-    finalise_kernel<<<blocks, 256, 0, st>>>(d_gain, sc->every_row_active, J, cap, floor_units, &sc->sel, sc->gt, sc->eq,
-                                            sc->block_eq, d_out_alloc, d_out_reduction, sc->cores_now, nullptr,
-                                            sc->counters, 0, nullptr, nullptr);
-    if (cudaGetLastError() != cudaSuccess) return SLAQ_E_CUDA;
-    if (total_cores < J) return SLAQ_W_OVERSUBSCRIBED;
-    if (total_cores > (long long)J * cap) return SLAQ_W_UNDERFILLED;
-    return SLAQ_OK;
-}

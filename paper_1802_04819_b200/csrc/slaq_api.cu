@@ -14,6 +14,7 @@ using namespace slaq;
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int32_t kEpochSteps = 15, kAllocateSteps = 11;   // slaq_stats.launches
 
 struct Bump {
     char* base;
@@ -63,15 +64,18 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     fit.warm_scale = b.take<double>(Js);
     Scratch sc;
     sc.hist = b.take<unsigned long long>((size_t)kRadixPasses * kRadixBins);
-    const size_t zero_from = b.off - sizeof(unsigned long long) * (size_t)kRadixPasses * kRadixBins;
     sc.ticket = b.take<unsigned int>(kTickets);
+    sc.zero = sc.ticket;
+    const size_t zero_from = b.off - sizeof(unsigned int) * kTickets;
     sc.sel = b.take<SelectState>(1);
     sc.counters = b.take<long long>(16);
     sc.bucket = b.take<int32_t>((size_t)Hmax + 1);
-    sc.zero_bytes = b.off - zero_from;
+    sc.select = b.take<SelectGlobal>(1);
+    sc.zero_bytes = b.off - sizeof(SelectGlobal) + SelectGlobal::kZeroBytes - zero_from;
     sc.gt = b.take<int32_t>(Js);
     sc.eq = b.take<int32_t>(Js);
     sc.block_eq = b.take<long long>(Js / 256 + 2);
+    sc.list = b.take<int32_t>(Js);
     sc.order = b.take<int32_t>(Js);
     sc.start = b.take<int32_t>((size_t)Hmax + 1);
     sc.cursor = b.take<int32_t>((size_t)Hmax + 1);
@@ -350,6 +354,7 @@ int check_device_errors(slaq_handle* h) {
         if (word & kErrSegment) what += " a candidate segment outside its row;";
         if (word & kErrBin) what += " a histogram bin out of range;";
         if (word & kErrJob) what += " a job id out of range;";
+        if (word & kErrBarrier) what += " the blocks of the selection launch did not all arrive in time;";
         if (word & kErrInput) what += " slaq_append_losses_device was given an id out of range, a job without losses, a value that is not finite or a core count below 1 (those entries were skipped);";
         cudaMemsetAsync(h->err_word, 0, sizeof word, h->stream);   // reported once: the next epoch starts clean
         return fail(h, SLAQ_E_CUDA, what);
@@ -387,6 +392,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     cudaDeviceProp prop;
     CK(cudaGetDeviceProperties(&prop, h->device), "cudaGetDeviceProperties");
     h->sm_count = prop.multiProcessorCount;
+    if (select_setup(&h->select_blocks_per_sm)) return fail(h, SLAQ_E_CUDA, "selection kernel setup failed");
     const size_t need = layout(nullptr, nullptr, max_jobs, max_hist, cap);
     if (ws) {
         if (bytes < need) return fail(h, SLAQ_E_NOMEM, "workspace smaller than slaq_workspace_bytes()");
@@ -408,7 +414,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     h->in_packed.assign((size_t)max_jobs, 0);
     h->hinted.assign((size_t)max_jobs, 0);
     for (auto& ev : h->ev) CK(cudaEventCreate(&ev), "cudaEventCreate");
-    CK(cudaMemsetAsync(h->scratch.hist, 0, h->scratch.zero_bytes, h->stream), "clear scratch");
+    CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, h->stream), "clear scratch");
     CK(cudaMemsetAsync(h->err_word, 0, 16, h->stream), "clear error word");
     const int threads = 256;
     init_jobs_kernel<<<(max_jobs + threads - 1) / threads, threads, 0, h->stream>>>(
@@ -576,9 +582,10 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
     return SLAQ_OK;
 }
 
-// Without a gain table: only the plain prediction (no envelope, no target-loss hints) has its gains in closed form.
-bool epoch_is_table_free(const slaq_handle* h, bool only_allocate) {
-    return !only_allocate && h->selection == 1 && !h->gain_envelope && h->n_hinted == 0;
+// The plain prediction happens inside the selection launch; its options (concave envelope, target-loss hints) need
+// whole rows, which the gain kernel writes first.
+bool gains_in_selection(const slaq_handle* h, bool only_allocate) {
+    return !only_allocate && !h->gain_envelope && h->n_hinted == 0;
 }
 
 // The launches of one epoch, put on h->stream in order.  Returns the number of kernels or -1.
@@ -589,21 +596,19 @@ int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32
     cudaStream_t st = h->stream;
     int launches = 0, k;
     if (with_events && cudaEventRecord(h->ev[0], st) != cudaSuccess) return -1;
-    if (cudaMemsetAsync(h->scratch.hist, 0, h->scratch.zero_bytes, st) != cudaSuccess) return -1;
+    if (cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st) != cudaSuccess) return -1;
     if (!only_allocate) {
         if ((k = launch_fit(h)) < 0) return -1;
         launches += k;
     }
     if (with_events && cudaEventRecord(h->ev[1], st) != cudaSuccess) return -1;
-    const bool table_free = epoch_is_table_free(h, only_allocate);
-    if (!only_allocate && !table_free) {
+    const bool from_curves = gains_in_selection(h, only_allocate);
+    if (!only_allocate && !from_curves) {
         if ((k = launch_gain(h, T, floor_units + 1)) < 0) return -1;
         launches += k;
     }
     if (with_events && cudaEventRecord(h->ev[2], st) != cudaSuccess) return -1;
-    if (table_free) k = launch_allocate_free(h, T, want, floor_units + 1, d_out);
-    else k = launch_allocate(h, want, floor_units + 1, !only_allocate, d_out);
-    if (k < 0) return -1;
+    if ((k = launch_select(h, T, want, floor_units + 1, from_curves, d_out)) < 0) return -1;
     launches += k;
     if (with_events && cudaEventRecord(h->ev[3], st) != cudaSuccess) return -1;
     return launches;
@@ -618,7 +623,7 @@ std::vector<long long> epoch_key(const slaq_handle* h, double T, int64_t want, i
     std::memcpy(&g_bits, &h->gamma, sizeof g_bits);
     return {t_bits, (long long)want, floor_units, (long long)(uintptr_t)d_out, only_allocate ? 1 : 0, h->n_active,
             h->max_cores, h->lm_trials, h->min_fit_points, h->warm_start ? 1 : 0, (long long)h->fit_slice_bytes,
-            (long long)h->fit_cluster_jobs, g_bits, h->gain_envelope ? 1 : 0, h->selection, h->n_hinted,
+            (long long)h->fit_cluster_jobs, g_bits, h->gain_envelope ? 1 : 0, h->n_hinted,
             (long long)(uintptr_t)h->job.packed_lo, (long long)(uintptr_t)h->job.packed_hi};
 }
 
@@ -695,10 +700,11 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     }
     h->have_epoch = true;
     h->last_launches = launches;
+    h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
     h->last_cores = usable;
-    // whether h->gain holds this epoch's rows (plain launches and a replayed graph alike), and what a later
+    // whether h->gain holds this epoch's whole rows (plain launches and a replayed graph alike), and what a later
     // request for them has to be predicted for
-    h->gain_table_current = !epoch_is_table_free(h, only_allocate);
+    h->gain_table_current = !gains_in_selection(h, only_allocate) || select_writes_whole_table(h, want);
     h->last_T = T;
     h->last_first_unit = floor_units + 1;
     if (active > 0 && C < active) return SLAQ_W_OVERSUBSCRIBED;
@@ -991,7 +997,8 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     int launches = 0, k;
     h->shard_first_unit = with_floor ? 2 : 1;
     h->last_epoch_was_graph = false;
-    CK(cudaMemsetAsync(h->scratch.hist, 0, h->scratch.zero_bytes, st), "clear scratch");
+    CK(cudaMemsetAsync(h->scratch.hist, 0, sizeof(unsigned long long) * kRadixPasses * kRadixBins, st), "clear scratch");
+    CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
     CK(cudaEventRecord(h->ev[0], st), "event");
     if ((k = launch_fit(h)) < 0) return SLAQ_E_CUDA;
     launches += k;
@@ -1001,7 +1008,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     CK(cudaEventRecord(h->ev[2], st), "event");
     CK(cudaEventRecord(h->ev[3], st), "event");
     h->have_epoch = true;
-    h->last_launches = launches;
+    h->last_launches = h->last_steps = launches;
     h->gain_table_current = true;
     h->last_T = epoch_seconds;
     h->last_first_unit = h->shard_first_unit;
@@ -1025,7 +1032,7 @@ int slaq_shard_pick(slaq_t* h, int32_t pass, int64_t want) {
     if (pass < 0 || pass >= kRadixPasses) return fail(h, SLAQ_E_ARG, "pass outside 0..5");
     const int k = launch_shard_pick(h, pass, want);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     return SLAQ_OK;
 }
 
@@ -1034,7 +1041,7 @@ int slaq_shard_pass(slaq_t* h, int32_t pass) {
     if (pass < 1 || pass >= kRadixPasses) return fail(h, SLAQ_E_ARG, "pass outside 1..5");
     const int k = launch_shard_pass(h, pass, h->shard_first_unit);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     return SLAQ_OK;
 }
 
@@ -1043,7 +1050,7 @@ int slaq_shard_count(slaq_t* h, int64_t* out_local_ties) {
     const long long* d_total = nullptr;
     const int k = launch_shard_count(h, h->shard_first_unit, &d_total);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     long long total = 0;
     CK(cudaMemcpyAsync(&total, d_total, sizeof total, cudaMemcpyDeviceToHost, h->stream), "read tie count");
     CK(cudaStreamSynchronize(h->stream), "read tie count");
@@ -1056,7 +1063,7 @@ int slaq_shard_count_device(slaq_t* h, int64_t* d_out_local_ties) {
     const long long* d_total = nullptr;
     const int k = launch_shard_count(h, h->shard_first_unit, &d_total);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     CK(cudaMemcpyAsync(d_out_local_ties, d_total, sizeof(long long), cudaMemcpyDeviceToDevice, h->stream), "export tie count");
     return SLAQ_OK;
 }
@@ -1066,7 +1073,7 @@ int slaq_shard_finalise_device(slaq_t* h, const int64_t* d_ties_before, int32_t*
     if (!out_alloc || !d_ties_before) return fail(h, SLAQ_E_ARG, "out_alloc or d_ties_before is null");
     const int k = launch_shard_finalise(h, h->shard_first_unit, 0, reinterpret_cast<const long long*>(d_ties_before), nullptr);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
        "copy allocation");
@@ -1079,7 +1086,7 @@ int slaq_shard_finalise(slaq_t* h, int64_t ties_before, int32_t* out_alloc) {
     if (ties_before < 0) return fail(h, SLAQ_E_ARG, "ties_before must not be negative");
     const int k = launch_shard_finalise(h, h->shard_first_unit, ties_before, nullptr, nullptr);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k;
+    h->last_launches += k, h->last_steps += k;
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
        "copy allocation");
@@ -1092,7 +1099,7 @@ int slaq_get_predictions(slaq_t* h, double* out_reduction, double* out_gain, int
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     const size_t J = (size_t)h->max_jobs;
     int rc = 0;
-    if (out_gain && !h->gain_table_current) {   // the last epoch ran without a table: write the rows now
+    if (out_gain && !h->gain_table_current) {   // the last epoch predicted rows only as far as it needed: write them now
         if (launch_gain(h, h->last_T, h->last_first_unit) < 0) return SLAQ_E_CUDA;
         h->gain_table_current = true;
     }
@@ -1450,7 +1457,8 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
         CK(cudaEventElapsedTime(&out->ms_gain, h->ev[1], h->ev[2]), "event time");
         CK(cudaEventElapsedTime(&out->ms_alloc, h->ev[2], h->ev[3]), "event time");
     }
-    out->launches = h->last_launches;
+    out->launches = h->last_steps;
+    out->kernel_launches = h->last_launches;
     out->active_jobs = h->n_active;
     out->points = counters[0];
     out->model_sweeps = counters[1];

@@ -74,10 +74,27 @@ struct SelectState {
     int done;                        // nothing is wanted: the threshold lies above every gain
 };
 
-// Scratch of one epoch; [hist, hist + zero_bytes) is cleared at the start of every epoch.
+constexpr int kSelectFineBins = 4096;
+constexpr int kSelectMaxGrid = 4096;
+
+// Global memory of the selection launch.  The leading part is cleared before every launch.
+struct SelectGlobal {
+    unsigned long long coarse[32];                        // first histogram: one total per power of two ..
+    unsigned long long fine[kSelectFineBins];             // .. and its 128 bins each
+    unsigned int barrier, ticket, n_list, pad;            // blocks that arrived; blocks that finished; listed rows
+    static constexpr size_t kZeroBytes = sizeof(unsigned long long) * (32 + kSelectFineBins) + 16;
+    unsigned long long narrow[kRadixPasses][kRadixBins];  // cleared by the kernel itself
+    long long block_eq[kSelectMaxGrid];                   // per block: candidates that equal the threshold
+};
+
+// Scratch of one epoch.  [zero, zero + zero_bytes) is cleared at the start of every epoch; the sharded steps
+// clear their histograms `hist` as well.
 struct Scratch {
-    unsigned long long* hist;        // [kRadixPasses][kRadixBins]
-    unsigned int* ticket;            // [kTickets]: block-completion counter per radix pass, work queue per fit class
+    unsigned long long* hist;        // [kRadixPasses][kRadixBins], sharded steps
+    void* zero;
+    SelectGlobal* select;            // its leading part is the end of the cleared region
+    int32_t* list;                   // [max_jobs] rows with candidates
+    unsigned int* ticket;            // [kTickets]: work queue of the fit
     SelectState* sel;
     long long* counters;             // [16] statistics accumulated by kernels
     size_t zero_bytes;
@@ -110,8 +127,8 @@ struct slaq_handle {
     int32_t lm_trials = 20, min_fit_points = 4;
     size_t fit_slice_bytes = 13824;       // shared memory one warp of the fit kernel may use (parked sums, up to 52 rows of 32 points, a spare row)
     bool warm_start = false;              // fits start from the last epoch's parameters where there are some
-    int selection = 0;                    // 0: selection over the written gain table, 1: gains evaluated on demand, no table
-    bool gain_table_current = false;      // h->gain holds the rows of the last epoch
+    int selection = 0;                    // SLAQ_P_SELECTION: kept for callers that ask, the launches are the same
+    bool gain_table_current = false;      // h->gain holds the whole rows of the last epoch
     double last_T = 0.0;                  // what the last epoch's gains were predicted for
     int last_first_unit = 2;
     std::vector<uint8_t> hinted;          // host mirror: job has a target-loss hint
@@ -139,7 +156,9 @@ struct slaq_handle {
     int32_t* err_word = nullptr;      // device error flags set by kernels
     cudaEvent_t ev[4] = {};
     bool have_epoch = false;
-    int32_t last_launches = 0;
+    int32_t last_launches = 0;            // kernels the last call launched
+    int32_t last_steps = 0;               // its steps, as slaq_stats counts them
+    int select_blocks_per_sm = 1;         // resident blocks of the selection kernel
     int64_t last_cores = 0;
     int sm_count = 148;
     std::vector<uint8_t> active;      // host mirror: job has at least one loss
@@ -165,8 +184,9 @@ namespace slaq {
 // kernel launchers: each returns the number of kernels it launched, or -1 after setting h->err
 int launch_fit(slaq_handle* h);
 int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit);
-int launch_allocate(slaq_handle* h, long long want, int first_unit, bool hist0_ready, int32_t* d_out_alloc);
-int launch_allocate_free(slaq_handle* h, double epoch_seconds, long long want, int first_unit, int32_t* d_out_alloc);
+int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc);
+bool select_writes_whole_table(const slaq_handle* h, long long want);
+int select_setup(int* blocks_per_sm);   // once per device before the first selection launch; 0 or -1
 int launch_normalise_export(slaq_handle* h, int32_t n, const int64_t* d_offsets, double* d_changes,
                             double* d_levels, double* d_largest);
 int launch_time_model(slaq_handle* h, double* d_s, double* d_w);

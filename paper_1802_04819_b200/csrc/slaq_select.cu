@@ -1,0 +1,824 @@
+// From fitted curves (or a table of gains) to the allocation in one cooperative launch.
+//
+// The paper starts every job at one core and then gives one core at a time to the job whose next core has the
+// largest predicted gain ("Scheduling Based on Quality Improvements").  Gain rows are non-increasing in n, so that
+// loop hands out exactly the `want` largest gains beyond the floor, and among equal gains it serves (job id
+// ascending, n ascending).  The 64-bit patterns of the gains (all >= +0) order like their values, and the threshold
+// is searched on them:
+//
+//   A  every block predicts (or reads) the gains of its own contiguous range of jobs and counts them in a histogram
+//      of 4096 bins: 128 per power of two from 2^-31 to 2, what lies below in bin 0, above in the last one.
+//      -- one grid barrier --
+//      Every block finds the bin of the want-th largest gain: the interval [lo, hi) the threshold lies in.
+//   B  every thread walks a row from its first core: gains >= hi are handed out, the row's gains inside [lo, hi) are
+//      its candidates.  A row without candidates is finished here.
+//   C  the last block to arrive ranks the candidates (normally a few hundred at most: a bin is 0.8 % wide) by (gain
+//      descending, job id, n) and completes their rows.  Only when there are more than kFinal of them do all blocks stay
+//      and narrow the interval by another 2048 bins at a time first; candidates that are all equal are handed out
+//      in job order with a prefix sum over the blocks.
+//
+// What bounds it: for up to a few thousand jobs the latency of its steps.  It replaces eleven launches (gain kernel,
+// six digits of a radix select over the whole table, counts, prefix sum, allocation) that took 90 to 110 us at every
+// size up to 33,000 jobs.
+//
+// How much of a row is looked at.  Jobs get few cores on average, so of a large table only the first `depth` cores
+// of each row enter the histogram; their bin bounds the threshold from below, and only the rows whose last gain
+// still reaches that bound are continued (once, until they fall below it) before the interval is taken again.  Gains
+// behind a row's first gain below the bound are below it too and can never be handed out.
+#include <math_constants.h>
+
+#include <algorithm>
+
+#include "slaq_gain_curve.cuh"
+#include "slaq_internal.cuh"
+
+namespace slaq {
+
+namespace {
+
+using namespace gaincurve;
+using u64 = unsigned long long;
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kSubBits = 7;                          // bins per power of two: 128
+constexpr int kFine = kSelectFineBins;               // 32 powers of two
+constexpr long long kBinBase = (long long)(1023 - 31) << kSubBits;
+constexpr int kBinShift = 52 - kSubBits;
+constexpr int kNarrowBins = kRadixBins;              // a narrowing step divides the interval by this
+constexpr int kFinal = 1024;                         // candidates one block ranks
+constexpr int kRankDirect = 256;                     // ranked against each other; more are narrowed in the block first
+constexpr u64 kTopKey = 1ull << 63;                  // above every key
+constexpr int kSpinLimit = 1 << 22;                  // polls of a barrier before it gives up (seconds)
+
+__device__ __forceinline__ int fine_bin(u64 key) {
+    const long long v = (long long)(key >> kBinShift) - kBinBase;
+    return v < 0 ? 0 : (v > kFine - 1 ? kFine - 1 : (int)v);
+}
+__device__ __forceinline__ u64 bin_edge(int b) {     // smallest key of bin b; b = kFine: above every key
+    return b <= 0 ? 0ull : (b >= kFine ? kTopKey : (u64)(b + kBinBase) << kBinShift);
+}
+__device__ __forceinline__ u64 key_of(double g) { return (u64)__double_as_longlong(g); }
+
+// The interval the threshold lies in, the same in every block.
+struct Interval {
+    u64 lo, hi;      // keys >= hi are handed out, [lo, hi) are candidates
+    u64 want;        // candidates still to hand out
+    u64 n;           // candidates in all rows
+};
+
+struct Shared {
+    union {
+        unsigned int hist[kFine];
+        struct {
+            u64 key[kFinal], pos[kFinal];
+        } cand;
+    };
+    unsigned int narrow[kNarrowBins];
+    unsigned short own[kFinal], idx[kFinal];
+    int take[kFinal];
+    Interval iv;
+    u64 scan[kWarps + 1];
+    int count, n_more, flag;
+};
+
+// Every block arrives; returns false (in every thread) if the others did not within the limit.
+__device__ bool grid_barrier(unsigned int* bar, unsigned int target, int* flag, int32_t* err_word) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int polls = 0;
+        unsigned int seen;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+        } while (seen < target && ++polls < kSpinLimit);
+        *flag = seen >= target;
+        if (seen < target && err_word) atomicOr(err_word, kErrBarrier);
+        __threadfence();
+    }
+    __syncthreads();
+    return *flag != 0;
+}
+
+__device__ __forceinline__ u64 warp_inclusive(u64 v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u64 up = __shfl_up_sync(kFull, v, o);
+        if (lane >= o) v += up;
+    }
+    return v;
+}
+
+// Exclusive prefix over the block's threads; every thread gets its own and *total.
+__device__ u64 block_exclusive(u64 v, Shared& sh, u64* total) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const u64 incl = warp_inclusive(v);
+    if (lane == 31) sh.scan[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const u64 w = lane < kWarps ? sh.scan[lane] : 0;
+        const u64 s = warp_inclusive(w);
+        if (lane < kWarps) sh.scan[lane] = s - w;
+        if (lane == kWarps - 1) sh.scan[kWarps] = s;
+    }
+    __syncthreads();
+    *total = sh.scan[kWarps];
+    const u64 out = sh.scan[warp] + incl - v;
+    __syncthreads();
+    return out;
+}
+
+// Warp 0: the bin of the want-th largest gain from the global histogram (octave totals first, then the 128 bins of one
+// octave).  Fewer gains than wanted: an interval below everything counted, n = 0.
+__device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
+    const int lane = threadIdx.x & 31;
+    const u64 c = __ldcg(&gl->coarse[31 - lane]);
+    const u64 incl = warp_inclusive(c);
+    const unsigned hit = __ballot_sync(kFull, incl >= want);
+    if (!hit) {
+        if (lane == 0) *iv = Interval{0, 0, want, 0};
+        return;
+    }
+    const int at = __ffs(hit) - 1;
+    const u64 above = __shfl_sync(kFull, incl - c, at);
+    const int top = (31 - at) * 128 + 127 - 4 * lane;
+    u64 v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]);
+    const u64 incl2 = warp_inclusive(sum);
+    const int at2 = __ffs(__ballot_sync(kFull, above + incl2 >= want)) - 1;
+    if (lane == at2) {
+        u64 run = above + incl2 - sum;
+        int k = 0;
+        while (k < 3 && run + v[k] < want) run += v[k++];
+        *iv = Interval{bin_edge(top - k), bin_edge(top - k + 1), want - run, v[k]};
+    }
+}
+
+__device__ __forceinline__ int narrow_shift(const Interval& iv) {
+    const u64 width = iv.hi - iv.lo;
+    const int bits = 64 - __clzll((long long)(width - 1));
+    return bits > kRadixBits ? bits - kRadixBits : 0;
+}
+
+// The bin of a narrowing step's histogram (counts(b), b = 0..2047) that holds the iv.want-th largest candidate.
+template <class Counts>
+__device__ void pick_narrow(Counts counts, Shared& sh) {
+    constexpr int per = kNarrowBins / kThreads;
+    const Interval iv = sh.iv;
+    const int shift = narrow_shift(iv);
+    u64 v[per], sum = 0;
+#pragma unroll
+    for (int k = 0; k < per; ++k) sum += v[k] = counts(kNarrowBins - 1 - ((int)threadIdx.x * per + k));
+    u64 total;
+    u64 run = block_exclusive(sum, sh, &total);
+    if (run < iv.want && iv.want <= run + sum) {
+        int k = 0;
+        while (k < per - 1 && run + v[k] < iv.want) run += v[k++];
+        const int b = kNarrowBins - 1 - ((int)threadIdx.x * per + k);
+        const u64 lo = iv.lo + ((u64)b << shift);
+        sh.iv = Interval{lo, min(lo + (1ull << shift), iv.hi), iv.want - run, v[k]};
+    }
+    __syncthreads();
+}
+
+// Adds a block's shared counts to the global ones.
+__device__ void flush_first(Shared& sh, SelectGlobal* gl) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int o = warp; o < 32; o += kWarps) {
+        unsigned int sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned int v = sh.hist[o * 128 + k * 32 + lane];
+            if (v) atomicAdd(&gl->fine[o * 128 + k * 32 + lane], (u64)v);
+            sum += v;
+        }
+        sum = __reduce_add_sync(kFull, sum);
+        if (lane == 0 && sum) atomicAdd(&gl->coarse[o], (u64)sum);
+    }
+}
+
+// One row's share of the histogram: gains that fall into bin 0 (zero, or below 2^-31) are counted in a register.
+__device__ __forceinline__ void count_gain(double g, bool counted, Shared& sh, unsigned int& low, int32_t* err_word) {
+    if (!counted) return;
+    const int b = fine_bin(key_of(g));
+    if (b == 0) ++low;
+    else if (index_ok(b, kFine, kErrBin, err_word)) atomicAdd(&sh.hist[b], 1u);
+}
+
+// A tile's curves in shared memory, one column per row.
+struct CurveTile {
+    double* v;       // [7][kThreads]
+    int* kind;       // [kThreads]; -1: inactive
+    __device__ void put(int r, const Curve& c, bool active) {
+        v[0 * kThreads + r] = c.p0;
+        v[1 * kThreads + r] = c.p1;
+        v[2 * kThreads + r] = c.p2;
+        v[3 * kThreads + r] = c.inv_span;
+        v[4 * kThreads + r] = c.s;
+        v[5 * kThreads + r] = c.w;
+        v[6 * kThreads + r] = c.step_scale;
+        kind[r] = active ? c.kind : -1;
+    }
+    __device__ Curve get(int r, double T) const {
+        Curve c;
+        c.kind = kind[r];
+        c.p0 = v[0 * kThreads + r];
+        c.p1 = v[1 * kThreads + r];
+        c.p2 = v[2 * kThreads + r];
+        c.inv_span = v[3 * kThreads + r];
+        c.s = v[4 * kThreads + r];
+        c.w = v[5 * kThreads + r];
+        c.step_scale = v[6 * kThreads + r];
+        c.T = T;
+        return c;
+    }
+};
+
+// Running minimum over the W lanes of a row (W a power of two, lanes aligned), continuing `carry`.  Most rows fall
+// already, which one look at the left neighbour shows.
+__device__ __forceinline__ double running_min(double g, double carry, int w, int W) {
+    double left = __shfl_up_sync(kFull, g, 1, W);
+    if (w == 0) left = carry;
+    if (__any_sync(kFull, g > left)) {
+        for (int o = 1; o < W; o <<= 1) {
+            const double up = __shfl_up_sync(kFull, g, o, W);
+            if (w >= o) g = fmin(g, up);
+        }
+        g = fmin(g, carry);
+    }
+    return g;
+}
+
+}  // namespace
+
+struct SelectArgs {
+    JobArrays job;
+    FitArrays fit;
+    const int32_t* count;    // active rows (count > 0); null: every row is active
+    double* gain;            // [J][cap]
+    int J, cap, first_unit;
+    int depth;               // cores per row that enter the first histogram
+    int W;                   // lanes per row (power of two)
+    int rows;                // rows per block
+    int stride;              // resident rows in shared memory: entries per row (0: rows stay in global memory)
+    double T;
+    long long want;
+    SelectGlobal* gl;
+    SelectState* sel;
+    long long* counters;
+    int32_t *gt, *eq, *list;
+    int32_t *alloc, *last_alloc, *out_alloc;
+    double* reduction;
+    int32_t* err_word;
+};
+
+namespace {
+
+__device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int cores, double R, bool active) {
+    a.alloc[j] = cores;
+    if (a.out_alloc) a.out_alloc[j] = cores;
+    if (active && a.last_alloc) a.last_alloc[j] = cores;
+    a.reduction[j] = R;
+}
+
+// The last block: hand out `iv.want` of the n <= kFinal candidates, best first, and complete their rows.
+__device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
+    const int tid = threadIdx.x;
+    const int rows = min((int)__ldcg(&a.gl->n_list), kFinal);
+    if (tid == 0) sh.count = 0;
+    __syncthreads();
+    for (int r = tid; r < rows; r += kThreads) {
+        const int j = __ldcg(&a.list[r]);
+        const int s = __ldcg(&a.gt[j]), c = __ldcg(&a.eq[j]);
+        sh.take[r] = 0;
+        const int off = atomicAdd(&sh.count, c);
+        for (int i = 0; i < c && off + i < kFinal; ++i) {
+            sh.cand.key[off + i] = key_of(__ldcg(&a.gain[(size_t)j * a.cap + s + i]));
+            sh.cand.pos[off + i] = ((u64)j << 10) | (u64)(s + i);
+            sh.own[off + i] = (unsigned short)r;
+            sh.idx[off + i] = (unsigned short)(off + i);
+        }
+    }
+    __syncthreads();
+    int n = min(sh.count, kFinal);
+    __syncthreads();
+    while (n > kRankDirect && sh.iv.hi - sh.iv.lo > 1) {
+        const int shift = narrow_shift(sh.iv);
+        const u64 lo = sh.iv.lo;
+        for (int b = tid; b < kNarrowBins; b += kThreads) sh.narrow[b] = 0;
+        if (tid == 0) sh.count = 0;
+        __syncthreads();
+        int mine[kFinal / kThreads];
+        int m = 0;
+        for (int i = tid; i < n; i += kThreads) {
+            mine[m++] = sh.idx[i];
+            atomicAdd(&sh.narrow[(sh.cand.key[sh.idx[i]] - lo) >> shift], 1u);
+        }
+        __syncthreads();
+        pick_narrow([&](int b) { return (u64)sh.narrow[b]; }, sh);
+        const u64 lo2 = sh.iv.lo, hi2 = sh.iv.hi;
+        for (int i = 0; i < m; ++i) {
+            const u64 key = sh.cand.key[mine[i]];
+            if (key >= hi2) atomicAdd(&sh.take[sh.own[mine[i]]], 1);
+            else if (key >= lo2) sh.idx[atomicAdd(&sh.count, 1)] = (unsigned short)mine[i];
+        }
+        __syncthreads();
+        n = sh.count;
+        __syncthreads();
+    }
+    // what is left is ranked outright
+    const u64 want = sh.iv.want;
+    if (tid == 0) sh.scan[0] = 0, sh.count = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += kThreads) {
+        const int e = sh.idx[i];
+        const u64 key = sh.cand.key[e], pos = sh.cand.pos[e];
+        u64 rank = 0;
+        for (int k = 0; k < n; ++k) {
+            const int f = sh.idx[k];
+            const u64 other = sh.cand.key[f];
+            rank += (other > key || (other == key && sh.cand.pos[f] < pos)) ? 1 : 0;
+        }
+        if (rank < want) atomicAdd(&sh.take[sh.own[e]], 1);
+        if (rank + 1 == want) sh.scan[0] = key;
+    }
+    __syncthreads();
+    const u64 tau = sh.scan[0];
+    int above = 0;   // all of them are taken; what is left of `want` goes to gains equal to tau
+    for (int i = tid; i < n; i += kThreads) above += sh.cand.key[sh.idx[i]] > tau ? 1 : 0;
+    if (above) atomicAdd(&sh.count, above);
+    __syncthreads();
+    if (tid == 0) {
+        a.sel->prefix = tau;
+        a.counters[7] = (long long)want - sh.count;
+    }
+    long long handed = 0;
+    for (int r = tid; r < rows; r += kThreads) {
+        const int j = __ldcg(&a.list[r]), s = __ldcg(&a.gt[j]), t = sh.take[r];
+        double R = __ldcg(&a.reduction[j]);
+        for (int i = 0; i < t; ++i) R += __ldcg(&a.gain[(size_t)j * a.cap + s + i]);
+        store_alloc(a, j, s + t, R, true);
+        handed += s + t;
+    }
+    if (handed) atomicAdd((u64*)&a.counters[6], (u64)handed);
+}
+
+// All blocks: narrow the interval over the rows' candidate segments (gt, eq) until kFinal candidates are left or all
+// are equal; equal ones are handed out here.  Returns whether the last block still has candidates to rank.
+__device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j1, unsigned int& arrived) {
+    const int tid = threadIdx.x;
+    for (int step = 0; sh.iv.hi - sh.iv.lo > 1 && sh.iv.n > kFinal && step < kRadixPasses; ++step) {
+        const int shift = narrow_shift(sh.iv);
+        const u64 lo = sh.iv.lo;
+        u64* global = a.gl->narrow[step];
+        for (int b = tid; b < kNarrowBins; b += kThreads) sh.narrow[b] = 0;
+        __syncthreads();
+        for (int j = j0 + tid; j < j1; j += kThreads) {
+            const int c = a.eq[j];
+            const double* row = a.gain + (size_t)j * a.cap + a.gt[j];
+            for (int i = 0; i < c; ++i) {
+                const u64 b = (key_of(__ldcg(row + i)) - lo) >> shift;
+                if (index_ok((long long)b, kNarrowBins, kErrBin, a.err_word)) atomicAdd(&sh.narrow[b], 1u);
+            }
+        }
+        __syncthreads();
+        for (int b = tid; b < kNarrowBins; b += kThreads)
+            if (sh.narrow[b]) atomicAdd(&global[b], (u64)sh.narrow[b]);
+        arrived += gridDim.x;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+        pick_narrow([&](int b) { return __ldcg(&global[b]); }, sh);
+        const u64 lo2 = sh.iv.lo, hi2 = sh.iv.hi;
+        for (int j = j0 + tid; j < j1; j += kThreads) {
+            const int c = a.eq[j], s = a.gt[j];
+            if (!c) continue;
+            const double* row = a.gain + (size_t)j * a.cap;
+            double R = a.reduction[j];
+            int i = s;
+            const int end = s + c;
+            while (i < end && key_of(__ldcg(row + i)) >= hi2) R += __ldcg(row + i++);
+            int left = 0;
+            while (i + left < end && key_of(__ldcg(row + i + left)) >= lo2) ++left;
+            a.gt[j] = i;
+            a.eq[j] = left;
+            a.reduction[j] = R;
+        }
+        __syncthreads();
+    }
+    const bool equal = sh.iv.n > kFinal;   // and the interval holds one key only
+    // rows in job order: the candidates before a row decide what it gets if all are equal, its list place otherwise
+    long long mine = 0;
+    for (int j = j0 + tid; j < j1; j += kThreads) mine += a.eq[j];
+    u64 total;
+    block_exclusive((u64)mine, sh, &total);
+    u64 before = 0;
+    if (equal) {
+        if (tid == 0) a.gl->block_eq[blockIdx.x] = (long long)total;
+        arrived += gridDim.x;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+        u64 part = 0;
+        for (int b = tid; b < (int)blockIdx.x; b += kThreads) part += (u64)__ldcg(&a.gl->block_eq[b]);
+        block_exclusive(part, sh, &before);
+    }
+    long long handed = 0, ties = 0;
+    for (int base = j0; base < j1; base += kThreads) {
+        const int j = base + tid;
+        const int c = j < j1 ? a.eq[j] : 0;
+        u64 tile;
+        const u64 ahead = before + block_exclusive((u64)c, sh, &tile);
+        before += tile;
+        if (j >= j1 || (a.count && a.count[j] <= 0)) continue;
+        const int s = a.gt[j];
+        if (!equal && c) {
+            a.list[atomicAdd(&a.gl->n_list, 1u)] = j;
+            continue;
+        }
+        const int take = ahead >= sh.iv.want ? 0 : (int)min((u64)c, sh.iv.want - ahead);
+        double R = a.reduction[j];
+        for (int i = 0; i < take; ++i) R += a.gain[(size_t)j * a.cap + s + i];
+        store_alloc(a, j, s + take, R, true);
+        handed += s + take;
+        ties += take;
+    }
+    u64 sum;
+    block_exclusive((u64)handed, sh, &sum);
+    if (tid == 0 && sum) atomicAdd((u64*)&a.counters[6], sum);
+    if (equal) {
+        block_exclusive((u64)ties, sh, &sum);
+        if (tid == 0 && sum) atomicAdd((u64*)&a.counters[7], sum);
+        if (tid == 0 && blockIdx.x == 0) a.sel->prefix = sh.iv.lo;
+    }
+    return !equal;
+}
+
+// kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
+// were continued); otherwise the table is read.
+template <bool kCurves>
+__global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_constant__ SelectArgs a) {
+    extern __shared__ double dyn[];
+    __shared__ Shared sh;
+    const int tid = threadIdx.x;
+    const int j0 = min((int)blockIdx.x * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
+    const bool resident = a.stride > 0;
+    CurveTile tile;
+    tile.v = dyn;
+    tile.kind = reinterpret_cast<int*>(dyn + 7 * kThreads);
+    double* const rows_sh = dyn + (kCurves ? 7 * kThreads + kThreads / 2 : 0);
+    unsigned int arrived = 0;
+
+    for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
+    // the narrowing histograms, should they be needed: cleared by all blocks before the first barrier
+    for (int i = blockIdx.x * kThreads + tid; i < kRadixPasses * kNarrowBins; i += gridDim.x * kThreads)
+        (&a.gl->narrow[0][0])[i] = 0;
+    __syncthreads();
+
+    // ---- A: the first `depth` gains of every row ----
+    unsigned int low = 0;
+    const int W = a.W, w = tid & (W - 1), groups = kThreads / W;
+    for (int base = j0; base < j1; base += kThreads) {
+        const int n_rows = min(kThreads, j1 - base);
+        if (kCurves) {
+            if (tid < n_rows) {
+                const int j = base + tid;
+                bool no_time = false;
+                const bool active = a.count[j] > 0;
+                const Curve c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
+                if (no_time) a.fit.status[j] = SLAQ_JOB_NO_TIME;
+                tile.put(tid, c, active);
+            }
+            __syncthreads();
+        }
+        for (int r0 = 0; r0 < n_rows; r0 += groups) {   // uniform trip count: the row steps use warp shuffles
+            const int r = r0 + tid / W;
+            const bool in = r < n_rows;
+            const int j = base + (in ? r : 0);
+            Curve c;
+            bool active = false;
+            if (kCurves) {
+                if (in) {
+                    c = tile.get(r, a.T);
+                    active = c.kind >= 0;
+                    if (!active) c.kind = 3;
+                }
+            } else if (in) {
+                active = !a.count || a.count[j] > 0;
+            }
+            double* const row = a.gain + (size_t)j * a.cap;
+            double carry = CUDART_INF;
+            for (int n0 = 0; n0 < a.depth; n0 += W) {
+                const int i = n0 + w;
+                const bool has = in && i < a.depth && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+                double g = 0.0;
+                if (kCurves) {
+                    if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
+                    g = running_min(has ? g : 0.0, carry, w, W);
+                    carry = __shfl_sync(kFull, g, W - 1, W);
+                    if (has) row[i] = g;
+                } else if (has) {
+                    g = row[i];
+                }
+                if (has && resident) rows_sh[(base - j0 + r) * a.stride + i] = g;
+                count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
+            }
+        }
+        __syncthreads();
+    }
+    low = __reduce_add_sync(kFull, low);
+    if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
+    __syncthreads();
+    flush_first(sh, a.gl);
+    arrived += gridDim.x;
+    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
+    if (a.want > 0) {
+        if (tid < 32) pick_first(a.gl, (u64)a.want, &sh.iv);
+    } else if (tid == 0) {
+        sh.iv = Interval{~0ull, ~0ull, 0, 0};   // nothing wanted: a threshold above every gain
+    }
+    __syncthreads();
+
+    // ---- rows that may reach the threshold beyond `depth` are continued ----
+    if (a.depth < a.cap && a.want > 0) {
+        const u64 bound = sh.iv.lo;
+        for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
+        low = 0;
+        for (int base = j0; base < j1; base += kThreads) {
+            if (tid == 0) sh.n_more = 0;
+            __syncthreads();
+            const int mine = base + tid;
+            if (mine < j1 && (!a.count || a.count[mine] > 0) &&
+                key_of(a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound)
+                sh.narrow[atomicAdd(&sh.n_more, 1)] = (unsigned int)mine;
+            __syncthreads();
+            const int n_more = sh.n_more;
+            for (int r0 = 0; r0 < n_more; r0 += groups) {
+                const int r = r0 + tid / W;
+                const bool in = r < n_more;
+                const int j = in ? (int)sh.narrow[r] : base;
+                double* const row = a.gain + (size_t)j * a.cap;
+                Curve c;
+                c.kind = 3;
+                double carry = CUDART_INF;
+                if (kCurves && in) {
+                    bool no_time = false;
+                    c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
+                    carry = row[a.depth - 1];
+                }
+                bool on = in;
+                for (int n0 = a.depth; n0 < a.cap && __any_sync(kFull, on); n0 += W) {
+                    const int i = n0 + w;
+                    const bool has = on && i < a.cap && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+                    double g = 0.0;
+                    if (kCurves) {
+                        if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
+                        g = running_min(g, carry, w, W);
+                        if (has) row[i] = g;
+                    } else if (has) {
+                        g = row[i];
+                    }
+                    count_gain(g, has && i + 1 >= a.first_unit, sh, low, a.err_word);
+                    carry = __shfl_sync(kFull, g, W - 1, W);
+                    on = on && key_of(carry) >= bound;
+                }
+            }
+            __syncthreads();
+        }
+        low = __reduce_add_sync(kFull, low);
+        if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
+        __syncthreads();
+        flush_first(sh, a.gl);
+        arrived += gridDim.x;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
+        if (tid < 32) pick_first(a.gl, (u64)a.want, &sh.iv);
+        __syncthreads();
+    }
+
+    // ---- B: every row up to the interval ----
+    const Interval iv = sh.iv;
+    const bool few = iv.n <= kFinal;
+    long long handed = 0;
+    for (int j = j0 + tid; j < j1; j += kThreads) {
+        const bool active = !a.count || a.count[j] > 0;
+        int s = 0, c = 0;
+        double R = 0.0;
+        if (active) {
+            const double* row = resident ? rows_sh + (size_t)(j - j0) * a.stride : a.gain + (size_t)j * a.cap;
+            if (a.first_unit == 2) R = row[0], s = 1;
+            while (s < a.cap) {
+                const double g = row[s];
+                if (key_of(g) < iv.hi) break;
+                R += g;
+                ++s;
+            }
+            while (s + c < a.cap && key_of(row[s + c]) >= iv.lo) ++c;
+        }
+        if (few && c == 0) {
+            store_alloc(a, j, s, R, active);
+            handed += s;
+        } else {
+            a.gt[j] = s;
+            a.eq[j] = c;
+            a.reduction[j] = R;
+            if (few) a.list[atomicAdd(&a.gl->n_list, 1u)] = j;
+            else if (!active) store_alloc(a, j, 0, 0.0, false);
+        }
+    }
+    if (few) {
+        u64 sum;
+        block_exclusive((u64)handed, sh, &sum);
+        if (tid == 0 && sum) atomicAdd((u64*)&a.counters[6], sum);
+    } else {
+        __syncthreads();
+        if (!narrow_on_the_grid(a, sh, j0, j1, arrived)) return;
+    }
+
+    // ---- C: the last block to get here ranks the candidates ----
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) sh.flag = atomicAdd(&a.gl->ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!sh.flag) return;
+    __threadfence();
+    if (sh.iv.n > 0) finish_candidates(a, sh);
+    else if (tid == 0) a.sel->prefix = ~0ull;
+}
+
+}  // namespace
+
+// Rule for the rows' home.  Up to kResidentGains gains per block (four evaluations per thread) all of them are predicted
+// at once, kept in shared memory and walked there; the whole table is written as well.  Beyond that prediction is what
+// costs (910 us for 128 gains of a million jobs each), so rows start with four times the average number of
+// cores handed out, at least 16, and only rows that need more are continued.
+constexpr int kResidentGains = 4 * kThreads;
+
+static size_t select_smem(bool curves, int rows, int stride) {
+    return sizeof(double) * ((curves ? 7 * kThreads + kThreads / 2 : 0) + (size_t)rows * stride);
+}
+
+int select_setup(int* blocks_per_sm) {
+    int per_sm = 1;
+    const size_t most = select_smem(true, kResidentGains, 2) + 1024;
+    if (cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
+    if (cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true>, kThreads, select_smem(true, 0, 0)) != cudaSuccess)
+        return -1;
+    *blocks_per_sm = per_sm < 1 ? 1 : per_sm;
+    return 0;
+}
+
+// Cores per row that enter the first histogram.
+static int select_depth(int J, int cap, long long want, int sm_count) {
+    if ((long long)J * cap <= (long long)kResidentGains * sm_count) return cap;
+    const long long average = (want + J - 1) / J + 1;
+    return (int)std::min<long long>(cap, std::max<long long>(16, (4 * average + 15) / 16 * 16));
+}
+
+// Fill the size-dependent part of the arguments and launch.
+static cudaError_t launch_select(SelectArgs& a, bool curves, int sm_count, int blocks_per_sm, cudaStream_t st) {
+    const long long gains = (long long)a.J * a.cap;
+    size_t smem;
+    int grid;
+    a.depth = select_depth(a.J, a.cap, a.want, sm_count);
+    if (gains <= (long long)kResidentGains * sm_count) {
+        a.W = 1;
+        while (a.W < 32 && a.W < a.cap) a.W <<= 1;
+        grid = (int)std::min<long long>(sm_count, std::max<long long>(1, (gains + kThreads - 1) / kThreads));
+        a.rows = (a.J + grid - 1) / grid;
+        grid = (a.J + a.rows - 1) / a.rows;
+        a.stride = a.cap | 1;   // odd: threads walking neighbouring rows meet different banks
+        smem = select_smem(curves, a.rows, a.stride);
+    } else {
+        a.W = 1;
+        while (a.W < 16 && a.W < a.cap) a.W <<= 1;
+        grid = sm_count * blocks_per_sm;
+        a.rows = (a.J + grid - 1) / grid;
+        grid = (a.J + a.rows - 1) / a.rows;
+        a.stride = 0;
+        smem = select_smem(curves, 0, 0);
+    }
+    void* args[] = {&a};
+    return cudaLaunchCooperativeKernel(curves ? (const void*)select_kernel<true> : (const void*)select_kernel<false>, dim3(grid),
+                                       dim3(kThreads), args, smem, st);
+}
+
+int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc) {
+    SelectArgs a;
+    a.job = h->job;
+    a.fit = h->fit;
+    a.count = h->job.count;
+    a.gain = h->gain;
+    a.J = h->max_jobs;
+    a.cap = h->max_cores;
+    a.first_unit = first_unit;
+    a.T = epoch_seconds;
+    a.want = want;
+    a.gl = h->scratch.select;
+    a.sel = h->scratch.sel;
+    a.counters = h->scratch.counters;
+    a.gt = h->scratch.gt;
+    a.eq = h->scratch.eq;
+    a.list = h->scratch.list;
+    a.alloc = h->alloc;
+    a.last_alloc = h->job.last_alloc;
+    a.out_alloc = d_out_alloc;
+    a.reduction = h->reduction;
+    a.err_word = h->err_word;
+    const cudaError_t e = launch_select(a, from_curves, h->sm_count, h->select_blocks_per_sm, h->stream);
+    if (e != cudaSuccess) {
+        h->err = std::string("selection launch: ") + cudaGetErrorString(e);
+        return -1;
+    }
+    return 1;
+}
+
+bool select_writes_whole_table(const slaq_handle* h, long long want) {
+    return select_depth(h->max_jobs, h->max_cores, want, h->sm_count) == h->max_cores;
+}
+
+// ---------------------------------------------------------------------------------
+// Allocation without any device allocation: the same kernel, its scratch in a static device array that ships with the
+// library image.
+// ---------------------------------------------------------------------------------
+namespace {
+
+constexpr int kStaticMaxJobs = 32768;
+
+struct StaticScratch {
+    SelectGlobal gl;                 // its leading part is cleared every call
+    SelectState sel;                 // rewritten every call
+    long long counters[16];
+    int32_t gt[kStaticMaxJobs], eq[kStaticMaxJobs], list[kStaticMaxJobs];   // written before they are read
+};
+
+static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
+
+struct StaticDevice {
+    StaticScratch* scratch;
+    int sm_count, blocks_per_sm;
+};
+
+// Device address of g_static_scratch on the current device and its launch limits, looked up once per device.
+// In host code the array's name only stands for the symbol; kernels need this address.
+int static_scratch_for_current_device(StaticDevice* out) {
+    constexpr int kMaxDevices = 64;
+    static StaticDevice cache[kMaxDevices] = {};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return SLAQ_E_CUDA;
+    StaticScratch* p = __atomic_load_n(&cache[dev].scratch, __ATOMIC_ACQUIRE);
+    if (!p) {
+        void* addr = nullptr;
+        int sm = 0, per_sm = 1;
+        if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || !addr) return SLAQ_E_CUDA;
+        if (cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SLAQ_E_CUDA;
+        if (select_setup(&per_sm)) return SLAQ_E_CUDA;
+        p = static_cast<StaticScratch*>(addr);
+        __atomic_store_n(&cache[dev].sm_count, sm, __ATOMIC_RELAXED);
+        __atomic_store_n(&cache[dev].blocks_per_sm, per_sm, __ATOMIC_RELAXED);
+        __atomic_store_n(&cache[dev].scratch, p, __ATOMIC_RELEASE);   // every thread finds the same values
+    }
+    out->scratch = p;
+    out->sm_count = __atomic_load_n(&cache[dev].sm_count, __ATOMIC_RELAXED);
+    out->blocks_per_sm = __atomic_load_n(&cache[dev].blocks_per_sm, __ATOMIC_RELAXED);
+    return SLAQ_OK;
+}
+
+}  // namespace
+
+}  // namespace slaq
+
+extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_t max_cores_per_job,
+                                    int64_t total_cores, int32_t* d_out_alloc, double* d_out_reduction,
+                                    void* cuda_stream) {
+    using namespace slaq;
+    if (!d_gain || !d_out_alloc || !d_out_reduction || n_jobs < 1 || max_cores_per_job < 1 || total_cores < 0)
+        return SLAQ_E_ARG;
+    if (n_jobs > kStaticMaxJobs || max_cores_per_job > kMaxCoresLimit) return SLAQ_E_RANGE;
+    StaticDevice dev;
+    const int rc = static_scratch_for_current_device(&dev);
+    if (rc) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    const int J = n_jobs, cap = max_cores_per_job;
+    const int floor_units = total_cores >= J ? 1 : 0;
+    const long long usable = total_cores < (long long)J * cap ? total_cores : (long long)J * cap;
+    // the array keeps the previous call's contents: clear what the kernel accumulates into
+    if (cudaMemsetAsync(&dev.scratch->gl, 0, SelectGlobal::kZeroBytes, st) != cudaSuccess) return SLAQ_E_CUDA;
+    SelectArgs a = {};
+    a.gain = const_cast<double*>(d_gain);   // only read: no gains are predicted here
+    a.J = J;
+    a.cap = cap;
+    a.first_unit = floor_units + 1;
+    a.want = usable - (long long)J * floor_units;
+    a.gl = &dev.scratch->gl;
+    a.sel = &dev.scratch->sel;
+    a.counters = dev.scratch->counters;
+    a.gt = dev.scratch->gt;
+    a.eq = dev.scratch->eq;
+    a.list = dev.scratch->list;
+    a.alloc = d_out_alloc;
+    a.reduction = d_out_reduction;
+    if (launch_select(a, false, dev.sm_count, dev.blocks_per_sm, st) != cudaSuccess) return SLAQ_E_CUDA;
+    if (total_cores < J) return SLAQ_W_OVERSUBSCRIBED;
+    if (total_cores > (long long)J * cap) return SLAQ_W_UNDERFILLED;
+    return SLAQ_OK;
+}
