@@ -82,10 +82,10 @@ enum {
                                      results agree bit for bit; 0 (default): the handle's own active jobs */
     SLAQ_P_EPOCH_GRAPH = 8,       /* 1: slaq_schedule / slaq_schedule_device replay the epoch's launches as one
                                      CUDA graph once two calls in a row had the same arguments, parameters and
-                                     number of active jobs (an epoch of a small cluster is bound by its sixteen
-                                     launches); 0: always plain launches; -1 (default): graph for handles
-                                     created for at most 20,000 jobs.  Results are the same either way.  Not
-                                     used while the handle's stream is itself being captured. */
+                                     number of active jobs; 0: always plain launches; -1 (default): what is faster,
+                                     which is plain launches at every size (an epoch is two to five of them).  Results
+                                     are the same either way.  Not used while the handle's stream is itself being
+                                     captured. */
     SLAQ_P_GAIN_ENVELOPE = 9,     /* 0 (default) or 1.  The greedy loop is exact when every job's predicted reduction
                                      R(n) is concave in its cores n, which a convex fitted curve gives.  Where a fit is
                                      not convex ahead of the newest point (the paper assumes convex losses: footnotes of

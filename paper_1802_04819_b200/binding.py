@@ -52,6 +52,17 @@ class SlaqError(RuntimeError):
 
 
 _libs = {}
+_fast = None       # the marshalling extension
+
+
+def _marshal():
+    global _fast
+    if _fast is None:
+        from .build import build_marshal
+        build_marshal()
+        from . import _marshal as mod
+        _fast = mod
+    return _fast
 
 
 def load_library(variant: str | None = None):
@@ -160,6 +171,9 @@ class Scheduler:
         self._h = c_void_p()
         self.max_jobs, self.max_hist, self.max_cores_per_job = int(max_jobs), int(max_hist), int(max_cores_per_job)
         self._workspace = workspace
+        self._calls = _marshal()
+        addr = lambda f: ctypes.cast(f, c_void_p).value   # noqa: E731
+        self._addr = (addr(self._lib.slaq_append_losses), addr(self._lib.slaq_append_losses_ex), addr(self._lib.slaq_schedule))
         if workspace is not None:
             rc = self._lib.slaq_create_in(c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size(),
                                           max_jobs, max_hist, max_cores_per_job, ctypes.byref(self._h))
@@ -210,6 +224,9 @@ class Scheduler:
         return out.value
 
     def append_losses(self, job_ids, losses, iter_times=None, cores_used=None):
+        rc = self._calls.append(self._addr[0], self._addr[1], self._h.value or 0, job_ids, losses, iter_times, cores_used)
+        if rc is not None:
+            return rc if rc >= 0 else self._check(rc)
         ids, ls = _arr(job_ids, np.int32), _arr(losses, np.float64)
         ts, cs = _arr(iter_times, np.float64), _arr(cores_used, np.int32)
         if cs is None:
@@ -245,7 +262,11 @@ class Scheduler:
     def schedule(self, epoch_seconds: float, total_cores: int, out_alloc=None):
         """Returns (alloc int32 [max_jobs], status) with status 0 or a warning code."""
         out = np.empty(self.max_jobs, np.int32) if out_alloc is None else out_alloc
-        rc = self._check(self._lib.slaq_schedule(self._h, float(epoch_seconds), int(total_cores), _ptr(out)))
+        rc = self._calls.schedule(self._addr[2], self._h.value or 0, float(epoch_seconds), int(total_cores), out, self.max_jobs)
+        if rc is None:   # not a plain int32 array: its address is taken as it is
+            rc = self._lib.slaq_schedule(self._h, float(epoch_seconds), int(total_cores), _ptr(out))
+        if rc < 0:
+            self._check(rc)
         return out, rc
 
     def schedule_device(self, epoch_seconds: float, total_cores: int, d_out_alloc=None):

@@ -3,12 +3,14 @@
 from __future__ import annotations
 
 import subprocess
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libslaq.so"
+MARSHAL = PKG / "_marshal.so"      # Python extension: argument marshalling of the loop's two calls
 SOURCES = ["slaq_api.cu", "slaq_fit.cu", "slaq_gain.cu", "slaq_alloc.cu", "slaq_select.cu"]
 
 
@@ -47,7 +49,16 @@ def is_stale(lib: Path = LIB) -> bool:
     return any(d.stat().st_mtime > built for d in deps)
 
 
+def build_marshal(force: bool = False) -> Path:
+    source = CSRC / "marshal.c"
+    if force or not MARSHAL.exists() or source.stat().st_mtime > MARSHAL.stat().st_mtime:
+        subprocess.run(["gcc", "-O2", "-Wall", "-Wextra", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
+                        "-o", str(MARSHAL), str(source)], check=True)
+    return MARSHAL
+
+
 def build(force: bool = False, verbose_ptxas: bool = False) -> Path:
+    build_marshal(force)
     if force or verbose_ptxas or is_stale():
         subprocess.run(nvcc_command(verbose_ptxas), check=True)
     return LIB

@@ -2,7 +2,10 @@
 // the scheduling epoch, and read-back of results.  The contract is in include/slaq.h.
 #include <math_constants.h>
 
+#include <immintrin.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -14,6 +17,7 @@ using namespace slaq;
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int32_t kMailAlways = 4096;   // entries of an append up to which asking where the arrays live costs more than it gives
 constexpr int32_t kEpochSteps = 15, kAllocateSteps = 11;   // slaq_stats.launches
 
 struct Bump {
@@ -75,7 +79,6 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     sc.gt = b.take<int32_t>(Js);
     sc.eq = b.take<int32_t>(Js);
     sc.block_eq = b.take<long long>(Js / 256 + 2);
-    sc.list = b.take<int32_t>(Js);
     sc.order = b.take<int32_t>(Js);
     sc.start = b.take<int32_t>((size_t)Hmax + 1);
     sc.cursor = b.take<int32_t>((size_t)Hmax + 1);
@@ -91,6 +94,8 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     int32_t* alloc = b.take<int32_t>(Js);
     double* reduction = b.take<double>(Js);
     int32_t* err_word = b.take<int32_t>(4);
+    sc.append_ticket = reinterpret_cast<unsigned int*>(err_word ? err_word + 2 : nullptr);
+    sc.published = b.take<long long>(16);
     job.max_jobs = J;
     job.ring_lo = ring;
     job.ring_hi = ring ? ring + Js * Hmax : nullptr;
@@ -165,28 +170,49 @@ __global__ void init_jobs_kernel(JobArrays job, FitArrays fit, double* ring, int
 // checked: the arrays come straight from the caller's device memory, unseen by the host - an id out of range,
 // a job without any loss yet, a loss or time that is not finite or a core count below 1 sets kErrInput and
 // that entry is skipped.
-__global__ void append_kernel(JobArrays job, FitArrays fit, int max_jobs, int n, const int32_t* ids,
-                              const double* losses, const double* times, const int32_t* cores, int checked) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// All loads of an entry are issued before anything is stored: the chain is then three memory latencies long (entry, job,
+// newest loss) instead of one per array.
+__device__ __forceinline__ void append_one(const JobArrays& job, const FitArrays& fit, int max_jobs, int i, const int32_t* ids,
+                                           const double* losses, const double* times, const int32_t* cores, int checked) {
     const int j = ids[i];
+    const double loss = losses[i];
+    const double t = times ? times[i] : 0.0;
+    int nc = times && cores ? cores[i] : 0;
     if (j < 0 || j >= max_jobs) {
         if (checked) atomicOr(job.err_word, kErrInput);
         return;
     }
-    const double loss = losses[i];
+    const size_t J = (size_t)max_jobs;
+    double* const row = job.row[j];
+    const int cap = job.cap[j];
+    int head = job.head[j];
+    const int count = job.count[j];
+    const int64_t k_last = job.k_last[j];
+    const double seen = job.m_seen[j];
+    const uint8_t fitted = fit.mask[j];
+    double both[8], tm[8];
+    double span = 1.0, scale = 1.0;
+    int64_t k_fit = 0;
+    if (fitted) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) both[k] = fit.both[8 * (size_t)j + k];
+        k_fit = fit.k_fit[j];
+        span = fit.span[j];
+        scale = fit.largest[j];
+    }
+    if (times) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) tm[k] = job.tm[k * J + j];
+        if (!cores) nc = job.last_alloc[j];
+    }
     if (checked) {
-        const bool bad = !(fabs(loss) <= 1.7976931348623157e308) || job.count[j] <= 0 ||
-                         (times && !(fabs(times[i]) <= 1.7976931348623157e308)) || (times && cores && cores[i] < 1);
+        const bool bad = !(fabs(loss) <= 1.7976931348623157e308) || count <= 0 ||
+                         (times && !(fabs(t) <= 1.7976931348623157e308)) || (times && cores && nc < 1);
         if (bad) {
             atomicOr(job.err_word, kErrInput);
             return;
         }
     }
-    double* row = job.row[j];
-    const int cap = job.cap[j];
-    int head = job.head[j];
-    const int count = job.count[j];
 #ifdef SLAQ_DEBUG_BOUNDS
     {   // the ring lies inside one of the pools and the write position inside the ring
         const bool in_ring = row >= job.ring_lo && row + cap <= job.ring_hi;
@@ -198,38 +224,57 @@ __global__ void append_kernel(JobArrays job, FitArrays fit, int max_jobs, int n,
     }
 #endif
     if (count > 0) {
-        const double prev = row[head == 0 ? cap - 1 : head - 1];
-        const double seen = job.m_seen[j], drop = prev - loss;
-        job.m_seen[j] = drop > seen ? drop : seen;
+        const double drop = row[head == 0 ? cap - 1 : head - 1] - loss;
+        if (drop > seen) job.m_seen[j] = drop;
     }
     row[head] = loss;
     head = head + 1 == cap ? 0 : head + 1;
     job.head[j] = head;
     job.count[j] = count < cap ? count + 1 : cap;
-    job.k_last[j] += 1;
+    job.k_last[j] = k_last + 1;
     // the history changes: what the last epoch fitted becomes the next fit's starting point
-    const uint8_t fitted = fit.mask[j];
     fit.warm_mask[j] = fitted;
     if (fitted) {
-        for (int k = 0; k < 8; ++k) fit.warm_p[8 * (size_t)j + k] = fit.both[8 * (size_t)j + k];
-        fit.warm_k[j] = fit.k_fit[j];
-        fit.warm_span[j] = fit.span[j];
-        fit.warm_scale[j] = fit.largest[j];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) fit.warm_p[8 * (size_t)j + k] = both[k];
+        fit.warm_k[j] = k_fit;
+        fit.warm_span[j] = span;
+        fit.warm_scale[j] = scale;
     }
     if (times) {
-        int nc = cores ? cores[i] : job.last_alloc[j];
         if (nc < 1) nc = 1;
-        const double t = times[i], nn = (double)nc, u = __ddiv_rn(1.0, nn);
-        const size_t J = (size_t)max_jobs;
-        double* tm = job.tm + j;
-        tm[0] = __dadd_rn(tm[0], 1.0);
-        tm[J] = __dadd_rn(tm[J], u);
-        tm[2 * J] = __dadd_rn(tm[2 * J], __dmul_rn(u, u));
-        tm[3 * J] = __dadd_rn(tm[3 * J], t);
-        tm[4 * J] = __dadd_rn(tm[4 * J], __dmul_rn(u, t));
-        tm[5 * J] = __dadd_rn(tm[5 * J], __dmul_rn(t, nn));
-        tm[6 * J] = fmin(tm[6 * J], u);
-        tm[7 * J] = fmax(tm[7 * J], u);
+        const double nn = (double)nc, u = __ddiv_rn(1.0, nn);
+        double* const sums = job.tm + j;
+        sums[0] = __dadd_rn(tm[0], 1.0);
+        sums[J] = __dadd_rn(tm[1], u);
+        sums[2 * J] = __dadd_rn(tm[2], __dmul_rn(u, u));
+        sums[3 * J] = __dadd_rn(tm[3], t);
+        sums[4 * J] = __dadd_rn(tm[4], __dmul_rn(u, t));
+        sums[5 * J] = __dadd_rn(tm[5], __dmul_rn(t, nn));
+        sums[6 * J] = fmin(tm[6], u);
+        sums[7 * J] = fmax(tm[7], u);
+    }
+}
+
+__global__ void append_kernel(JobArrays job, FitArrays fit, int max_jobs, int n, const int32_t* ids,
+                              const double* losses, const double* times, const int32_t* cores, int checked,
+                              Mailbox* mail, uint32_t seq, unsigned int* ticket) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) append_one(job, fit, max_jobs, i, ids, losses, times, cores, checked);
+    if (!mail) return;
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {   // the last block tells the host
+        last = true;
+        if (gridDim.x > 1) {
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
+        if (last) {
+            *ticket = 0;
+            __threadfence_system();
+            mail->done = seq;
+        }
     }
 }
 
@@ -310,11 +355,23 @@ int check_device(slaq_handle* h) {
     return SLAQ_OK;
 }
 
+// Mark the listed ids with a new stamp.
+void stamp_ids(slaq_handle* h, int32_t n, const int32_t* ids) {
+    if (++h->stamp_epoch == 0) {
+        std::fill(h->stamp.begin(), h->stamp.end(), 0u);
+        h->stamp_epoch = 1;
+    }
+    for (int32_t i = 0; i < n; ++i) h->stamp[ids[i]] = h->stamp_epoch;
+}
+
+bool strictly_increasing(const int32_t* ids, int32_t n);
+
 int check_ids(slaq_handle* h, int32_t n, const int32_t* ids, bool forbid_dups) {
     if (const int rc = check_device(h)) return rc;
     if (n < 0) return fail(h, SLAQ_E_ARG, "negative count");
     if (n > 0 && !ids) return fail(h, SLAQ_E_ARG, "job_ids is null");
     if (n > h->max_jobs) return fail(h, SLAQ_E_ARG, "more entries than job ids");
+    if (n > 0 && ids[0] >= 0 && ids[n - 1] < h->max_jobs && strictly_increasing(ids, n)) return SLAQ_OK;
     if (++h->stamp_epoch == 0) {
         std::fill(h->stamp.begin(), h->stamp.end(), 0u);
         h->stamp_epoch = 1;
@@ -357,9 +414,46 @@ int check_device_errors(slaq_handle* h) {
         if (word & kErrBarrier) what += " the blocks of the selection launch did not all arrive in time;";
         if (word & kErrInput) what += " slaq_append_losses_device was given an id out of range, a job without losses, a value that is not finite or a core count below 1 (those entries were skipped);";
         cudaMemsetAsync(h->err_word, 0, sizeof word, h->stream);   // reported once: the next epoch starts clean
+        h->scratch_clean = false;
         return fail(h, SLAQ_E_CUDA, what);
     }
     return SLAQ_OK;
+}
+
+// Wait until the kernel that carries this call's number has reported to the mailbox.  Watching host memory sees the end of
+// a kernel a few microseconds before a stream synchronisation returns; the stream is asked now and then, for errors.
+int wait_mailbox(slaq_handle* h, const char* what) {
+    for (int spins = 0; h->mailbox->done != h->call_seq;) {
+        _mm_pause();
+        if (++spins < 2000) continue;
+        spins = 0;
+        const cudaError_t e = cudaStreamQuery(h->stream);
+        if (e == cudaErrorNotReady) continue;
+        if (e != cudaSuccess) return cuda_fail(h, e, what);
+        if (h->mailbox->done != h->call_seq) {   // the kernel gave up: the error word says why
+            if (const int rc = check_device_errors(h)) return rc;
+            return fail(h, SLAQ_E_CUDA, std::string(what) + ": the kernel did not report its end");
+        }
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return SLAQ_OK;
+}
+
+// Checks of whole arrays, in a form the compiler vectorises.
+bool all_finite(const double* p, size_t n) {
+    double acc[8] = {};
+    size_t i = 0;
+    for (; i + 8 <= n; i += 8)
+        for (int k = 0; k < 8; ++k) acc[k] += p[i + k] * 0.0;   // NaN as soon as one is NaN or infinite
+    for (; i < n; ++i) acc[0] += p[i] * 0.0;
+    double sum = 0.0;
+    for (double a : acc) sum += a;
+    return sum == 0.0;
+}
+bool strictly_increasing(const int32_t* ids, int32_t n) {
+    int32_t bad = 0;
+    for (int32_t i = 1; i < n; ++i) bad |= ids[i] <= ids[i - 1];
+    return bad == 0;
 }
 
 // Device scratch for calls that move caller data of a size unknown at creation (a bulk load into
@@ -409,6 +503,17 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     }
     h->ws_bytes = need;
     layout(h, static_cast<char*>(h->ws), max_jobs, max_hist, cap);
+    h->mailbox_jobs = std::min(max_jobs, kMailboxJobs);
+    {
+        const size_t mail = sizeof(Mailbox) + (size_t)h->mailbox_jobs * 28 + 64;
+        const cudaError_t e = cudaHostAlloc(&h->mailbox_mem, mail, cudaHostAllocPortable);
+        if (e != cudaSuccess) {
+            h->mailbox_mem = nullptr;
+            return fail(h, SLAQ_E_NOMEM, std::string("cudaHostAlloc of the mailbox: ") + cudaGetErrorString(e));
+        }
+        h->mailbox = new (h->mailbox_mem) Mailbox();   // unified addressing: kernels use the same pointer
+    }
+    if (fit_setup()) return fail(h, SLAQ_E_CUDA, "fit kernel setup failed");
     h->active.assign((size_t)max_jobs, 0);
     h->stamp.assign((size_t)max_jobs, 0u);
     h->in_packed.assign((size_t)max_jobs, 0);
@@ -421,6 +526,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
         h->job, h->fit, h->ring_pool, max_jobs, max_hist, nullptr, max_jobs, h->alloc, h->reduction);
     CK(cudaGetLastError(), "init kernel");
     CK(cudaStreamSynchronize(h->stream), "init kernel");
+    h->scratch_clean = true;
     return SLAQ_OK;
 }
 
@@ -436,34 +542,57 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
     if (n < 0) return fail(h, SLAQ_E_ARG, "negative count");
     if (n > 0 && !ids) return fail(h, SLAQ_E_ARG, "job_ids is null");
     if (n > h->max_jobs) return fail(h, SLAQ_E_ARG, "more entries than job ids");
+    if (n == 0) return SLAQ_OK;
     cudaStream_t st = h->stream;
-    // The copies into the staging arrays go first: from pinned memory they run while the host
-    // checks the arguments below.  Nothing reads the staging arrays unless the checks pass.
-    if (n > 0) {
+    const int threads = 256, blocks = (n + threads - 1) / threads;
+    const int32_t *d_ids = h->stage.ids, *d_cores = times && cores ? h->stage.cores : nullptr;
+    const double *d_losses = h->stage.losses, *d_times = times ? h->stage.times : nullptr;
+    // Small calls: the arrays are copied into the mailbox and the kernel reads them there.  Larger ones are copied to the
+    // device; from page-locked memory that runs while the host checks the arguments, so those copies go first.
+    // Nothing reads the staging arrays unless the checks pass.
+    bool mailed = n <= h->mailbox_jobs;
+    if (mailed && n > kMailAlways) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, losses) != cudaSuccess) cudaGetLastError();
+        else mailed = attr.type != cudaMemoryTypeHost;
+    }
+    if (!mailed) {
         CK(cudaMemcpyAsync(h->stage.ids, ids, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy job ids");
         CK(cudaMemcpyAsync(h->stage.losses, losses, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy losses");
-        if (times)
-            CK(cudaMemcpyAsync(h->stage.times, times, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy times");
-        if (times && cores)
-            CK(cudaMemcpyAsync(h->stage.cores, cores, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy cores");
+        if (d_times) CK(cudaMemcpyAsync(h->stage.times, times, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy times");
+        if (d_cores) CK(cudaMemcpyAsync(h->stage.cores, cores, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy cores");
     }
     int bad = check_ids(h, n, ids, true);
-    for (int32_t i = 0; i < n && !bad; ++i) {
-        if (!std::isfinite(losses[i])) bad = fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
-        else if (times && !std::isfinite(times[i])) bad = fail(h, SLAQ_E_NONFINITE, "an iteration time is not finite");
-        else if (cores && cores[i] < 1) bad = fail(h, SLAQ_E_ARG, "cores_used must be at least 1");
+    if (!bad && !(all_finite(losses, n) && (!times || all_finite(times, n)))) {   // which comes first says the message
+        for (int32_t i = 0; i < n && !bad; ++i) {
+            if (!std::isfinite(losses[i])) bad = fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
+            else if (times && !std::isfinite(times[i])) bad = fail(h, SLAQ_E_NONFINITE, "an iteration time is not finite");
+            else if (cores && cores[i] < 1) bad = fail(h, SLAQ_E_ARG, "cores_used must be at least 1");
+        }
+    }
+    if (!bad && cores) {
+        int32_t least = 1;
+        for (int32_t i = 0; i < n; ++i) least = cores[i] < least ? cores[i] : least;
+        if (least < 1) bad = fail(h, SLAQ_E_ARG, "cores_used must be at least 1");
     }
     if (bad) {
-        cudaStreamSynchronize(st);   // the caller's buffers are free again; the state is untouched
+        if (!mailed) cudaStreamSynchronize(st);   // the caller's buffers are free again; the state is untouched
         return bad;
     }
-    if (n == 0) return SLAQ_OK;
-    const int threads = 256;
-    append_kernel<<<(n + threads - 1) / threads, threads, 0, st>>>(
-        h->job, h->fit, h->max_jobs, n, h->stage.ids, h->stage.losses, times ? h->stage.times : nullptr,
-        (times && cores) ? h->stage.cores : nullptr, 0);
+    if (mailed) {
+        std::memcpy(h->mail_ids(), ids, sizeof(int32_t) * n);
+        std::memcpy(h->mail_losses(), losses, sizeof(double) * n);
+        if (d_times) std::memcpy(h->mail_times(), times, sizeof(double) * n);
+        if (d_cores) std::memcpy(h->mail_cores(), cores, sizeof(int32_t) * n);
+        d_ids = h->mail_ids();
+        d_losses = h->mail_losses();
+        if (d_times) d_times = h->mail_times();
+        if (d_cores) d_cores = h->mail_cores();
+    }
+    append_kernel<<<blocks, threads, 0, st>>>(h->job, h->fit, h->max_jobs, n, d_ids, d_losses, d_times, d_cores, 0, h->mailbox,
+                                              ++h->call_seq, h->scratch.append_ticket);
     CK(cudaGetLastError(), "append kernel");
-    CK(cudaStreamSynchronize(st), "append");   // the caller may reuse its buffers
+    if (const int rc = wait_mailbox(h, "append")) return rc;   // the caller may reuse its buffers
     if (h->n_active < h->max_jobs) {   // nothing to do once every id is active
         for (int32_t i = 0; i < n; ++i) {
             if (!h->active[ids[i]]) {
@@ -496,6 +625,7 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
     double* d_src = nullptr;
     double* old_pool = nullptr;
     if (packed) {
+        stamp_ids(h, n, ids);
         // The new pool is allocated before anything changes, so a failed allocation leaves the handle
         // as it was.  Jobs of the old pool that are listed again are re-pointed by the load kernel and
         // keep their time sums, time law and core count; those that are not listed lose their
@@ -509,7 +639,7 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
         if (h->packed_pool) {
             std::vector<int32_t> gone;
             for (int32_t j = 0; j < h->max_jobs; ++j)
-                if (h->in_packed[j] && h->stamp[j] != h->stamp_epoch) gone.push_back(j);   // check_ids stamped the listed ids
+                if (h->in_packed[j] && h->stamp[j] != h->stamp_epoch) gone.push_back(j);   // the listed ids are stamped
             const int32_t m = (int32_t)gone.size();
             if (m > 0) {
                 cudaError_t e = cudaMemcpyAsync(h->stage.ids, gone.data(), sizeof(int32_t) * m, cudaMemcpyHostToDevice, st);
@@ -592,11 +722,10 @@ bool gains_in_selection(const slaq_handle* h, bool only_allocate) {
 // with_events: the stage boundaries are marked with the handle's events (left out of a captured
 // graph: events recorded by a graph cannot be timed).
 int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32_t* d_out, bool only_allocate,
-                  bool with_events) {
+                  bool with_events, uint32_t seq) {
     cudaStream_t st = h->stream;
     int launches = 0, k;
     if (with_events && cudaEventRecord(h->ev[0], st) != cudaSuccess) return -1;
-    if (cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st) != cudaSuccess) return -1;
     if (!only_allocate) {
         if ((k = launch_fit(h)) < 0) return -1;
         launches += k;
@@ -608,7 +737,7 @@ int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32
         launches += k;
     }
     if (with_events && cudaEventRecord(h->ev[2], st) != cudaSuccess) return -1;
-    if ((k = launch_select(h, T, want, floor_units + 1, from_curves, d_out)) < 0) return -1;
+    if ((k = launch_select(h, T, want, floor_units + 1, from_curves, d_out, seq)) < 0) return -1;
     launches += k;
     if (with_events && cudaEventRecord(h->ev[3], st) != cudaSuccess) return -1;
     return launches;
@@ -627,7 +756,9 @@ std::vector<long long> epoch_key(const slaq_handle* h, double T, int64_t want, i
             (long long)(uintptr_t)h->job.packed_lo, (long long)(uintptr_t)h->job.packed_hi};
 }
 
-int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_allocate) {
+// to_mailbox: the launches report to the mailbox under the call number h->call_seq, unless a graph is replayed
+// (h->last_epoch_was_graph says so).
+int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_allocate, bool to_mailbox) {
     if (!only_allocate && !(T > 0.0 && std::isfinite(T))) return fail(h, SLAQ_E_ARG, "epoch_seconds must be positive");
     if (C < 0) return fail(h, SLAQ_E_ARG, "total_cores must not be negative");
     if (const int dc = check_device(h)) return dc;
@@ -639,7 +770,12 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     const int64_t want = usable - active * floor_units;
     cudaStream_t st = h->stream;
 
-    bool graph_ok = h->epoch_graph == 1 || (h->epoch_graph < 0 && h->max_jobs <= kGraphAutoJobs);
+    if (!h->scratch_clean) {
+        CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone) h->scratch_clean = true;
+    }
+    bool graph_ok = h->epoch_graph == 1;
     if (graph_ok) {   // not while the caller captures this stream into a graph of its own
         cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone) graph_ok = false;
@@ -660,7 +796,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
                 CK(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking), "create capture stream");
             CK(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeRelaxed), "begin capture");
             h->stream = h->capture_stream;
-            const int n = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, false);
+            const int n = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, false, 0);
             h->stream = st;
             cudaGraph_t graph = nullptr;
             const cudaError_t e_end = cudaStreamEndCapture(h->capture_stream, &graph);
@@ -692,13 +828,13 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
         h->seen_key = key;
     }
     if (launches < 0) {
-        launches = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, true);
+        launches = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, true, to_mailbox ? ++h->call_seq : 0);
         if (launches < 0) {
             if (h->err.empty()) h->err = "an epoch launch failed";
             return SLAQ_E_CUDA;
         }
     }
-    h->have_epoch = true;
+    h->have_epoch = h->stats_published = true;
     h->last_launches = launches;
     h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
     h->last_cores = usable;
@@ -710,6 +846,30 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     if (active > 0 && C < active) return SLAQ_W_OVERSUBSCRIBED;
     if (C > active * cap) return SLAQ_W_UNDERFILLED;
     return SLAQ_OK;
+}
+
+// An epoch whose allocation goes to a host array.
+int epoch_to_host(slaq_handle* h, double T, int64_t C, int32_t* out_alloc, bool only_allocate) {
+    const int rc = run_epoch(h, T, C, nullptr, only_allocate, true);
+    if (rc < 0) return rc;
+    const size_t bytes = sizeof(int32_t) * (size_t)h->max_jobs;
+    if (h->last_epoch_was_graph || h->max_jobs > h->mailbox_jobs) {
+        CK(cudaMemcpyAsync(out_alloc, h->alloc, bytes, cudaMemcpyDeviceToHost, h->stream), "copy allocation");
+        if (h->last_epoch_was_graph) {
+            const int ec = check_device_errors(h);   // its synchronisation also completes the copy above
+            return ec ? ec : rc;
+        }
+        CK(cudaStreamSynchronize(h->stream), "epoch");
+        if (const int wc = wait_mailbox(h, "epoch")) return wc;
+    } else {
+        if (const int wc = wait_mailbox(h, "epoch")) return wc;
+        std::memcpy(out_alloc, h->mail_alloc(), bytes);
+    }
+    if (h->mailbox->err) {
+        const int ec = check_device_errors(h);
+        return ec ? ec : rc;
+    }
+    return rc;
 }
 
 template <class T>
@@ -755,6 +915,7 @@ int slaq_destroy(slaq_t* h) {
         if (ev) cudaEventDestroy(ev);
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
+    if (h->mailbox_mem) cudaFreeHost(h->mailbox_mem);
     if (h->packed_pool) cudaFree(h->packed_pool);
     if (h->call_buf) cudaFree(h->call_buf);
     if (h->owns_ws && h->ws) cudaFree(h->ws);
@@ -858,7 +1019,7 @@ int slaq_append_losses_device(slaq_t* h, int32_t n, const int32_t* d_job_ids, co
     if (n == 0) return SLAQ_OK;
     const int threads = 256;
     append_kernel<<<(n + threads - 1) / threads, threads, 0, h->stream>>>(h->job, h->fit, h->max_jobs, n, d_job_ids, d_losses,
-                                                                        d_iter_times, d_cores_used, 1);
+                                                                        d_iter_times, d_cores_used, 1, nullptr, 0, nullptr);
     CK(cudaGetLastError(), "append kernel");
     return SLAQ_OK;
 }
@@ -945,18 +1106,13 @@ int slaq_remove_jobs(slaq_t* h, int32_t n, const int32_t* job_ids) {
 
 int slaq_schedule_device(slaq_t* h, double epoch_seconds, int64_t total_cores, int32_t* d_out_alloc) {
     if (!h) return SLAQ_E_ARG;
-    return run_epoch(h, epoch_seconds, total_cores, d_out_alloc, false);
+    return run_epoch(h, epoch_seconds, total_cores, d_out_alloc, false, false);
 }
 
 int slaq_schedule(slaq_t* h, double epoch_seconds, int64_t total_cores, int32_t* out_alloc) {
     if (!h) return SLAQ_E_ARG;
     if (!out_alloc) return fail(h, SLAQ_E_ARG, "out_alloc is null");
-    const int rc = run_epoch(h, epoch_seconds, total_cores, nullptr, false);
-    if (rc < 0) return rc;
-    CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
-       "copy allocation");
-    const int ec = check_device_errors(h);   // its synchronisation also completes the copy above
-    return ec ? ec : rc;
+    return epoch_to_host(h, epoch_seconds, total_cores, out_alloc, false);
 }
 
 int slaq_set_gains(slaq_t* h, const double* gain) {
@@ -971,12 +1127,7 @@ int slaq_set_gains(slaq_t* h, const double* gain) {
 int slaq_allocate_only(slaq_t* h, int64_t total_cores, int32_t* out_alloc) {
     if (!h) return SLAQ_E_ARG;
     if (!out_alloc) return fail(h, SLAQ_E_ARG, "out_alloc is null");
-    const int rc = run_epoch(h, 1.0, total_cores, nullptr, true);
-    if (rc < 0) return rc;
-    CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
-       "copy allocation");
-    CK(cudaStreamSynchronize(h->stream), "copy allocation");
-    return rc;
+    return epoch_to_host(h, 1.0, total_cores, out_alloc, true);
 }
 
 // ---- one cluster sharded over several GPUs ----
@@ -999,6 +1150,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     h->last_epoch_was_graph = false;
     CK(cudaMemsetAsync(h->scratch.hist, 0, sizeof(unsigned long long) * kRadixPasses * kRadixBins, st), "clear scratch");
     CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
+    h->scratch_clean = h->stats_published = false;   // these steps leave their counts where they were added up
     CK(cudaEventRecord(h->ev[0], st), "event");
     if ((k = launch_fit(h)) < 0) return SLAQ_E_CUDA;
     launches += k;
@@ -1436,7 +1588,8 @@ int slaq_get_fit_phase_cycles(slaq_t* h, int64_t* out_cycles) {
     if (!h || !out_cycles) return SLAQ_E_ARG;
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     long long counters[16];
-    CK(cudaMemcpyAsync(counters, h->scratch.counters, sizeof counters, cudaMemcpyDeviceToHost, h->stream), "copy counters");
+    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters, sizeof counters,
+                       cudaMemcpyDeviceToHost, h->stream), "copy counters");
     CK(cudaStreamSynchronize(h->stream), "copy phase cycles");
     for (int i = 0; i < 6; ++i) out_cycles[i] = counters[8 + i];
     return SLAQ_OK;
@@ -1448,9 +1601,11 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
     std::memset(out, 0, sizeof *out);
     long long counters[16];
     SelectState sel;
-    CK(cudaMemcpyAsync(counters, h->scratch.counters, sizeof counters, cudaMemcpyDeviceToHost, h->stream), "copy counters");
-    CK(cudaMemcpyAsync(&sel, h->scratch.sel, sizeof sel, cudaMemcpyDeviceToHost, h->stream), "copy selection state");
+    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters, sizeof counters,
+                       cudaMemcpyDeviceToHost, h->stream), "copy counters");
+    if (!h->stats_published) CK(cudaMemcpyAsync(&sel, h->scratch.sel, sizeof sel, cudaMemcpyDeviceToHost, h->stream), "copy selection state");
     CK(cudaStreamSynchronize(h->stream), "copy statistics");
+    if (h->stats_published) sel.prefix = (unsigned long long)counters[15];
     CK(cudaEventElapsedTime(&out->ms_total, h->ev[0], h->ev[3]), "event time");
     if (!h->last_epoch_was_graph) {   // a replayed graph has no stage boundaries to time
         CK(cudaEventElapsedTime(&out->ms_fit, h->ev[0], h->ev[1]), "event time");

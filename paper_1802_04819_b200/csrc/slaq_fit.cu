@@ -658,7 +658,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         int run = 0;
         for (int c = 0; c < cls.n; ++c) {
             slot_base[c] = run;
-            const int jobs = start[cls.h_lo[c]] - start[cls.h_hi[c]], per_slot = 32 / cls.L[c];
+            const int jobs = order ? start[cls.h_lo[c]] - start[cls.h_hi[c]] : job.max_jobs, per_slot = 32 / cls.L[c];
             run += (jobs + per_slot - 1) / per_slot;
         }
         for (int c = cls.n; c <= kMaxFitClasses; ++c) slot_base[c] = run;
@@ -684,10 +684,10 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         const int G = 32 / L, g = lane / L;
         S.park = slice + 2 * g + (lane & 1);
         S.y = slice + kParked * 2 * G;
-        const int last = start[cls.h_lo[c]];
-        const int base = start[h_hi] + (slot - slot_base[c]) * G;
+        const int last = order ? start[cls.h_lo[c]] : job.max_jobs;
+        const int base = (order ? start[h_hi] : 0) + (slot - slot_base[c]) * G;
         const int idx = base + g;
-        int j = idx < last && index_ok(idx, job.max_jobs, kErrJob, err_word) ? order[idx] : -1;
+        int j = idx < last && index_ok(idx, job.max_jobs, kErrJob, err_word) ? (order ? order[idx] : idx) : -1;
         if (j >= 0 && !index_ok(j, job.max_jobs, kErrJob, err_word)) j = -1;
         __syncwarp();
         const int H = stage_window(job, j, h_hi, S, err_word);
@@ -1048,27 +1048,91 @@ length_scatter_kernel(const int32_t* __restrict__ count, int max_jobs, int max_h
     }
 }
 
+// The same in one block for few jobs: count, scan and scatter in shared memory.
+constexpr int kOneBlockSort = 16384;
+
+__global__ void __launch_bounds__(1024) length_sort_kernel(const int32_t* __restrict__ count, int max_jobs, int max_hist,
+                                                           int32_t* start, int32_t* order, int32_t* err_word) {
+    extern __shared__ int sh_one[];     // [max_hist + 1] jobs per length, then [max_hist + 1] next free position
+    __shared__ int warp_sum[32];
+    int* const bins = sh_one;
+    int* const next = sh_one + (max_hist + 1);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, n = max_hist + 1;
+    for (int i = t; i < n; i += 1024) bins[i] = 0;
+    __syncthreads();
+    int H[kOneBlockSort / 1024];
+#pragma unroll
+    for (int k = 0; k < kOneBlockSort / 1024; ++k) {
+        const int j = k * 1024 + t;
+        H[k] = j < max_jobs ? clamped_length(count, j, max_hist) : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < kOneBlockSort / 1024; ++k) {
+        if (k * 1024 >= max_jobs) break;
+        const unsigned peers = __match_any_sync(kFull, H[k]);
+        if (H[k] >= 0 && __ffs(peers) - 1 == lane) atomicAdd(&bins[H[k]], __popc(peers));
+    }
+    __syncthreads();
+    // thread t owns lengths max_hist - (t * per + i): from the longest down, the jobs before its first length
+    const int per = (n + 1023) / 1024;
+    int sum = 0;
+    for (int i = 0; i < per; ++i) {
+        const int h = max_hist - (t * per + i);
+        if (h >= 0) sum += bins[h];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    int run = incl - sum;
+    for (int i = 0; i < warp; ++i) run += warp_sum[i];
+    for (int i = 0; i < per; ++i) {
+        const int h = max_hist - (t * per + i);
+        if (h < 0) break;
+        start[h] = run;
+        next[h] = run;
+        run += bins[h];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kOneBlockSort / 1024; ++k) {
+        if (k * 1024 >= max_jobs) break;
+        const unsigned peers = __match_any_sync(kFull, H[k]);
+        const int leader = __ffs(peers) - 1;
+        int first = 0;
+        if (H[k] >= 0 && lane == leader) first = atomicAdd(&next[H[k]], __popc(peers));
+        first = __shfl_sync(kFull, first, leader);
+        const int at = first + __popc(peers & ((1u << lane) - 1u));
+        if (H[k] >= 0 && index_ok(at, max_jobs, kErrJob, err_word)) order[at] = k * 1024 + t;
+    }
+}
+
 size_t fit_smem_bytes(const FitClasses& c, int warps) {
     return sizeof(double) * ((size_t)c.h_max + (size_t)warps * (size_t)c.slice);
 }
 
 }  // namespace
 
+int fit_setup() {
+    const int most = (int)kSmemLimit;
+    bool ok = true;
+    for (const void* k : {(const void*)fit_kernel<false>, (const void*)fit_kernel<true>})
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
+             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    for (const void* k : {(const void*)length_scatter_kernel, (const void*)length_sort_kernel})
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(2 * sizeof(int) * (kMaxHistLimit + 1))) == cudaSuccess;
+    return ok ? 0 : -1;
+}
+
 int launch_fit(slaq_handle* h) {
     cudaStream_t st = h->stream;
     const int J = h->max_jobs, Hmax = h->max_hist;
     int launches = 0;
-    // work list
-    {
-        const int blocks = (J + kSortJobsPerBlock - 1) / kSortJobsPerBlock;
-        const size_t one = sizeof(int) * ((size_t)Hmax + 1);
-        cudaFuncSetAttribute(length_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * one));
-        length_count_kernel<<<blocks, kSortThreads, one, st>>>(h->job.count, J, Hmax, h->scratch.bucket);
-        length_scan_kernel<<<1, 1024, 0, st>>>(h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
-        length_scatter_kernel<<<blocks, kSortThreads, 2 * one, st>>>(h->job.count, J, Hmax, h->scratch.cursor,
-                                                                     h->scratch.order, h->err_word);
-        launches += 3;
-    }
     // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked
     // doubles per job and family), the window rows of 32 points and one spare row; with L lanes
     // per job that leaves rows_at(L) rows.  The class with L = 32, 16, .. 2 lanes per job takes
@@ -1099,32 +1163,41 @@ int launch_fit(slaq_handle* h) {
         h_hi = h_lo;
     }
     for (int c = cls.n; c < kMaxFitClasses; ++c) cls.h_lo[c] = cls.h_hi[c] = 0, cls.L[c] = 32;
+    // The work list: job ids, longest window first.  A job per warp of the GPU and no more: every job starts at once,
+    // so their order means nothing and none is made.  Up to kOneBlockSort jobs one block sorts (one launch of about 5 us
+    // instead of three of 3 to 4 us each), beyond that a block per 2048 jobs.
+    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= h->sm_count * kMaxWarpsPerBlock;
+    const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
+    if (in_order) {
+    } else if (J <= kOneBlockSort) {
+        length_sort_kernel<<<1, 1024, 2 * bins, st>>>(h->job.count, J, Hmax, h->scratch.start, h->scratch.order, h->err_word);
+        launches += 1;
+    } else {
+        const int sort_blocks = (J + kSortJobsPerBlock - 1) / kSortJobsPerBlock;
+        length_count_kernel<<<sort_blocks, kSortThreads, bins, st>>>(h->job.count, J, Hmax, h->scratch.bucket);
+        length_scan_kernel<<<1, 1024, 0, st>>>(h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
+        length_scatter_kernel<<<sort_blocks, kSortThreads, 2 * bins, st>>>(h->job.count, J, Hmax, h->scratch.cursor,
+                                                                          h->scratch.order, h->err_word);
+        launches += 3;
+    }
     int warps = kMaxWarpsPerBlock;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
+    if (in_order) warps = std::min(warps, (J + h->sm_count - 1) / h->sm_count);   // few jobs: spread over all SMs
     const size_t smem = fit_smem_bytes(cls, warps);
     if (smem > kSmemLimit) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
     const auto kernel = h->warm_start ? fit_kernel<true> : fit_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        h->err = std::string("fit kernel shared memory: ") + cudaGetErrorString(e);
-        return -1;
-    }
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, warps * 32, smem);
-    if (per_sm < 1) per_sm = 1;
-    int blocks = h->sm_count * per_sm;
+    int blocks = h->sm_count;   // one block per SM: its registers and shared memory fill one
     const int needed = (J + warps - 1) / warps;   // at least one job per slot
     if (blocks > needed) blocks = needed;
     if (blocks < 1) blocks = 1;
-    kernel<<<blocks, warps * 32, smem, st>>>(h->job, h->fit, h->wtab, h->scratch.order, h->scratch.start, cls,
+    kernel<<<blocks, warps * 32, smem, st>>>(h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order, h->scratch.start, cls,
                                             h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase,
                                             h->scratch.counters, h->err_word);
     ++launches;
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
         return -1;

@@ -20,7 +20,6 @@ constexpr int kRadixPasses = 6;       // 11 + 11 + 11 + 11 + 11 + 9 bits, most s
 constexpr int kMaxFitClasses = 8;     // window-length classes of the fit (one launch each)
 constexpr int kFitQueueBase = 8;      // ticket[kFitQueueBase + c]: work queue head of class c
 constexpr int kTickets = 16;
-constexpr int kGraphAutoJobs = 20000;  // handles up to this size replay the epoch as a CUDA graph unless told otherwise
 
 // Device-side state of one job, structure of arrays (index = job id).
 struct JobArrays {
@@ -74,18 +73,29 @@ struct SelectState {
     int done;                        // nothing is wanted: the threshold lies above every gain
 };
 
-constexpr int kSelectFineBins = 4096;
+constexpr int kSelectFineBins = 2048;
+constexpr int kSelectCandidates = 2048;
 constexpr int kSelectMaxGrid = 4096;
 
 // Global memory of the selection launch.  The leading part is cleared before every launch.
 struct SelectGlobal {
     unsigned long long coarse[32];                        // first histogram: one total per power of two ..
-    unsigned long long fine[kSelectFineBins];             // .. and its 128 bins each
-    unsigned int barrier, ticket, n_list, pad;            // blocks that arrived; blocks that finished; listed rows
+    unsigned long long fine[kSelectFineBins];             // .. and its 64 bins each
+    unsigned int barrier, ticket, n_cand, pad;            // blocks that arrived; blocks that finished; listed candidates
     static constexpr size_t kZeroBytes = sizeof(unsigned long long) * (32 + kSelectFineBins) + 16;
     unsigned long long narrow[kRadixPasses][kRadixBins];  // cleared by the kernel itself
+    unsigned long long cand_key[kSelectCandidates];       // the candidates the last block ranks ..
+    unsigned long long cand_pos[kSelectCandidates];       // .. and their (candidates of the row, job, n)
     long long block_eq[kSelectMaxGrid];                   // per block: candidates that equal the threshold
 };
+
+// Page-locked host memory of a handle that kernels write and read directly: a call is over when `done` holds its number.
+struct Mailbox {
+    volatile uint32_t done;
+    volatile int32_t err;            // the device error word when the call finished
+    uint32_t pad[14];
+};
+constexpr int32_t kMailboxJobs = 32768;   // most entries per call that pass through the mailbox's arrays
 
 // Scratch of one epoch.  [zero, zero + zero_bytes) is cleared at the start of every epoch; the sharded steps
 // clear their histograms `hist` as well.
@@ -93,10 +103,11 @@ struct Scratch {
     unsigned long long* hist;        // [kRadixPasses][kRadixBins], sharded steps
     void* zero;
     SelectGlobal* select;            // its leading part is the end of the cleared region
-    int32_t* list;                   // [max_jobs] rows with candidates
     unsigned int* ticket;            // [kTickets]: work queue of the fit
     SelectState* sel;
-    long long* counters;             // [16] statistics accumulated by kernels
+    long long* counters;             // [16] statistics accumulated by kernels during an epoch
+    long long* published;            // [16] those of the last finished epoch
+    unsigned int* append_ticket;     // blocks of the append kernel that are done
     size_t zero_bytes;
     int32_t* gt;                     // per job: during the passes the start of its candidate segment, then gains above the threshold
     int32_t* eq;                     // per job: during the passes the end of its segment, then gains equal to the threshold
@@ -154,6 +165,17 @@ struct slaq_handle {
     int32_t* alloc = nullptr;
     double* reduction = nullptr;
     int32_t* err_word = nullptr;      // device error flags set by kernels
+    void* mailbox_mem = nullptr;      // page-locked: Mailbox, then ids, losses, times, cores in and the allocation out
+    slaq::Mailbox* mailbox = nullptr;
+    int32_t mailbox_jobs = 0;         // entries of each of those arrays
+    int32_t* mail_ids() const { return reinterpret_cast<int32_t*>(mailbox + 1); }
+    int32_t* mail_cores() const { return mail_ids() + mailbox_jobs; }
+    int32_t* mail_alloc() const { return mail_cores() + mailbox_jobs; }
+    double* mail_losses() const { return reinterpret_cast<double*>(mail_alloc() + mailbox_jobs + (mailbox_jobs & 1)); }
+    double* mail_times() const { return mail_losses() + mailbox_jobs; }
+    uint32_t call_seq = 0;            // number of the last call that reports to the mailbox
+    bool stats_published = true;      // the last epoch's statistics are in scratch.published (sharded steps: where they are counted)
+    bool scratch_clean = false;       // the last epoch left its scratch cleared for the next one
     cudaEvent_t ev[4] = {};
     bool have_epoch = false;
     int32_t last_launches = 0;            // kernels the last call launched
@@ -170,7 +192,7 @@ struct slaq_handle {
     // The epoch as a CUDA graph: what the captured launches depended on, the instantiated graph,
     // and the stream the capture runs on (the caller's stream may be the legacy default stream,
     // which cannot capture).
-    int epoch_graph = -1;             // 0 never, 1 always, -1: for handles of at most kGraphAutoJobs jobs
+    int epoch_graph = -1;             // 1: replay the launches as a graph; 0, -1: plain launches
     std::vector<long long> graph_key, seen_key;
     cudaGraphExec_t graph_exec = nullptr;
     cudaStream_t capture_stream = nullptr;
@@ -182,9 +204,12 @@ struct slaq_handle {
 namespace slaq {
 
 // kernel launchers: each returns the number of kernels it launched, or -1 after setting h->err
+int fit_setup();   // once per device before the first fit; 0 or -1
 int launch_fit(slaq_handle* h);
 int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit);
-int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc);
+// seq != 0: the kernel reports to the handle's mailbox under that number, and writes the allocation there too if it fits
+int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
+                  uint32_t seq);
 bool select_writes_whole_table(const slaq_handle* h, long long want);
 int select_setup(int* blocks_per_sm);   // once per device before the first selection launch; 0 or -1
 int launch_normalise_export(slaq_handle* h, int32_t n, const int64_t* d_offsets, double* d_changes,

@@ -7,12 +7,12 @@
 // is searched on them:
 //
 //   A  every block predicts (or reads) the gains of its own contiguous range of jobs and counts them in a histogram
-//      of 4096 bins: 128 per power of two from 2^-31 to 2, what lies below in bin 0, above in the last one.
+//      of 2048 bins: 64 per power of two from 2^-31 to 2, what lies below in bin 0, above in the last one.
 //      -- one grid barrier --
 //      Every block finds the bin of the want-th largest gain: the interval [lo, hi) the threshold lies in.
 //   B  every thread walks a row from its first core: gains >= hi are handed out, the row's gains inside [lo, hi) are
 //      its candidates.  A row without candidates is finished here.
-//   C  the last block to arrive ranks the candidates (normally a few hundred at most: a bin is 0.8 % wide) by (gain
+//   C  the last block to arrive ranks the candidates (normally a few hundred at most: a bin is 1.6 % wide) by (gain
 //      descending, job id, n) and completes their rows.  Only when there are more than kFinal of them do all blocks stay
 //      and narrow the interval by another 2048 bins at a time first; candidates that are all equal are handed out
 //      in job order with a prefix sum over the blocks.
@@ -39,15 +39,18 @@ namespace {
 using namespace gaincurve;
 using u64 = unsigned long long;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 1024;                       // one block per SM: half the arrivals and histogram flushes of two
 constexpr int kWarps = kThreads / 32;
-constexpr int kSubBits = 7;                          // bins per power of two: 128
+constexpr int kSubBits = 6;                          // bins per power of two: 64 (twice as many: the flush of 148 blocks
+                                                     // costs more than the candidates it saves)
+constexpr int kSub = 1 << kSubBits;
 constexpr int kFine = kSelectFineBins;               // 32 powers of two
 constexpr long long kBinBase = (long long)(1023 - 31) << kSubBits;
 constexpr int kBinShift = 52 - kSubBits;
 constexpr int kNarrowBins = kRadixBins;              // a narrowing step divides the interval by this
-constexpr int kFinal = 1024;                         // candidates one block ranks
+constexpr int kFinal = kSelectCandidates;            // candidates one block ranks
 constexpr int kRankDirect = 256;                     // ranked against each other; more are narrowed in the block first
+constexpr int kShortWalk = 16;                       // gains of a row its own thread walks; its warp continues
 constexpr u64 kTopKey = 1ull << 63;                  // above every key
 constexpr int kSpinLimit = 1 << 22;                  // polls of a barrier before it gives up (seconds)
 
@@ -75,8 +78,8 @@ struct Shared {
         } cand;
     };
     unsigned int narrow[kNarrowBins];
-    unsigned short own[kFinal], idx[kFinal];
-    int take[kFinal];
+    unsigned short idx[kFinal];
+    unsigned char taken[kFinal];
     Interval iv;
     u64 scan[kWarps + 1];
     int count, n_more, flag;
@@ -130,8 +133,7 @@ __device__ u64 block_exclusive(u64 v, Shared& sh, u64* total) {
     return out;
 }
 
-// Warp 0: the bin of the want-th largest gain from the global histogram (octave totals first, then the 128 bins of one
-// octave).  Fewer gains than wanted: an interval below everything counted, n = 0.
+// Warp 0: the bin of the want-th largest gain from the global histogram (octave totals first, then the bins of one octave).  Fewer gains than wanted: an interval below everything counted, n = 0.
 __device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
     const int lane = threadIdx.x & 31;
     const u64 c = __ldcg(&gl->coarse[31 - lane]);
@@ -143,16 +145,17 @@ __device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
     }
     const int at = __ffs(hit) - 1;
     const u64 above = __shfl_sync(kFull, incl - c, at);
-    const int top = (31 - at) * 128 + 127 - 4 * lane;
-    u64 v[4], sum = 0;
+    constexpr int per = kSub / 32;
+    const int top = (31 - at) * kSub + kSub - 1 - per * lane;
+    u64 v[per], sum = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]);
+    for (int k = 0; k < per; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]);
     const u64 incl2 = warp_inclusive(sum);
     const int at2 = __ffs(__ballot_sync(kFull, above + incl2 >= want)) - 1;
     if (lane == at2) {
         u64 run = above + incl2 - sum;
         int k = 0;
-        while (k < 3 && run + v[k] < want) run += v[k++];
+        while (k < per - 1 && run + v[k] < want) run += v[k++];
         *iv = Interval{bin_edge(top - k), bin_edge(top - k + 1), want - run, v[k]};
     }
 }
@@ -190,9 +193,9 @@ __device__ void flush_first(Shared& sh, SelectGlobal* gl) {
     for (int o = warp; o < 32; o += kWarps) {
         unsigned int sum = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const unsigned int v = sh.hist[o * 128 + k * 32 + lane];
-            if (v) atomicAdd(&gl->fine[o * 128 + k * 32 + lane], (u64)v);
+        for (int k = 0; k < kSub / 32; ++k) {
+            const unsigned int v = sh.hist[o * kSub + k * 32 + lane];
+            if (v) atomicAdd(&gl->fine[o * kSub + k * 32 + lane], (u64)v);
             sum += v;
         }
         sum = __reduce_add_sync(kFull, sum);
@@ -264,15 +267,23 @@ struct SelectArgs {
     int W;                   // lanes per row (power of two)
     int rows;                // rows per block
     int stride;              // resident rows in shared memory: entries per row (0: rows stay in global memory)
+    int keep_last;           // rows in global memory: the last gain of each row is kept in shared memory
     double T;
     long long want;
     SelectGlobal* gl;
     SelectState* sel;
     long long* counters;
-    int32_t *gt, *eq, *list;
+    int32_t *gt, *eq;
     int32_t *alloc, *last_alloc, *out_alloc;
     double* reduction;
     int32_t* err_word;
+    // after the last row: what the next epoch finds cleared, the published statistics, and the host's mailbox
+    void* zero;
+    int zero_words;
+    long long* published;
+    Mailbox* mail;
+    int32_t* mail_alloc;
+    uint32_t seq;
 };
 
 namespace {
@@ -280,30 +291,33 @@ namespace {
 __device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int cores, double R, bool active) {
     a.alloc[j] = cores;
     if (a.out_alloc) a.out_alloc[j] = cores;
+    if (a.mail_alloc) a.mail_alloc[j] = cores;
     if (active && a.last_alloc) a.last_alloc[j] = cores;
     a.reduction[j] = R;
 }
 
+// A row's candidates, entries s .. s+c-1, for the block that ranks them.  The first of them carries the row's count.
+__device__ __forceinline__ void list_candidates(const SelectArgs& a, int j, int s, int c, const double* row) {
+    const int at = (int)atomicAdd(&a.gl->n_cand, (unsigned int)c);
+    for (int k = 0; k < c && at + k < kFinal; ++k) {
+        a.gl->cand_key[at + k] = key_of(row[s + k]);
+        a.gl->cand_pos[at + k] = ((u64)(k == 0 ? c : 0) << 48) | ((u64)j << 10) | (u64)(s + k);
+    }
+}
+
+constexpr u64 kPosMask = (1ull << 48) - 1;
+
 // The last block: hand out `iv.want` of the n <= kFinal candidates, best first, and complete their rows.
 __device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
     const int tid = threadIdx.x;
-    const int rows = min((int)__ldcg(&a.gl->n_list), kFinal);
-    if (tid == 0) sh.count = 0;
-    __syncthreads();
-    for (int r = tid; r < rows; r += kThreads) {
-        const int j = __ldcg(&a.list[r]);
-        const int s = __ldcg(&a.gt[j]), c = __ldcg(&a.eq[j]);
-        sh.take[r] = 0;
-        const int off = atomicAdd(&sh.count, c);
-        for (int i = 0; i < c && off + i < kFinal; ++i) {
-            sh.cand.key[off + i] = key_of(__ldcg(&a.gain[(size_t)j * a.cap + s + i]));
-            sh.cand.pos[off + i] = ((u64)j << 10) | (u64)(s + i);
-            sh.own[off + i] = (unsigned short)r;
-            sh.idx[off + i] = (unsigned short)(off + i);
-        }
+    const int all = min((int)__ldcg(&a.gl->n_cand), kFinal);
+    for (int i = tid; i < all; i += kThreads) {
+        sh.cand.key[i] = __ldcg(&a.gl->cand_key[i]);
+        sh.cand.pos[i] = __ldcg(&a.gl->cand_pos[i]);
+        sh.idx[i] = (unsigned short)i;
+        sh.taken[i] = 0;
     }
-    __syncthreads();
-    int n = min(sh.count, kFinal);
+    int n = all;
     __syncthreads();
     while (n > kRankDirect && sh.iv.hi - sh.iv.lo > 1) {
         const int shift = narrow_shift(sh.iv);
@@ -312,63 +326,81 @@ __device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
         if (tid == 0) sh.count = 0;
         __syncthreads();
         int mine[kFinal / kThreads];
-        int m = 0;
-        for (int i = tid; i < n; i += kThreads) {
-            mine[m++] = sh.idx[i];
-            atomicAdd(&sh.narrow[(sh.cand.key[sh.idx[i]] - lo) >> shift], 1u);
+#pragma unroll
+        for (int m = 0; m < kFinal / kThreads; ++m) {
+            const int i = tid + m * kThreads;
+            mine[m] = i < n ? sh.idx[i] : -1;
+            if (i < n) atomicAdd(&sh.narrow[(sh.cand.key[mine[m]] - lo) >> shift], 1u);
         }
         __syncthreads();
         pick_narrow([&](int b) { return (u64)sh.narrow[b]; }, sh);
         const u64 lo2 = sh.iv.lo, hi2 = sh.iv.hi;
-        for (int i = 0; i < m; ++i) {
-            const u64 key = sh.cand.key[mine[i]];
-            if (key >= hi2) atomicAdd(&sh.take[sh.own[mine[i]]], 1);
-            else if (key >= lo2) sh.idx[atomicAdd(&sh.count, 1)] = (unsigned short)mine[i];
+#pragma unroll
+        for (int m = 0; m < kFinal / kThreads; ++m) {
+            if (mine[m] < 0) continue;
+            const u64 key = sh.cand.key[mine[m]];
+            if (key >= hi2) sh.taken[mine[m]] = 1;
+            else if (key >= lo2) sh.idx[atomicAdd(&sh.count, 1)] = (unsigned short)mine[m];
         }
         __syncthreads();
         n = sh.count;
         __syncthreads();
     }
-    // what is left is ranked outright
+    // what is left is ranked outright: 2^k threads share a candidate's comparisons
     const u64 want = sh.iv.want;
     if (tid == 0) sh.scan[0] = 0, sh.count = 0;
+    for (int i = tid; i < n; i += kThreads) sh.narrow[i] = 0;
+    __syncthreads();
+    int share = 1;
+    while (share < 32 && 2 * share * n <= kThreads) share <<= 1;
+    for (int i = tid / share; i < n; i += kThreads / share) {
+        const int e = sh.idx[i];
+        const u64 key = sh.cand.key[e], pos = sh.cand.pos[e] & kPosMask;
+        unsigned int rank = 0;
+#pragma unroll 4
+        for (int k = tid & (share - 1); k < n; k += share) {
+            const int f = sh.idx[k];
+            const u64 other = sh.cand.key[f], other_pos = sh.cand.pos[f] & kPosMask;
+            rank += (other > key || (other == key && other_pos < pos)) ? 1 : 0;
+        }
+        if (rank) atomicAdd(&sh.narrow[i], rank);
+    }
     __syncthreads();
     for (int i = tid; i < n; i += kThreads) {
-        const int e = sh.idx[i];
-        const u64 key = sh.cand.key[e], pos = sh.cand.pos[e];
-        u64 rank = 0;
-        for (int k = 0; k < n; ++k) {
-            const int f = sh.idx[k];
-            const u64 other = sh.cand.key[f];
-            rank += (other > key || (other == key && sh.cand.pos[f] < pos)) ? 1 : 0;
-        }
-        if (rank < want) atomicAdd(&sh.take[sh.own[e]], 1);
-        if (rank + 1 == want) sh.scan[0] = key;
+        const u64 rank = sh.narrow[i];
+        if (rank < want) sh.taken[sh.idx[i]] = 1;
+        if (rank + 1 == want) sh.scan[0] = sh.cand.key[sh.idx[i]];
     }
     __syncthreads();
     const u64 tau = sh.scan[0];
     int above = 0;   // all of them are taken; what is left of `want` goes to gains equal to tau
     for (int i = tid; i < n; i += kThreads) above += sh.cand.key[sh.idx[i]] > tau ? 1 : 0;
     if (above) atomicAdd(&sh.count, above);
-    __syncthreads();
-    if (tid == 0) {
-        a.sel->prefix = tau;
-        a.counters[7] = (long long)want - sh.count;
-    }
     long long handed = 0;
-    for (int r = tid; r < rows; r += kThreads) {
-        const int j = __ldcg(&a.list[r]), s = __ldcg(&a.gt[j]), t = sh.take[r];
+    for (int i = tid; i < all; i += kThreads) {
+        const u64 pos = sh.cand.pos[i];
+        const int c = (int)(pos >> 48);
+        if (c == 0) continue;          // not the first candidate of its row
+        const int j = (int)((pos & kPosMask) >> 10), s = (int)(pos & 1023);
         double R = __ldcg(&a.reduction[j]);
-        for (int i = 0; i < t; ++i) R += __ldcg(&a.gain[(size_t)j * a.cap + s + i]);
+        int t = 0;                     // the taken ones of a row are its first
+        while (t < c && sh.taken[i + t]) R += __longlong_as_double((long long)sh.cand.key[i + t++]);
         store_alloc(a, j, s + t, R, true);
         handed += s + t;
     }
-    if (handed) atomicAdd((u64*)&a.counters[6], (u64)handed);
+    u64 sum;
+    block_exclusive((u64)handed, sh, &sum);
+    if (tid == 0) {
+        atomicAdd((u64*)&a.counters[6], sum);
+        a.sel->prefix = tau;
+        a.counters[7] = (long long)want - sh.count;
+    }
 }
 
 // All blocks: narrow the interval over the rows' candidate segments (gt, eq) until kFinal candidates are left or all
-// are equal; equal ones are handed out here.  Returns whether the last block still has candidates to rank.
-__device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j1, unsigned int& arrived) {
+// are equal; equal ones are handed out here.  Returns whether the last block still has candidates to rank, -1 after a
+// barrier that was not reached.
+__device__ int narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j1, unsigned int& arrived) {
     const int tid = threadIdx.x;
     for (int step = 0; sh.iv.hi - sh.iv.lo > 1 && sh.iv.n > kFinal && step < kRadixPasses; ++step) {
         const int shift = narrow_shift(sh.iv);
@@ -388,7 +420,7 @@ __device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int 
         for (int b = tid; b < kNarrowBins; b += kThreads)
             if (sh.narrow[b]) atomicAdd(&global[b], (u64)sh.narrow[b]);
         arrived += gridDim.x;
-        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return -1;
         pick_narrow([&](int b) { return __ldcg(&global[b]); }, sh);
         const u64 lo2 = sh.iv.lo, hi2 = sh.iv.hi;
         for (int j = j0 + tid; j < j1; j += kThreads) {
@@ -417,7 +449,7 @@ __device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int 
     if (equal) {
         if (tid == 0) a.gl->block_eq[blockIdx.x] = (long long)total;
         arrived += gridDim.x;
-        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return -1;
         u64 part = 0;
         for (int b = tid; b < (int)blockIdx.x; b += kThreads) part += (u64)__ldcg(&a.gl->block_eq[b]);
         block_exclusive(part, sh, &before);
@@ -432,7 +464,7 @@ __device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int 
         if (j >= j1 || (a.count && a.count[j] <= 0)) continue;
         const int s = a.gt[j];
         if (!equal && c) {
-            a.list[atomicAdd(&a.gl->n_list, 1u)] = j;
+            list_candidates(a, j, s, c, a.gain + (size_t)j * a.cap);
             continue;
         }
         const int take = ahead >= sh.iv.want ? 0 : (int)min((u64)c, sh.iv.want - ahead);
@@ -450,13 +482,45 @@ __device__ bool narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int 
         if (tid == 0 && sum) atomicAdd((u64*)&a.counters[7], sum);
         if (tid == 0 && blockIdx.x == 0) a.sel->prefix = sh.iv.lo;
     }
-    return !equal;
+    return equal ? 0 : 1;
+}
+
+// Whether this is the last block to get here; it then sees what the others wrote.
+__device__ bool arrive_last(const SelectArgs& a, Shared& sh) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (a.mail_alloc) __threadfence_system();   // the block's share of the allocation is on its way to the host
+        else __threadfence();
+        sh.flag = atomicAdd(&a.gl->ticket, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return sh.flag != 0;
+}
+
+// The last block, after everything else: publish the statistics, tell the host, clear the scratch for the next epoch.
+__device__ void finish_epoch(const SelectArgs& a) {
+    const int tid = threadIdx.x;
+    __syncthreads();
+    if (a.published && tid < 16)
+        a.published[tid] = tid == 15 ? (long long)__ldcg(&a.sel->prefix) : __ldcg(&a.counters[tid]);
+    if (a.mail) {
+        if (tid == 0) {
+            a.mail->err = __ldcg(a.err_word);
+            __threadfence_system();
+            a.mail->done = a.seq;
+        }
+    }
+    if (a.zero) {
+        __syncthreads();
+        for (int i = tid; i < a.zero_words; i += kThreads) static_cast<u64*>(a.zero)[i] = 0;
+    }
 }
 
 // kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
 // were continued); otherwise the table is read.
 template <bool kCurves>
-__global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_constant__ SelectArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_constant__ SelectArgs a) {
     extern __shared__ double dyn[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
@@ -465,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_consta
     CurveTile tile;
     tile.v = dyn;
     tile.kind = reinterpret_cast<int*>(dyn + 7 * kThreads);
-    double* const rows_sh = dyn + (kCurves ? 7 * kThreads + kThreads / 2 : 0);
+    double* const rows_sh = dyn + (kCurves ? 7 * kThreads + kThreads / 2 : 0);   // resident rows, or each row's last gain
     unsigned int arrived = 0;
 
     for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
@@ -520,6 +584,7 @@ __global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_consta
                     g = row[i];
                 }
                 if (has && resident) rows_sh[(base - j0 + r) * a.stride + i] = g;
+                else if (has && a.keep_last && i == a.depth - 1) rows_sh[base - j0 + r] = g;
                 count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
             }
         }
@@ -548,7 +613,7 @@ __global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_consta
             __syncthreads();
             const int mine = base + tid;
             if (mine < j1 && (!a.count || a.count[mine] > 0) &&
-                key_of(a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound)
+                key_of(a.keep_last ? rows_sh[mine - j0] : a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound)
                 sh.narrow[atomicAdd(&sh.n_more, 1)] = (unsigned int)mine;
             __syncthreads();
             const int n_more = sh.n_more;
@@ -598,30 +663,66 @@ __global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_consta
     const Interval iv = sh.iv;
     const bool few = iv.n <= kFinal;
     long long handed = 0;
-    for (int j = j0 + tid; j < j1; j += kThreads) {
-        const bool active = !a.count || a.count[j] > 0;
+    const int lane = tid & 31;
+    // a few rows per block are spread over its warps, one per warp at first
+    const int pitch = j1 - j0 <= kThreads / 4 ? kWarps : 1;
+    const int slot0 = pitch == 1 ? tid & ~31 : tid >> 5, slot = slot0 + pitch * lane;
+    for (int base = j0; base < j1; base += kThreads) {   // uniform trip count: a warp finishes its long rows together
+        const int j = base + slot;
+        const bool in = j < j1, active = in && (!a.count || a.count[j] > 0);
+        const double* row = resident ? rows_sh + (size_t)(j - j0) * a.stride : a.gain + (size_t)j * a.cap;
         int s = 0, c = 0;
         double R = 0.0;
+        bool more = false;
         if (active) {
-            const double* row = resident ? rows_sh + (size_t)(j - j0) * a.stride : a.gain + (size_t)j * a.cap;
             if (a.first_unit == 2) R = row[0], s = 1;
-            while (s < a.cap) {
-                const double g = row[s];
-                if (key_of(g) < iv.hi) break;
-                R += g;
-                ++s;
+            const int end = min(a.cap, kShortWalk);
+            more = s < a.cap;
+            while (more && s < end) {
+                double g[4];   // four loads in flight; entries behind a row's first gain below the interval mean nothing
+#pragma unroll
+                for (int k = 0; k < 4; ++k) g[k] = s + k < end ? row[s + k] : 0.0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (more && s < end) {
+                        if (key_of(g[k]) >= iv.hi) R += g[k], ++s;
+                        else more = false;
+                    }
+                }
             }
-            while (s + c < a.cap && key_of(row[s + c]) >= iv.lo) ++c;
+            more = more && s < a.cap;   // every gain so far is handed out
         }
+        for (unsigned todo = __ballot_sync(kFull, more); todo; todo &= todo - 1) {
+            const int r = __ffs(todo) - 1;
+            const int jr = base + slot0 + pitch * r;
+            const double* far = resident ? rows_sh + (size_t)(jr - j0) * a.stride : a.gain + (size_t)jr * a.cap;
+            int at = __shfl_sync(kFull, s, r);
+            double sum = __shfl_sync(kFull, R, r);
+            for (bool on = true; on && at < a.cap;) {
+                const double g = at + lane < a.cap ? far[at + lane] : 0.0;
+                const unsigned stop = __ballot_sync(kFull, at + lane >= a.cap || key_of(g) < iv.hi);
+                const int n = stop ? __ffs(stop) - 1 : 32;
+                for (int k = 0; k < n; ++k) sum += __shfl_sync(kFull, g, k);   // in order, as the row's own thread adds
+                at += n;
+                on = n == 32;
+            }
+            if (lane == r) s = at, R = sum;
+        }
+        if (!in) continue;
+        if (active)
+            while (s + c < a.cap && key_of(row[s + c]) >= iv.lo) ++c;
         if (few && c == 0) {
             store_alloc(a, j, s, R, active);
             handed += s;
         } else {
-            a.gt[j] = s;
-            a.eq[j] = c;
             a.reduction[j] = R;
-            if (few) a.list[atomicAdd(&a.gl->n_list, 1u)] = j;
-            else if (!active) store_alloc(a, j, 0, 0.0, false);
+            if (few) {
+                list_candidates(a, j, s, c, row);
+            } else {
+                a.gt[j] = s;
+                a.eq[j] = c;
+                if (!active) store_alloc(a, j, 0, 0.0, false);
+            }
         }
     }
     if (few) {
@@ -630,27 +731,29 @@ __global__ void __launch_bounds__(kThreads, 2) select_kernel(const __grid_consta
         if (tid == 0 && sum) atomicAdd((u64*)&a.counters[6], sum);
     } else {
         __syncthreads();
-        if (!narrow_on_the_grid(a, sh, j0, j1, arrived)) return;
+        const int next = narrow_on_the_grid(a, sh, j0, j1, arrived);
+        if (next < 0) return;
+        if (next == 0) {
+            if (arrive_last(a, sh)) finish_epoch(a);
+            return;
+        }
     }
 
     // ---- C: the last block to get here ranks the candidates ----
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) sh.flag = atomicAdd(&a.gl->ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!sh.flag) return;
-    __threadfence();
+    if (!arrive_last(a, sh)) return;
     if (sh.iv.n > 0) finish_candidates(a, sh);
     else if (tid == 0) a.sel->prefix = ~0ull;
+    finish_epoch(a);
 }
 
 }  // namespace
 
-// Rule for the rows' home.  Up to kResidentGains gains per block (four evaluations per thread) all of them are predicted
+// Rule for the rows' home.  Up to kResidentGains gains per block (two evaluations per thread) all of them are predicted
 // at once, kept in shared memory and walked there; the whole table is written as well.  Beyond that prediction is what
 // costs (910 us for 128 gains of a million jobs each), so rows start with four times the average number of
 // cores handed out, at least 16, and only rows that need more are continued.
-constexpr int kResidentGains = 4 * kThreads;
+constexpr int kResidentGains = 2048;
+constexpr int kKeepLast = 8192;
 
 static size_t select_smem(bool curves, int rows, int stride) {
     return sizeof(double) * ((curves ? 7 * kThreads + kThreads / 2 : 0) + (size_t)rows * stride);
@@ -658,10 +761,10 @@ static size_t select_smem(bool curves, int rows, int stride) {
 
 int select_setup(int* blocks_per_sm) {
     int per_sm = 1;
-    const size_t most = select_smem(true, kResidentGains, 2) + 1024;
+    const size_t most = select_smem(true, kKeepLast, 1);
     if (cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
     if (cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true>, kThreads, select_smem(true, 0, 0)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true>, kThreads, most) != cudaSuccess)
         return -1;
     *blocks_per_sm = per_sm < 1 ? 1 : per_sm;
     return 0;
@@ -686,6 +789,7 @@ static cudaError_t launch_select(SelectArgs& a, bool curves, int sm_count, int b
         grid = (int)std::min<long long>(sm_count, std::max<long long>(1, (gains + kThreads - 1) / kThreads));
         a.rows = (a.J + grid - 1) / grid;
         grid = (a.J + a.rows - 1) / a.rows;
+        a.keep_last = 0;
         a.stride = a.cap | 1;   // odd: threads walking neighbouring rows meet different banks
         smem = select_smem(curves, a.rows, a.stride);
     } else {
@@ -695,14 +799,16 @@ static cudaError_t launch_select(SelectArgs& a, bool curves, int sm_count, int b
         a.rows = (a.J + grid - 1) / grid;
         grid = (a.J + a.rows - 1) / a.rows;
         a.stride = 0;
-        smem = select_smem(curves, 0, 0);
+        a.keep_last = a.depth < a.cap && a.rows <= kKeepLast;
+        smem = select_smem(curves, a.keep_last ? a.rows : 0, 1);
     }
     void* args[] = {&a};
     return cudaLaunchCooperativeKernel(curves ? (const void*)select_kernel<true> : (const void*)select_kernel<false>, dim3(grid),
                                        dim3(kThreads), args, smem, st);
 }
 
-int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc) {
+int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
+                  uint32_t seq) {
     SelectArgs a;
     a.job = h->job;
     a.fit = h->fit;
@@ -718,12 +824,17 @@ int launch_select(slaq_handle* h, double epoch_seconds, long long want, int firs
     a.counters = h->scratch.counters;
     a.gt = h->scratch.gt;
     a.eq = h->scratch.eq;
-    a.list = h->scratch.list;
     a.alloc = h->alloc;
     a.last_alloc = h->job.last_alloc;
     a.out_alloc = d_out_alloc;
     a.reduction = h->reduction;
     a.err_word = h->err_word;
+    a.zero = h->scratch.zero;
+    a.zero_words = (int)(h->scratch.zero_bytes / sizeof(u64));
+    a.published = h->scratch.published;
+    a.mail = seq ? h->mailbox : nullptr;
+    a.mail_alloc = seq && h->max_jobs <= h->mailbox_jobs ? h->mail_alloc() : nullptr;
+    a.seq = seq;
     const cudaError_t e = launch_select(a, from_curves, h->sm_count, h->select_blocks_per_sm, h->stream);
     if (e != cudaSuccess) {
         h->err = std::string("selection launch: ") + cudaGetErrorString(e);
@@ -748,7 +859,7 @@ struct StaticScratch {
     SelectGlobal gl;                 // its leading part is cleared every call
     SelectState sel;                 // rewritten every call
     long long counters[16];
-    int32_t gt[kStaticMaxJobs], eq[kStaticMaxJobs], list[kStaticMaxJobs];   // written before they are read
+    int32_t gt[kStaticMaxJobs], eq[kStaticMaxJobs];   // written before they are read
 };
 
 static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
@@ -814,7 +925,6 @@ extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_
     a.counters = dev.scratch->counters;
     a.gt = dev.scratch->gt;
     a.eq = dev.scratch->eq;
-    a.list = dev.scratch->list;
     a.alloc = d_out_alloc;
     a.reduction = d_out_reduction;
     if (launch_select(a, false, dev.sm_count, dev.blocks_per_sm, st) != cudaSuccess) return SLAQ_E_CUDA;
