@@ -262,9 +262,19 @@ sweep_loop_kernel(const double* __restrict__ g_wtab, int L, int rows, int n_swee
             if (kVariant == 1) sweep_tables(S, kTable, fam, H, rows, inv_span, pI, true, pII, true, sums);
             else if (kVariant == 2) sweep_products(S, fam, H, rows, inv_span, pI, true, pII, true, sums);
             else slaq::sweep(S, fam, H, rows, inv_span, pI, true, pII, true, sums);
-            check += sums.v[fam ? 8 : 12];
-            if (it == n_sweeps - 1 && blockIdx.x == 0 && warp == 0)
-                for (int i = 0; i < 13; ++i) last_sums[lane * 13 + i] = (i < 9 || !fam) ? sums.v[i] : 0.0;
+            check += kVariant == 0 ? sums.S : sums.v[fam ? 8 : 12];
+            if (it == n_sweeps - 1 && blockIdx.x == 0 && warp == 0) {
+                if (kVariant == 0) {   // a lane holds its share of the sums: written down for all lanes of its group and family
+                    int from, own;
+                    S.held(from, own);
+                    for (int i = 0; i < 13; ++i)
+                        if (i < own)
+                            for (int q = fam; q < 32; q += 2)
+                                if ((S.group() >> q) & 1u) last_sums[q * 13 + from + i] = sums.v[i];
+                } else {
+                    for (int i = 0; i < 13; ++i) last_sums[lane * 13 + i] = (i < 9 || !fam) ? sums.v[i] : 0.0;
+                }
+            }
             // move the points a little, as accepted trials do (keeps every sweep's arithmetic live)
             pI[2] = fma(pI[2], 1.0 + 1e-9, sums.usable ? 0.0 : 1e-12);
             pII[0] = fma(pII[0], 1.0 - 1e-9, 0.0);

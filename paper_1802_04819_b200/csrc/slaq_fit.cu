@@ -260,8 +260,9 @@ __device__ bool ldl_solve(const Sym4& B, const double (&r)[4], double (&x)[4]) {
     const double l32 = t32 * i2;
     const double d3 = fma(-l32, t32, fma(-l31, t31, fma(-l30, B.a03, B.a33)));
     const double i3 = fast_rcp(d3);
-    bool ok = d0 > 0.0 && d1 > 0.0 && d2 > 0.0 && d3 > 0.0 && finite_d(d0) && finite_d(d1) && finite_d(d2) &&
-              finite_d(d3);
+    // positive and finite, read off the high words (a subnormal pivot counts as zero: its reciprocal is not finite)
+    const int h0 = __double2hiint(d0), h1 = __double2hiint(d1), h2 = __double2hiint(d2), h3 = __double2hiint(d3);
+    bool ok = min(min(h0, h1), min(h2, h3)) > 0 && max(max(h0, h1), max(h2, h3)) < 0x7ff00000;
     const double z0 = r[0];
     const double z1 = fma(-l10, z0, r[1]);
     const double z2 = fma(-l21, z1, fma(-l20, z0, r[2]));
@@ -270,7 +271,9 @@ __device__ bool ldl_solve(const Sym4& B, const double (&r)[4], double (&x)[4]) {
     x[2] = fma(-l32, x[3], z2 * i2);
     x[1] = fma(-l31, x[3], fma(-l21, x[2], z1 * i1));
     x[0] = fma(-l30, x[3], fma(-l20, x[2], fma(-l10, x[1], z0 * i0)));
-    ok = ok && finite_d(x[0]) && finite_d(x[1]) && finite_d(x[2]) && finite_d(x[3]);
+    const int m = 0x7ff00000;
+    ok = ok && max(max(__double2hiint(x[0]) & m, __double2hiint(x[1]) & m),
+                   max(__double2hiint(x[2]) & m, __double2hiint(x[3]) & m)) < m;
     return ok;
 }
 
@@ -288,20 +291,14 @@ struct Family {
     bool has_trial;    // the running sweep evaluates the trial point
 };
 
-// Lower bounds.  Family I (fam 0): a >= 0, b >= 0, c >= 1e-12 keep the curve non-increasing ahead
-// of the newest point and its denominator positive there.  Family II (fam 1): beta >= 0.
-__device__ __forceinline__ double lower_bound_of(int fam, int a) {
-    if (fam == 0) return a == 3 ? -CUDART_INF : (a == 2 ? 1e-12 : 0.0);
-    return a == 1 ? 0.0 : -CUDART_INF;
-}
-
 // One Levenberg-Marquardt trial up to the point where the model must be evaluated: freeze
 // parameters that sit on their bound while the descent direction or the solved step points
 // outside (and keep them frozen from then on), solve (A + lambda diag A) step = g over the
 // rest, clip the trial point to the bounds, and record the reduction the quadratic model
-// promises.  `busy` = this lane has a trial to prepare; the re-solve loop runs while any
-// lane of the warp needs another round.  Family II has three parameters: its fourth row is
-// a fixed identity row.
+// promises.  Lower bounds: a >= 0, b >= 0, c >= 1e-12 of family I keep the curve non-increasing ahead of the newest
+// point and its denominator positive there; beta >= 0 of family II.  `busy` = this lane has a trial to prepare; the
+// re-solve loop runs while any lane of the warp needs another round (each freezes at least one more of the three
+// bounded parameters).  Family II has three parameters: its fourth row is a fixed identity row.
 __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&g)[4], bool busy, double sum_wy2,
                               double (&trial)[4]) {
     F.has_trial = false;
@@ -309,25 +306,25 @@ __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&
         F.done = true;
         busy = false;
     }
-    const int P = fam == 0 ? 4 : 3;
-    double lo[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) lo[a] = lower_bound_of(fam, a);
-    unsigned frozen = fam == 0 ? 0u : 8u;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-        if (a < P && F.p[a] <= lo[a] && (g[a] < 0.0 || ((F.was_frozen >> a) & 1u))) frozen |= 1u << a;
+    const bool one = fam == 0;
+    const bool at0 = one && F.p[0] <= 0.0, at1 = F.p[1] <= 0.0, at2 = one && F.p[2] <= 1e-12;   // on their bounds
+    unsigned frozen = one ? 0u : 8u;
+    if (at0 && (g[0] < 0.0 || (F.was_frozen & 1u))) frozen |= 1u;
+    if (at1 && (g[1] < 0.0 || (F.was_frozen & 2u))) frozen |= 2u;
+    if (at2 && (g[2] < 0.0 || (F.was_frozen & 4u))) frozen |= 4u;
+    // the damped diagonal
+    auto damped = [&](double d) { return fma(F.lambda, d < 1e-300 ? 1e-300 : d, d); };
+    const double D0 = damped(A.a00), D1 = damped(A.a11), D2 = damped(A.a22), D3 = damped(A.a33);
     double step[4] = {0.0, 0.0, 0.0, 0.0};
     bool solved = false, again = busy;
-    for (int round = 0; round <= 4; ++round) {
-        if (!__any_sync(kFull, again)) break;
-        if (again && round <= P) {
+    while (__any_sync(kFull, again)) {
+        if (again) {
             const bool f0 = frozen & 1u, f1 = frozen & 2u, f2 = frozen & 4u, f3 = frozen & 8u;
             Sym4 B;
-            B.a00 = f0 ? 1.0 : fma(F.lambda, fmax(A.a00, 1e-300), A.a00);
-            B.a11 = f1 ? 1.0 : fma(F.lambda, fmax(A.a11, 1e-300), A.a11);
-            B.a22 = f2 ? 1.0 : fma(F.lambda, fmax(A.a22, 1e-300), A.a22);
-            B.a33 = f3 ? 1.0 : fma(F.lambda, fmax(A.a33, 1e-300), A.a33);
+            B.a00 = f0 ? 1.0 : D0;
+            B.a11 = f1 ? 1.0 : D1;
+            B.a22 = f2 ? 1.0 : D2;
+            B.a33 = f3 ? 1.0 : D3;
             B.a01 = (f0 || f1) ? 0.0 : A.a01;
             B.a02 = (f0 || f2) ? 0.0 : A.a02;
             B.a03 = (f0 || f3) ? 0.0 : A.a03;
@@ -337,15 +334,12 @@ __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&
             const double rhs[4] = {f0 ? 0.0 : g[0], f1 ? 0.0 : g[1], f2 ? 0.0 : g[2], f3 ? 0.0 : g[3]};
             solved = ldl_solve(B, rhs, step);
             unsigned grow = 0;
-            if (solved) {
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-                    if (a < P && !((frozen >> a) & 1u) && F.p[a] <= lo[a] && step[a] < 0.0) grow |= 1u << a;
-            }
+            if (at0 && step[0] < 0.0) grow |= 1u;
+            if (at1 && step[1] < 0.0) grow |= 2u;
+            if (at2 && step[2] < 0.0) grow |= 4u;
+            grow = solved ? grow & ~frozen : 0u;
             frozen |= grow;
-            again = solved && grow != 0;
-        } else {
-            again = false;
+            again = grow != 0;
         }
     }
     if (!busy) return;
@@ -357,10 +351,12 @@ __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&
     }
     double d[4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        trial[a] = a < P ? fmax(F.p[a] + step[a], lo[a]) : 0.0;
-        d[a] = trial[a] - F.p[a];
-    }
+    for (int a = 0; a < 4; ++a) trial[a] = F.p[a] + step[a];
+    if (one && trial[0] < 0.0) trial[0] = 0.0;
+    if (trial[1] < 0.0) trial[1] = 0.0;
+    if (one && trial[2] < 1e-12) trial[2] = 1e-12;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) d[a] = trial[a] - F.p[a];
     const double dg = fma(d[0], g[0], fma(d[1], g[1], fma(d[2], g[2], d[3] * g[3])));
     const double Ad0 = fma(A.a00, d[0], fma(A.a01, d[1], fma(A.a02, d[2], A.a03 * d[3])));
     const double Ad1 = fma(A.a01, d[0], fma(A.a11, d[1], fma(A.a12, d[2], A.a13 * d[3])));
@@ -396,15 +392,27 @@ __device__ __forceinline__ bool finish_trial(Family& F, const double (&trial)[4]
 }
 
 // The sums of the last accepted point live in shared memory between sweeps, one column per job
-// and family: after the reduction every lane of a group's parity holds the same sums, so the
-// group's first two lanes write them for all.  Every lane of the warp calls this; `keep` says
+// and family: every lane writes the ones it holds.  Every lane of the warp calls this; `keep` says
 // whether the lane's family has new sums to park.
 __device__ __forceinline__ void park(const Lanes& S, const SweepSums& s, bool keep) {
-    if (keep && S.l < 2) {
+    if (keep) {
         const int n = S.park_stride();
+        if (S.L == 2) {
 #pragma unroll
-        for (int k = 0; k < kParked; ++k)
-            if (S.holds(S.park + k * n)) S.park[k * n] = s.v[k];
+            for (int k = 0; k < kParked; ++k)
+                if (S.holds(S.park + k * n)) S.park[k * n] = s.v[k];
+        } else {
+            int from, own;
+            S.held(from, own);
+            own = min(own, kParked - from);   // the objective of family I is not parked
+            double* const at = S.park + from * n;
+            const int most = S.L == 32 ? 1 : S.L == 16 ? 2 : S.L == 8 ? 4 : 7;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                if (k >= most) break;
+                if (k < own && S.holds(at + k * n)) at[k * n] = s.v[k];
+            }
+        }
     }
     __syncwarp();
 }
@@ -750,7 +758,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
 #pragma unroll
             for (int a = 0; a < 4; ++a) F.p[a] = fam ? pII[a] : pI[a];
             F.ok = fits && sums.usable;
-            F.S = sums.v[fam ? 8 : 12];
+            F.S = sums.S;
             F.lambda = kLambda0;
             F.nu = 2.0;
             F.was_frozen = 0;
@@ -778,7 +786,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
                     pII[a] = __shfl_sync(kFull, trial[a], oddl);
                 }
                 sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
-                park(S, sums, finish_trial(F, trial, sums.usable, sums.v[fam ? 8 : 12]));
+                park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
                 SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
             }
             // both results of the job, in every lane

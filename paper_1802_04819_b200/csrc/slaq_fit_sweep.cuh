@@ -36,6 +36,21 @@ struct Lanes {
     const double* wtab;
     int lane, L, l;
     __device__ __forceinline__ int park_stride() const { return 64 >> (__ffs(L) - 1); }   // 2 * (32 / L), L a power of two
+    // Which of its family's 13 sums the lane holds after a sweep's reduction (see halve): `n` of them from the `from`-th on.
+    __device__ __forceinline__ void held(int& from, int& n) const {
+        from = 0, n = 13;
+        if (L >= 4) { const int b = (lane >> 1) & 1; from = 7 * b; n = 7 - b; }
+        if (L >= 8) { const int b = (lane >> 2) & 1; from += 4 * b; n = b ? n - 4 : 4; }
+        if (L >= 16) { const int b = (lane >> 3) & 1; from += 2 * b; n = b ? max(n - 2, 0) : min(n, 2); }
+        if (L >= 32) { const int b = (lane >> 4) & 1; from += b; n = b ? max(n - 1, 0) : min(n, 1); }
+    }
+    // Where the steps of the reduction leave the objective: sum 12 of family I, sum 8 of family II.
+    __device__ __forceinline__ int objective_lane() const {
+        return (lane & -L) + (lane & 1) + 2 + (L >= 8 && !(lane & 1) ? 4 : 0) + (L >= 32 ? 16 : 0);
+    }
+    __device__ __forceinline__ unsigned group() const {   // the lanes of this lane's job
+        return (0xffffffffu >> (32 - L)) << (lane & -L);
+    }
     // extents, read by the bounds build only: the warp's slice [slice, slice + slice_len) and the weight table
     const double* slice;
     int slice_len, wtab_len;
@@ -61,13 +76,14 @@ __device__ __forceinline__ double older_neighbour(const Lanes& S, int k) {
     return S.holds(p) ? *p : 0.0;
 }
 
-// What a lane keeps of one sweep: the sums of ITS family over the whole window.
+// What a lane keeps of one sweep: its share of the sums of ITS family over the whole window (see Lanes::held), and the objective.
 // Family I (u = 1/q^2, J = (-u x^2, -u x, -u, 1)): v[0..4] = sum w u^2 x^k, v[5..7] = sum w u x^k,
 // v[8..10] = sum w u r x^k, v[11] = sum w r, v[12] = S.
 // Family II (J = (e, -x e, 1)): v[0..2] = sum w e^2 x^k, v[3..4] = sum w e x^k, v[5..6] = sum w e r x^k,
 // v[7] = sum w r, v[8] = S.
 struct SweepSums {
     double v[13];
+    double S;      // the objective
     bool usable;   // the model was defined at every point and all sums are finite
 };
 
@@ -168,12 +184,26 @@ __device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all,
         if (i <= k_last) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);   // row k_last - i >= 0
 }
 
+// One step of the reduction over the lanes of a group: of N sums a lane keeps the lower K (bit `o` of its number clear) or
+// the upper N - K (set), and adds the partner's.
+template <int K, int N>
+__device__ __forceinline__ void halve(double (&v)[13], int o, int lane) {
+    const bool upper = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const double hi = K + k < N ? v[K + k] : 0.0;
+        const double give = upper ? v[k] : hi;
+        v[k] = (upper ? hi : v[k]) + __shfl_xor_sync(kFull, give, o);
+    }
+}
+
 // One sweep over the window: both families at once, each at its own point.  A lane adds up
 // both families over its points, oldest first, as running sums (see chains_to_powers: in the loop
 // every accumulation but the two objectives is an addition of two registers, which the fp64 pipe
 // issues in two cycles where a fused multiply-add on three registers takes three); the first
 // reduction step hands each lane of a pair the other lane's partial sums of its own family, the
-// remaining steps run over lanes of the same parity.
+// remaining steps run over lanes of the same parity.  With few rows per lane these steps are most of a sweep: exchanging
+// all 13 sums in each took 840 of the 5,300 cycles of a trial at 32 lanes and one row per lane.
 __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all, double inv_span,
                                       const double (&pI)[4], bool doI, const double (&pII)[4], bool doII,
                                       SweepSums& out) {
@@ -189,7 +219,6 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     }
     double (&m)[5] = a.m, (&n)[3] = a.n, (&h)[3] = a.h, (&ee)[3] = a.ee, (&f)[2] = a.f, (&kk)[2] = a.kk;
     const double gd = a.gd, sI = a.sI, gc = a.gc, sII = a.sII;
-    int feasible = a.q_signs >= 0 ? 1 : 0;
     const double dL = (double)S.L;
     const double x_l = -(double)S.l * inv_span, g = -dL * inv_span;
     chains_to_powers(m, x_l, g);
@@ -206,23 +235,48 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     SLAQ_PAIR(4, m[4], f[1]); SLAQ_PAIR(5, n[0], kk[0]); SLAQ_PAIR(6, n[1], kk[1]); SLAQ_PAIR(7, n[2], gc);
     SLAQ_PAIR(8, h[0], sII);
 #undef SLAQ_PAIR
-    v[9] = h[1] + __shfl_xor_sync(kFull, h[1], 1);    // family I only: odd lanes carry these along unused
+    // family I only: an odd lane has no such sums
+    v[9] = h[1] + __shfl_xor_sync(kFull, h[1], 1);
     v[10] = h[2] + __shfl_xor_sync(kFull, h[2], 1);
     v[11] = gd + __shfl_xor_sync(kFull, gd, 1);
     v[12] = sI + __shfl_xor_sync(kFull, sI, 1);
-    feasible &= __shfl_xor_sync(kFull, feasible, 1);
-    for (int o = 2; o < S.L; o <<= 1) {
+    if (odd) v[9] = v[10] = v[11] = v[12] = 0.0;
+    // Remaining steps over the lanes of the same parity: in each a lane hands over one half of its sums and keeps the
+    // other, 7 + 4 + 2 + 1 exchanges instead of 13 in every step, and every sum ends in one lane.
+    double chk, objective;
+    if (S.L == 2) {
+        objective = odd ? v[8] : v[12];
+        chk = 0.0;
 #pragma unroll
-        for (int k = 0; k < 13; ++k) v[k] += __shfl_xor_sync(kFull, v[k], o);
-        feasible &= __shfl_xor_sync(kFull, feasible, o);
+        for (int k = 0; k < 13; ++k) chk += v[k];
+    } else {
+        halve<7, 13>(v, 2, S.lane);
+        if (S.L == 4) {
+            objective = odd ? v[1] : v[5];
+            chk = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + v[6]);
+        } else {
+            halve<4, 7>(v, 4, S.lane);
+            if (S.L == 8) {
+                objective = v[1];
+                chk = (v[0] + v[1]) + (v[2] + v[3]);
+            } else {
+                halve<2, 4>(v, 8, S.lane);
+                objective = v[1];
+                chk = v[0] + v[1];
+                if (S.L == 32) {
+                    halve<1, 2>(v, 16, S.lane);
+                    objective = chk = v[0];
+                }
+            }
+        }
+        objective = __shfl_sync(kFull, objective, S.objective_lane());
     }
-    double chk = 0.0;
 #pragma unroll
-    for (int k = 0; k < 13; ++k) {
-        out.v[k] = v[k];
-        if (k < 9 || !odd) chk += v[k];
-    }
-    out.usable = finite_d(chk) && (odd || feasible);
+    for (int k = 0; k < 13; ++k) out.v[k] = v[k];
+    out.S = objective;
+    const unsigned broken = __ballot_sync(kFull, !finite_d(chk)), negative = __ballot_sync(kFull, a.q_signs < 0);
+    const unsigned group = S.group();
+    out.usable = !(broken & group & (odd ? 0xaaaaaaaau : 0x55555555u)) && (odd || !(negative & group));
 }
 
 }  // namespace slaq
