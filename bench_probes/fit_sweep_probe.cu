@@ -28,7 +28,7 @@ namespace {
 // tables every accumulation is one fused multiply-add of (table entry, value, sum), the products with
 // w, x and x^2 disappear from the loop, and the sums are scaled once after it.  q is evaluated in
 // the point index as well: q = (a / span^2) m^2 - (b / span) m + c.
-__device__ __forceinline__ void sweep_tables(const slaq::Lanes& S, int ts, int fam, int H, int k_all, double inv_span,
+__device__ __forceinline__ void sweep_tables(const slaq::LanesOf<0>& S, int ts, int fam, int H, int k_all, double inv_span,
                                              const double (&pI)[4], bool doI, const double (&pII)[4], bool doII,
                                              slaq::SweepSums& out) {
     double m0 = 0, m1 = 0, m2 = 0, m3 = 0, m4 = 0, n0 = 0, n1 = 0, n2 = 0, h0 = 0, h1 = 0, h2 = 0, gd = 0, sI = 0;
@@ -37,15 +37,15 @@ __device__ __forceinline__ void sweep_tables(const slaq::Lanes& S, int ts, int f
     double e = 0.0, ratio = 1.0;
     if (doII) {
         e = exp(fma(pII[1], (double)S.l * inv_span, pII[0]));
-        ratio = exp(pII[1] * ((double)S.L * inv_span));
+        ratio = exp(pII[1] * ((double)S.L() * inv_span));
     }
     const double qa = pI[0] * inv_span * inv_span, qb = -pI[1] * inv_span, qc = pI[2], dI = pI[3], cII = pII[2];
     double md = (double)S.l;
-    const double dL = (double)S.L;
+    const double dL = (double)S.L();
     const double* yp = S.y + S.lane;
     const double* tp = S.wtab + S.l;
 #pragma unroll 1
-    for (int k = 0, m = S.l; k < k_all; ++k, m += S.L, md += dL, yp += 32, tp += S.L) {
+    for (int k = 0, m = S.l; k < k_all; ++k, m += S.L(), md += dL, yp += 32, tp += S.L()) {
         if (m < H) {
             const bool ok = (m < S.wtab_len);
             const double t0 = ok ? tp[0] : 0.0, t1 = ok ? tp[ts] : 0.0, t2 = ok ? tp[2 * ts] : 0.0;
@@ -107,7 +107,7 @@ __device__ __forceinline__ void sweep_tables(const slaq::Lanes& S, int ts, int f
     v[11] = gd + __shfl_xor_sync(slaq::kFull, gd, 1);
     v[12] = sI + __shfl_xor_sync(slaq::kFull, sI, 1);
     feasible &= __shfl_xor_sync(slaq::kFull, feasible, 1);
-    for (int o = 2; o < S.L; o <<= 1) {
+    for (int o = 2; o < S.L(); o <<= 1) {
 #pragma unroll
         for (int k = 0; k < 13; ++k) v[k] += __shfl_xor_sync(slaq::kFull, v[k], o);
         feasible &= __shfl_xor_sync(slaq::kFull, feasible, o);
@@ -124,7 +124,7 @@ __device__ __forceinline__ void sweep_tables(const slaq::Lanes& S, int ts, int f
 // A second alternative, the library's sweep until the running sums replaced it: the powers of x multiplied out
 // point by point (x, x^2 and w u^2 x^2 formed in the loop, 13 of the 22 accumulations fused multiply-adds on three
 // different registers): 46 fp64 instructions per point instead of 43, 19 fused multiply-adds instead of 8.
-__device__ __forceinline__ void sweep_products(const slaq::Lanes& S, int fam, int H, int k_all, double inv_span,
+__device__ __forceinline__ void sweep_products(const slaq::LanesOf<0>& S, int fam, int H, int k_all, double inv_span,
                                                const double (&pI)[4], bool doI, const double (&pII)[4], bool doII,
                                                slaq::SweepSums& out) {
     double m0 = 0, m1 = 0, m2 = 0, m3 = 0, m4 = 0, n0 = 0, n1 = 0, n2 = 0, h0 = 0, h1 = 0, h2 = 0, gd = 0, sI = 0;
@@ -136,13 +136,13 @@ __device__ __forceinline__ void sweep_products(const slaq::Lanes& S, int fam, in
     double e = 0.0, ratio = 1.0;
     if (doII) {
         e = exp(fma(pII[1], (double)S.l * inv_span, pII[0]));
-        ratio = exp(pII[1] * ((double)S.L * inv_span));
+        ratio = exp(pII[1] * ((double)S.L() * inv_span));
     }
     double md = (double)S.l;
-    const double dL = (double)S.L;
+    const double dL = (double)S.L();
     const double* yp = S.y + S.lane;
 #pragma unroll 1   // unrolling only adds register pressure here: the body already holds 22 independent sums
-    for (int k = 0, m = S.l; k < k_all; ++k, m += S.L, md += dL, yp += 32) {
+    for (int k = 0, m = S.l; k < k_all; ++k, m += S.L(), md += dL, yp += 32) {
         if (m < H) {
             const double x = -md * inv_span;
             const double w = S.weight(m);
@@ -198,7 +198,7 @@ __device__ __forceinline__ void sweep_products(const slaq::Lanes& S, int fam, in
     v[11] = gd + __shfl_xor_sync(slaq::kFull, gd, 1);
     v[12] = sI + __shfl_xor_sync(slaq::kFull, sI, 1);
     feasible &= __shfl_xor_sync(slaq::kFull, feasible, 1);
-    for (int o = 2; o < S.L; o <<= 1) {
+    for (int o = 2; o < S.L(); o <<= 1) {
 #pragma unroll
         for (int k = 0; k < 13; ++k) v[k] += __shfl_xor_sync(slaq::kFull, v[k], o);
         feasible &= __shfl_xor_sync(slaq::kFull, feasible, o);
@@ -228,10 +228,10 @@ sweep_loop_kernel(const double* __restrict__ g_wtab, int L, int rows, int n_swee
     constexpr int kTabs = kVariant == 1 ? 5 : 1;
     for (int i = threadIdx.x; i < kTabs * kTable; i += blockDim.x) wtab[i] = g_wtab[i];
     double* const slice = smem + kTabs * kTable + (size_t)warp * slice_doubles;
-    slaq::Lanes S;
+    slaq::LanesOf<0> S;
     S.wtab = wtab;
     S.lane = lane;
-    S.L = L;
+    S.any_L = L;
     S.l = lane & (L - 1);
     const int G = 32 / L;
     S.park = slice + 2 * (lane / L) + (lane & 1);

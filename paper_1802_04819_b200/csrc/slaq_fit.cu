@@ -79,6 +79,7 @@ __device__ __forceinline__ void copy_async_8(double* dst_shared, const double* s
 
 // Copy the job's window into the lane columns (ring storage: the newest loss sits just before
 // `head`).  Returns H, or 0 after flagging storage that cannot be right.
+template <class Lanes>
 __device__ int stage_window(const JobArrays& job, int j, int h_cap, const Lanes& S, int32_t* err_word) {
     if (j < 0) return 0;
     const double* row = job.row[j];
@@ -105,7 +106,7 @@ __device__ int stage_window(const JobArrays& job, int j, int h_cap, const Lanes&
     // asynchronous 8-byte copies straight into the lane's column: all of a lane's points are in
     // flight at once, and nothing passes through registers
     double* dst = S.y + S.lane;
-    for (int m = S.l; m < H; m += S.L, dst += 32) {
+    for (int m = S.l; m < H; m += S.L(), dst += 32) {
         int pos = newest - m;
         pos += pos < 0 ? cap : 0;
         if (index_ok(pos, cap, kErrStorage, err_word) && S.holds(dst)) copy_async_8(dst, row + pos);
@@ -125,6 +126,7 @@ struct Normalised {
 // normalised change; then the window is scaled in place to levels y = l / M.  k_all: uniform
 // trip count of the warp.  changes_out (optional, global, indexed oldest first) receives the
 // normalised changes.
+template <class Lanes>
 __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double m_seen, int min_fit_points,
                                        double* changes_out) {
     Normalised out;
@@ -133,11 +135,11 @@ __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double 
     // Rows of the lane with a point (m < H), and with a point that has an older neighbour (m + 1 < H).  The rows
     // that every lane of the warp has are walked without a test per row (a branch in these loops costs issue
     // slots on every row), the ragged rest with one.
-    const int shift = __ffs(S.L) - 1;
+    const int shift = __ffs(S.L()) - 1;
     const int rows = H - 1 - S.l >= 0 ? ((H - 1 - S.l) >> shift) + 1 : 0;
     const int rows_nb = H - 2 - S.l >= 0 ? ((H - 2 - S.l) >> shift) + 1 : 0;
     const int full_nb = __reduce_min_sync(kFull, rows_nb);
-    const int nb_off = S.l + 1 < S.L ? 1 : 32 - (S.L - 1);   // from a point to its older neighbour
+    const int nb_off = S.l + 1 < S.L() ? 1 : 32 - (S.L() - 1);   // from a point to its older neighbour
     int fin = 1;
     double dmax = -CUDART_INF;
     {
@@ -158,8 +160,8 @@ __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double 
             }
         }
     }
-    fin = group_and(fin, S.L);
-    dmax = group_max(dmax, S.L);
+    fin = group_and(fin, S.L());
+    dmax = group_max(dmax, S.L());
     if (H <= 0) {
         out.status = SLAQ_JOB_INACTIVE;
     } else if (!fin || m_seen != m_seen || m_seen == CUDART_INF) {
@@ -177,7 +179,7 @@ __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double 
     double num = 0.0, den = 0.0;
     if (__any_sync(kFull, want_changes)) {
         for (int k = 0; k < k_all; ++k) {
-            const int m = S.l + S.L * k;
+            const int m = S.l + S.L() * k;
             if (want_changes && m + 1 < H) {
                 const double change = __ddiv_rn(older_neighbour(S, k) - S.level(k), M);
                 const double w = S.weight(m);
@@ -187,8 +189,8 @@ __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double 
             }
         }
         if (changes_out && usable && S.l == 0) changes_out[0] = 0.0;
-        num = group_sum(num, S.L);
-        den = group_sum(den, S.L);
+        num = group_sum(num, S.L());
+        den = group_sum(den, S.L());
         out.rho = fmax(num / den, 0.0);
     }
     __syncwarp();   // all neighbour reads are done before the window is overwritten
@@ -215,26 +217,27 @@ __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double 
             }
         }
     }
-    out.ymin = group_min(lo, S.L);
-    out.ymax = group_max(hi, S.L);
+    out.ymin = group_min(lo, S.L());
+    out.ymax = group_max(hi, S.L());
     __syncwarp();
     return out;
 }
 
 // Weighted mean normalised change per iteration from the scaled window (used when a window long
 // enough for a fit ends without one): sum w (y_{i-1} - y_i) / sum w.
+template <class Lanes>
 __device__ double mean_change_of_levels(const Lanes& S, int H, int k_all) {
     double num = 0.0, den = 0.0;
     for (int k = 0; k < k_all; ++k) {
-        const int m = S.l + S.L * k;
+        const int m = S.l + S.L() * k;
         if (m + 1 < H) {
             const double w = S.weight(m);
             num = fma(w, older_neighbour(S, k) - S.level(k), num);
             den += w;
         }
     }
-    num = group_sum(num, S.L);
-    den = group_sum(den, S.L);
+    num = group_sum(num, S.L());
+    den = group_sum(den, S.L());
     return fmax(num / den, 0.0);
 }
 
@@ -394,10 +397,11 @@ __device__ __forceinline__ bool finish_trial(Family& F, const double (&trial)[4]
 // The sums of the last accepted point live in shared memory between sweeps, one column per job
 // and family: every lane writes the ones it holds.  Every lane of the warp calls this; `keep` says
 // whether the lane's family has new sums to park.
+template <class Lanes>
 __device__ __forceinline__ void park(const Lanes& S, const SweepSums& s, bool keep) {
     if (keep) {
         const int n = S.park_stride();
-        if (S.L == 2) {
+        if (S.L() == 2) {
 #pragma unroll
             for (int k = 0; k < kParked; ++k)
                 if (S.holds(S.park + k * n)) S.park[k * n] = s.v[k];
@@ -406,7 +410,7 @@ __device__ __forceinline__ void park(const Lanes& S, const SweepSums& s, bool ke
             S.held(from, own);
             own = min(own, kParked - from);   // the objective of family I is not parked
             double* const at = S.park + from * n;
-            const int most = S.L == 32 ? 1 : S.L == 16 ? 2 : S.L == 8 ? 4 : 7;
+            const int most = S.L() == 32 ? 1 : S.L() == 16 ? 2 : S.L() == 8 ? 4 : 7;
 #pragma unroll
             for (int k = 0; k < 7; ++k) {
                 if (k >= most) break;
@@ -418,6 +422,7 @@ __device__ __forceinline__ void park(const Lanes& S, const SweepSums& s, bool ke
 }
 
 // Normal equations A = sum w J J^T, g = sum w J r of the lane's family from the parked sums.
+template <class Lanes>
 __device__ __forceinline__ void normal_equations(const Lanes& S, int fam, double sw, Sym4& A, double (&g)[4]) {
     const double* c = S.park;
     const int n = S.park_stride();
@@ -454,7 +459,7 @@ struct GuessSums {
 
 // One point of the first-guess pass.  kI / kII: the transformed values of family I (1 / (y - d0)) and of
 // family II (log(y - d0)) are wanted by some lane of the warp.
-template <bool kI, bool kII>
+template <bool kI, bool kII, class Lanes>
 __device__ __forceinline__ void guess_point(const Lanes& S, const double* wp, const double* yp, double md, double inv_span,
                                             double d0, GuessSums& g) {
     const double x = -md * inv_span;
@@ -483,26 +488,27 @@ __device__ __forceinline__ void guess_point(const Lanes& S, const double* wp, co
 }
 
 // The rows every lane of the warp has without a test per row, the ragged rest with one.
-template <bool kI, bool kII>
+template <bool kI, bool kII, class Lanes>
 __device__ __forceinline__ void guess_rows(const Lanes& S, int own, int k_all, double inv_span, double d0, GuessSums& g) {
     const int full = __reduce_min_sync(kFull, own);
     const double* yp = S.y + S.lane;
     const double* wp = S.wtab + S.l;
     double md = (double)S.l;
-    const double dL = (double)S.L;
+    const double dL = (double)S.L();
     int k = 0;
 #pragma unroll 1
-    for (; k < full; ++k, md += dL, yp += 32, wp += S.L) guess_point<kI, kII>(S, wp, yp, md, inv_span, d0, g);
+    for (; k < full; ++k, md += dL, yp += 32, wp += S.L()) guess_point<kI, kII>(S, wp, yp, md, inv_span, d0, g);
 #pragma unroll 1
-    for (; k < k_all; ++k, md += dL, yp += 32, wp += S.L)
+    for (; k < k_all; ++k, md += dL, yp += 32, wp += S.L())
         if (k < own) guess_point<kI, kII>(S, wp, yp, md, inv_span, d0, g);
 }
 
+template <class Lanes>
 __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span, double ymin, double ymax, bool busy,
                               bool needI, bool needII, Moments& mom, double (&pI)[4], double (&pII)[4]) {
     const double d0 = ymax > ymin ? ymin - 0.1 * (ymax - ymin) : ymin - 1e-3 * fmax(fabs(ymin), 1.0);
     GuessSums g = {};
-    const int shift = __ffs(S.L) - 1;
+    const int shift = __ffs(S.L()) - 1;
     const int own = busy && H - 1 - S.l >= 0 ? ((H - 1 - S.l) >> shift) + 1 : 0;   // the lane's rows
     // a family that no lane of the warp wants a guess for is left out of the pass; a lane that does not want
     // what the warp computes gets sums it does not use
@@ -516,7 +522,7 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
     }
     double sw = g.sw, swx = g.swx, swx2 = g.swx2, swx3 = g.swx3, swx4 = g.swx4, swy2 = g.swy2;
     double r0 = g.r0, r1 = g.r1, r2 = g.r2, su = g.su, sxu = g.sxu;
-    for (int o = S.L >> 1; o > 0; o >>= 1) {
+    for (int o = S.L() >> 1; o > 0; o >>= 1) {
         sw += __shfl_xor_sync(kFull, sw, o); swx += __shfl_xor_sync(kFull, swx, o);
         swx2 += __shfl_xor_sync(kFull, swx2, o); swx3 += __shfl_xor_sync(kFull, swx3, o);
         swx4 += __shfl_xor_sync(kFull, swx4, o); swy2 += __shfl_xor_sync(kFull, swy2, o);
@@ -538,7 +544,7 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
         {
             const int mine = needI ? own : 0;
             const int full = __reduce_min_sync(kFull, mine);
-            const double dL = (double)S.L;
+            const double dL = (double)S.L();
             double md = (double)S.l;
             int k = 0;
             for (; k < full; ++k, md += dL) {
@@ -552,11 +558,11 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
                 }
             }
         }
-        pos = group_and(pos, S.L);
+        pos = group_and(pos, S.L());
         good = good && pos;
         // the oldest point (m = H - 1) and the newest (m = 0), read from the lanes that own them
         const int m_old = max(H - 1, 0);
-        const double* at_old = S.y + (m_old / S.L) * 32 + (S.lane - S.l) + (m_old & (S.L - 1));
+        const double* at_old = S.y + (m_old / S.L()) * 32 + (S.lane - S.l) + (m_old & (S.L() - 1));
         const double y_old = S.holds(at_old) ? *at_old : 0.0;
         const double y_new = S.holds(S.y + S.lane - S.l) ? S.y[S.lane - S.l] : 0.0;
         if (good) {
@@ -610,6 +616,7 @@ __device__ void carry_over(const FitArrays& fit, const JobArrays& job, int j, do
 
 // The second round of a warm start: the families whose carried-over point had no finite
 // residual (`redo`, per lane for its own family) take their first guesses and are swept again.
+template <class Lanes>
 __device__ __noinline__ void restart_from_first_guesses(const Lanes& S, int fam, int H, int k_all, double inv_span,
                                                         double ymin, double ymax, bool fits, bool redo, double* pI,
                                                         double* pII, SweepSums* sums) {
@@ -643,8 +650,10 @@ struct FitClasses {
 };
 
 // kWarm: families may start from last epoch's parameters (a separate instantiation, so that the
-// plain one carries none of that code).
-template <bool kWarm>
+// plain one carries none of that code).  kL: lanes per job if the launch has one length class - every cluster with
+// windows of up to about 80 points, or with few jobs - as a constant, which takes branches and index arithmetic out of
+// every step of a trial; 0 where several classes share the launch.
+template <bool kWarm, int kL>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1)
 fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
            const int32_t* __restrict__ start, FitClasses cls, int lm_trials, int min_fit_points,
@@ -654,7 +663,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     double* wtab = smem;                                   // [h_max]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* const slice = smem + cls.h_max + (size_t)warp * cls.slice;   // this warp's: parked sums, then the window rows
-    Lanes S;
+    LanesOf<kL> S;
     S.wtab = wtab;
     S.lane = lane;
     S.slice = slice;
@@ -686,8 +695,8 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         if (slot >= slot_base[cls.n]) break;
         int c = 0;
         while (slot >= slot_base[c + 1]) ++c;
-        const int L = cls.L[c], h_hi = cls.h_hi[c];
-        S.L = L;
+        const int L = kL ? kL : cls.L[c], h_hi = cls.h_hi[c];
+        S.any_L = L;
         S.l = lane & (L - 1);
         const int G = 32 / L, g = lane / L;
         S.park = slice + 2 * g + (lane & 1);
@@ -905,7 +914,7 @@ normalise_export_kernel(JobArrays job, const int32_t* __restrict__ ids, const in
     double* wtab = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k_cap = (max_hist + 31) / 32;
-    Lanes S;
+    LanesOf<32> S;
     S.y = smem + max_hist + (size_t)warp * (k_cap + 1) * 32;
     S.slice = S.y;
     S.slice_len = (k_cap + 1) * 32;
@@ -914,7 +923,7 @@ normalise_export_kernel(JobArrays job, const int32_t* __restrict__ ids, const in
     S.park = nullptr;
     S.wtab = wtab;
     S.lane = lane;
-    S.L = 32;
+    S.any_L = 32;
     S.l = lane;
     for (int i = threadIdx.x; i < max_hist; i += blockDim.x) wtab[i] = g_wtab[i];
     __syncthreads();
@@ -1125,12 +1134,17 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 
 }  // namespace
 
+using FitKernel = decltype(&fit_kernel<false, 0>);
+static FitKernel const kFitKernels[2][6] = {
+    {fit_kernel<false, 0>, fit_kernel<false, 2>, fit_kernel<false, 4>, fit_kernel<false, 8>, fit_kernel<false, 16>, fit_kernel<false, 32>},
+    {fit_kernel<true, 0>, fit_kernel<true, 2>, fit_kernel<true, 4>, fit_kernel<true, 8>, fit_kernel<true, 16>, fit_kernel<true, 32>}};
+
 int fit_setup() {
-    const int most = (int)kSmemLimit;
     bool ok = true;
-    for (const void* k : {(const void*)fit_kernel<false>, (const void*)fit_kernel<true>})
-        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
-             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    for (const auto& row : kFitKernels)
+        for (FitKernel k : row)
+            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
+                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
     for (const void* k : {(const void*)length_scatter_kernel, (const void*)length_sort_kernel})
         ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)(2 * sizeof(int) * (kMaxHistLimit + 1))) == cudaSuccess;
@@ -1196,7 +1210,7 @@ int launch_fit(slaq_handle* h) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
-    const auto kernel = h->warm_start ? fit_kernel<true> : fit_kernel<false>;
+    const FitKernel kernel = kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
     int blocks = h->sm_count;   // one block per SM: its registers and shared memory fill one
     const int needed = (J + warps - 1) / warps;   // at least one job per slot
     if (blocks > needed) blocks = needed;

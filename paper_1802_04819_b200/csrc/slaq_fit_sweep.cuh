@@ -30,26 +30,30 @@ __device__ __forceinline__ double fast_rcp(double q) {
 // Shared-memory view of one warp.  Point m of a lane's job (m = distance from the newest
 // point, m = l + L k for the lane with index l in its group) sits at y[k * 32 + lane]:
 // every access of the sweeps is lane-private and free of bank conflicts.
-struct Lanes {
+// kL: the lanes per job where all jobs of a launch have the same (a constant for the compiler), else 0.
+template <int kL>
+struct LanesOf {
     double* y;         // [k_cap + 1][32]
     double* park;      // this lane's family of its job in [kParked][2 * jobs per warp] (one column per job and family)
     const double* wtab;
-    int lane, L, l;
-    __device__ __forceinline__ int park_stride() const { return 64 >> (__ffs(L) - 1); }   // 2 * (32 / L), L a power of two
+    int lane, l;
+    int any_L;         // lanes per job (kL == 0)
+    __device__ __forceinline__ int L() const { return kL ? kL : any_L; }
+    __device__ __forceinline__ int park_stride() const { return 64 >> (__ffs(L()) - 1); }   // 2 * (32 / L), L() a power of two
     // Which of its family's 13 sums the lane holds after a sweep's reduction (see halve): `n` of them from the `from`-th on.
     __device__ __forceinline__ void held(int& from, int& n) const {
         from = 0, n = 13;
-        if (L >= 4) { const int b = (lane >> 1) & 1; from = 7 * b; n = 7 - b; }
-        if (L >= 8) { const int b = (lane >> 2) & 1; from += 4 * b; n = b ? n - 4 : 4; }
-        if (L >= 16) { const int b = (lane >> 3) & 1; from += 2 * b; n = b ? max(n - 2, 0) : min(n, 2); }
-        if (L >= 32) { const int b = (lane >> 4) & 1; from += b; n = b ? max(n - 1, 0) : min(n, 1); }
+        if (L() >= 4) { const int b = (lane >> 1) & 1; from = 7 * b; n = 7 - b; }
+        if (L() >= 8) { const int b = (lane >> 2) & 1; from += 4 * b; n = b ? n - 4 : 4; }
+        if (L() >= 16) { const int b = (lane >> 3) & 1; from += 2 * b; n = b ? max(n - 2, 0) : min(n, 2); }
+        if (L() >= 32) { const int b = (lane >> 4) & 1; from += b; n = b ? max(n - 1, 0) : min(n, 1); }
     }
     // Where the steps of the reduction leave the objective: sum 12 of family I, sum 8 of family II.
     __device__ __forceinline__ int objective_lane() const {
-        return (lane & -L) + (lane & 1) + 2 + (L >= 8 && !(lane & 1) ? 4 : 0) + (L >= 32 ? 16 : 0);
+        return (lane & -L()) + (lane & 1) + 2 + (L() >= 8 && !(lane & 1) ? 4 : 0) + (L() >= 32 ? 16 : 0);
     }
     __device__ __forceinline__ unsigned group() const {   // the lanes of this lane's job
-        return (0xffffffffu >> (32 - L)) << (lane & -L);
+        return (0xffffffffu >> (32 - L())) << (lane & -L());
     }
     // extents, read by the bounds build only: the warp's slice [slice, slice + slice_len) and the weight table
     const double* slice;
@@ -71,12 +75,13 @@ struct Lanes {
 };
 
 // The window value at distance m + 1 from the newest point, seen from the lane that owns m.
+template <class Lanes>
 __device__ __forceinline__ double older_neighbour(const Lanes& S, int k) {
-    const double* p = S.l + 1 < S.L ? S.y + k * 32 + S.lane + 1 : S.y + (k + 1) * 32 + S.lane - (S.L - 1);
+    const double* p = S.l + 1 < S.L() ? S.y + k * 32 + S.lane + 1 : S.y + (k + 1) * 32 + S.lane - (S.L() - 1);
     return S.holds(p) ? *p : 0.0;
 }
 
-// What a lane keeps of one sweep: its share of the sums of ITS family over the whole window (see Lanes::held), and the objective.
+// What a lane keeps of one sweep: its share of the sums of ITS family over the whole window (see LanesOf::held), and the objective.
 // Family I (u = 1/q^2, J = (-u x^2, -u x, -u, 1)): v[0..4] = sum w u^2 x^k, v[5..7] = sum w u x^k,
 // v[8..10] = sum w u r x^k, v[11] = sum w r, v[12] = S.
 // Family II (J = (e, -x e, 1)): v[0..2] = sum w e^2 x^k, v[3..4] = sum w e x^k, v[5..6] = sum w e r x^k,
@@ -119,7 +124,7 @@ struct LaneSums {
 };
 
 // One point of a lane's walk: both families' values at the point and their running sums.
-template <bool kI, bool kII>
+template <bool kI, bool kII, class Lanes>
 __device__ __forceinline__ void add_point(const Lanes& S, const double* wp, const double* yp, double x,
                                           const double (&pI)[4], const double (&pII)[4], double& e, double ratio,
                                           LaneSums& a) {
@@ -154,12 +159,12 @@ __device__ __forceinline__ void add_point(const Lanes& S, const double* wp, cons
 // the whole warp, so that the loop has no branch per family (a lane whose family has no trial computes it at
 // parameters nobody uses and its sums are discarded).  Branches inside the loop cost issue slots on every row:
 // the rows that every lane of the warp has are walked without a test, only the ragged rest with one.
-template <bool kI, bool kII>
+template <bool kI, bool kII, class Lanes>
 __device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all, double inv_span,
                                           const double (&pI)[4], const double (&pII)[4], LaneSums& a) {
-    const int mi = S.l + k_last * S.L;
+    const int mi = S.l + k_last * S.L();
     const double md = (double)mi;
-    const double dL = (double)S.L;
+    const double dL = (double)S.L();
     // x from the lane's oldest point by one addition per row (its rounding, at most a few 1e-15 absolute at the
     // newest point, moves the predictions as little as the exponential's recurrence does: measured)
     double x = -md * inv_span;
@@ -178,9 +183,9 @@ __device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all,
     const int k_min = __reduce_min_sync(kFull, k_last);
     int i = 0;
 #pragma unroll 1   // unrolling was measured (2 rows per step): slower, more spills
-    for (; i <= k_min; ++i, x += hx, yp -= 32, wp -= S.L) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);
+    for (; i <= k_min; ++i, x += hx, yp -= 32, wp -= S.L()) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);
 #pragma unroll 1
-    for (; i < k_all; ++i, x += hx, yp -= 32, wp -= S.L)
+    for (; i < k_all; ++i, x += hx, yp -= 32, wp -= S.L())
         if (i <= k_last) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);   // row k_last - i >= 0
 }
 
@@ -204,11 +209,12 @@ __device__ __forceinline__ void halve(double (&v)[13], int o, int lane) {
 // reduction step hands each lane of a pair the other lane's partial sums of its own family, the
 // remaining steps run over lanes of the same parity.  With few rows per lane these steps are most of a sweep: exchanging
 // all 13 sums in each took 840 of the 5,300 cycles of a trial at 32 lanes and one row per lane.
+template <class Lanes>
 __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all, double inv_span,
                                       const double (&pI)[4], bool doI, const double (&pII)[4], bool doII,
                                       SweepSums& out) {
     LaneSums a = {};
-    const int shift = __ffs(S.L) - 1;                                      // L is a power of two
+    const int shift = __ffs(S.L()) - 1;                                      // L is a power of two
     const int k_last = H - 1 - S.l >= 0 ? (H - 1 - S.l) >> shift : -1;     // the row of the lane's oldest point
     const bool anyI = __any_sync(kFull, doI), anyII = __any_sync(kFull, doII);
     if (anyI && anyII) {
@@ -219,7 +225,7 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     }
     double (&m)[5] = a.m, (&n)[3] = a.n, (&h)[3] = a.h, (&ee)[3] = a.ee, (&f)[2] = a.f, (&kk)[2] = a.kk;
     const double gd = a.gd, sI = a.sI, gc = a.gc, sII = a.sII;
-    const double dL = (double)S.L;
+    const double dL = (double)S.L();
     const double x_l = -(double)S.l * inv_span, g = -dL * inv_span;
     chains_to_powers(m, x_l, g);
     chains_to_powers(n, x_l, g);
@@ -244,26 +250,26 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     // Remaining steps over the lanes of the same parity: in each a lane hands over one half of its sums and keeps the
     // other, 7 + 4 + 2 + 1 exchanges instead of 13 in every step, and every sum ends in one lane.
     double chk, objective;
-    if (S.L == 2) {
+    if (S.L() == 2) {
         objective = odd ? v[8] : v[12];
         chk = 0.0;
 #pragma unroll
         for (int k = 0; k < 13; ++k) chk += v[k];
     } else {
         halve<7, 13>(v, 2, S.lane);
-        if (S.L == 4) {
+        if (S.L() == 4) {
             objective = odd ? v[1] : v[5];
             chk = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + v[6]);
         } else {
             halve<4, 7>(v, 4, S.lane);
-            if (S.L == 8) {
+            if (S.L() == 8) {
                 objective = v[1];
                 chk = (v[0] + v[1]) + (v[2] + v[3]);
             } else {
                 halve<2, 4>(v, 8, S.lane);
                 objective = v[1];
                 chk = v[0] + v[1];
-                if (S.L == 32) {
+                if (S.L() == 32) {
                     halve<1, 2>(v, 16, S.lane);
                     objective = chk = v[0];
                 }
