@@ -3,6 +3,8 @@
 from __future__ import annotations
 
 import ctypes
+import math
+import weakref
 from ctypes import POINTER, c_double, c_float, c_int, c_int8, c_int32, c_int64, c_size_t, c_void_p, c_char_p
 
 import numpy as np
@@ -51,6 +53,7 @@ class SlaqError(RuntimeError):
         self.code = code
 
 
+_F8, _I8, _I4, _I1, _U1 = (np.dtype(t) for t in (np.float64, np.int64, np.int32, np.int8, np.uint8))
 _libs = {}
 _fast = None       # the marshalling extension
 
@@ -117,6 +120,8 @@ def load_library(variant: str | None = None):
         "slaq_shard_count_device": (c_int, [vp, vp]),
         "slaq_shard_finalise_device": (c_int, [vp, vp, vp]),
     }
+    sig["slaq_result_take"] = (vp, [c_size_t])      # page-locked memory for results, internal to the binding
+    sig["slaq_result_give"] = (None, [vp])
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
         fn.restype, fn.argtypes = res, args
@@ -149,6 +154,26 @@ def allocate_static(d_gain, total_cores: int, d_out_alloc, d_out_reduction, stre
                     -5: "a CUDA call failed"}
         raise SlaqError(rc, messages.get(rc, "error"))
     return rc
+
+
+def _results(lib, fields):
+    """Uninitialised arrays for results: ``fields`` = (name, shape, dtype) each, in one block of page-locked memory where
+    the library has one to give (it goes back when the last array is gone), else ordinary ones."""
+    at, places = 0, []
+    for name, shape, dtype in fields:
+        count = shape if isinstance(shape, int) else math.prod(shape)
+        places.append((name, shape, dtype, count, at))
+        at += (count * dtype.itemsize + 63) & ~63
+    address = lib.slaq_result_take(at)
+    if not address:
+        return {name: np.empty(shape, dtype) for name, shape, dtype in fields}
+    block = (ctypes.c_char * max(1, at)).from_address(address)
+    weakref.finalize(block, lib.slaq_result_give, address).atexit = False
+    out = {}
+    for name, shape, dtype, count, start in places:
+        flat = np.frombuffer(block, dtype, count, start)
+        out[name] = flat if isinstance(shape, int) else flat.reshape(shape)
+    return out
 
 
 def _arr(a, dtype):
@@ -276,11 +301,11 @@ class Scheduler:
 
     def get_predictions(self, want_gain=True):
         J, cap = self.max_jobs, self.max_cores_per_job
-        out = dict(
-            R=np.empty(J), gain=np.empty((J, cap)) if want_gain else None, family=np.empty(J, np.int8),
-            params=np.empty((J, 4)), S=np.empty((J, 2)), status=np.empty(J, np.int32),
-            evals=np.empty((J, 2), np.int32), M=np.empty(J),
-        )
+        f8, i4 = _F8, _I4
+        fields = [("R", J, f8), ("family", J, _I1), ("params", (J, 4), f8), ("S", (J, 2), f8), ("status", J, i4),
+                  ("evals", (J, 2), i4), ("M", J, f8)]
+        out = _results(self._lib, fields + [("gain", (J, cap), f8)] if want_gain else fields)
+        out.setdefault("gain")
         self._check(self._lib.slaq_get_predictions(
             self._h, _ptr(out["R"]), _ptr(out["gain"]), _ptr(out["family"]), _ptr(out["params"]), _ptr(out["S"]),
             _ptr(out["status"]), _ptr(out["evals"]), _ptr(out["M"])))
@@ -304,8 +329,7 @@ class Scheduler:
     def get_fit_state(self):
         """Both families' end points of the last epoch: dict(p [J, 8], valid uint8 [J], K int64 [J], span, M)."""
         J = self.max_jobs
-        st = dict(p=np.empty((J, 8)), valid=np.empty(J, np.uint8), K=np.empty(J, np.int64), span=np.empty(J),
-                  M=np.empty(J))
+        st = _results(self._lib, [("p", (J, 8), _F8), ("valid", J, _U1), ("K", J, _I8), ("span", J, _F8), ("M", J, _F8)])
         self._check(self._lib.slaq_get_fit_state(self._h, _ptr(st["p"]), _ptr(st["valid"]), _ptr(st["K"]),
                                                  _ptr(st["span"]), _ptr(st["M"])))
         return st
@@ -362,7 +386,7 @@ class Scheduler:
         """The whole per-job state of the handle as one blob (uint8 array)."""
         n = c_size_t()
         self._check(self._lib.slaq_export_state_bytes(self._h, ctypes.byref(n)))
-        blob = np.zeros(n.value, np.uint8)
+        blob = _results(self._lib, [("blob", n.value, _U1)])["blob"]   # written as a whole
         self._check(self._lib.slaq_export_state(self._h, _ptr(blob), blob.size))
         return blob
 

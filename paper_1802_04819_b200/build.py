@@ -11,7 +11,7 @@ ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libslaq.so"
 MARSHAL = PKG / "_marshal.so"      # Python extension: argument marshalling of the loop's two calls
-SOURCES = ["slaq_api.cu", "slaq_fit.cu", "slaq_gain.cu", "slaq_alloc.cu", "slaq_select.cu"]
+SOURCES = ["slaq_api.cu", "slaq_fit.cu", "slaq_gain.cu", "slaq_alloc.cu", "slaq_select.cu", "slaq_pipe.cu"]
 
 
 # Instrumented builds of the same sources, each a library of its own beside libslaq.so.

@@ -11,12 +11,14 @@
 #include <new>
 
 #include "slaq_internal.cuh"
+#include "slaq_pipe.cuh"
 
 using namespace slaq;
 
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int64_t kCheckOnHost = 32768;   // losses of a bulk load up to which the host checks them
 constexpr int32_t kMailAlways = 4096;   // entries of an append up to which asking where the arrays live costs more than it gives
 constexpr int32_t kEpochSteps = 15, kAllocateSteps = 11;   // slaq_stats.launches
 
@@ -95,6 +97,7 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     double* reduction = b.take<double>(Js);
     int32_t* err_word = b.take<int32_t>(4);
     sc.append_ticket = reinterpret_cast<unsigned int*>(err_word ? err_word + 2 : nullptr);
+    sc.load_flag = err_word ? err_word + 1 : nullptr;
     sc.published = b.take<long long>(16);
     job.max_jobs = J;
     job.ring_lo = ring;
@@ -170,6 +173,25 @@ __global__ void init_jobs_kernel(JobArrays job, FitArrays fit, double* ring, int
 // checked: the arrays come straight from the caller's device memory, unseen by the host - an id out of range,
 // a job without any loss yet, a loss or time that is not finite or a core count below 1 sets kErrInput and
 // that entry is skipped.
+// Called by every thread of a kernel at its end: the last block to get here tells the host.
+__device__ __forceinline__ void report(Mailbox* mail, uint32_t seq, unsigned int* ticket, int32_t* flag) {
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const unsigned int blocks = gridDim.x * gridDim.y;
+    if (blocks > 1) {
+        __threadfence();
+        if (atomicAdd(ticket, 1u) != blocks - 1) return;
+        *ticket = 0;
+        __threadfence();
+    }
+    if (flag) {
+        mail->err = *(volatile int32_t*)flag;
+        *flag = 0;
+    }
+    __threadfence_system();
+    mail->done = seq;
+}
+
 // All loads of an entry are issued before anything is stored: the chain is then three memory latencies long (entry, job,
 // newest loss) instead of one per array.
 __device__ __forceinline__ void append_one(const JobArrays& job, const FitArrays& fit, int max_jobs, int i, const int32_t* ids,
@@ -261,31 +283,24 @@ __global__ void append_kernel(JobArrays job, FitArrays fit, int max_jobs, int n,
                               Mailbox* mail, uint32_t seq, unsigned int* ticket) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) append_one(job, fit, max_jobs, i, ids, losses, times, cores, checked);
-    if (!mail) return;
-    __shared__ bool last;
-    __syncthreads();
-    if (threadIdx.x == 0) {   // the last block tells the host
-        last = true;
-        if (gridDim.x > 1) {
-            __threadfence();
-            last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-        }
-        if (last) {
-            *ticket = 0;
-            __threadfence_system();
-            mail->done = seq;
-        }
-    }
+    if (mail) report(mail, seq, ticket, nullptr);
+}
+
+// Sets *flag if a value is not finite; with a mailbox the flag is reported (and cleared).
+__global__ void __launch_bounds__(256) finite_kernel(const double* __restrict__ v, size_t n, int32_t* flag, Mailbox* mail, uint32_t seq,
+                                                     unsigned int* ticket) {
+    int top = 0;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        top = max(top, __double2hiint(v[i]) & 0x7ff00000);
+    if (top == 0x7ff00000) *flag = 1;
+    if (mail) report(mail, seq, ticket, flag);
 }
 
 // Bulk load: one warp per listed job copies (ring mode) or adopts (packed mode) its row.
-__global__ void load_kernel(JobArrays job, FitArrays fit, double* ring, int max_jobs, int max_hist, int n,
-                            const int32_t* ids,
-                            const int64_t* offsets, const double* src, const int64_t* k_last, const double* m_seen,
-                            int packed) {
-    const int slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (slot >= n) return;
-    const int j = ids[slot];
+__device__ __forceinline__ void load_one(const JobArrays& job, const FitArrays& fit, double* ring, int max_jobs, int max_hist, int slot,
+                                         int lane, const int32_t* ids, const int64_t* offsets, const double* src,
+                                         const int64_t* k_last, const double* m_seen, int packed) {
+    const int j = ids ? ids[slot] : slot;   // no list: every job in order
     if (j < 0 || j >= max_jobs) return;
     const int64_t lo = offsets[slot], hi = offsets[slot + 1];
     int64_t H = hi - lo;
@@ -312,6 +327,81 @@ __global__ void load_kernel(JobArrays job, FitArrays fit, double* ring, int max_
     }
 }
 
+__global__ void load_kernel(JobArrays job, FitArrays fit, double* ring, int max_jobs, int max_hist, int n,
+                            const int32_t* ids,
+                            const int64_t* offsets, const double* src, const int64_t* k_last, const double* m_seen,
+                            int packed, Mailbox* mail, uint32_t seq, unsigned int* ticket, int32_t* flag) {
+    const int slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (slot < n && *(volatile int32_t*)flag == 0)   // nothing is applied if a loss is not finite
+        load_one(job, fit, ring, max_jobs, max_hist, slot, lane, ids, offsets, src, k_last, m_seen, packed);
+    if (mail) report(mail, seq, ticket, flag);
+}
+
+// Where every job's window goes in an export (offsets[max_jobs] in all), the longest window, both reported to the host.
+__global__ void __launch_bounds__(1024) window_offsets_kernel(const int32_t* __restrict__ count, int max_jobs, int64_t* offsets,
+                                                              Mailbox* mail, uint32_t seq) {
+    __shared__ long long warp_sum[32];
+    __shared__ int warp_max[32];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int per = (max_jobs + 1023) / 1024, lo = min(t * per, max_jobs), hi = min(lo + per, max_jobs);
+    long long sum = 0;
+    int longest = 0;
+    for (int j = lo; j < hi; ++j) {
+        const int c = max(count[j], 0);
+        sum += c;
+        longest = max(longest, c);
+    }
+    long long incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+    }
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if (lane == 31) warp_sum[warp] = incl, warp_max[warp] = longest;
+    __syncthreads();
+    long long run = incl - sum;
+    for (int w = 0; w < warp; ++w) run += warp_sum[w];
+    for (int j = lo; j < hi; ++j) {
+        offsets[j] = run;
+        run += max(count[j], 0);
+    }
+    if (t == 1023) {
+        offsets[max_jobs] = run;
+        for (int w = 0; w < 32; ++w) longest = max(longest, warp_max[w]);
+        mail->points = run;
+        mail->longest = longest;
+    }
+    report(mail, seq, nullptr, nullptr);
+}
+
+// Copies up to kMaxPieces arrays, one per blockIdx.y, in 8-byte words (both sides 8-byte aligned) and trailing bytes; skipped
+// if *flag is set.
+constexpr int kMaxPieces = 20;
+struct Pieces {
+    void* dst[kMaxPieces];
+    const void* src[kMaxPieces];
+    size_t bytes[kMaxPieces];
+    int n = 0;
+    void add(void* to, const void* from, size_t size) {
+        dst[n] = to;
+        src[n] = from;
+        bytes[n++] = size;
+    }
+};
+__global__ void __launch_bounds__(256) pieces_kernel(const __grid_constant__ Pieces p, Mailbox* mail, uint32_t seq, unsigned int* ticket,
+                                                     int32_t* flag) {
+    const int k = blockIdx.y;
+    if (!flag || *(volatile int32_t*)flag == 0) {
+        const size_t words = p.bytes[k] / 8, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, pitch = (size_t)gridDim.x * blockDim.x;
+        for (size_t i = first; i < words; i += pitch)
+            static_cast<unsigned long long*>(p.dst[k])[i] = static_cast<const unsigned long long*>(p.src[k])[i];
+        for (size_t i = 8 * words + first; i < p.bytes[k]; i += pitch)
+            static_cast<unsigned char*>(p.dst[k])[i] = static_cast<const unsigned char*>(p.src[k])[i];
+    }
+    if (mail) report(mail, seq, ticket, flag);
+}
+
 // Export: one warp per job copies its window, oldest point first, to out[offsets[j] ..].
 __global__ void export_windows_kernel(JobArrays job, int max_jobs, const int64_t* offsets, double* out) {
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -330,13 +420,17 @@ __global__ void export_windows_kernel(JobArrays job, int max_jobs, const int64_t
 }
 
 __global__ void set_time_kernel(JobArrays job, int max_jobs, int n, const int32_t* ids, const double* s,
-                                const double* w) {
+                                const double* w, Mailbox* mail, uint32_t seq, unsigned int* ticket) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int j = ids[i];
-    if (j < 0 || j >= max_jobs) return;
-    job.s_set[j] = s[i];
-    job.w_set[j] = w[i];
+    if (i < n) {
+        const int j = ids[i];
+        const double si = s[i], wi = w[i];
+        if (j >= 0 && j < max_jobs) {
+            job.s_set[j] = si;
+            job.w_set[j] = wi;
+        }
+    }
+    report(mail, seq, ticket, nullptr);
 }
 
 __global__ void set_target_kernel(JobArrays job, int max_jobs, int n, const int32_t* ids, const double* targets) {
@@ -503,6 +597,8 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     }
     h->ws_bytes = need;
     layout(h, static_cast<char*>(h->ws), max_jobs, max_hist, cap);
+    pipe_retain();
+    h->pipe_user = true;
     h->mailbox_jobs = std::min(max_jobs, kMailboxJobs);
     {
         const size_t mail = sizeof(Mailbox) + (size_t)h->mailbox_jobs * 28 + 64;
@@ -615,8 +711,9 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
     for (int32_t i = 0; i < n; ++i)
         if (offsets[i + 1] < offsets[i]) return fail(h, SLAQ_E_ARG, "offsets must not decrease");
     const int64_t lo = offsets[0], total = offsets[n] - lo;
-    for (int64_t i = 0; i < total; ++i)
-        if (!std::isfinite(losses[lo + i])) return fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
+    // many losses are checked on the device, where they are anyway before anything is applied
+    const bool check_here = total <= kCheckOnHost;
+    if (check_here && !all_finite(losses + lo, (size_t)total)) return fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
     if (m_seen)
         for (int32_t i = 0; i < n; ++i)
             if (std::isnan(m_seen[i]) || m_seen[i] == INFINITY)
@@ -635,6 +732,18 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
             const cudaError_t e = cudaMalloc(&new_pool, sizeof(double) * (size_t)total);
             if (e != cudaSuccess)
                 return fail(h, SLAQ_E_NOMEM, std::string("cudaMalloc of the packed pool: ") + cudaGetErrorString(e));
+            int rc_new = pipe_to_device(h, {{new_pool, losses + lo, sizeof(double) * (size_t)total}});
+            if (!rc_new && !check_here) {
+                finite_kernel<<<h->sm_count * 4, 256, 0, st>>>(new_pool, (size_t)total, h->scratch.load_flag, h->mailbox,
+                                                               ++h->call_seq, h->scratch.append_ticket);
+                rc_new = wait_mailbox(h, "check of the losses");
+                if (!rc_new && h->mailbox->err) rc_new = fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
+            }
+            if (rc_new) {
+                cudaStreamSynchronize(st);
+                cudaFree(new_pool);
+                return rc_new;
+            }
         }
         if (h->packed_pool) {
             std::vector<int32_t> gone;
@@ -679,25 +788,30 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
     }
     int status = SLAQ_OK;
     {
-        cudaError_t e = cudaSuccess;
-        if (total > 0) e = cudaMemcpyAsync(d_src, losses + lo, sizeof(double) * (size_t)total, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h->stage.ids, ids, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st);
-        std::vector<int64_t> rel((size_t)n + 1);
-        for (int32_t i = 0; i <= n; ++i) rel[i] = offsets[i] - lo;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h->stage.offsets, rel.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h->stage.k_last, k_last, sizeof(int64_t) * n, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess && m_seen)
-            e = cudaMemcpyAsync(h->stage.m_seen, m_seen, sizeof(double) * n, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) {
+        std::vector<int64_t> shifted;
+        if (lo != 0) {
+            shifted.resize((size_t)n + 1);
+            for (int32_t i = 0; i <= n; ++i) shifted[i] = offsets[i] - lo;
+        }
+        std::vector<Segment> up = {{h->stage.ids, ids, sizeof(int32_t) * n},
+                                   {h->stage.offsets, lo != 0 ? shifted.data() : offsets, sizeof(int64_t) * ((size_t)n + 1)},
+                                   {h->stage.k_last, k_last, sizeof(int64_t) * n}};
+        if (m_seen) up.push_back({h->stage.m_seen, m_seen, sizeof(double) * n});
+        if (!packed) up.push_back({d_src, losses + lo, sizeof(double) * (size_t)total});
+        status = pipe_to_device(h, up);
+        if (!status) {
+            if (!packed && !check_here)
+                finite_kernel<<<h->sm_count * 4, 256, 0, st>>>(d_src, (size_t)total, h->scratch.load_flag, nullptr, 0, nullptr);
             const int threads = 256, warps = threads / 32;
             load_kernel<<<(n + warps - 1) / warps, threads, 0, st>>>(
                 h->job, h->fit, h->ring_pool, h->max_jobs, h->max_hist, n, h->stage.ids, h->stage.offsets, d_src,
-                h->stage.k_last, m_seen ? h->stage.m_seen : nullptr, packed ? 1 : 0);
-            e = cudaGetLastError();
+                h->stage.k_last, m_seen ? h->stage.m_seen : nullptr, packed ? 1 : 0, h->mailbox, ++h->call_seq,
+                h->scratch.append_ticket, h->scratch.load_flag);
+            const cudaError_t e = cudaGetLastError();
+            status = e == cudaSuccess ? wait_mailbox(h, "bulk load") : cuda_fail(h, e, "bulk load");
+            if (!status && h->mailbox->err) status = fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // `rel` and the caller's buffers are free again
-        if (e != cudaSuccess) status = cuda_fail(h, e, "bulk load");
+        if (status) cudaStreamSynchronize(st);   // the caller's buffers are free again
     }
     if (old_pool) cudaFree(old_pool);   // the stream is idle: nothing points into the old pool any more
     if (status) return status;
@@ -848,6 +962,24 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     return SLAQ_OK;
 }
 
+// Results into host arrays.  Arrays in one of the binding's result blocks are written by one kernel, which reports to the
+// mailbox; anything else is copied.
+int results_to_host(slaq_handle* h, const std::vector<Segment>& segments) {
+    Pieces p;
+    size_t bytes = 0;
+    for (const Segment& s : segments) {
+        if (!s.dst) continue;
+        if (p.n == kMaxPieces || reinterpret_cast<uintptr_t>(s.dst) % 8 || !in_result_block(s.dst, s.bytes)) return pipe_to_host(h, segments);
+        p.add(s.dst, s.src, s.bytes);
+        bytes += s.bytes;
+    }
+    if (p.n == 0) return SLAQ_OK;
+    const unsigned blocks = (unsigned)std::min<size_t>(64, 1 + bytes / 32768);
+    pieces_kernel<<<dim3(blocks, p.n), 256, 0, h->stream>>>(p, h->mailbox, ++h->call_seq, h->scratch.append_ticket, nullptr);
+    CK(cudaGetLastError(), "results");
+    return wait_mailbox(h, "results");
+}
+
 // An epoch whose allocation goes to a host array.
 int epoch_to_host(slaq_handle* h, double T, int64_t C, int32_t* out_alloc, bool only_allocate) {
     const int rc = run_epoch(h, T, C, nullptr, only_allocate, true);
@@ -870,13 +1002,6 @@ int epoch_to_host(slaq_handle* h, double T, int64_t C, int32_t* out_alloc, bool 
         return ec ? ec : rc;
     }
     return rc;
-}
-
-template <class T>
-int fetch(slaq_handle* h, T* host, const T* dev, size_t n, const char* what) {
-    if (!host) return SLAQ_OK;
-    CK(cudaMemcpyAsync(host, dev, sizeof(T) * n, cudaMemcpyDeviceToHost, h->stream), what);
-    return SLAQ_OK;
 }
 
 }  // namespace
@@ -911,6 +1036,7 @@ int slaq_create(int32_t max_jobs, int32_t max_hist, slaq_t** out) {
 int slaq_destroy(slaq_t* h) {
     if (!h) return SLAQ_OK;
     if (h->ws) cudaStreamSynchronize(h->stream);
+    if (h->pipe_user) pipe_release();
     for (auto& ev : h->ev)
         if (ev) cudaEventDestroy(ev);
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
@@ -1039,20 +1165,26 @@ int slaq_set_time_model(slaq_t* h, int32_t n, const int32_t* job_ids, const doub
     if (n > 0 && (!s || !w)) return fail(h, SLAQ_E_ARG, "s or w is null");
     const int rc = check_ids(h, n, job_ids, true);
     if (rc) return rc;
-    for (int32_t i = 0; i < n; ++i)
-        if (!(std::isfinite(s[i]) && std::isfinite(w[i]) && s[i] >= 0.0 && w[i] > 0.0))
-            return fail(h, SLAQ_E_ARG, "time law needs finite s >= 0 and w > 0");
+    int32_t bad = all_finite(s, n) && all_finite(w, n) ? 0 : 1;
+    for (int32_t i = 0; i < n; ++i) bad |= (s[i] < 0.0) | (w[i] <= 0.0);
+    if (bad) return fail(h, SLAQ_E_ARG, "time law needs finite s >= 0 and w > 0");
     if (n == 0) return SLAQ_OK;
-    cudaStream_t st = h->stream;
-    CK(cudaMemcpyAsync(h->stage.ids, job_ids, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy job ids");
-    CK(cudaMemcpyAsync(h->stage.losses, s, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy s");
-    CK(cudaMemcpyAsync(h->stage.times, w, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy w");
+    const bool mailed = n <= h->mailbox_jobs;
+    int32_t* const d_ids = mailed ? h->mail_ids() : h->stage.ids;
+    double* const d_s = mailed ? h->mail_losses() : h->stage.losses;
+    double* const d_w = mailed ? h->mail_times() : h->stage.times;
+    if (mailed) {
+        std::memcpy(d_ids, job_ids, sizeof(int32_t) * n);
+        std::memcpy(d_s, s, sizeof(double) * n);
+        std::memcpy(d_w, w, sizeof(double) * n);
+    } else if (const int up = pipe_to_device(h, {{d_ids, job_ids, sizeof(int32_t) * n}, {d_s, s, sizeof(double) * n}, {d_w, w, sizeof(double) * n}})) {
+        return up;
+    }
     const int threads = 256;
-    set_time_kernel<<<(n + threads - 1) / threads, threads, 0, st>>>(h->job, h->max_jobs, n, h->stage.ids, h->stage.losses,
-                                                                    h->stage.times);
+    set_time_kernel<<<(n + threads - 1) / threads, threads, 0, h->stream>>>(h->job, h->max_jobs, n, d_ids, d_s, d_w, h->mailbox,
+                                                                           ++h->call_seq, h->scratch.append_ticket);
     CK(cudaGetLastError(), "time law kernel");
-    CK(cudaStreamSynchronize(st), "time law");
-    return SLAQ_OK;
+    return wait_mailbox(h, "time law");
 }
 
 int slaq_set_target_loss(slaq_t* h, int32_t n, const int32_t* job_ids, const double* targets) {
@@ -1117,9 +1249,7 @@ int slaq_schedule(slaq_t* h, double epoch_seconds, int64_t total_cores, int32_t*
 
 int slaq_set_gains(slaq_t* h, const double* gain) {
     if (!h || !gain) return SLAQ_E_ARG;
-    CK(cudaMemcpyAsync(h->gain, gain, sizeof(double) * (size_t)h->max_jobs * h->max_cores, cudaMemcpyHostToDevice,
-                       h->stream),
-       "copy gains");
+    if (const int rc = pipe_to_device(h, {{h->gain, gain, sizeof(double) * (size_t)h->max_jobs * h->max_cores}})) return rc;
     CK(cudaStreamSynchronize(h->stream), "copy gains");
     return SLAQ_OK;
 }
@@ -1250,21 +1380,18 @@ int slaq_get_predictions(slaq_t* h, double* out_reduction, double* out_gain, int
     if (!h) return SLAQ_E_ARG;
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     const size_t J = (size_t)h->max_jobs;
-    int rc = 0;
     if (out_gain && !h->gain_table_current) {   // the last epoch predicted rows only as far as it needed: write them now
         if (launch_gain(h, h->last_T, h->last_first_unit) < 0) return SLAQ_E_CUDA;
         h->gain_table_current = true;
     }
-    if ((rc = fetch(h, out_reduction, h->reduction, J, "copy reductions"))) return rc;
-    if ((rc = fetch(h, out_gain, h->gain, J * h->max_cores, "copy gains"))) return rc;
-    if ((rc = fetch(h, out_family, h->fit.family, J, "copy families"))) return rc;
-    if ((rc = fetch(h, out_params, h->fit.params, 4 * J, "copy parameters"))) return rc;
-    if ((rc = fetch(h, out_residual, h->fit.residual, 2 * J, "copy residuals"))) return rc;
-    if ((rc = fetch(h, out_status, h->fit.status, J, "copy status"))) return rc;
-    if ((rc = fetch(h, out_sweeps, h->fit.sweeps, 2 * J, "copy sweeps"))) return rc;
-    if ((rc = fetch(h, out_largest, h->fit.largest, J, "copy largest reductions"))) return rc;
-    CK(cudaStreamSynchronize(h->stream), "copy predictions");
-    return SLAQ_OK;
+    return results_to_host(h, {{out_gain, h->gain, 8 * J * h->max_cores},
+                               {out_reduction, h->reduction, 8 * J},
+                               {out_family, h->fit.family, J},
+                               {out_params, h->fit.params, 8 * 4 * J},
+                               {out_residual, h->fit.residual, 8 * 2 * J},
+                               {out_status, h->fit.status, 4 * J},
+                               {out_sweeps, h->fit.sweeps, 4 * 2 * J},
+                               {out_largest, h->fit.largest, 8 * J}});
 }
 
 int slaq_get_normalised(slaq_t* h, int32_t n, const int32_t* job_ids, int64_t capacity, int64_t* out_offsets,
@@ -1330,14 +1457,11 @@ int slaq_get_fit_state(slaq_t* h, double* out_params, uint8_t* out_mask, int64_t
     if (!h || !out_params || !out_mask || !out_k || !out_span || !out_scale) return SLAQ_E_ARG;
     if (const int rc = check_device(h)) return rc;
     const size_t J = (size_t)h->max_jobs;
-    int rc;
-    if ((rc = fetch(h, out_params, h->fit.both, 8 * J, "copy fitted parameters"))) return rc;
-    if ((rc = fetch(h, out_mask, h->fit.mask, J, "copy fit masks"))) return rc;
-    if ((rc = fetch(h, out_k, h->fit.k_fit, J, "copy fit iteration indices"))) return rc;
-    if ((rc = fetch(h, out_span, h->fit.span, J, "copy fit spans"))) return rc;
-    if ((rc = fetch(h, out_scale, h->fit.largest, J, "copy fit scales"))) return rc;
-    CK(cudaStreamSynchronize(h->stream), "copy fit state");
-    return SLAQ_OK;
+    return results_to_host(h, {{out_params, h->fit.both, 8 * 8 * J},
+                               {out_mask, h->fit.mask, J},
+                               {out_k, h->fit.k_fit, 8 * J},
+                               {out_span, h->fit.span, 8 * J},
+                               {out_scale, h->fit.largest, 8 * J}});
 }
 
 int slaq_set_fit_state(slaq_t* h, const double* params, const uint8_t* mask, const int64_t* k, const double* span,
@@ -1395,6 +1519,8 @@ struct StateLayout {
     size_t off_offsets, off_losses, bytes;
 };
 
+constexpr int kPieceBlocks = 16;   // blocks per array of a blob
+
 StateLayout state_layout(int32_t max_jobs, int64_t total_points) {
     StateLayout L;
     L.J8 = ((size_t)max_jobs + 7) / 8 * 8;
@@ -1424,18 +1550,46 @@ StateLayout state_layout(int32_t max_jobs, int64_t total_points) {
     return L;
 }
 
-int read_counts(slaq_handle* h, std::vector<int32_t>& counts, int64_t* total, int32_t* longest) {
-    counts.resize((size_t)h->max_jobs);
-    CK(cudaMemcpyAsync(counts.data(), h->job.count, sizeof(int32_t) * counts.size(), cudaMemcpyDeviceToHost, h->stream),
-       "read window lengths");
-    CK(cudaStreamSynchronize(h->stream), "read window lengths");
-    *total = 0;
-    *longest = 0;
-    for (int32_t c : counts) {
-        *total += c > 0 ? c : 0;
-        *longest = std::max(*longest, c);
-    }
+// Offsets of all windows into h->stage.offsets; their total and the longest to the host.
+int window_offsets(slaq_handle* h, int64_t* total, int32_t* longest) {
+    window_offsets_kernel<<<1, 1024, 0, h->stream>>>(h->job.count, h->max_jobs, h->stage.offsets, h->mailbox, ++h->call_seq);
+    CK(cudaGetLastError(), "window lengths");
+    if (const int rc = wait_mailbox(h, "window lengths")) return rc;
+    *total = h->mailbox->points;
+    *longest = h->mailbox->longest;
     return SLAQ_OK;
+}
+
+// The arrays of a blob besides the windows, between the handle's state and the blob's image on the device.
+Pieces state_pieces(const slaq_handle* h, const StateLayout& L, char* image, bool into_image) {
+    const size_t J = (size_t)h->max_jobs;
+    Pieces p;
+    auto add = [&](size_t off, void* array, size_t bytes) {
+        if (into_image) p.add(image + off, array, bytes);
+        else p.add(array, image + off, bytes);
+    };
+    add(L.off_tm, h->job.tm, 8 * 8 * J);
+    add(L.off_s_set, h->job.s_set, 8 * J);
+    add(L.off_w_set, h->job.w_set, 8 * J);
+    add(L.off_last_alloc, h->job.last_alloc, 4 * J);
+    add(L.off_target, h->job.target, 8 * J);
+    add(L.off_both, h->fit.both, 8 * 8 * J);
+    add(L.off_mask, h->fit.mask, J);
+    add(L.off_k_fit, h->fit.k_fit, 8 * J);
+    add(L.off_span, h->fit.span, 8 * J);
+    add(L.off_largest, h->fit.largest, 8 * J);
+    add(L.off_warm_p, h->fit.warm_p, 8 * 8 * J);
+    add(L.off_warm_mask, h->fit.warm_mask, J);
+    add(L.off_warm_k, h->fit.warm_k, 8 * J);
+    add(L.off_warm_span, h->fit.warm_span, 8 * J);
+    add(L.off_warm_scale, h->fit.warm_scale, 8 * J);
+    if (into_image) {   // an import takes these through the bulk load
+        p.add(image + L.off_count, h->job.count, 4 * J);
+        p.add(image + L.off_k_last, h->job.k_last, 8 * J);
+        p.add(image + L.off_m_seen, h->job.m_seen, 8 * J);
+        p.add(image + L.off_offsets, h->stage.offsets, 8 * (J + 1));
+    }
+    return p;
 }
 
 }  // namespace
@@ -1443,10 +1597,9 @@ int read_counts(slaq_handle* h, std::vector<int32_t>& counts, int64_t* total, in
 int slaq_export_state_bytes(slaq_t* h, size_t* out_bytes) {
     if (!h || !out_bytes) return SLAQ_E_ARG;
     if (const int rc = check_device(h)) return rc;
-    std::vector<int32_t> counts;
     int64_t total = 0;
     int32_t longest = 0;
-    if (const int rc = read_counts(h, counts, &total, &longest)) return rc;
+    if (const int rc = window_offsets(h, &total, &longest)) return rc;
     *out_bytes = state_layout(h->max_jobs, total).bytes;
     return SLAQ_OK;
 }
@@ -1454,51 +1607,28 @@ int slaq_export_state_bytes(slaq_t* h, size_t* out_bytes) {
 int slaq_export_state(slaq_t* h, void* out_blob, size_t capacity) {
     if (!h || !out_blob) return SLAQ_E_ARG;
     if (const int rc = check_device(h)) return rc;
-    std::vector<int32_t> counts;
     int64_t total = 0;
     int32_t longest = 0;
-    if (const int rc = read_counts(h, counts, &total, &longest)) return rc;
+    if (const int rc = window_offsets(h, &total, &longest)) return rc;
     const StateLayout L = state_layout(h->max_jobs, total);
     if (capacity < L.bytes) return fail(h, SLAQ_E_RANGE, "blob capacity below slaq_export_state_bytes()");
-    char* blob = static_cast<char*>(out_blob);
-    std::memset(blob, 0, L.bytes);
-    StateHeader hd{kStateMagic, kStateVersion, h->max_jobs, longest, 0, total, (uint64_t)L.bytes};
-    std::memcpy(blob, &hd, sizeof hd);
-    const size_t J = (size_t)h->max_jobs;
-    int64_t* offsets = reinterpret_cast<int64_t*>(blob + L.off_offsets);
-    offsets[0] = 0;
-    for (size_t j = 0; j < J; ++j) offsets[j + 1] = offsets[j] + (counts[j] > 0 ? counts[j] : 0);
+    // the blob is put together on the device and comes over in one piece
     cudaStream_t st = h->stream;
-    const cudaMemcpyKind down = cudaMemcpyDeviceToHost;
-    std::memcpy(blob + L.off_count, counts.data(), 4 * J);
-    CK(cudaMemcpyAsync(blob + L.off_k_last, h->job.k_last, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_m_seen, h->job.m_seen, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_tm, h->job.tm, 8 * 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_s_set, h->job.s_set, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_w_set, h->job.w_set, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_last_alloc, h->job.last_alloc, 4 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_target, h->job.target, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_both, h->fit.both, 8 * 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_mask, h->fit.mask, J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_k_fit, h->fit.k_fit, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_span, h->fit.span, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_largest, h->fit.largest, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_warm_p, h->fit.warm_p, 8 * 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_warm_mask, h->fit.warm_mask, J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_warm_k, h->fit.warm_k, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_warm_span, h->fit.warm_span, 8 * J, down, st), "export state");
-    CK(cudaMemcpyAsync(blob + L.off_warm_scale, h->fit.warm_scale, 8 * J, down, st), "export state");
+    void* buf = nullptr;
+    if (const int rc = ensure_call_buffer(h, L.bytes, &buf)) return rc;
+    char* const image = static_cast<char*>(buf);
+    CK(cudaMemsetAsync(image, 0, L.bytes, st), "export state");   // the gaps between the arrays
+    const Pieces p = state_pieces(h, L, image, true);
+    pieces_kernel<<<dim3(kPieceBlocks, p.n), 256, 0, st>>>(p, nullptr, 0, nullptr, nullptr);
     if (total > 0) {
-        void* buf = nullptr;
-        if (const int rc = ensure_call_buffer(h, 8 * (size_t)total, &buf)) return rc;
-        CK(cudaMemcpyAsync(h->stage.offsets, offsets, 8 * (J + 1), cudaMemcpyHostToDevice, st), "export state");
         const int threads = 256, warps = threads / 32;
         export_windows_kernel<<<(h->max_jobs + warps - 1) / warps, threads, 0, st>>>(h->job, h->max_jobs, h->stage.offsets,
-                                                                                  static_cast<double*>(buf));
-        CK(cudaGetLastError(), "export kernel");
-        CK(cudaMemcpyAsync(blob + L.off_losses, buf, 8 * (size_t)total, down, st), "export state");
+                                                                                  reinterpret_cast<double*>(image + L.off_losses));
     }
-    CK(cudaStreamSynchronize(st), "export state");
+    CK(cudaGetLastError(), "export kernels");
+    if (const int rc = pipe_to_host(h, {{out_blob, image, L.bytes}})) return rc;
+    const StateHeader hd{kStateMagic, kStateVersion, h->max_jobs, longest, 0, total, (uint64_t)L.bytes};
+    std::memcpy(out_blob, &hd, sizeof hd);
     return SLAQ_OK;
 }
 
@@ -1518,7 +1648,6 @@ int slaq_import_state(slaq_t* h, const void* blob_in, size_t bytes) {
     const size_t J = (size_t)h->max_jobs;
     const int32_t* counts = reinterpret_cast<const int32_t*>(blob + L.off_count);
     const int64_t* offsets = reinterpret_cast<const int64_t*>(blob + L.off_offsets);
-    const int64_t* k_last = reinterpret_cast<const int64_t*>(blob + L.off_k_last);
     const double* m_seen = reinterpret_cast<const double*>(blob + L.off_m_seen);
     const uint8_t* mask = reinterpret_cast<const uint8_t*>(blob + L.off_mask);
     const uint8_t* warm_mask = reinterpret_cast<const uint8_t*>(blob + L.off_warm_mask);
@@ -1530,57 +1659,51 @@ int slaq_import_state(slaq_t* h, const void* blob_in, size_t bytes) {
         if (std::isnan(m_seen[j]) || m_seen[j] == INFINITY) return fail(h, SLAQ_E_NONFINITE, "state blob: m_seen must be a number below +infinity");
         if (mask[j] > 3 || warm_mask[j] > 3) return fail(h, SLAQ_E_ARG, "state blob: fit mask above 3");
     }
-    // everything the handle holds goes; then the windows come in as a bulk load into rings (which checks the losses)
+    // everything the handle holds goes; then the windows come in as a bulk load into rings (which checks the losses), and the
+    // other arrays are unpacked over it
     cudaStream_t st = h->stream;
-    {
-        const int threads = 256;
-        init_jobs_kernel<<<(h->max_jobs + threads - 1) / threads, threads, 0, st>>>(
-            h->job, h->fit, h->ring_pool, h->max_jobs, h->max_hist, nullptr, h->max_jobs, h->alloc, h->reduction);
-        CK(cudaGetLastError(), "import: reset kernel");
-        CK(cudaStreamSynchronize(st), "import: reset");
-        std::fill(h->active.begin(), h->active.end(), 0);
-        std::fill(h->in_packed.begin(), h->in_packed.end(), 0);
-        std::fill(h->hinted.begin(), h->hinted.end(), 0);
-        h->n_hinted = 0;
-        h->n_active = 0;
-        if (h->packed_pool) {
-            cudaFree(h->packed_pool);
-            h->packed_pool = nullptr;
-            h->packed_len = 0;
-            h->job.packed_lo = h->job.packed_hi = nullptr;
+    void* buf = nullptr;
+    if (const int rc = ensure_call_buffer(h, L.bytes, &buf)) return rc;
+    char* const image = static_cast<char*>(buf);
+    if (const int rc = pipe_to_device(h, {{image, blob, L.bytes}})) return rc;
+    const int threads = 256, warps = threads / 32;
+    init_jobs_kernel<<<(h->max_jobs + threads - 1) / threads, threads, 0, st>>>(
+        h->job, h->fit, h->ring_pool, h->max_jobs, h->max_hist, nullptr, h->max_jobs, h->alloc, h->reduction);
+    std::fill(h->active.begin(), h->active.end(), 0);
+    std::fill(h->in_packed.begin(), h->in_packed.end(), 0);
+    std::fill(h->hinted.begin(), h->hinted.end(), 0);
+    h->n_hinted = 0;
+    h->n_active = 0;
+    h->have_epoch = false;
+    const double* const d_losses = reinterpret_cast<const double*>(image + L.off_losses);
+    if (hd.total_points > 0)
+        finite_kernel<<<h->sm_count * 4, 256, 0, st>>>(d_losses, (size_t)hd.total_points, h->scratch.load_flag, nullptr, 0, nullptr);
+    load_kernel<<<(h->max_jobs + warps - 1) / warps, threads, 0, st>>>(
+        h->job, h->fit, h->ring_pool, h->max_jobs, h->max_hist, h->max_jobs, nullptr, reinterpret_cast<const int64_t*>(image + L.off_offsets),
+        d_losses, reinterpret_cast<const int64_t*>(image + L.off_k_last), reinterpret_cast<const double*>(image + L.off_m_seen), 0, nullptr, 0,
+        nullptr, h->scratch.load_flag);
+    const Pieces p = state_pieces(h, L, image, false);
+    pieces_kernel<<<dim3(kPieceBlocks, p.n), 256, 0, st>>>(p, h->mailbox, ++h->call_seq, h->scratch.append_ticket, h->scratch.load_flag);
+    CK(cudaGetLastError(), "import kernels");
+    if (const int rc = wait_mailbox(h, "import")) return rc;
+    if (h->packed_pool) {   // nothing points into it any more
+        cudaFree(h->packed_pool);
+        h->packed_pool = nullptr;
+        h->packed_len = 0;
+        h->job.packed_lo = h->job.packed_hi = nullptr;
+    }
+    if (h->mailbox->err) return fail(h, SLAQ_E_NONFINITE, "a loss is not finite");
+    const double* target = reinterpret_cast<const double*>(blob + L.off_target);
+    for (size_t j = 0; j < J; ++j) {
+        if (offsets[j + 1] > offsets[j]) {
+            h->active[j] = 1;
+            h->n_active += 1;
         }
-        h->have_epoch = false;
+        if (!std::isnan(target[j])) {
+            h->hinted[j] = 1;
+            h->n_hinted += 1;
+        }
     }
-    std::vector<int32_t> ids(J);
-    for (size_t j = 0; j < J; ++j) ids[j] = (int32_t)j;
-    const int rc = do_load(h, h->max_jobs, ids.data(), offsets, reinterpret_cast<const double*>(blob + L.off_losses), k_last,
-                           m_seen, false);
-    if (rc) return rc;
-    const cudaMemcpyKind up = cudaMemcpyHostToDevice;
-    CK(cudaMemcpyAsync(h->job.tm, blob + L.off_tm, 8 * 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->job.s_set, blob + L.off_s_set, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->job.w_set, blob + L.off_w_set, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->job.last_alloc, blob + L.off_last_alloc, 4 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->job.target, blob + L.off_target, 8 * J, up, st), "import state");
-    {
-        const double* target = reinterpret_cast<const double*>(blob + L.off_target);
-        for (size_t j = 0; j < J; ++j)
-            if (!std::isnan(target[j])) {
-                h->hinted[j] = 1;
-                h->n_hinted += 1;
-            }
-    }
-    CK(cudaMemcpyAsync(h->fit.both, blob + L.off_both, 8 * 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.mask, blob + L.off_mask, J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.k_fit, blob + L.off_k_fit, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.span, blob + L.off_span, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.largest, blob + L.off_largest, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.warm_p, blob + L.off_warm_p, 8 * 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.warm_mask, blob + L.off_warm_mask, J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.warm_k, blob + L.off_warm_k, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.warm_span, blob + L.off_warm_span, 8 * J, up, st), "import state");
-    CK(cudaMemcpyAsync(h->fit.warm_scale, blob + L.off_warm_scale, 8 * J, up, st), "import state");
-    CK(cudaStreamSynchronize(st), "import state");
     return SLAQ_OK;
 }
 

@@ -92,8 +92,10 @@ struct SelectGlobal {
 // Page-locked host memory of a handle that kernels write and read directly: a call is over when `done` holds its number.
 struct Mailbox {
     volatile uint32_t done;
-    volatile int32_t err;            // the device error word when the call finished
-    uint32_t pad[14];
+    volatile int32_t err;            // the device error word when the call finished; a bulk load: a loss is not finite
+    volatile int64_t points;         // state export: stored losses in all, and the longest window
+    volatile int32_t longest;
+    uint32_t pad[11];
 };
 constexpr int32_t kMailboxJobs = 32768;   // most entries per call that pass through the mailbox's arrays
 
@@ -107,7 +109,8 @@ struct Scratch {
     SelectState* sel;
     long long* counters;             // [16] statistics accumulated by kernels during an epoch
     long long* published;            // [16] those of the last finished epoch
-    unsigned int* append_ticket;     // blocks of the append kernel that are done
+    unsigned int* append_ticket;     // blocks of a reporting kernel that are done
+    int32_t* load_flag;              // a bulk load brought a loss that is not finite
     size_t zero_bytes;
     int32_t* gt;                     // per job: during the passes the start of its candidate segment, then gains above the threshold
     int32_t* eq;                     // per job: during the passes the end of its segment, then gains equal to the threshold
@@ -165,6 +168,7 @@ struct slaq_handle {
     int32_t* alloc = nullptr;
     double* reduction = nullptr;
     int32_t* err_word = nullptr;      // device error flags set by kernels
+    bool pipe_user = false;           // counted among the users of the bulk copies' buffers
     void* mailbox_mem = nullptr;      // page-locked: Mailbox, then ids, losses, times, cores in and the allocation out
     slaq::Mailbox* mailbox = nullptr;
     int32_t mailbox_jobs = 0;         // entries of each of those arrays

@@ -1,0 +1,232 @@
+// Bulk copies between ordinary (pageable) host memory and the device.
+//
+// The driver moves pageable memory through its own staging buffer with one thread, at 6 to 9 GB/s, several times below
+// what the link does.  Here up to kPipeThreads threads each take every n-th chunk, copy it into (or out of) one of their
+// two page-locked buffers and queue the transfer of that buffer, so that copies of one chunk run beside transfers of
+// others.  Measured on 16 MB of histories: 1.6 ms by cudaMemcpyAsync, 0.5 ms so.  Page-locked memory is handed to the copy engine
+// as it is.  Below kPipeFrom bytes starting threads costs more than it gives and the driver's path is taken.
+#include "slaq_pipe.cuh"
+
+#include <algorithm>
+#include <atomic>
+#include <cstring>
+#include <mutex>
+#include <system_error>
+#include <thread>
+
+#include <map>
+
+#include "slaq_internal.cuh"
+
+namespace slaq {
+
+namespace {
+
+constexpr int kPipeThreads = 8, kPipeBuffers = 2;
+constexpr size_t kPipeChunk = 256 * 1024;
+constexpr size_t kResultBytes = 64 << 20, kResultLeast = 64 << 10;
+constexpr size_t kPipeFrom = 256 * 1024;
+
+struct Pool {
+    std::mutex lock;         // one bulk copy of the process at a time uses the buffers
+    std::mutex count_lock;
+    int handles = 0;
+    char* memory = nullptr;
+    // result blocks by address (guarded by count_lock)
+    struct Block {
+        size_t bytes;
+        bool taken;
+    };
+    std::map<const char*, Block> blocks;
+    size_t block_bytes = 0;
+};
+
+Pool& pool() {
+    static Pool p;
+    return p;
+}
+
+bool page_locked(const void* p) {
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return attr.type == cudaMemoryTypeHost;
+}
+
+int failed(slaq_handle* h, cudaError_t e) {
+    h->err = std::string("bulk copy: ") + cudaGetErrorString(e);
+    return SLAQ_E_CUDA;
+}
+
+// Copies chunk after chunk of one direction; what `thread` of `threads` does.
+void work(slaq_handle* h, const std::vector<Segment>& chunks, bool down, int thread, int threads, std::atomic<int>& error) {
+    cudaError_t e = cudaSetDevice(h->device);   // a new thread starts on device 0
+    cudaEvent_t done[kPipeBuffers] = {};
+    for (int b = 0; b < kPipeBuffers && e == cudaSuccess; ++b) e = cudaEventCreateWithFlags(&done[b], cudaEventDisableTiming);
+    char* const base = pool().memory + (size_t)thread * kPipeBuffers * kPipeChunk;
+    const Segment* flying[kPipeBuffers] = {};   // chunk whose transfer was last queued on each buffer
+    int b = 0;
+    auto land = [&](int k) {                    // wait for a buffer's transfer; downwards, empty it
+        if (!flying[k]) return;
+        e = cudaEventSynchronize(done[k]);
+        if (e == cudaSuccess && down) std::memcpy(flying[k]->dst, base + k * kPipeChunk, flying[k]->bytes);
+        flying[k] = nullptr;
+    };
+    for (size_t c = thread; c < chunks.size() && e == cudaSuccess && !error.load(); c += threads, b = (b + 1) % kPipeBuffers) {
+        char* const buffer = base + b * kPipeChunk;
+        land(b);
+        if (e != cudaSuccess) break;
+        if (!down) std::memcpy(buffer, chunks[c].src, chunks[c].bytes);
+        e = down ? cudaMemcpyAsync(buffer, chunks[c].src, chunks[c].bytes, cudaMemcpyDeviceToHost, h->stream)
+                 : cudaMemcpyAsync(chunks[c].dst, buffer, chunks[c].bytes, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(done[b], h->stream);
+        flying[b] = &chunks[c];
+    }
+    for (int k = 0; k < kPipeBuffers && e == cudaSuccess; ++k, b = (b + 1) % kPipeBuffers) land(b);   // the buffers are free again
+    for (cudaEvent_t d : done)
+        if (d) cudaEventDestroy(d);
+    if (e != cudaSuccess) error.store((int)e);
+}
+
+int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
+    std::vector<Segment> chunks;
+    size_t total = 0;
+    for (const Segment& s : segments) {
+        const void* const host = down ? s.dst : s.src;
+        if (s.bytes == 0 || !host) continue;
+        if (s.bytes >= kPipeFrom && page_locked(host)) {
+            const cudaError_t e = cudaMemcpyAsync(s.dst, s.src, s.bytes, down ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, h->stream);
+            if (e != cudaSuccess) return failed(h, e);
+            continue;
+        }
+        total += s.bytes;
+        for (size_t at = 0; at < s.bytes; at += kPipeChunk)
+            chunks.push_back({static_cast<char*>(s.dst) + at, static_cast<const char*>(s.src) + at, std::min(kPipeChunk, s.bytes - at)});
+    }
+    Pool& p = pool();
+    std::unique_lock<std::mutex> hold(p.lock, std::defer_lock);
+    if (total >= kPipeFrom) {
+        hold.lock();
+        if (!p.memory &&
+            cudaHostAlloc(reinterpret_cast<void**>(&p.memory), kPipeThreads * kPipeBuffers * kPipeChunk, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            p.memory = nullptr;   // no page-locked memory to be had: the driver's path does
+        }
+    }
+    if (total < kPipeFrom || !p.memory) {
+        for (const Segment& s : chunks) {
+            const cudaError_t e = cudaMemcpyAsync(s.dst, s.src, s.bytes, down ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, h->stream);
+            if (e != cudaSuccess) return failed(h, e);
+        }
+    } else {
+        const int cores = std::max(1, (int)std::thread::hardware_concurrency());
+        const int threads = (int)std::min<size_t>({(size_t)kPipeThreads, (size_t)cores, (total + kPipeFrom - 1) / kPipeFrom, chunks.size()});
+        std::atomic<int> error{0};
+        std::thread helper[kPipeThreads];
+        int started = 1;
+        // a helper that cannot be started leaves its chunks to be done here afterwards
+        for (; started < threads; ++started) {
+            try {
+                helper[started] = std::thread(work, h, std::cref(chunks), down, started, threads, std::ref(error));
+            } catch (const std::system_error&) {
+                break;
+            }
+        }
+        work(h, chunks, down, 0, threads, error);
+        for (int t = 1; t < started; ++t) helper[t].join();
+        for (int t = started; t < threads; ++t) work(h, chunks, down, t, threads, error);
+        if (error.load()) return failed(h, (cudaError_t)error.load());
+    }
+    if (down) {
+        const cudaError_t e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) return failed(h, e);
+    }
+    return SLAQ_OK;
+}
+
+}  // namespace
+
+int pipe_to_device(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, false); }
+int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, true); }
+
+void pipe_retain() {
+    std::lock_guard<std::mutex> hold(pool().count_lock);
+    ++pool().handles;
+}
+
+void pipe_release() {
+    Pool& p = pool();
+    std::lock_guard<std::mutex> hold(p.count_lock);
+    if (--p.handles > 0) return;
+    std::lock_guard<std::mutex> use(p.lock);
+    if (p.memory) cudaFreeHost(p.memory);
+    p.memory = nullptr;
+    for (auto it = p.blocks.begin(); it != p.blocks.end();) {
+        if (it->second.taken) {
+            ++it;   // freed when it is given back
+            continue;
+        }
+        p.block_bytes -= it->second.bytes;
+        cudaFreeHost(const_cast<char*>(it->first));
+        it = p.blocks.erase(it);
+    }
+}
+
+bool in_result_block(const void* q, size_t bytes) {
+    Pool& p = pool();
+    std::lock_guard<std::mutex> hold(p.count_lock);
+    const char* const at = static_cast<const char*>(q);
+    auto it = p.blocks.upper_bound(at);
+    if (it == p.blocks.begin()) return false;
+    --it;
+    return it->second.taken && at + bytes <= it->first + it->second.bytes;
+}
+
+}  // namespace slaq
+
+void* slaq_result_take(size_t bytes) {
+    using namespace slaq;
+    size_t size = kResultLeast;
+    while (size < bytes) size <<= 1;
+    Pool& p = pool();
+    std::lock_guard<std::mutex> hold(p.count_lock);
+    for (auto& b : p.blocks)
+        if (!b.second.taken && b.second.bytes == size) {
+            b.second.taken = true;
+            return const_cast<char*>(b.first);
+        }
+    if (p.handles == 0 || size > kResultBytes) return nullptr;
+    for (auto it = p.blocks.begin(); it != p.blocks.end() && p.block_bytes + size > kResultBytes;) {   // make room
+        if (it->second.taken) {
+            ++it;
+            continue;
+        }
+        p.block_bytes -= it->second.bytes;
+        cudaFreeHost(const_cast<char*>(it->first));
+        it = p.blocks.erase(it);
+    }
+    if (p.block_bytes + size > kResultBytes) return nullptr;
+    void* m = nullptr;
+    if (cudaHostAlloc(&m, size, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    p.blocks[static_cast<char*>(m)] = {size, true};
+    p.block_bytes += size;
+    return m;
+}
+
+void slaq_result_give(void* block) {
+    using namespace slaq;
+    Pool& p = pool();
+    std::lock_guard<std::mutex> hold(p.count_lock);
+    auto it = p.blocks.find(static_cast<char*>(block));
+    if (it == p.blocks.end()) return;
+    it->second.taken = false;
+    if (p.handles > 0) return;
+    p.block_bytes -= it->second.bytes;
+    p.blocks.erase(it);
+    cudaFreeHost(block);
+}

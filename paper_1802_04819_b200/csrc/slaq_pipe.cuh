@@ -1,0 +1,36 @@
+// Bulk copies between ordinary host memory and the device.
+#pragma once
+
+#include <cstddef>
+#include <vector>
+
+struct slaq_handle;
+
+namespace slaq {
+
+struct Segment {
+    void* dst;
+    const void* src;
+    size_t bytes;
+};
+
+// Copy all segments, queued on the handle's stream.  to_device: returns once the sources have been read (the copies may
+// still run).  to_host: returns once everything has arrived.  Returns 0, or a status with the handle's message set.
+int pipe_to_device(slaq_handle* h, const std::vector<Segment>& segments);
+int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments);
+
+// A handle begins / ends its life: the page-locked buffers behind the copies are shared by all handles of the process
+// and released with the last of them.
+void pipe_retain();
+void pipe_release();
+
+// Whether [p, p + bytes) lies in a block handed out by slaq_result_take.
+bool in_result_block(const void* p, size_t bytes);
+
+}  // namespace slaq
+
+// Page-locked memory for results the binding hands to its caller: the device writes them where they are read, and memory
+// that is used again has its pages.  At most 64 MB at a time, in blocks of a power of two; NULL beyond that (the binding
+// then takes ordinary memory).  A block that is given back is kept for the next call until the last handle ends.
+extern "C" void* slaq_result_take(size_t bytes);
+extern "C" void slaq_result_give(void* block);
