@@ -577,9 +577,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     h->cap_alloc = cap;
     h->max_cores = cap;
     CK(cudaGetDevice(&h->device), "cudaGetDevice");
-    cudaDeviceProp prop;
-    CK(cudaGetDeviceProperties(&prop, h->device), "cudaGetDeviceProperties");
-    h->sm_count = prop.multiProcessorCount;
+    CK(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device), "cudaDeviceGetAttribute");
     if (select_setup(&h->select_blocks_per_sm)) return fail(h, SLAQ_E_CUDA, "selection kernel setup failed");
     const size_t need = layout(nullptr, nullptr, max_jobs, max_hist, cap);
     if (ws) {
@@ -602,12 +600,9 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     h->mailbox_jobs = std::min(max_jobs, kMailboxJobs);
     {
         const size_t mail = sizeof(Mailbox) + (size_t)h->mailbox_jobs * 28 + 64;
-        const cudaError_t e = cudaHostAlloc(&h->mailbox_mem, mail, cudaHostAllocPortable);
-        if (e != cudaSuccess) {
-            h->mailbox_mem = nullptr;
-            return fail(h, SLAQ_E_NOMEM, std::string("cudaHostAlloc of the mailbox: ") + cudaGetErrorString(e));
-        }
-        h->mailbox = new (h->mailbox_mem) Mailbox();   // unified addressing: kernels use the same pointer
+        h->mailbox_mem = page_locked_alloc(mail);
+        if (!h->mailbox_mem) return fail(h, SLAQ_E_NOMEM, "page-locked memory of the mailbox");
+        h->mailbox = new (h->mailbox_mem) Mailbox();
     }
     if (fit_setup()) return fail(h, SLAQ_E_CUDA, "fit kernel setup failed");
     h->active.assign((size_t)max_jobs, 0);
@@ -1041,7 +1036,7 @@ int slaq_destroy(slaq_t* h) {
         if (ev) cudaEventDestroy(ev);
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
-    if (h->mailbox_mem) cudaFreeHost(h->mailbox_mem);
+    page_locked_free(h->mailbox_mem);
     if (h->packed_pool) cudaFree(h->packed_pool);
     if (h->call_buf) cudaFree(h->call_buf);
     if (h->owns_ws && h->ws) cudaFree(h->ws);

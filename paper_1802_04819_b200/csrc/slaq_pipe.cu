@@ -1,20 +1,26 @@
 // Bulk copies between ordinary (pageable) host memory and the device.
 //
-// The driver moves pageable memory through its own staging buffer with one thread, at 6 to 9 GB/s, several times below
+// The driver moves pageable memory through its own staging buffer with one thread, at 6 to 10 GB/s, several times below
 // what the link does.  Here up to kPipeThreads threads each take every n-th chunk, copy it into (or out of) one of their
 // two page-locked buffers and queue the transfer of that buffer, so that copies of one chunk run beside transfers of
-// others.  Measured on 16 MB of histories: 1.6 ms by cudaMemcpyAsync, 0.5 ms so.  Page-locked memory is handed to the copy engine
-// as it is.  Below kPipeFrom bytes starting threads costs more than it gives and the driver's path is taken.
+// others.  16 MB to the device: 1,530 us by cudaMemcpyAsync, 530 us with 4 threads and chunks of 1 MB (640 us with 512 KB,
+// 850 us with 256 KB: a chunk's event and queueing cost more than its copy then), 313 us from page-locked memory, which
+// is handed to the copy engine as it is.  Below kPipeFrom bytes starting threads costs more than it gives and the
+// driver's path is taken.
+//
+// Page-locking costs milliseconds, which a process that loads once should not pay.  So the buffers are made once
+// kPipeEarned bytes have gone (or are about to go) the slow way, and a result block once kResultEarned requests of its
+// size have been answered with ordinary memory: about when they would have paid for themselves.
 #include "slaq_pipe.cuh"
 
 #include <algorithm>
 #include <atomic>
+#include <cstdlib>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <system_error>
 #include <thread>
-
-#include <map>
 
 #include "slaq_internal.cuh"
 
@@ -22,8 +28,10 @@ namespace slaq {
 
 namespace {
 
-constexpr int kPipeThreads = 8, kPipeBuffers = 2;
-constexpr size_t kPipeChunk = 256 * 1024;
+constexpr int kPipeThreads = 4, kPipeBuffers = 2;
+constexpr size_t kPipeChunk = 1024 * 1024, kPipeLeastChunk = 256 * 1024;
+constexpr size_t kPipeEarned = 64 << 20;
+constexpr int kResultEarned = 8;
 constexpr size_t kResultBytes = 64 << 20, kResultLeast = 64 << 10;
 constexpr size_t kPipeFrom = 256 * 1024;
 
@@ -32,6 +40,8 @@ struct Pool {
     std::mutex count_lock;
     int handles = 0;
     char* memory = nullptr;
+    size_t earned = 0;       // bytes that went the driver's way (guarded by lock)
+    std::map<size_t, int> asked;   // requests for result blocks by size, answered with ordinary memory
     // result blocks by address (guarded by count_lock)
     struct Block {
         size_t bytes;
@@ -91,7 +101,7 @@ void work(slaq_handle* h, const std::vector<Segment>& chunks, bool down, int thr
 }
 
 int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
-    std::vector<Segment> chunks;
+    std::vector<Segment> pageable;
     size_t total = 0;
     for (const Segment& s : segments) {
         const void* const host = down ? s.dst : s.src;
@@ -102,25 +112,30 @@ int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
             continue;
         }
         total += s.bytes;
-        for (size_t at = 0; at < s.bytes; at += kPipeChunk)
-            chunks.push_back({static_cast<char*>(s.dst) + at, static_cast<const char*>(s.src) + at, std::min(kPipeChunk, s.bytes - at)});
+        pageable.push_back(s);
     }
     Pool& p = pool();
     std::unique_lock<std::mutex> hold(p.lock, std::defer_lock);
     if (total >= kPipeFrom) {
         hold.lock();
-        if (!p.memory &&
-            cudaHostAlloc(reinterpret_cast<void**>(&p.memory), kPipeThreads * kPipeBuffers * kPipeChunk, cudaHostAllocPortable) != cudaSuccess) {
-            cudaGetLastError();
-            p.memory = nullptr;   // no page-locked memory to be had: the driver's path does
+        p.earned += p.memory ? 0 : total;
+        if (!p.memory && p.earned >= kPipeEarned) {
+            p.earned = 0;
+            p.memory = static_cast<char*>(page_locked_alloc(kPipeThreads * kPipeBuffers * kPipeChunk));
         }
     }
     if (total < kPipeFrom || !p.memory) {
-        for (const Segment& s : chunks) {
+        for (const Segment& s : pageable) {
             const cudaError_t e = cudaMemcpyAsync(s.dst, s.src, s.bytes, down ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, h->stream);
             if (e != cudaSuccess) return failed(h, e);
         }
     } else {
+        const size_t share = (total / (2 * kPipeThreads) + 4095) / 4096 * 4096;   // two chunks per thread, within limits
+        const size_t chunk = std::min(kPipeChunk, std::max(kPipeLeastChunk, share));
+        std::vector<Segment> chunks;
+        for (const Segment& s : pageable)
+            for (size_t at = 0; at < s.bytes; at += chunk)
+                chunks.push_back({static_cast<char*>(s.dst) + at, static_cast<const char*>(s.src) + at, std::min(chunk, s.bytes - at)});
         const int cores = std::max(1, (int)std::thread::hardware_concurrency());
         const int threads = (int)std::min<size_t>({(size_t)kPipeThreads, (size_t)cores, (total + kPipeFrom - 1) / kPipeFrom, chunks.size()});
         std::atomic<int> error{0};
@@ -148,6 +163,28 @@ int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
 
 }  // namespace
 
+// Ordinary memory that is page-locked afterwards: a third of what cudaHostAlloc takes at the sizes used here (0.3 to 0.5 ms
+// against 1.2 to 2.5 ms up to 1 MB).
+void* page_locked_alloc(size_t bytes) {
+    const size_t size = (bytes + 4095) / 4096 * 4096;
+    void* const m = std::aligned_alloc(4096, size);
+    void* seen = nullptr;
+    if (!m) return nullptr;
+    if (cudaHostRegister(m, size, cudaHostRegisterPortable | cudaHostRegisterMapped) == cudaSuccess) {
+        if (cudaHostGetDevicePointer(&seen, m, 0) == cudaSuccess && seen == m) return m;   // kernels use the same address
+        cudaHostUnregister(m);
+    }
+    cudaGetLastError();
+    std::free(m);
+    return nullptr;
+}
+
+void page_locked_free(void* m) {
+    if (!m) return;
+    cudaHostUnregister(m);
+    std::free(m);
+}
+
 int pipe_to_device(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, false); }
 int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, true); }
 
@@ -161,15 +198,17 @@ void pipe_release() {
     std::lock_guard<std::mutex> hold(p.count_lock);
     if (--p.handles > 0) return;
     std::lock_guard<std::mutex> use(p.lock);
-    if (p.memory) cudaFreeHost(p.memory);
+    if (p.memory) page_locked_free(p.memory);
     p.memory = nullptr;
+    p.earned = 0;
+    p.asked.clear();
     for (auto it = p.blocks.begin(); it != p.blocks.end();) {
         if (it->second.taken) {
             ++it;   // freed when it is given back
             continue;
         }
         p.block_bytes -= it->second.bytes;
-        cudaFreeHost(const_cast<char*>(it->first));
+        page_locked_free(const_cast<char*>(it->first));
         it = p.blocks.erase(it);
     }
 }
@@ -197,22 +236,19 @@ void* slaq_result_take(size_t bytes) {
             b.second.taken = true;
             return const_cast<char*>(b.first);
         }
-    if (p.handles == 0 || size > kResultBytes) return nullptr;
+    if (p.handles == 0 || size > kResultBytes || ++p.asked[size] <= kResultEarned) return nullptr;
     for (auto it = p.blocks.begin(); it != p.blocks.end() && p.block_bytes + size > kResultBytes;) {   // make room
         if (it->second.taken) {
             ++it;
             continue;
         }
         p.block_bytes -= it->second.bytes;
-        cudaFreeHost(const_cast<char*>(it->first));
+        page_locked_free(const_cast<char*>(it->first));
         it = p.blocks.erase(it);
     }
     if (p.block_bytes + size > kResultBytes) return nullptr;
-    void* m = nullptr;
-    if (cudaHostAlloc(&m, size, cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
+    void* const m = page_locked_alloc(size);
+    if (!m) return nullptr;
     p.blocks[static_cast<char*>(m)] = {size, true};
     p.block_bytes += size;
     return m;
@@ -228,5 +264,5 @@ void slaq_result_give(void* block) {
     if (p.handles > 0) return;
     p.block_bytes -= it->second.bytes;
     p.blocks.erase(it);
-    cudaFreeHost(block);
+    page_locked_free(block);
 }

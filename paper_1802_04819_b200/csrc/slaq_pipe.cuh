@@ -24,6 +24,10 @@ int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments);
 void pipe_retain();
 void pipe_release();
 
+// Page-locked memory at the same address for host and device; null if there is none to be had.
+void* page_locked_alloc(size_t bytes);
+void page_locked_free(void* m);
+
 // Whether [p, p + bytes) lies in a block handed out by slaq_result_take.
 bool in_result_block(const void* p, size_t bytes);
 
