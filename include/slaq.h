@@ -424,6 +424,16 @@ int slaq_get_fit_phase_cycles(slaq_t* h, int64_t* out_cycles);
  * waits for the device once, when the allocation is copied out.
  */
 int slaq_get_active_count(slaq_t* h, int32_t* out_active);
+/*
+ * The same epoch for shards that live on ONE GPU: handles[0..n-1] in global order (at most 8, distinct, all on one stream
+ * and with one max_cores_per_job), out_alloc[s] a host array of handles[s]'s max_jobs entries.  The fits run beside one
+ * another and one launch does the selection for all.  Equal to the steps below and to slaq_schedule on one handle
+ * holding all jobs, provided SLAQ_P_FIT_CLUSTER_JOBS is set as there.  Messages are those of handles[0].  Errors:
+ * SLAQ_E_ARG; SLAQ_E_RANGE before anything is queued (more than 8 handles, or a handle with a prediction option: use the
+ * steps); SLAQ_E_CUDA.  Warnings as slaq_schedule, for the cluster.
+ */
+int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds, int64_t total_cores,
+                        int32_t* const* out_alloc);
 int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor);
 int slaq_shard_histogram(slaq_t* h, int32_t pass, uint64_t* d_hist, int32_t import_it);
 int slaq_shard_pick(slaq_t* h, int32_t pass, int64_t want);

@@ -30,7 +30,7 @@ EXPORTED_SYMBOLS = [
     "slaq_get_stats", "slaq_get_fit_phase_cycles", "slaq_export_state_bytes", "slaq_export_state",
     "slaq_import_state", "slaq_allocate_static", "slaq_get_active_count", "slaq_shard_predict", "slaq_shard_histogram",
     "slaq_shard_pick", "slaq_shard_pass", "slaq_shard_count", "slaq_shard_finalise", "slaq_shard_count_device",
-    "slaq_shard_finalise_device",
+    "slaq_shard_finalise_device", "slaq_schedule_group",
 ]
 
 
@@ -119,6 +119,7 @@ def load_library(variant: str | None = None):
         "slaq_shard_finalise": (c_int, [vp, c_int64, vp]),
         "slaq_shard_count_device": (c_int, [vp, vp]),
         "slaq_shard_finalise_device": (c_int, [vp, vp, vp]),
+        "slaq_schedule_group": (c_int, [vp, c_int32, c_double, c_int64, vp]),
     }
     sig["slaq_result_take"] = (vp, [c_size_t])      # page-locked memory for results, internal to the binding
     sig["slaq_result_give"] = (None, [vp])
@@ -134,6 +135,22 @@ def workspace_bytes(max_jobs: int, max_hist: int, max_cores_per_job: int) -> int
 
 
 STATIC_MAX_JOBS = 32768
+
+
+def schedule_group(shards, epoch_seconds: float, total_cores: int):
+    """slaq_schedule_group on ``Scheduler`` handles of one GPU, all on one stream.  Returns the list of their allocations,
+    or None if such handles have to be scheduled step by step."""
+    lib, n = shards[0]._lib, len(shards)
+    if any(s._lib is not lib for s in shards):
+        return None
+    out = [np.empty(s.max_jobs, np.int32) for s in shards]
+    handles = (c_void_p * n)(*[s._h.value for s in shards])
+    rows = (c_void_p * n)(*[a.ctypes.data for a in out])
+    rc = lib.slaq_schedule_group(handles, n, float(epoch_seconds), int(total_cores), rows)
+    if rc == -2:
+        return None
+    shards[0]._check(rc)
+    return out
 
 
 def allocate_static(d_gain, total_cores: int, d_out_alloc, d_out_reduction, stream=None) -> int:

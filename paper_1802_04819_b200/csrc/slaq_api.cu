@@ -836,7 +836,7 @@ int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32
     int launches = 0, k;
     if (with_events && cudaEventRecord(h->ev[0], st) != cudaSuccess) return -1;
     if (!only_allocate) {
-        if ((k = launch_fit(h)) < 0) return -1;
+        if ((k = launch_fit(h, st, h->sm_count)) < 0) return -1;
         launches += k;
     }
     if (with_events && cudaEventRecord(h->ev[1], st) != cudaSuccess) return -1;
@@ -1036,6 +1036,7 @@ int slaq_destroy(slaq_t* h) {
         if (ev) cudaEventDestroy(ev);
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
+    if (h->side_stream) cudaStreamDestroy(h->side_stream);
     page_locked_free(h->mailbox_mem);
     if (h->packed_pool) cudaFree(h->packed_pool);
     if (h->call_buf) cudaFree(h->call_buf);
@@ -1255,6 +1256,100 @@ int slaq_allocate_only(slaq_t* h, int64_t total_cores, int32_t* out_alloc) {
     return epoch_to_host(h, 1.0, total_cores, out_alloc, true);
 }
 
+// ---- one cluster in several handles of this GPU ----
+
+int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds, int64_t total_cores, int32_t* const* out_alloc) {
+    if (!handles || n < 1 || !handles[0]) return SLAQ_E_ARG;
+    slaq_t* const h = handles[0];
+    if (!out_alloc) return fail(h, SLAQ_E_ARG, "out_alloc is null");
+    if (!(epoch_seconds > 0.0 && std::isfinite(epoch_seconds))) return fail(h, SLAQ_E_ARG, "epoch_seconds must be positive");
+    if (total_cores < 0) return fail(h, SLAQ_E_ARG, "total_cores must not be negative");
+    if (n > kMaxGroup) return fail(h, SLAQ_E_RANGE, "more handles than one group takes");
+    int64_t active = 0;
+    for (int32_t s = 0; s < n; ++s) {
+        slaq_t* const g = handles[s];
+        if (!g || !out_alloc[s]) return fail(h, SLAQ_E_ARG, "a handle or its out_alloc is null");
+        for (int32_t t = 0; t < s; ++t)
+            if (handles[t] == g) return fail(h, SLAQ_E_ARG, "a handle is listed twice");
+        if (check_device(g)) return fail(h, SLAQ_E_ARG, "a handle was created on another device than the current one");
+        if (g->stream != h->stream) return fail(h, SLAQ_E_ARG, "the handles of a group work on one stream");
+        if (g->max_cores != h->max_cores) return fail(h, SLAQ_E_ARG, "the handles of a group have one max_cores_per_job");
+        if (g->gain_envelope || g->n_hinted > 0) return fail(h, SLAQ_E_RANGE, "prediction options need the single steps");
+        active += g->n_active;
+    }
+    cudaStream_t st = h->stream;
+    const int64_t cap = h->max_cores, usable = std::min<int64_t>(total_cores, active * cap);
+    const int floor_units = total_cores >= active ? 1 : 0;
+    const int64_t want = usable - active * floor_units;
+    for (int32_t s = 0; s < n; ++s) {
+        slaq_t* const g = handles[s];
+        if (const int rc = ensure_weights(g)) return fail(h, rc, g->err);
+        if (!g->scratch_clean) CK(cudaMemsetAsync(g->scratch.zero, 0, g->scratch.zero_bytes, st), "clear scratch");
+        g->scratch_clean = false;   // until the last launch is queued
+        CK(cudaEventRecord(g->ev[0], st), "event");
+    }
+    // The fits run beside one another.  Few jobs: each gets SMs in proportion to its jobs, so that no fit waits for another's
+    // last windows; many jobs: each may use the whole GPU and starts where the one before it runs out of work.
+    const bool split = active * fit_least_lanes(h) <= 4LL * 32 * 16 * h->sm_count;
+    int free_sms = h->sm_count;
+    for (int32_t s = 0; s < n; ++s) {
+        slaq_t* const g = handles[s];
+        int blocks = h->sm_count;
+        if (split) {
+            blocks = s + 1 == n ? free_sms : (int)(active > 0 ? h->sm_count * (int64_t)g->n_active / active : 1);
+            blocks = std::max(1, std::min(blocks, free_sms - (n - 1 - s)));
+            free_sms -= blocks;
+        }
+        cudaStream_t side = st;
+        if (s > 0) {
+            if (!g->side_stream) CK(cudaStreamCreateWithFlags(&g->side_stream, cudaStreamNonBlocking), "create side stream");
+            side = g->side_stream;
+            CK(cudaStreamWaitEvent(side, handles[n - 1]->ev[0], 0), "fork");
+        }
+        const int k = launch_fit(g, side, blocks);
+        if (k < 0) return fail(h, SLAQ_E_CUDA, g->err);
+        g->last_launches = k;
+        CK(cudaEventRecord(g->ev[1], side), "event");
+    }
+    for (int32_t s = 0; s < n; ++s) {
+        if (s > 0) CK(cudaStreamWaitEvent(st, handles[s]->ev[1], 0), "join");
+        CK(cudaEventRecord(handles[s]->ev[2], st), "event");
+    }
+    bool whole_table = false;
+    const int k = launch_select_group(handles, n, epoch_seconds, want, floor_units + 1, ++h->call_seq, &whole_table);
+    if (k < 0) return SLAQ_E_CUDA;
+    for (int32_t s = 0; s < n; ++s) {
+        slaq_t* const g = handles[s];
+        CK(cudaEventRecord(g->ev[3], st), "event");
+        g->scratch_clean = true;
+        g->have_epoch = g->stats_published = true;
+        g->last_epoch_was_graph = false;
+        g->last_launches += s == 0 ? k : 0;
+        g->last_steps = kEpochSteps;
+        g->gain_table_current = whole_table;
+        g->last_T = epoch_seconds;
+        g->last_first_unit = floor_units + 1;
+    }
+    bool copied = false;
+    for (int32_t s = 0; s < n; ++s)
+        if (handles[s]->max_jobs > handles[s]->mailbox_jobs) {
+            CK(cudaMemcpyAsync(out_alloc[s], handles[s]->alloc, sizeof(int32_t) * (size_t)handles[s]->max_jobs, cudaMemcpyDeviceToHost, st),
+               "copy allocation");
+            copied = true;
+        }
+    if (copied) CK(cudaStreamSynchronize(st), "epoch");
+    if (const int wc = wait_mailbox(h, "epoch")) return wc;
+    for (int32_t s = 0; s < n; ++s)
+        if (handles[s]->max_jobs <= handles[s]->mailbox_jobs)
+            std::memcpy(out_alloc[s], handles[s]->mail_alloc(), sizeof(int32_t) * (size_t)handles[s]->max_jobs);
+    if (h->mailbox->err)
+        for (int32_t s = 0; s < n; ++s)
+            if (const int ec = check_device_errors(handles[s])) return fail(h, ec, handles[s]->err);
+    if (active > 0 && total_cores < active) return SLAQ_W_OVERSUBSCRIBED;
+    if (total_cores > active * cap) return SLAQ_W_UNDERFILLED;
+    return SLAQ_OK;
+}
+
 // ---- one cluster sharded over several GPUs ----
 
 int slaq_get_active_count(slaq_t* h, int32_t* out_active) {
@@ -1277,7 +1372,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
     h->scratch_clean = h->stats_published = false;   // these steps leave their counts where they were added up
     CK(cudaEventRecord(h->ev[0], st), "event");
-    if ((k = launch_fit(h)) < 0) return SLAQ_E_CUDA;
+    if ((k = launch_fit(h, st, h->sm_count)) < 0) return SLAQ_E_CUDA;
     launches += k;
     CK(cudaEventRecord(h->ev[1], st), "event");
     if ((k = launch_gain(h, epoch_seconds, h->shard_first_unit)) < 0) return SLAQ_E_CUDA;

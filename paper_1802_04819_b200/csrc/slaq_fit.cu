@@ -1151,8 +1151,20 @@ int fit_setup() {
     return ok ? 0 : -1;
 }
 
-int launch_fit(slaq_handle* h) {
-    cudaStream_t st = h->stream;
+static long long jobs_for_lanes(const slaq_handle* h) {
+    return h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : (long long)h->n_active;
+}
+
+// With few active jobs every job gets more lanes, so that the warps of the GPU all have work: the fewest lanes at which
+// the jobs fill about two slots per warp.
+int fit_least_lanes(const slaq_handle* h) {
+    const long long lanes_wanted = 64LL * h->sm_count * kMaxWarpsPerBlock;
+    int L = 2;
+    while (L < 32 && jobs_for_lanes(h) * L < lanes_wanted) L <<= 1;
+    return L;
+}
+
+int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     int launches = 0;
     // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked
@@ -1167,12 +1179,7 @@ int launch_fit(slaq_handle* h) {
     cls.slice = (int)(h->fit_slice_bytes / sizeof(double));
     cls.slice = std::max(cls.slice, kParked * 2 + ((Hmax + 31) / 32 + 1) * 32);
     auto rows_at = [&](int L) { return (cls.slice - kParked * (64 / L)) / 32 - 1; };
-    // With few active jobs every job gets more lanes, so that the warps of the GPU all have work:
-    // the fewest lanes at which the jobs fill about two slots per warp.
-    const long long jobs_for_lanes = h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : (long long)h->n_active;
-    const long long lanes_wanted = 64LL * h->sm_count * kMaxWarpsPerBlock;
-    int L_min = 2;
-    while (L_min < 32 && jobs_for_lanes * L_min < lanes_wanted) L_min <<= 1;
+    const int L_min = fit_least_lanes(h);
     int h_hi = Hmax;
     for (int L = 32; L >= L_min && h_hi > 0; L >>= 1) {
         const int h_lo = L > L_min ? std::max(rows_at(L / 2), 0) * (L / 2) : 0;
@@ -1188,7 +1195,7 @@ int launch_fit(slaq_handle* h) {
     // The work list: job ids, longest window first.  A job per warp of the GPU and no more: every job starts at once,
     // so their order means nothing and none is made.  Up to kOneBlockSort jobs one block sorts (one launch of about 5 us
     // instead of three of 3 to 4 us each), beyond that a block per 2048 jobs.
-    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= h->sm_count * kMaxWarpsPerBlock;
+    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * kMaxWarpsPerBlock;
     const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
     if (in_order) {
     } else if (J <= kOneBlockSort) {
@@ -1204,14 +1211,14 @@ int launch_fit(slaq_handle* h) {
     }
     int warps = kMaxWarpsPerBlock;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
-    if (in_order) warps = std::min(warps, (J + h->sm_count - 1) / h->sm_count);   // few jobs: spread over all SMs
+    if (in_order) warps = std::min(warps, (J + max_blocks - 1) / max_blocks);   // few jobs: spread over all SMs
     const size_t smem = fit_smem_bytes(cls, warps);
     if (smem > kSmemLimit) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
     const FitKernel kernel = kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
-    int blocks = h->sm_count;   // one block per SM: its registers and shared memory fill one
+    int blocks = max_blocks;   // one block per SM: its registers and shared memory fill one
     const int needed = (J + warps - 1) / warps;   // at least one job per slot
     if (blocks > needed) blocks = needed;
     if (blocks < 1) blocks = 1;

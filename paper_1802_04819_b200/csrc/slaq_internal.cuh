@@ -200,6 +200,7 @@ struct slaq_handle {
     std::vector<long long> graph_key, seen_key;
     cudaGraphExec_t graph_exec = nullptr;
     cudaStream_t capture_stream = nullptr;
+    cudaStream_t side_stream = nullptr;   // the fit of a handle that is scheduled together with others
     int32_t graph_launches = 0;
     bool last_epoch_was_graph = false;
     std::string err;
@@ -209,11 +210,17 @@ namespace slaq {
 
 // kernel launchers: each returns the number of kernels it launched, or -1 after setting h->err
 int fit_setup();   // once per device before the first fit; 0 or -1
-int launch_fit(slaq_handle* h);
+// on `st`, with at most max_blocks blocks
+int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks);
+int fit_least_lanes(const slaq_handle* h);
 int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit);
 // seq != 0: the kernel reports to the handle's mailbox under that number, and writes the allocation there too if it fits
 int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
                   uint32_t seq);
+// one cluster whose jobs are held by n handles of this GPU (n <= kMaxGroup), on the first one's stream; reports to its mailbox
+constexpr int kMaxGroup = 8;
+int launch_select_group(slaq_handle* const* hs, int n, double epoch_seconds, long long want, int first_unit, uint32_t seq,
+                        bool* whole_table);
 bool select_writes_whole_table(const slaq_handle* h, long long want);
 int select_setup(int* blocks_per_sm);   // once per device before the first selection launch; 0 or -1
 int launch_normalise_export(slaq_handle* h, int32_t n, const int64_t* d_offsets, double* d_changes,

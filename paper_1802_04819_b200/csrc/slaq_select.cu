@@ -83,6 +83,7 @@ struct Shared {
     Interval iv;
     u64 scan[kWarps + 1];
     int count, n_more, flag;
+    unsigned int handed[kMaxGroup][2];   // per handle: cores of the rows with candidates, candidates taken at the threshold
 };
 
 // Every block arrives; returns false (in every thread) if the others did not within the limit.
@@ -286,6 +287,32 @@ struct SelectArgs {
     uint32_t seq;
 };
 
+// One handle's jobs, or those of several handles on this GPU that share one cluster's cores: each owns a run of blocks, in
+// order, and all count into the first one's SelectGlobal.
+constexpr int kMaxShards = kMaxGroup;
+struct OneHandle {
+    SelectArgs a;
+    __device__ __forceinline__ int shards() const { return 1; }
+    __device__ __forceinline__ const SelectArgs& of(int) const { return a; }
+    __device__ __forceinline__ int mine(int* block) const {
+        *block = blockIdx.x;
+        return 0;
+    }
+};
+struct ManyHandles {
+    SelectArgs a[kMaxShards];
+    int first_block[kMaxShards + 1];
+    int n;
+    __device__ __forceinline__ int shards() const { return n; }
+    __device__ __forceinline__ const SelectArgs& of(int s) const { return a[s]; }
+    __device__ __forceinline__ int mine(int* block) const {
+        int s = 0;
+        while (s + 1 < n && (int)blockIdx.x >= first_block[s + 1]) ++s;
+        *block = blockIdx.x - first_block[s];
+        return s;
+    }
+};
+
 namespace {
 
 __device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int cores, double R, bool active) {
@@ -297,23 +324,26 @@ __device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int core
 }
 
 // A row's candidates, entries s .. s+c-1, for the block that ranks them.  The first of them carries the row's count.
-__device__ __forceinline__ void list_candidates(const SelectArgs& a, int j, int s, int c, const double* row) {
+__device__ __forceinline__ void list_candidates(const SelectArgs& a, int shard, int j, int s, int c, const double* row) {
     const int at = (int)atomicAdd(&a.gl->n_cand, (unsigned int)c);
     for (int k = 0; k < c && at + k < kFinal; ++k) {
         a.gl->cand_key[at + k] = key_of(row[s + k]);
-        a.gl->cand_pos[at + k] = ((u64)(k == 0 ? c : 0) << 48) | ((u64)j << 10) | (u64)(s + k);
+        a.gl->cand_pos[at + k] = ((u64)(k == 0 ? c : 0) << 48) | ((u64)shard << 41) | ((u64)j << 10) | (u64)(s + k);
     }
 }
 
 constexpr u64 kPosMask = (1ull << 48) - 1;
 
 // The last block: hand out `iv.want` of the n <= kFinal candidates, best first, and complete their rows.
-__device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
+template <class Args>
+__device__ void finish_candidates(const Args& args, Shared& sh) {
     const int tid = threadIdx.x;
-    const int all = min((int)__ldcg(&a.gl->n_cand), kFinal);
+    const SelectGlobal* const gl = args.of(0).gl;
+    const int all = min((int)__ldcg(&gl->n_cand), kFinal);
+    if (tid < 2 * kMaxShards) sh.handed[tid >> 1][tid & 1] = 0;
     for (int i = tid; i < all; i += kThreads) {
-        sh.cand.key[i] = __ldcg(&a.gl->cand_key[i]);
-        sh.cand.pos[i] = __ldcg(&a.gl->cand_pos[i]);
+        sh.cand.key[i] = __ldcg(&gl->cand_key[i]);
+        sh.cand.pos[i] = __ldcg(&gl->cand_pos[i]);
         sh.idx[i] = (unsigned short)i;
         sh.taken[i] = 0;
     }
@@ -348,7 +378,7 @@ __device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
     }
     // what is left is ranked outright: 2^k threads share a candidate's comparisons
     const u64 want = sh.iv.want;
-    if (tid == 0) sh.scan[0] = 0, sh.count = 0;
+    if (tid == 0) sh.scan[0] = 0;
     for (int i = tid; i < n; i += kThreads) sh.narrow[i] = 0;
     __syncthreads();
     int share = 1;
@@ -373,34 +403,32 @@ __device__ void finish_candidates(const SelectArgs& a, Shared& sh) {
     }
     __syncthreads();
     const u64 tau = sh.scan[0];
-    int above = 0;   // all of them are taken; what is left of `want` goes to gains equal to tau
-    for (int i = tid; i < n; i += kThreads) above += sh.cand.key[sh.idx[i]] > tau ? 1 : 0;
-    if (above) atomicAdd(&sh.count, above);
-    long long handed = 0;
     for (int i = tid; i < all; i += kThreads) {
         const u64 pos = sh.cand.pos[i];
+        const int shard = (int)((pos >> 41) & 31);
+        if (sh.taken[i] && sh.cand.key[i] == tau) atomicAdd(&sh.handed[shard][1], 1u);
         const int c = (int)(pos >> 48);
         if (c == 0) continue;          // not the first candidate of its row
-        const int j = (int)((pos & kPosMask) >> 10), s = (int)(pos & 1023);
+        const SelectArgs& a = args.of(shard);
+        const int j = (int)((pos >> 10) & 0x7fffffff), s = (int)(pos & 1023);
         double R = __ldcg(&a.reduction[j]);
         int t = 0;                     // the taken ones of a row are its first
         while (t < c && sh.taken[i + t]) R += __longlong_as_double((long long)sh.cand.key[i + t++]);
         store_alloc(a, j, s + t, R, true);
-        handed += s + t;
+        atomicAdd(&sh.handed[shard][0], (unsigned int)(s + t));
     }
-    u64 sum;
-    block_exclusive((u64)handed, sh, &sum);
-    if (tid == 0) {
-        atomicAdd((u64*)&a.counters[6], sum);
-        a.sel->prefix = tau;
-        a.counters[7] = (long long)want - sh.count;
+    __syncthreads();
+    if (tid == 0) args.of(0).sel->prefix = tau;
+    if (tid < args.shards()) {
+        atomicAdd((u64*)&args.of(tid).counters[6], (u64)sh.handed[tid][0]);
+        args.of(tid).counters[7] = sh.handed[tid][1];
     }
 }
 
 // All blocks: narrow the interval over the rows' candidate segments (gt, eq) until kFinal candidates are left or all
 // are equal; equal ones are handed out here.  Returns whether the last block still has candidates to rank, -1 after a
 // barrier that was not reached.
-__device__ int narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j1, unsigned int& arrived) {
+__device__ int narrow_on_the_grid(const SelectArgs& a, int shard, SelectState* sel, Shared& sh, int j0, int j1, unsigned int& arrived) {
     const int tid = threadIdx.x;
     for (int step = 0; sh.iv.hi - sh.iv.lo > 1 && sh.iv.n > kFinal && step < kRadixPasses; ++step) {
         const int shift = narrow_shift(sh.iv);
@@ -464,7 +492,7 @@ __device__ int narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j
         if (j >= j1 || (a.count && a.count[j] <= 0)) continue;
         const int s = a.gt[j];
         if (!equal && c) {
-            list_candidates(a, j, s, c, a.gain + (size_t)j * a.cap);
+            list_candidates(a, shard, j, s, c, a.gain + (size_t)j * a.cap);
             continue;
         }
         const int take = ahead >= sh.iv.want ? 0 : (int)min((u64)c, sh.iv.want - ahead);
@@ -480,7 +508,7 @@ __device__ int narrow_on_the_grid(const SelectArgs& a, Shared& sh, int j0, int j
     if (equal) {
         block_exclusive((u64)ties, sh, &sum);
         if (tid == 0 && sum) atomicAdd((u64*)&a.counters[7], sum);
-        if (tid == 0 && blockIdx.x == 0) a.sel->prefix = sh.iv.lo;
+        if (tid == 0 && blockIdx.x == 0) sel->prefix = sh.iv.lo;
     }
     return equal ? 0 : 1;
 }
@@ -499,32 +527,42 @@ __device__ bool arrive_last(const SelectArgs& a, Shared& sh) {
 }
 
 // The last block, after everything else: publish the statistics, tell the host, clear the scratch for the next epoch.
-__device__ void finish_epoch(const SelectArgs& a) {
+template <class Args>
+__device__ void finish_epoch(const Args& args) {
     const int tid = threadIdx.x;
     __syncthreads();
-    if (a.published && tid < 16)
-        a.published[tid] = tid == 15 ? (long long)__ldcg(&a.sel->prefix) : __ldcg(&a.counters[tid]);
-    if (a.mail) {
-        if (tid == 0) {
-            a.mail->err = __ldcg(a.err_word);
-            __threadfence_system();
-            a.mail->done = a.seq;
-        }
+    const SelectArgs& first = args.of(0);
+    for (int s = 0; s < args.shards(); ++s) {
+        const SelectArgs& a = args.of(s);
+        if (a.published && tid < 16)
+            a.published[tid] = tid == 15 ? (long long)__ldcg(&first.sel->prefix) : __ldcg(&a.counters[tid]);
     }
-    if (a.zero) {
-        __syncthreads();
-        for (int i = tid; i < a.zero_words; i += kThreads) static_cast<u64*>(a.zero)[i] = 0;
+    if (first.mail && tid == 0) {
+        int32_t err = 0;
+        for (int s = 0; s < args.shards(); ++s) err |= __ldcg(args.of(s).err_word);
+        first.mail->err = err;
+        __threadfence_system();
+        first.mail->done = first.seq;
+    }
+    __syncthreads();
+    for (int s = 0; s < args.shards(); ++s) {
+        const SelectArgs& a = args.of(s);
+        if (a.zero)
+            for (int i = tid; i < a.zero_words; i += kThreads) static_cast<u64*>(a.zero)[i] = 0;
     }
 }
 
 // kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
 // were continued); otherwise the table is read.
-template <bool kCurves>
-__global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_constant__ SelectArgs a) {
+template <bool kCurves, class Args>
+__global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_constant__ Args args) {
     extern __shared__ double dyn[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
-    const int j0 = min((int)blockIdx.x * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
+    int block;
+    const int shard = args.mine(&block);
+    const SelectArgs& a = args.of(shard);
+    const int j0 = min(block * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
     const bool resident = a.stride > 0;
     CurveTile tile;
     tile.v = dyn;
@@ -717,7 +755,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         } else {
             a.reduction[j] = R;
             if (few) {
-                list_candidates(a, j, s, c, row);
+                list_candidates(a, shard, j, s, c, row);
             } else {
                 a.gt[j] = s;
                 a.eq[j] = c;
@@ -731,19 +769,19 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         if (tid == 0 && sum) atomicAdd((u64*)&a.counters[6], sum);
     } else {
         __syncthreads();
-        const int next = narrow_on_the_grid(a, sh, j0, j1, arrived);
+        const int next = narrow_on_the_grid(a, shard, args.of(0).sel, sh, j0, j1, arrived);
         if (next < 0) return;
         if (next == 0) {
-            if (arrive_last(a, sh)) finish_epoch(a);
+            if (arrive_last(a, sh)) finish_epoch(args);
             return;
         }
     }
 
     // ---- C: the last block to get here ranks the candidates ----
     if (!arrive_last(a, sh)) return;
-    if (sh.iv.n > 0) finish_candidates(a, sh);
-    else if (tid == 0) a.sel->prefix = ~0ull;
-    finish_epoch(a);
+    if (sh.iv.n > 0) finish_candidates(args, sh);
+    else if (tid == 0) args.of(0).sel->prefix = ~0ull;
+    finish_epoch(args);
 }
 
 }  // namespace
@@ -762,53 +800,67 @@ static size_t select_smem(bool curves, int rows, int stride) {
 int select_setup(int* blocks_per_sm) {
     int per_sm = 1;
     const size_t most = select_smem(true, kKeepLast, 1);
-    if (cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
-    if (cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true>, kThreads, most) != cudaSuccess)
-        return -1;
+    for (const void* k : {(const void*)select_kernel<true, OneHandle>, (const void*)select_kernel<false, OneHandle>,
+                          (const void*)select_kernel<true, ManyHandles>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true, ManyHandles>, kThreads, most) != cudaSuccess) return -1;
     *blocks_per_sm = per_sm < 1 ? 1 : per_sm;
     return 0;
 }
 
 // Cores per row that enter the first histogram.
-static int select_depth(int J, int cap, long long want, int sm_count) {
-    if ((long long)J * cap <= (long long)kResidentGains * sm_count) return cap;
+static int select_depth(long long J, int cap, long long want, int sm_count) {
+    if (J * cap <= (long long)kResidentGains * sm_count) return cap;
     const long long average = (want + J - 1) / J + 1;
     return (int)std::min<long long>(cap, std::max<long long>(16, (4 * average + 15) / 16 * 16));
 }
 
-// Fill the size-dependent part of the arguments and launch.
-static cudaError_t launch_select(SelectArgs& a, bool curves, int sm_count, int blocks_per_sm, cudaStream_t st) {
-    const long long gains = (long long)a.J * a.cap;
+// The part of the arguments that depends on the sizes, the same for all handles of a launch (J: their rows in all).
+struct SelectPlan {
+    int depth, W, rows, stride, keep_last;
     size_t smem;
-    int grid;
-    a.depth = select_depth(a.J, a.cap, a.want, sm_count);
+};
+static void set_rows(SelectPlan& p, int rows, int cap, bool curves) {
+    p.rows = rows;
+    p.keep_last = p.stride == 0 && p.depth < cap && rows <= kKeepLast;
+    p.smem = select_smem(curves, p.stride > 0 || p.keep_last ? rows : 0, p.stride > 0 ? p.stride : 1);
+}
+static SelectPlan plan_select(long long J, int cap, long long want, bool curves, int sm_count, int blocks_per_sm) {
+    SelectPlan p;
+    const long long gains = J * cap;
+    p.depth = select_depth(J, cap, want, sm_count);
+    p.W = 1;
+    long long grid;
     if (gains <= (long long)kResidentGains * sm_count) {
-        a.W = 1;
-        while (a.W < 32 && a.W < a.cap) a.W <<= 1;
-        grid = (int)std::min<long long>(sm_count, std::max<long long>(1, (gains + kThreads - 1) / kThreads));
-        a.rows = (a.J + grid - 1) / grid;
-        grid = (a.J + a.rows - 1) / a.rows;
-        a.keep_last = 0;
-        a.stride = a.cap | 1;   // odd: threads walking neighbouring rows meet different banks
-        smem = select_smem(curves, a.rows, a.stride);
+        while (p.W < 32 && p.W < cap) p.W <<= 1;
+        grid = std::min<long long>(sm_count, std::max<long long>(1, (gains + kThreads - 1) / kThreads));
+        p.stride = cap | 1;   // odd: threads walking neighbouring rows meet different banks
     } else {
-        a.W = 1;
-        while (a.W < 16 && a.W < a.cap) a.W <<= 1;
-        grid = sm_count * blocks_per_sm;
-        a.rows = (a.J + grid - 1) / grid;
-        grid = (a.J + a.rows - 1) / a.rows;
-        a.stride = 0;
-        a.keep_last = a.depth < a.cap && a.rows <= kKeepLast;
-        smem = select_smem(curves, a.keep_last ? a.rows : 0, 1);
+        while (p.W < 16 && p.W < cap) p.W <<= 1;
+        grid = (long long)sm_count * blocks_per_sm;
+        p.stride = 0;
     }
-    void* args[] = {&a};
-    return cudaLaunchCooperativeKernel(curves ? (const void*)select_kernel<true> : (const void*)select_kernel<false>, dim3(grid),
-                                       dim3(kThreads), args, smem, st);
+    set_rows(p, (int)((J + grid - 1) / grid), cap, curves);
+    return p;
+}
+static void apply_plan(SelectArgs& a, const SelectPlan& p) {
+    a.depth = p.depth;
+    a.W = p.W;
+    a.rows = p.rows;
+    a.stride = p.stride;
+    a.keep_last = p.keep_last;
 }
 
-int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
-                  uint32_t seq) {
+static cudaError_t launch_one(OneHandle& one, bool curves, int sm_count, int blocks_per_sm, cudaStream_t st) {
+    SelectArgs& a = one.a;
+    const SelectPlan p = plan_select(a.J, a.cap, a.want, curves, sm_count, blocks_per_sm);
+    apply_plan(a, p);
+    void* args[] = {&one};
+    return cudaLaunchCooperativeKernel(curves ? (const void*)select_kernel<true, OneHandle> : (const void*)select_kernel<false, OneHandle>,
+                                       dim3((a.J + p.rows - 1) / p.rows), dim3(kThreads), args, p.smem, st);
+}
+
+static SelectArgs handle_args(slaq_handle* h, double epoch_seconds, long long want, int first_unit, int32_t* d_out_alloc, uint32_t seq) {
     SelectArgs a;
     a.job = h->job;
     a.fit = h->fit;
@@ -835,7 +887,51 @@ int launch_select(slaq_handle* h, double epoch_seconds, long long want, int firs
     a.mail = seq ? h->mailbox : nullptr;
     a.mail_alloc = seq && h->max_jobs <= h->mailbox_jobs ? h->mail_alloc() : nullptr;
     a.seq = seq;
-    const cudaError_t e = launch_select(a, from_curves, h->sm_count, h->select_blocks_per_sm, h->stream);
+    return a;
+}
+
+int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
+                  uint32_t seq) {
+    OneHandle one{handle_args(h, epoch_seconds, want, first_unit, d_out_alloc, seq)};
+    const cudaError_t e = launch_one(one, from_curves, h->sm_count, h->select_blocks_per_sm, h->stream);
+    if (e != cudaSuccess) {
+        h->err = std::string("selection launch: ") + cudaGetErrorString(e);
+        return -1;
+    }
+    return 1;
+}
+
+int launch_select_group(slaq_handle* const* hs, int n, double epoch_seconds, long long want, int first_unit, uint32_t seq,
+                        bool* whole_table) {
+    slaq_handle* const h = hs[0];
+    ManyHandles many;
+    long long J = 0;
+    for (int s = 0; s < n; ++s) J += hs[s]->max_jobs;
+    SelectPlan p = plan_select(J, h->max_cores, want, true, h->sm_count, h->select_blocks_per_sm);
+    // a handle's last block may be partly empty: a few more rows per block until all blocks are resident at once
+    int blocks;
+    for (int rows = p.rows;; ++rows) {
+        blocks = 0;
+        for (int s = 0; s < n; ++s) blocks += (hs[s]->max_jobs + rows - 1) / rows;
+        set_rows(p, rows, h->max_cores, true);
+        if (blocks <= h->sm_count * h->select_blocks_per_sm) break;
+    }
+    *whole_table = p.depth == h->max_cores;
+    many.n = n;
+    many.first_block[0] = 0;
+    for (int s = 0; s < kMaxShards; ++s) {
+        if (s < n) {
+            SelectArgs& a = many.a[s];
+            a = handle_args(hs[s], epoch_seconds, want, first_unit, nullptr, seq);
+            a.gl = h->scratch.select;
+            a.mail = h->mailbox;
+            apply_plan(a, p);
+        }
+        many.first_block[s + 1] = many.first_block[s] + (s < n ? (hs[s]->max_jobs + p.rows - 1) / p.rows : 0);
+    }
+    void* args[] = {&many};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)select_kernel<true, ManyHandles>, dim3(blocks), dim3(kThreads), args, p.smem,
+                                                      h->stream);
     if (e != cudaSuccess) {
         h->err = std::string("selection launch: ") + cudaGetErrorString(e);
         return -1;
@@ -914,7 +1010,8 @@ extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_
     const long long usable = total_cores < (long long)J * cap ? total_cores : (long long)J * cap;
     // the array keeps the previous call's contents: clear what the kernel accumulates into
     if (cudaMemsetAsync(&dev.scratch->gl, 0, SelectGlobal::kZeroBytes, st) != cudaSuccess) return SLAQ_E_CUDA;
-    SelectArgs a = {};
+    OneHandle one = {};
+    SelectArgs& a = one.a;
     a.gain = const_cast<double*>(d_gain);   // only read: no gains are predicted here
     a.J = J;
     a.cap = cap;
@@ -927,7 +1024,7 @@ extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_
     a.eq = dev.scratch->eq;
     a.alloc = d_out_alloc;
     a.reduction = d_out_reduction;
-    if (launch_select(a, false, dev.sm_count, dev.blocks_per_sm, st) != cudaSuccess) return SLAQ_E_CUDA;
+    if (launch_one(one, false, dev.sm_count, dev.blocks_per_sm, st) != cudaSuccess) return SLAQ_E_CUDA;
     if (total_cores < J) return SLAQ_W_OVERSUBSCRIBED;
     if (total_cores > (long long)J * cap) return SLAQ_W_UNDERFILLED;
     return SLAQ_OK;

@@ -12,7 +12,7 @@ at the end one gather of each shard's number of threshold-equal gains.  Two ways
 
 from __future__ import annotations
 
-from .binding import P_FIT_CLUSTER_JOBS
+from .binding import P_FIT_CLUSTER_JOBS, schedule_group
 
 N_PASSES = 6
 N_BINS = 2048
@@ -75,7 +75,8 @@ def schedule_sharded(shards, exchange, epoch_seconds: float, total_cores: int):
 
     Every shard works on torch's current stream, on which torch orders its collectives as well: the
     exchanges between the steps are stream-ordered, and the host waits for the device only twice, for
-    the cluster's job count before anything is queued and for the allocation at the end."""
+    the cluster's job count before anything is queued and for the allocation at the end.  Shards that all live in this
+    process (``LocalExchange``) are scheduled by one call, to the same result."""
     import torch
     on_gpu = str(exchange.device).startswith("cuda")
     if on_gpu:
@@ -90,6 +91,10 @@ def schedule_sharded(shards, exchange, epoch_seconds: float, total_cores: int):
     with_floor = total_cores >= n_jobs
     for s in shards:                      # every shard fits with the lanes per job the undivided cluster would use
         s.set_param(P_FIT_CLUSTER_JOBS, n_jobs)
+    if type(exchange) is LocalExchange:   # all shards are here: nothing has to be exchanged between the steps
+        together = schedule_group(shards, epoch_seconds, total_cores)
+        if together is not None:
+            return together
     want = min(total_cores, n_jobs * cap) - (n_jobs if with_floor else 0)
     for s in shards:
         s.shard_predict(epoch_seconds, with_floor)
