@@ -10,8 +10,8 @@
 // Work split.  Jobs are sorted by window length (counting sort, longest first) and cut into
 // length classes.  In class c a group of L lanes (L = 2, 4, .. 32: the fewest lanes at which
 // the window fits the rows of a warp's shared-memory slice) owns one job (so a warp carries
-// 32/L jobs; with few active jobs L is raised so that every warp of the GPU has work).  One
-// persistent launch (one block of 16 warps per SM) serves all classes from one work queue,
+// 32/L jobs; with fewer jobs L is raised where a shorter chain of rows is worth the work, see
+// fit_least_lanes).  One persistent launch (one block of 16 warps per SM) serves all classes from one work queue,
 // longest windows first.  A lane walks its job's points m = l, l + L, l + 2L, ... counted
 // from the newest one; both families
 // are evaluated in the same sweep over the window; the partial sums of the normal equations
@@ -21,6 +21,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "slaq_internal.cuh"
 #include "slaq_fit_sweep.cuh"
@@ -659,7 +660,8 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
            const int32_t* __restrict__ start, FitClasses cls, int lm_trials, int min_fit_points,
            unsigned int* queue, long long* counters, int32_t* err_word) {
     extern __shared__ double smem[];
-    __shared__ int slot_base[kMaxFitClasses + 1];
+    __shared__ int slot_base[kMaxFitClasses + 1], dealt;
+    __shared__ unsigned long long tally[kMaxWarpsPerBlock][6];   // statistics of a warp's jobs, out of its registers
     double* wtab = smem;                                   // [h_max]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* const slice = smem + cls.h_max + (size_t)warp * cls.slice;   // this warp's: parked sums, then the window rows
@@ -671,7 +673,9 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     S.wtab_len = cls.h_max;
     S.err_word = err_word;
     for (int i = threadIdx.x; i < cls.h_max; i += blockDim.x) wtab[i] = g_wtab[i];
+    if (lane < 6) tally[warp][lane] = 0;
     if (threadIdx.x == 0) {   // queue slots of each class: one slot = one warp's worth of jobs
+        dealt = 0;
         int run = 0;
         for (int c = 0; c < cls.n; ++c) {
             slot_base[c] = run;
@@ -684,12 +688,16 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     const int fam = lane & 1;             // even lanes solve family I, odd lanes family II
     const int even = lane & ~1, oddl = lane | 1;
 
-    long long n_points = 0, n_sweep_points = 0;
-    int n_fit = 0, n_sub = 0, n_exp = 0, n_fallback = 0, n_nonconvex = 0;
     SLAQ_PHASE_DECL;
+    // The first slots are dealt out to the SMs in turn: slots are sorted by length, and the warps of a block, which draw
+    // together, would get neighbours - the longest windows all on one SM (4,000 windows of up to 200 at 16 lanes: 133 us
+    // drawn, 113 dealt).  The rest are drawn.
     for (;;) {
         int slot = 0;
-        if (lane == 0) slot = (int)atomicAdd(queue, 1u);
+        if (lane == 0) {
+            const int i = atomicAdd(&dealt, 1), warps = blockDim.x >> 5;
+            slot = i < warps ? i * (int)gridDim.x + (int)blockIdx.x : warps * (int)gridDim.x + (int)atomicAdd(queue, 1u);
+        }
         slot = __shfl_sync(kFull, slot, 0);
         SLAQ_PHASE(5);   // between jobs: statistics, record tail, queue
         if (slot >= slot_base[cls.n]) break;
@@ -779,22 +787,23 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
             SLAQ_PHASE(1);   // first guesses and the sweep at the starting points
             for (int t = 0; t < lm_trials; ++t) {
                 if (!__any_sync(kFull, !F.done)) break;
-                double trial[4] = {0.0, 0.0, 0.0, 0.0};
                 {
                     Sym4 A;
-                    double gr[4];
+                    double gr[4], trial[4] = {0.0, 0.0, 0.0, 0.0};
                     normal_equations(S, fam, mom.sw, A, gr);
                     prepare_trial(F, fam, A, gr, !F.done, mom.swy2, trial);
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
+                        pI[a] = __shfl_sync(kFull, trial[a], even);
+                        pII[a] = a < 3 ? __shfl_sync(kFull, trial[a], oddl) : 0.0;
+                    }
                 }
                 const unsigned trying = __ballot_sync(kFull, F.has_trial);
                 SLAQ_PHASE(2);   // solver step of a trial
                 if (!trying) continue;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
-                    pI[a] = __shfl_sync(kFull, trial[a], even);
-                    pII[a] = __shfl_sync(kFull, trial[a], oddl);
-                }
                 sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
+                // the lane's own trial point is one of the two it swept: not kept a second time across the sweep
+                const double trial[4] = {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]};
                 park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
                 SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
             }
@@ -847,18 +856,18 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
             p_out[1] = y_new > 0.0 ? y_new : CUDART_INF;
             p_out[2] = p_out[3] = CUDART_NAN;
         }
+        {   // the slot's share of the statistics, one entry per lane
+            const bool own = S.l == 0 && H > 0, curve = own && status == SLAQ_JOB_FITTED;
+            const unsigned points = __reduce_add_sync(kFull, own ? (unsigned)H : 0u);
+            const unsigned swept = __reduce_add_sync(kFull, own ? (unsigned)H * (unsigned)(sweeps_out[0] + sweeps_out[1]) : 0u);
+            const unsigned sub = __ballot_sync(kFull, curve && family == 0), expo = __ballot_sync(kFull, curve && family == 1);
+            const unsigned other = __ballot_sync(kFull, own && (status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW || status == SLAQ_JOB_FIT_FAILED));
+            // 1/(a x^2 + b x + c) is convex for all x >= 0 exactly when b^2 >= a c
+            const unsigned bent = __ballot_sync(kFull, curve && family == 0 && p_out[1] * p_out[1] < p_out[0] * p_out[2]);
+            if (lane < 6)
+                tally[warp][lane] += lane == 0 ? points : lane == 1 ? swept : __popc(lane == 2 ? sub : lane == 3 ? expo : lane == 4 ? other : bent);
+        }
         if (S.l == 0 && H > 0) {
-            n_points += H;
-            n_sweep_points += (long long)H * (sweeps_out[0] + sweeps_out[1]);
-            if (status == SLAQ_JOB_FITTED) {
-                n_fit += 1;
-                n_sub += family == 0;
-                n_exp += family == 1;
-                // 1/(a x^2 + b x + c) is convex for all x >= 0 exactly when b^2 >= a c
-                n_nonconvex += family == 0 && p_out[1] * p_out[1] < p_out[0] * p_out[2];
-            } else if (status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW || status == SLAQ_JOB_FIT_FAILED) {
-                n_fallback += 1;
-            }
             fit.status[j] = status;
             fit.mask[j] = (uint8_t)ended;
             if (any_ended) {   // what the next epoch may start from
@@ -879,24 +888,13 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         __syncwarp();
         SLAQ_PHASE(4);   // winner, fallback, the job's record
     }
-    // per-warp totals of the statistics
-    for (int o = 16; o > 0; o >>= 1) {
-        n_points += __shfl_xor_sync(kFull, n_points, o);
-        n_sweep_points += __shfl_xor_sync(kFull, n_sweep_points, o);
-        n_fit += __shfl_xor_sync(kFull, n_fit, o);
-        n_sub += __shfl_xor_sync(kFull, n_sub, o);
-        n_exp += __shfl_xor_sync(kFull, n_exp, o);
-        n_fallback += __shfl_xor_sync(kFull, n_fallback, o);
-        n_nonconvex += __shfl_xor_sync(kFull, n_nonconvex, o);
-    }
-    if (lane == 0 && n_points > 0) {
-        atomicAdd((unsigned long long*)&counters[0], (unsigned long long)n_points);
-        atomicAdd((unsigned long long*)&counters[1], (unsigned long long)n_sweep_points);
-        atomicAdd((unsigned long long*)&counters[2], (unsigned long long)n_fit);
-        atomicAdd((unsigned long long*)&counters[3], (unsigned long long)n_sub);
-        atomicAdd((unsigned long long*)&counters[4], (unsigned long long)n_exp);
-        atomicAdd((unsigned long long*)&counters[5], (unsigned long long)n_fallback);
-        atomicAdd((unsigned long long*)&counters[14], (unsigned long long)n_nonconvex);
+    // counters 0, 1: points, points swept; 2: fitted jobs; 3, 4: of family I, II; 5: jobs without a curve; 14: not convex ahead
+    if (lane < 6) {
+        const unsigned long long v = tally[warp][lane];
+        if (v) {
+            atomicAdd((unsigned long long*)&counters[lane < 2 ? lane : lane == 5 ? 14 : lane + 1], v);
+            if (lane == 2 || lane == 3) atomicAdd((unsigned long long*)&counters[2], v);
+        }
     }
 #ifdef SLAQ_PHASE_CLOCKS
     if (lane == 0)
@@ -1155,34 +1153,52 @@ static long long jobs_for_lanes(const slaq_handle* h) {
     return h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : (long long)h->n_active;
 }
 
-// With few active jobs every job gets more lanes, so that the warps of the GPU all have work: the fewest lanes at which
-// the jobs fill about two slots per warp.
+// Doubles of shared memory per warp: the parked sums, the window rows and one spare row.  It grows if the longest window
+// does not fit at 32 lanes.
+static int fit_slice(const slaq_handle* h) {
+    return std::max((int)(h->fit_slice_bytes / sizeof(double)), kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32);
+}
+static int rows_at(int slice, int L) { return (slice - kParked * (64 / L)) / 32 - 1; }
+
+// The fewest lanes a job gets.  Fewer lanes are less work - the solver's step and the reductions of a trial cost a warp
+// the same whatever it carries - and longer chains of rows.  Cycles per trial, fitted to clusters of 1,000 to 32,000 jobs
+// with windows of up to 12 to 1,000 points, full or ragged, at 2 to 32 lanes each: a warp alone takes 2500 + 142 per row,
+// and a sub-partition can issue 1500 + 106 per row for each of its warps; the longer of the two decides, over the lane
+// counts at which every window fits.  That choice is within 1 % of the best on average and 13 % at worst; filling
+// every warp of the GPU twice, the rule before, cost 36 % (fit of 8,000 windows of up to 100: 282 -> 118 us).  Beyond one
+// slot per warp of the GPU more lanes only add work, although the longest windows then get more lanes than
+// the others (100,000 windows of up to 1,000: 4.9 ms with 32 lanes for all, 4.0 with 2 and up).
 int fit_least_lanes(const slaq_handle* h) {
-    const long long lanes_wanted = 64LL * h->sm_count * kMaxWarpsPerBlock;
-    int L = 2;
-    while (L < 32 && jobs_for_lanes(h) * L < lanes_wanted) L <<= 1;
-    return L;
+    const int slice = fit_slice(h), Hmax = h->max_hist;
+    const double jobs = (double)std::max(1LL, jobs_for_lanes(h));
+    int best = 32;
+    double least = 0.0;
+    for (int L = 32; L >= 2 && rows_at(slice, L) * L >= Hmax; L >>= 1) {
+        const int rows = (Hmax + L - 1) / L;
+        double warps = std::ceil(jobs * L / 32.0) / (4.0 * h->sm_count);   // per sub-partition
+        if (warps < 4.0) warps = std::ceil(warps);
+        const double cycles = std::max(2500.0 + 142.0 * rows, warps * (1500.0 + 106.0 * rows));
+        if (L == 32 || cycles <= least) best = L, least = cycles;
+    }
+    while (best > 2 && jobs * (best / 2) >= 32.0 * kMaxWarpsPerBlock * h->sm_count) best >>= 1;
+    return best;
 }
 
 int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     int launches = 0;
-    // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked
-    // doubles per job and family), the window rows of 32 points and one spare row; with L lanes
-    // per job that leaves rows_at(L) rows.  The class with L = 32, 16, .. 2 lanes per job takes
-    // the windows that do not fit at L/2 lanes.  The slice grows if the longest window does not
-    // fit at 32 lanes.
+    // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked doubles per job and
+    // family), the window rows of 32 points and one spare row.  The class with L = 32, 16, .. lanes per job takes
+    // the windows that do not fit at L/2 lanes; the last one has the fewest lanes and takes the rest.
     FitClasses cls;
     cls.n = 0;
     cls.rows = 1;
     cls.h_max = Hmax;
-    cls.slice = (int)(h->fit_slice_bytes / sizeof(double));
-    cls.slice = std::max(cls.slice, kParked * 2 + ((Hmax + 31) / 32 + 1) * 32);
-    auto rows_at = [&](int L) { return (cls.slice - kParked * (64 / L)) / 32 - 1; };
+    cls.slice = fit_slice(h);
     const int L_min = fit_least_lanes(h);
     int h_hi = Hmax;
     for (int L = 32; L >= L_min && h_hi > 0; L >>= 1) {
-        const int h_lo = L > L_min ? std::max(rows_at(L / 2), 0) * (L / 2) : 0;
+        const int h_lo = L > L_min ? std::max(rows_at(cls.slice, L / 2), 0) * (L / 2) : 0;
         if (h_lo >= h_hi) continue;
         cls.h_lo[cls.n] = h_lo;
         cls.h_hi[cls.n] = h_hi;
@@ -1209,19 +1225,19 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
                                                                           h->scratch.order, h->err_word);
         launches += 3;
     }
+    // One block per SM: its registers and shared memory fill one.  Where there are fewer slots than warps every SM gets
+    // its share of them.
+    const long long slots = ((long long)J * cls.L[0] + 31) / 32;   // at most
+    const int blocks = (int)std::max(1LL, std::min((long long)max_blocks, slots));
     int warps = kMaxWarpsPerBlock;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
-    if (in_order) warps = std::min(warps, (J + max_blocks - 1) / max_blocks);   // few jobs: spread over all SMs
+    warps = (int)std::min((long long)warps, (slots + blocks - 1) / blocks);
     const size_t smem = fit_smem_bytes(cls, warps);
     if (smem > kSmemLimit) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
     const FitKernel kernel = kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
-    int blocks = max_blocks;   // one block per SM: its registers and shared memory fill one
-    const int needed = (J + warps - 1) / warps;   // at least one job per slot
-    if (blocks > needed) blocks = needed;
-    if (blocks < 1) blocks = 1;
     kernel<<<blocks, warps * 32, smem, st>>>(h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order, h->scratch.start, cls,
                                             h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase,
                                             h->scratch.counters, h->err_word);
