@@ -265,12 +265,16 @@ sweep_loop_kernel(const double* __restrict__ g_wtab, int L, int rows, int n_swee
             check += kVariant == 0 ? sums.S : sums.v[fam ? 8 : 12];
             if (it == n_sweeps - 1 && blockIdx.x == 0 && warp == 0) {
                 if (kVariant == 0) {   // a lane holds its share of the sums: written down for all lanes of its group and family
+                    // where the alternatives have family II's sums, and the signs the library keeps them with (0: not one of its sums)
+                    const int place[13] = {9, 4, 2, 1, 0, 3, 10, 11, 7, 6, 5, 12, 8};
+                    const double sign[13] = {0, -1, 1, -1, 1, 1, 0, 0, -1, 1, -1, 0, 1};
                     int from, own;
                     S.held(from, own);
                     for (int i = 0; i < 13; ++i)
                         if (i < own)
                             for (int q = fam; q < 32; q += 2)
-                                if ((S.group() >> q) & 1u) last_sums[q * 13 + from + i] = sums.v[i];
+                                if ((S.group() >> q) & 1u)
+                                    last_sums[q * 13 + (fam ? place[from + i] : from + i)] = fam ? sign[from + i] * sums.v[i] : sums.v[i];
                 } else {
                     for (int i = 0; i < 13; ++i) last_sums[lane * 13 + i] = (i < 9 || !fam) ? sums.v[i] : 0.0;
                 }
@@ -317,7 +321,7 @@ int main(int argc, char** argv) {
     std::vector<double> last_lib(5 * 32 * 13, 0.0), last(32 * 13);
     const char* const names[3] = {"the library's sweep (powers of x by running sums)", "weighted powers from tables",
                                   "powers of x multiplied in the loop"};
-    const double kInstr[3] = {43.0, 41.0, 46.0};   // fp64 arithmetic instructions per point in the loop, from the source
+    const double kInstr[3] = {42.0, 40.0, 45.0};   // fp64 arithmetic instructions per point in the loop, from the source
     for (int variant = 0; variant < 3; ++variant) {
         // the tables take 4 x kTable doubles more of the SM's shared memory: the sixteen slices shrink accordingly
         const int slice_doubles = variant != 1 ? kSliceDoubles : (kSliceDoubles * kWarps - 4 * kTable) / kWarps / 32 * 32;

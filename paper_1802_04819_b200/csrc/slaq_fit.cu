@@ -249,23 +249,28 @@ struct Sym4 {   // symmetric 4x4, upper triangle
 };
 
 // Solve B x = r for symmetric positive definite B by the root-free Cholesky factorisation
-// B = L D L^T.  False if a pivot is not positive and finite or the solution is not finite.
-__device__ bool ldl_solve(const Sym4& B, const double (&r)[4], double (&x)[4]) {
+// B = L D L^T.  False if a pivot is not positive and finite or the solution is not finite.  Unknowns whose bit is set
+// in `fixed` (of the first three) are left out and come back as 0: a pivot's reciprocal taken as 0 removes its row and
+// column.
+__device__ bool ldl_solve(const Sym4& B, const double (&r)[4], unsigned fixed, double (&x)[4]) {
+    const bool f0 = fixed & 1u, f1 = fixed & 2u, f2 = fixed & 4u;
     const double d0 = B.a00;
-    const double i0 = fast_rcp(d0);
+    const double i0 = f0 ? 0.0 : fast_rcp(d0);
     const double l10 = B.a01 * i0, l20 = B.a02 * i0, l30 = B.a03 * i0;
     const double d1 = fma(-l10, B.a01, B.a11);
-    const double i1 = fast_rcp(d1);
+    const double i1 = f1 ? 0.0 : fast_rcp(d1);
     const double t21 = fma(-l20, B.a01, B.a12), t31 = fma(-l30, B.a01, B.a13);
     const double l21 = t21 * i1, l31 = t31 * i1;
     const double d2 = fma(-l21, t21, fma(-l20, B.a02, B.a22));
-    const double i2 = fast_rcp(d2);
+    const double i2 = f2 ? 0.0 : fast_rcp(d2);
     const double t32 = fma(-l31, t21, fma(-l30, B.a02, B.a23));
     const double l32 = t32 * i2;
     const double d3 = fma(-l32, t32, fma(-l31, t31, fma(-l30, B.a03, B.a33)));
     const double i3 = fast_rcp(d3);
     // positive and finite, read off the high words (a subnormal pivot counts as zero: its reciprocal is not finite)
-    const int h0 = __double2hiint(d0), h1 = __double2hiint(d1), h2 = __double2hiint(d2), h3 = __double2hiint(d3);
+    const int fine = 0x3ff00000;
+    const int h0 = f0 ? fine : __double2hiint(d0), h1 = f1 ? fine : __double2hiint(d1), h2 = f2 ? fine : __double2hiint(d2);
+    const int h3 = __double2hiint(d3);
     bool ok = min(min(h0, h1), min(h2, h3)) > 0 && max(max(h0, h1), max(h2, h3)) < 0x7ff00000;
     const double z0 = r[0];
     const double z1 = fma(-l10, z0, r[1]);
@@ -302,45 +307,34 @@ struct Family {
 // promises.  Lower bounds: a >= 0, b >= 0, c >= 1e-12 of family I keep the curve non-increasing ahead of the newest
 // point and its denominator positive there; beta >= 0 of family II.  `busy` = this lane has a trial to prepare; the
 // re-solve loop runs while any lane of the warp needs another round (each freezes at least one more of the three
-// bounded parameters).  Family II has three parameters: its fourth row is a fixed identity row.
-__device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&g)[4], bool busy, double sum_wy2,
+// bounded parameters).  Family II has three parameters: the fourth row of its system is empty but for the diagonal.
+__device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&g)[4], bool busy, double tiny_S,
                               double (&trial)[4]) {
     F.has_trial = false;
-    if (busy && F.S <= 1e-28 * sum_wy2) {   // residual is zero to rounding
+    if (busy && F.S <= tiny_S) {   // residual is zero to rounding
         F.done = true;
         busy = false;
     }
     const bool one = fam == 0;
-    const bool at0 = one && F.p[0] <= 0.0, at1 = F.p[1] <= 0.0, at2 = one && F.p[2] <= 1e-12;   // on their bounds
-    unsigned frozen = one ? 0u : 8u;
-    if (at0 && (g[0] < 0.0 || (F.was_frozen & 1u))) frozen |= 1u;
-    if (at1 && (g[1] < 0.0 || (F.was_frozen & 2u))) frozen |= 2u;
-    if (at2 && (g[2] < 0.0 || (F.was_frozen & 4u))) frozen |= 4u;
-    // the damped diagonal
-    auto damped = [&](double d) { return fma(F.lambda, d < 1e-300 ? 1e-300 : d, d); };
-    const double D0 = damped(A.a00), D1 = damped(A.a11), D2 = damped(A.a22), D3 = damped(A.a33);
+    // on their bounds; no parameter with bound 0 is ever below it, so the high word tells (subnormals count as 0)
+    const bool at0 = one && __double2hiint(F.p[0]) <= 0, at1 = __double2hiint(F.p[1]) <= 0, at2 = one && F.p[2] <= 1e-12;
+    unsigned frozen = 0;
+    if (at0 && (__double2hiint(g[0]) < 0 || (F.was_frozen & 1u))) frozen |= 1u;
+    if (at1 && (__double2hiint(g[1]) < 0 || (F.was_frozen & 2u))) frozen |= 2u;
+    if (at2 && (__double2hiint(g[2]) < 0 || (F.was_frozen & 4u))) frozen |= 4u;
+    // the damped diagonal; 0x01a56e1f is the high word of 1e-300
+    auto damped = [&](double d) { return fma(F.lambda, __double2hiint(d) < 0x01a56e1f ? 1e-300 : d, d); };
+    Sym4 B = A;
+    B.a00 = damped(A.a00), B.a11 = damped(A.a11), B.a22 = damped(A.a22), B.a33 = damped(A.a33);
     double step[4] = {0.0, 0.0, 0.0, 0.0};
     bool solved = false, again = busy;
     while (__any_sync(kFull, again)) {
         if (again) {
-            const bool f0 = frozen & 1u, f1 = frozen & 2u, f2 = frozen & 4u, f3 = frozen & 8u;
-            Sym4 B;
-            B.a00 = f0 ? 1.0 : D0;
-            B.a11 = f1 ? 1.0 : D1;
-            B.a22 = f2 ? 1.0 : D2;
-            B.a33 = f3 ? 1.0 : D3;
-            B.a01 = (f0 || f1) ? 0.0 : A.a01;
-            B.a02 = (f0 || f2) ? 0.0 : A.a02;
-            B.a03 = (f0 || f3) ? 0.0 : A.a03;
-            B.a12 = (f1 || f2) ? 0.0 : A.a12;
-            B.a13 = (f1 || f3) ? 0.0 : A.a13;
-            B.a23 = (f2 || f3) ? 0.0 : A.a23;
-            const double rhs[4] = {f0 ? 0.0 : g[0], f1 ? 0.0 : g[1], f2 ? 0.0 : g[2], f3 ? 0.0 : g[3]};
-            solved = ldl_solve(B, rhs, step);
+            solved = ldl_solve(B, g, frozen, step);
             unsigned grow = 0;
-            if (at0 && step[0] < 0.0) grow |= 1u;
-            if (at1 && step[1] < 0.0) grow |= 2u;
-            if (at2 && step[2] < 0.0) grow |= 4u;
+            if (at0 && __double2hiint(step[0]) < 0) grow |= 1u;
+            if (at1 && __double2hiint(step[1]) < 0) grow |= 2u;
+            if (at2 && __double2hiint(step[2]) < 0) grow |= 4u;
             grow = solved ? grow & ~frozen : 0u;
             frozen |= grow;
             again = grow != 0;
@@ -356,8 +350,8 @@ __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&
     double d[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) trial[a] = F.p[a] + step[a];
-    if (one && trial[0] < 0.0) trial[0] = 0.0;
-    if (trial[1] < 0.0) trial[1] = 0.0;
+    if (one && __double2hiint(trial[0]) < 0) trial[0] = 0.0;
+    if (__double2hiint(trial[1]) < 0) trial[1] = 0.0;
     if (one && trial[2] < 1e-12) trial[2] = 1e-12;
 #pragma unroll
     for (int a = 0; a < 4; ++a) d[a] = trial[a] - F.p[a];
@@ -409,7 +403,7 @@ __device__ __forceinline__ void park(const Lanes& S, const SweepSums& s, bool ke
         } else {
             int from, own;
             S.held(from, own);
-            own = min(own, kParked - from);   // the objective of family I is not parked
+            own = min(own, kParked - from);   // the objective is not parked
             double* const at = S.park + from * n;
             const int most = S.L() == 32 ? 1 : S.L() == 16 ? 2 : S.L() == 8 ? 4 : 7;
 #pragma unroll
@@ -432,16 +426,11 @@ __device__ __forceinline__ void normal_equations(const Lanes& S, int fam, double
         g[0] = g[1] = g[2] = g[3] = 0.0;
         return;
     }
-    if (fam == 0) {
-        A.a00 = c[4 * n]; A.a01 = c[3 * n]; A.a02 = c[2 * n]; A.a11 = c[2 * n]; A.a12 = c[1 * n];
-        A.a22 = c[0];
-        A.a03 = -c[7 * n]; A.a13 = -c[6 * n]; A.a23 = -c[5 * n]; A.a33 = sw;
-        g[0] = -c[10 * n]; g[1] = -c[9 * n]; g[2] = -c[8 * n]; g[3] = c[11 * n];
-    } else {
-        A.a00 = c[0]; A.a01 = -c[1 * n]; A.a11 = c[2 * n]; A.a02 = c[3 * n]; A.a12 = -c[4 * n]; A.a22 = sw;
-        A.a03 = 0.0; A.a13 = 0.0; A.a23 = 0.0; A.a33 = 1.0;
-        g[0] = c[5 * n]; g[1] = -c[6 * n]; g[2] = c[7 * n]; g[3] = 0.0;
-    }
+    const bool one = fam == 0;
+    const double c0 = c[0], c2 = c[2 * n], c5 = c[5 * n];
+    A.a00 = c[4 * n]; A.a01 = c[3 * n]; A.a02 = one ? c2 : c5; A.a11 = c2; A.a12 = c[1 * n]; A.a22 = one ? c0 : sw;
+    A.a03 = -c[7 * n]; A.a13 = -c[6 * n]; A.a23 = one ? -c5 : 0.0; A.a33 = sw;
+    g[0] = -c[10 * n]; g[1] = -c[9 * n]; g[2] = -c[8 * n]; g[3] = c[11 * n];
 }
 
 struct Moments {
@@ -540,7 +529,7 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
         B.a03 = B.a13 = B.a23 = 0.0; B.a33 = 1.0;
         const double rhs[4] = {r0, r1, r2, 0.0};
         double sol[4] = {0.0, 0.0, 0.0, 0.0};
-        bool good = needI && ldl_solve(B, rhs, sol) && sol[0] >= 0.0 && sol[1] >= 0.0;
+        bool good = needI && ldl_solve(B, rhs, 0u, sol) && sol[0] >= 0.0 && sol[1] >= 0.0;
         int pos = 1;
         {
             const int mine = needI ? own : 0;
@@ -785,13 +774,14 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
             F.predicted = 0.0;
             park(S, sums, true);
             SLAQ_PHASE(1);   // first guesses and the sweep at the starting points
+            const double tiny_S = 1e-28 * mom.swy2;
             for (int t = 0; t < lm_trials; ++t) {
                 if (!__any_sync(kFull, !F.done)) break;
                 {
                     Sym4 A;
                     double gr[4], trial[4] = {0.0, 0.0, 0.0, 0.0};
                     normal_equations(S, fam, mom.sw, A, gr);
-                    prepare_trial(F, fam, A, gr, !F.done, mom.swy2, trial);
+                    prepare_trial(F, fam, A, gr, !F.done, tiny_S, trial);
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
                         pI[a] = __shfl_sync(kFull, trial[a], even);
@@ -801,10 +791,20 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
                 const unsigned trying = __ballot_sync(kFull, F.has_trial);
                 SLAQ_PHASE(2);   // solver step of a trial
                 if (!trying) continue;
-                sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
                 // the lane's own trial point is one of the two it swept: not kept a second time across the sweep
-                const double trial[4] = {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]};
-                park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
+#define SLAQ_OWN_TRIAL {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]}
+                if (t + 1 < lm_trials) {
+                    sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
+                    const double trial[4] = SLAQ_OWN_TRIAL;
+                    park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
+                } else {   // no step follows: the objective decides, the normal equations are not needed
+                    bool usable;
+                    double objective;
+                    sweep_objective(S, fam, H, k_all, inv_span, pI, pII, usable, objective);
+                    const double trial[4] = SLAQ_OWN_TRIAL;
+                    finish_trial(F, trial, usable, objective);
+                }
+#undef SLAQ_OWN_TRIAL
                 SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
             }
             // both results of the job, in every lane

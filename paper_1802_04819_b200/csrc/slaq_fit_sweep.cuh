@@ -15,16 +15,15 @@ constexpr int kParked = 12;                 // doubles per job and family kept i
 
 __device__ __forceinline__ bool finite_d(double v) { return fabs(v) <= 1.7976931348623157e308; }
 
-// Reciprocal to about one ulp: hardware seed and two Newton steps (no special-case paths;
+// Reciprocal to about one ulp: hardware seed (2^-20 or better) and one step of third order, x (1 + e + e^2) with
+// e = 1 - q x, which takes one instruction fewer than two Newton steps (no special-case paths;
 // a zero, subnormal or non-finite argument gives a non-finite or zero result, which the
 // callers treat as "not usable").
 __device__ __forceinline__ double fast_rcp(double q) {
     double x;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(q));
-    double e = fma(-q, x, 1.0);
-    x = fma(x, e, x);
-    e = fma(-q, x, 1.0);
-    return fma(x, e, x);
+    const double e = fma(-q, x, 1.0);
+    return fma(x, fma(e, e, e), x);
 }
 
 // Shared-memory view of one warp.  Point m of a lane's job (m = distance from the newest
@@ -48,9 +47,9 @@ struct LanesOf {
         if (L() >= 16) { const int b = (lane >> 3) & 1; from += 2 * b; n = b ? max(n - 2, 0) : min(n, 2); }
         if (L() >= 32) { const int b = (lane >> 4) & 1; from += b; n = b ? max(n - 1, 0) : min(n, 1); }
     }
-    // Where the steps of the reduction leave the objective: sum 12 of family I, sum 8 of family II.
+    // Where the steps of the reduction leave the objective, sum 12 of either family.
     __device__ __forceinline__ int objective_lane() const {
-        return (lane & -L()) + (lane & 1) + 2 + (L() >= 8 && !(lane & 1) ? 4 : 0) + (L() >= 32 ? 16 : 0);
+        return (lane & -L()) + (lane & 1) + 2 + (L() >= 8 ? 4 : 0) + (L() >= 32 ? 16 : 0);
     }
     __device__ __forceinline__ unsigned group() const {   // the lanes of this lane's job
         return (0xffffffffu >> (32 - L())) << (lane & -L());
@@ -84,8 +83,9 @@ __device__ __forceinline__ double older_neighbour(const Lanes& S, int k) {
 // What a lane keeps of one sweep: its share of the sums of ITS family over the whole window (see LanesOf::held), and the objective.
 // Family I (u = 1/q^2, J = (-u x^2, -u x, -u, 1)): v[0..4] = sum w u^2 x^k, v[5..7] = sum w u x^k,
 // v[8..10] = sum w u r x^k, v[11] = sum w r, v[12] = S.
-// Family II (J = (e, -x e, 1)): v[0..2] = sum w e^2 x^k, v[3..4] = sum w e x^k, v[5..6] = sum w e r x^k,
-// v[7] = sum w r, v[8] = S.
+// Family II (J = (e, -x e, 1)) has its entries of the normal equations where family I has the same ones, with the sign
+// family I's are read with, so that both solvers read one layout: v[4], -v[3], v[2] = sum w e^2 x^k, v[5], -v[1] = sum w e
+// x^k, -v[10], v[9] = sum w e r x^k, v[8] = -sum w r, v[12] = S, the others 0.
 struct SweepSums {
     double v[13];
     double S;      // the objective
@@ -237,28 +237,27 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     const bool odd = fam != 0;
     double v[13];
 #define SLAQ_PAIR(k, a, b) v[k] = (odd ? (b) : (a)) + __shfl_xor_sync(kFull, odd ? (a) : (b), 1)
-    SLAQ_PAIR(0, m[0], ee[0]); SLAQ_PAIR(1, m[1], ee[1]); SLAQ_PAIR(2, m[2], ee[2]); SLAQ_PAIR(3, m[3], f[0]);
-    SLAQ_PAIR(4, m[4], f[1]); SLAQ_PAIR(5, n[0], kk[0]); SLAQ_PAIR(6, n[1], kk[1]); SLAQ_PAIR(7, n[2], gc);
-    SLAQ_PAIR(8, h[0], sII);
+    SLAQ_PAIR(1, m[1], -f[1]); SLAQ_PAIR(2, m[2], ee[2]); SLAQ_PAIR(3, m[3], -ee[1]); SLAQ_PAIR(4, m[4], ee[0]);
+    SLAQ_PAIR(5, n[0], f[0]); SLAQ_PAIR(8, h[0], -gc); SLAQ_PAIR(9, h[1], kk[1]); SLAQ_PAIR(10, h[2], -kk[0]);
+    SLAQ_PAIR(12, sI, sII);
 #undef SLAQ_PAIR
     // family I only: an odd lane has no such sums
-    v[9] = h[1] + __shfl_xor_sync(kFull, h[1], 1);
-    v[10] = h[2] + __shfl_xor_sync(kFull, h[2], 1);
+    v[0] = m[0] + __shfl_xor_sync(kFull, m[0], 1);
+    v[6] = n[1] + __shfl_xor_sync(kFull, n[1], 1);
+    v[7] = n[2] + __shfl_xor_sync(kFull, n[2], 1);
     v[11] = gd + __shfl_xor_sync(kFull, gd, 1);
-    v[12] = sI + __shfl_xor_sync(kFull, sI, 1);
-    if (odd) v[9] = v[10] = v[11] = v[12] = 0.0;
+    if (odd) v[0] = v[6] = v[7] = v[11] = 0.0;
     // Remaining steps over the lanes of the same parity: in each a lane hands over one half of its sums and keeps the
     // other, 7 + 4 + 2 + 1 exchanges instead of 13 in every step, and every sum ends in one lane.
     double chk, objective;
     if (S.L() == 2) {
-        objective = odd ? v[8] : v[12];
-        chk = 0.0;
-#pragma unroll
-        for (int k = 0; k < 13; ++k) chk += v[k];
+        // these bound the others: |x| <= 1, and sum |w u r x^k| <= sqrt(sum w u^2 . sum w r^2)
+        objective = v[12];
+        chk = (v[0] + v[4]) + v[12];
     } else {
         halve<7, 13>(v, 2, S.lane);
         if (S.L() == 4) {
-            objective = odd ? v[1] : v[5];
+            objective = v[5];
             chk = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + v[6]);
         } else {
             halve<4, 7>(v, 4, S.lane);
@@ -283,6 +282,46 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     const unsigned broken = __ballot_sync(kFull, !finite_d(chk)), negative = __ballot_sync(kFull, a.q_signs < 0);
     const unsigned group = S.group();
     out.usable = !(broken & group & (odd ? 0xaaaaaaaau : 0x55555555u)) && (odd || !(negative & group));
+}
+
+// The objectives alone, for a trial after which no further step is taken: a third of the sweep's arithmetic per point, and
+// nothing to reduce but the objective.  Added up in the sweep's order, so the same to the bit.  A point at which the model
+// is not defined makes its objective non-finite or its denominator negative; the other sums are bounded by the
+// objective and the finite denominators.
+template <class Lanes>
+__device__ __forceinline__ void sweep_objective(const Lanes& S, int fam, int H, int k_all, double inv_span,
+                                                const double (&pI)[4], const double (&pII)[4], bool& usable, double& objective) {
+    const int shift = __ffs(S.L()) - 1;
+    const int k_last = H - 1 - S.l >= 0 ? (H - 1 - S.l) >> shift : -1;
+    const int mi = S.l + k_last * S.L();
+    const double md = (double)mi, dL = (double)S.L();
+    double x = -md * inv_span;
+    const double hx = dL * inv_span;
+    double e = exp(fma(pII[1], md * inv_span, pII[0]));
+    const double ratio = exp(-pII[1] * (dL * inv_span));
+    double sI = 0.0, sII = 0.0;
+    int q_signs = 0;
+    const double* yp = S.y + S.lane + k_last * 32;
+    const double* wp = S.wtab + mi;
+#pragma unroll 1
+    for (int i = 0; i < k_all; ++i, x += hx, yp -= 32, wp -= S.L()) {
+        if (i <= k_last) {
+            const double w = S.weight(wp);
+            const double y = S.holds(yp) ? *yp : 0.0;
+            const double q = fma(fma(pI[0], x, pI[1]), x, pI[2]);
+            q_signs |= __double2hiint(q);
+            const double rI = y - (fast_rcp(q) + pI[3]), rII = y - (e + pII[2]);
+            sI = fma(w * rI, rI, sI);
+            sII = fma(w * rII, rII, sII);
+            e *= ratio;
+        }
+    }
+    const bool odd = fam != 0;
+    double v = (odd ? sII : sI) + __shfl_xor_sync(kFull, odd ? sI : sII, 1);
+    for (int o = 2; o < S.L(); o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+    objective = v;
+    const unsigned negative = __ballot_sync(kFull, q_signs < 0);
+    usable = finite_d(v) && (odd || !(negative & S.group()));
 }
 
 }  // namespace slaq
