@@ -516,21 +516,32 @@ int check_device_errors(slaq_handle* h) {
 
 // Wait until the kernel that carries this call's number has reported to the mailbox.  Watching host memory sees the end of
 // a kernel a few microseconds before a stream synchronisation returns; the stream is asked now and then, for errors.
-int wait_mailbox(slaq_handle* h, const char* what) {
-    for (int spins = 0; h->mailbox->done != h->call_seq;) {
+int wait_mailbox_for(slaq_handle* h, uint32_t seq, const char* what) {
+    // the number is written by kernels of one stream in order, so a later one says that this one is over too
+    for (int spins = 0; (int32_t)(h->mailbox->done - seq) < 0;) {
         _mm_pause();
         if (++spins < 2000) continue;
         spins = 0;
         const cudaError_t e = cudaStreamQuery(h->stream);
         if (e == cudaErrorNotReady) continue;
         if (e != cudaSuccess) return cuda_fail(h, e, what);
-        if (h->mailbox->done != h->call_seq) {   // the kernel gave up: the error word says why
+        if ((int32_t)(h->mailbox->done - seq) < 0) {   // the kernel gave up: the error word says why
             if (const int rc = check_device_errors(h)) return rc;
             return fail(h, SLAQ_E_CUDA, std::string(what) + ": the kernel did not report its end");
         }
     }
     std::atomic_thread_fence(std::memory_order_acquire);
     return SLAQ_OK;
+}
+
+int wait_mailbox(slaq_handle* h, const char* what) { return wait_mailbox_for(h, h->call_seq, what); }
+
+// The mailbox's arrays are free once the append that was given its entries there has read them.  That append itself does not
+// wait: its caller's arrays were copied, and the epoch that follows is queued while it runs (8 jobs: 10 us per pass).
+int mail_arrays_free(slaq_handle* h) {
+    if (!h->mail_in_use) return SLAQ_OK;
+    h->mail_in_use = false;
+    return wait_mailbox_for(h, h->mail_seq, "append");
 }
 
 // Checks of whole arrays, in a form the compiler vectorises.
@@ -671,6 +682,7 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
         return bad;
     }
     if (mailed) {
+        if (const int rc = mail_arrays_free(h)) return rc;
         std::memcpy(h->mail_ids(), ids, sizeof(int32_t) * n);
         std::memcpy(h->mail_losses(), losses, sizeof(double) * n);
         if (d_times) std::memcpy(h->mail_times(), times, sizeof(double) * n);
@@ -683,7 +695,12 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
     append_kernel<<<blocks, threads, 0, st>>>(h->job, h->fit, h->max_jobs, n, d_ids, d_losses, d_times, d_cores, 0, h->mailbox,
                                               ++h->call_seq, h->scratch.append_ticket);
     CK(cudaGetLastError(), "append kernel");
-    if (const int rc = wait_mailbox(h, "append")) return rc;   // the caller may reuse its buffers
+    if (mailed) {
+        h->mail_in_use = true;
+        h->mail_seq = h->call_seq;
+    } else if (const int rc = wait_mailbox(h, "append")) {   // the caller may reuse its buffers
+        return rc;
+    }
     if (h->n_active < h->max_jobs) {   // nothing to do once every id is active
         for (int32_t i = 0; i < n; ++i) {
             if (!h->active[ids[i]]) {
@@ -1170,6 +1187,7 @@ int slaq_set_time_model(slaq_t* h, int32_t n, const int32_t* job_ids, const doub
     double* const d_s = mailed ? h->mail_losses() : h->stage.losses;
     double* const d_w = mailed ? h->mail_times() : h->stage.times;
     if (mailed) {
+        if (const int busy = mail_arrays_free(h)) return busy;
         std::memcpy(d_ids, job_ids, sizeof(int32_t) * n);
         std::memcpy(d_s, s, sizeof(double) * n);
         std::memcpy(d_w, w, sizeof(double) * n);

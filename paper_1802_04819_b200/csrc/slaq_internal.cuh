@@ -178,6 +178,8 @@ struct slaq_handle {
     double* mail_losses() const { return reinterpret_cast<double*>(mail_alloc() + mailbox_jobs + (mailbox_jobs & 1)); }
     double* mail_times() const { return mail_losses() + mailbox_jobs; }
     uint32_t call_seq = 0;            // number of the last call that reports to the mailbox
+    uint32_t mail_seq = 0;            // number of the append that reads its entries from the mailbox's arrays
+    bool mail_in_use = false;         // and whether it may still be reading them
     bool stats_published = true;      // the last epoch's statistics are in scratch.published (sharded steps: where they are counted)
     bool scratch_clean = false;       // the last epoch left its scratch cleared for the next one
     cudaEvent_t ev[4] = {};
