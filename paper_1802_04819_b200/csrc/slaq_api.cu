@@ -98,7 +98,8 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     int32_t* err_word = b.take<int32_t>(4);
     sc.append_ticket = reinterpret_cast<unsigned int*>(err_word ? err_word + 2 : nullptr);
     sc.load_flag = err_word ? err_word + 1 : nullptr;
-    sc.published = b.take<long long>(16);
+    sc.published = b.take<long long>(20);
+    sc.stamps = sc.published ? sc.published + 16 : nullptr;
     job.max_jobs = J;
     job.ring_lo = ring;
     job.ring_hi = ring ? ring + Js * Hmax : nullptr;
@@ -845,27 +846,19 @@ bool gains_in_selection(const slaq_handle* h, bool only_allocate) {
 }
 
 // The launches of one epoch, put on h->stream in order.  Returns the number of kernels or -1.
-// with_events: the stage boundaries are marked with the handle's events (left out of a captured
-// graph: events recorded by a graph cannot be timed).
-int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32_t* d_out, bool only_allocate,
-                  bool with_events, uint32_t seq) {
-    cudaStream_t st = h->stream;
+int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32_t* d_out, bool only_allocate, uint32_t seq) {
     int launches = 0, k;
-    if (with_events && cudaEventRecord(h->ev[0], st) != cudaSuccess) return -1;
     if (!only_allocate) {
-        if ((k = launch_fit(h, st, h->sm_count)) < 0) return -1;
+        if ((k = launch_fit(h, h->stream, h->sm_count)) < 0) return -1;
         launches += k;
     }
-    if (with_events && cudaEventRecord(h->ev[1], st) != cudaSuccess) return -1;
     const bool from_curves = gains_in_selection(h, only_allocate);
     if (!only_allocate && !from_curves) {
         if ((k = launch_gain(h, T, floor_units + 1)) < 0) return -1;
         launches += k;
     }
-    if (with_events && cudaEventRecord(h->ev[2], st) != cudaSuccess) return -1;
     if ((k = launch_select(h, T, want, floor_units + 1, from_curves, d_out, seq)) < 0) return -1;
     launches += k;
-    if (with_events && cudaEventRecord(h->ev[3], st) != cudaSuccess) return -1;
     return launches;
 }
 
@@ -922,7 +915,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
                 CK(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking), "create capture stream");
             CK(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeRelaxed), "begin capture");
             h->stream = h->capture_stream;
-            const int n = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, false, 0);
+            const int n = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, 0);
             h->stream = st;
             cudaGraph_t graph = nullptr;
             const cudaError_t e_end = cudaStreamEndCapture(h->capture_stream, &graph);
@@ -954,13 +947,16 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
         h->seen_key = key;
     }
     if (launches < 0) {
-        launches = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, true, to_mailbox ? ++h->call_seq : 0);
+        launches = enqueue_epoch(h, T, want, floor_units, d_out, only_allocate, to_mailbox ? ++h->call_seq : 0);
         if (launches < 0) {
             if (h->err.empty()) h->err = "an epoch launch failed";
             return SLAQ_E_CUDA;
         }
     }
     h->have_epoch = h->stats_published = true;
+    h->last_epoch_stamped = !h->last_epoch_was_graph;
+    h->last_gain_launch = !only_allocate && !gains_in_selection(h, only_allocate);
+    h->last_fit_launch = !only_allocate;
     h->last_launches = launches;
     h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
     h->last_cores = usable;
@@ -1050,6 +1046,8 @@ int slaq_destroy(slaq_t* h) {
     if (h->ws) cudaStreamSynchronize(h->stream);
     if (h->pipe_user) pipe_release();
     for (auto& ev : h->ev)
+        if (ev) cudaEventDestroy(ev);
+    for (auto& ev : h->order_ev)
         if (ev) cudaEventDestroy(ev);
     if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
@@ -1304,8 +1302,8 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
         if (const int rc = ensure_weights(g)) return fail(h, rc, g->err);
         if (!g->scratch_clean) CK(cudaMemsetAsync(g->scratch.zero, 0, g->scratch.zero_bytes, st), "clear scratch");
         g->scratch_clean = false;   // until the last launch is queued
-        CK(cudaEventRecord(g->ev[0], st), "event");
     }
+    if (n > 1) CK(cudaEventRecord(h->order_event(0), st), "event");
     // The fits run beside one another.  Few jobs: each gets SMs in proportion to its jobs, so that no fit waits for another's
     // last windows; many jobs: each may use the whole GPU and starts where the one before it runs out of work.
     const bool split = active * fit_least_lanes(h) <= 4LL * 32 * 16 * h->sm_count;
@@ -1322,25 +1320,22 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
         if (s > 0) {
             if (!g->side_stream) CK(cudaStreamCreateWithFlags(&g->side_stream, cudaStreamNonBlocking), "create side stream");
             side = g->side_stream;
-            CK(cudaStreamWaitEvent(side, handles[n - 1]->ev[0], 0), "fork");
+            CK(cudaStreamWaitEvent(side, h->order_event(0), 0), "fork");
         }
         const int k = launch_fit(g, side, blocks);
         if (k < 0) return fail(h, SLAQ_E_CUDA, g->err);
         g->last_launches = k;
-        CK(cudaEventRecord(g->ev[1], side), "event");
+        if (s > 0) CK(cudaEventRecord(g->order_event(1), side), "event");
     }
-    for (int32_t s = 0; s < n; ++s) {
-        if (s > 0) CK(cudaStreamWaitEvent(st, handles[s]->ev[1], 0), "join");
-        CK(cudaEventRecord(handles[s]->ev[2], st), "event");
-    }
+    for (int32_t s = 1; s < n; ++s) CK(cudaStreamWaitEvent(st, handles[s]->order_event(1), 0), "join");
     bool whole_table = false;
     const int k = launch_select_group(handles, n, epoch_seconds, want, floor_units + 1, ++h->call_seq, &whole_table);
     if (k < 0) return SLAQ_E_CUDA;
     for (int32_t s = 0; s < n; ++s) {
         slaq_t* const g = handles[s];
-        CK(cudaEventRecord(g->ev[3], st), "event");
         g->scratch_clean = true;
-        g->have_epoch = g->stats_published = true;
+        g->have_epoch = g->stats_published = g->last_epoch_stamped = g->last_fit_launch = true;
+        g->last_gain_launch = false;
         g->last_epoch_was_graph = false;
         g->last_launches += s == 0 ? k : 0;
         g->last_steps = kEpochSteps;
@@ -1385,7 +1380,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     cudaStream_t st = h->stream;
     int launches = 0, k;
     h->shard_first_unit = with_floor ? 2 : 1;
-    h->last_epoch_was_graph = false;
+    h->last_epoch_was_graph = h->last_epoch_stamped = false;
     CK(cudaMemsetAsync(h->scratch.hist, 0, sizeof(unsigned long long) * kRadixPasses * kRadixBins, st), "clear scratch");
     CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
     h->scratch_clean = h->stats_published = false;   // these steps leave their counts where they were added up
@@ -1830,18 +1825,28 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
     if (!h || !out) return SLAQ_E_ARG;
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     std::memset(out, 0, sizeof *out);
-    long long counters[16];
+    long long counters[20];
     SelectState sel;
-    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters, sizeof counters,
-                       cudaMemcpyDeviceToHost, h->stream), "copy counters");
+    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters,
+                       sizeof(long long) * (h->stats_published ? 20 : 16), cudaMemcpyDeviceToHost, h->stream), "copy counters");
     if (!h->stats_published) CK(cudaMemcpyAsync(&sel, h->scratch.sel, sizeof sel, cudaMemcpyDeviceToHost, h->stream), "copy selection state");
     CK(cudaStreamSynchronize(h->stream), "copy statistics");
     if (h->stats_published) sel.prefix = (unsigned long long)counters[15];
-    CK(cudaEventElapsedTime(&out->ms_total, h->ev[0], h->ev[3]), "event time");
-    if (!h->last_epoch_was_graph) {   // a replayed graph has no stage boundaries to time
-        CK(cudaEventElapsedTime(&out->ms_fit, h->ev[0], h->ev[1]), "event time");
-        CK(cudaEventElapsedTime(&out->ms_gain, h->ev[1], h->ev[2]), "event time");
-        CK(cudaEventElapsedTime(&out->ms_alloc, h->ev[2], h->ev[3]), "event time");
+    if (h->last_epoch_stamped) {
+        const long long* const at = counters + 16;
+        auto ms = [](long long ns) { return (float)((double)(ns > 0 ? ns : 0) * 1e-6); };
+        const long long first = h->last_fit_launch ? at[0] : at[2], gains = h->last_gain_launch ? at[1] : at[2];
+        out->ms_total = ms(at[3] - first);
+        out->ms_fit = ms(gains - first);
+        out->ms_gain = ms(at[2] - gains);
+        out->ms_alloc = ms(at[3] - at[2]);
+    } else {
+        CK(cudaEventElapsedTime(&out->ms_total, h->ev[0], h->ev[3]), "event time");
+        if (!h->last_epoch_was_graph) {   // a replayed graph has no stage boundaries to time
+            CK(cudaEventElapsedTime(&out->ms_fit, h->ev[0], h->ev[1]), "event time");
+            CK(cudaEventElapsedTime(&out->ms_gain, h->ev[1], h->ev[2]), "event time");
+            CK(cudaEventElapsedTime(&out->ms_alloc, h->ev[2], h->ev[3]), "event time");
+        }
     }
     out->launches = h->last_steps;
     out->kernel_launches = h->last_launches;

@@ -647,7 +647,7 @@ template <bool kWarm, int kL>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1)
 fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
            const int32_t* __restrict__ start, FitClasses cls, int lm_trials, int min_fit_points,
-           unsigned int* queue, long long* counters, int32_t* err_word) {
+           unsigned int* queue, long long* counters, long long* stamp, int32_t* err_word) {
     extern __shared__ double smem[];
     __shared__ int slot_base[kMaxFitClasses + 1], dealt;
     __shared__ unsigned long long tally[kMaxWarpsPerBlock][6];   // statistics of a warp's jobs, out of its registers
@@ -663,6 +663,8 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     S.err_word = err_word;
     for (int i = threadIdx.x; i < cls.h_max; i += blockDim.x) wtab[i] = g_wtab[i];
     if (lane < 6) tally[warp][lane] = 0;
+    after_previous();
+    note_time(stamp);
     if (threadIdx.x == 0) {   // queue slots of each class: one slot = one warp's worth of jobs
         dealt = 0;
         int run = 0;
@@ -966,8 +968,10 @@ __device__ __forceinline__ int clamped_length(const int32_t* __restrict__ count,
 }
 
 __global__ void __launch_bounds__(kSortThreads)
-length_count_kernel(const int32_t* __restrict__ count, int max_jobs, int max_hist, int32_t* bucket) {
+length_count_kernel(const int32_t* __restrict__ count, int max_jobs, int max_hist, int32_t* bucket, long long* stamp) {
     extern __shared__ int sh_count[];   // [max_hist + 1]
+    after_previous();
+    note_time(stamp);
     for (int i = threadIdx.x; i <= max_hist; i += blockDim.x) sh_count[i] = 0;
     __syncthreads();
     const int lo = blockIdx.x * kSortJobsPerBlock, hi = min(lo + kSortJobsPerBlock, max_jobs);
@@ -992,6 +996,7 @@ length_count_kernel(const int32_t* __restrict__ count, int max_jobs, int max_his
 __global__ void __launch_bounds__(1024) length_scan_kernel(const int32_t* __restrict__ bucket, int max_hist,
                                                            int32_t* start, int32_t* cursor) {
     __shared__ int sh[1024];
+    after_previous();
     const int t = threadIdx.x, n = max_hist + 1;
     const int per = (n + 1023) / 1024;
     // thread t owns lengths h = max_hist - (t * per + i): it walks from the longest down
@@ -1026,6 +1031,7 @@ length_scatter_kernel(const int32_t* __restrict__ count, int max_jobs, int max_h
     extern __shared__ int sh_sort[];    // [max_hist + 1] counts, then [max_hist + 1] next free position
     int* sh_count = sh_sort;
     int* sh_next = sh_sort + (max_hist + 1);
+    after_previous();
     for (int i = threadIdx.x; i <= max_hist; i += blockDim.x) sh_count[i] = 0;
     __syncthreads();
     const int lo = blockIdx.x * kSortJobsPerBlock, hi = min(lo + kSortJobsPerBlock, max_jobs);
@@ -1067,7 +1073,7 @@ length_scatter_kernel(const int32_t* __restrict__ count, int max_jobs, int max_h
 constexpr int kOneBlockSort = 16384;
 
 __global__ void __launch_bounds__(1024) length_sort_kernel(const int32_t* __restrict__ count, int max_jobs, int max_hist,
-                                                           int32_t* start, int32_t* order, int32_t* err_word) {
+                                                           int32_t* start, int32_t* order, long long* stamp, int32_t* err_word) {
     extern __shared__ int sh_one[];     // [max_hist + 1] jobs per length, then [max_hist + 1] next free position
     __shared__ int warp_sum[32];
     int* const bins = sh_one;
@@ -1075,6 +1081,8 @@ __global__ void __launch_bounds__(1024) length_sort_kernel(const int32_t* __rest
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31, n = max_hist + 1;
     for (int i = t; i < n; i += 1024) bins[i] = 0;
     __syncthreads();
+    after_previous();
+    note_time(stamp);
     int H[kOneBlockSort / 1024];
 #pragma unroll
     for (int k = 0; k < kOneBlockSort / 1024; ++k) {
@@ -1213,16 +1221,19 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     // instead of three of 3 to 4 us each), beyond that a block per 2048 jobs.
     const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * kMaxWarpsPerBlock;
     const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
+    long long* const stamp = h->scratch.stamps;
+    cudaError_t e = cudaSuccess;
     if (in_order) {
     } else if (J <= kOneBlockSort) {
-        length_sort_kernel<<<1, 1024, 2 * bins, st>>>(h->job.count, J, Hmax, h->scratch.start, h->scratch.order, h->err_word);
+        e = launch_behind(length_sort_kernel, 1, 1024, 2 * bins, st, h->job.count, J, Hmax, h->scratch.start, h->scratch.order, stamp, h->err_word);
         launches += 1;
     } else {
         const int sort_blocks = (J + kSortJobsPerBlock - 1) / kSortJobsPerBlock;
-        length_count_kernel<<<sort_blocks, kSortThreads, bins, st>>>(h->job.count, J, Hmax, h->scratch.bucket);
-        length_scan_kernel<<<1, 1024, 0, st>>>(h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
-        length_scatter_kernel<<<sort_blocks, kSortThreads, 2 * bins, st>>>(h->job.count, J, Hmax, h->scratch.cursor,
-                                                                          h->scratch.order, h->err_word);
+        e = launch_behind(length_count_kernel, sort_blocks, kSortThreads, bins, st, h->job.count, J, Hmax, h->scratch.bucket, stamp);
+        if (e == cudaSuccess) e = launch_behind(length_scan_kernel, 1, 1024, 0, st, h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
+        if (e == cudaSuccess)
+            e = launch_behind(length_scatter_kernel, sort_blocks, kSortThreads, 2 * bins, st, h->job.count, J, Hmax, h->scratch.cursor,
+                              h->scratch.order, h->err_word);
         launches += 3;
     }
     // One block per SM: its registers and shared memory fill one.  Where there are fewer slots than warps every SM gets
@@ -1232,17 +1243,18 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     int warps = kMaxWarpsPerBlock;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
     warps = (int)std::min((long long)warps, (slots + blocks - 1) / blocks);
-    const size_t smem = fit_smem_bytes(cls, warps);
+    // more than half of an SM's shared memory: no SM gets two blocks while another one still holds the kernel before
+    const size_t smem = std::max(fit_smem_bytes(cls, warps), kSmemLimit / 2 + 4096);
     if (smem > kSmemLimit) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
     const FitKernel kernel = kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
-    kernel<<<blocks, warps * 32, smem, st>>>(h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order, h->scratch.start, cls,
-                                            h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase,
-                                            h->scratch.counters, h->err_word);
+    if (e == cudaSuccess)
+        e = launch_behind(kernel, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
+                          h->scratch.start, cls, h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase, h->scratch.counters,
+                          in_order ? stamp : nullptr, h->err_word);
     ++launches;
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
         return -1;

@@ -54,8 +54,9 @@ __device__ void envelope_of_row(double* row, int cap, unsigned short* stack) {
 // running minimum; target-loss hints are read per job.
 template <bool kOptions>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-gain_kernel(JobArrays job, FitArrays fit, int max_jobs, int cap, double T, int first_unit, double* __restrict__ gain,
+gain_kernel(JobArrays job, FitArrays fit, int max_jobs, int cap, double T, int first_unit, double* __restrict__ gain, long long* stamp,
             unsigned long long* __restrict__ hist0, int options) {
+    note_time(stamp);
     __shared__ unsigned int sh_hist[kRadixBins];
     __shared__ unsigned short sh_stack[kOptions ? kWarpsPerBlock : 1][kOptions ? kMaxCoresLimit + 1 : 1];
     const bool envelope = kOptions && (options & 1) != 0;
@@ -202,7 +203,7 @@ int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit) {
     if (blocks > needed) blocks = needed;
     const auto kernel = (h->gain_envelope || h->n_hinted > 0) ? gain_kernel<true> : gain_kernel<false>;
     kernel<<<blocks, kWarpsPerBlock * 32, 0, h->stream>>>(h->job, h->fit, h->max_jobs, h->max_cores, epoch_seconds,
-                                                         first_unit, h->gain, h->scratch.hist, h->gain_envelope ? 1 : 0);
+                                                         first_unit, h->gain, h->scratch.stamps + 1, h->scratch.hist, h->gain_envelope ? 1 : 0);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->err = std::string("gain kernel launch: ") + cudaGetErrorString(e);

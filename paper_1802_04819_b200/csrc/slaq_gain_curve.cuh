@@ -18,16 +18,24 @@ __device__ __forceinline__ bool finite_d(double v) { return fabs(v) <= 1.7976931
 // Iteration-time law of job j: the fixed one if set, else ordinary least squares of the
 // sampled seconds on u = 1/cores from the running sums.  s and w are left untouched if the
 // job has neither; returns whether the law can be used (s >= 0, w > 0, finite).
+// kEager: all loads are issued before any is used, for callers that wait for every one of them.
+template <bool kEager = false>
 __device__ inline bool time_law(const JobArrays& job, int j, int max_jobs, double& s, double& w) {
     const double s_fix = job.s_set[j], w_fix = job.w_set[j];
+    double early[8];
+    if (kEager) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) early[k] = job.tm[k * (size_t)max_jobs + j];
+    }
     if (finite_d(s_fix) && finite_d(w_fix)) {
         s = s_fix;
         w = w_fix;
     } else {
         const double* tm = job.tm + j;
         const size_t J = (size_t)max_jobs;
-        const double cnt = tm[0], su = tm[J], suu = tm[2 * J], st = tm[3 * J], sut = tm[4 * J], stn = tm[5 * J];
-        const double umin = tm[6 * J], umax = tm[7 * J];
+        auto sum = [&](int k) { return kEager ? early[k] : tm[k * J]; };
+        const double cnt = sum(0), su = sum(1), suu = sum(2), st = sum(3), sut = sum(4), stn = sum(5);
+        const double umin = sum(6), umax = sum(7);
         if (!(cnt > 0.0)) return false;
         bool fitted = false;
         if (umax > umin) {
@@ -93,26 +101,37 @@ __device__ inline double raw_gain(const Curve& c, int n) {
 // The curve of job j for this epoch.  Sets kind 3 (no gain) for jobs that predict nothing; a job
 // that could predict but has no usable time law gets status SLAQ_JOB_NO_TIME, which the caller
 // records (*no_time).
+template <bool kEager = false>
 __device__ inline Curve load_curve(const JobArrays& job, const FitArrays& fit, int j, int max_jobs, double T,
                                    bool* no_time) {
     const int status = fit.status[j];
     const bool active = job.count[j] > 0;
+    double p[3];
+    int family = 0;
+    bool law = false;
     Curve c;
+    c.s = c.w = 0.0;
+    if (kEager) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) p[k] = fit.params[4 * (size_t)j + k];
+        family = fit.family[j];
+        law = time_law<true>(job, j, max_jobs, c.s, c.w);
+    }
     c.kind = 3;
     c.T = T;
     c.inv_span = 1.0 / fit.span[j];
-    c.s = c.w = c.p0 = c.p1 = c.p2 = c.step_scale = 0.0;
+    c.p0 = c.p1 = c.p2 = c.step_scale = 0.0;
     *no_time = false;
     const bool predicts = status == SLAQ_JOB_FITTED || status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW ||
                           status == SLAQ_JOB_FIT_FAILED;
     if (active && status != SLAQ_JOB_NONFINITE && status != SLAQ_JOB_FLAT) {
-        if (!time_law(job, j, max_jobs, c.s, c.w)) {
+        if (!(kEager ? law : time_law(job, j, max_jobs, c.s, c.w))) {
             *no_time = true;
         } else if (predicts) {
-            c.p0 = fit.params[4 * (size_t)j];
-            c.p1 = fit.params[4 * (size_t)j + 1];
-            c.p2 = fit.params[4 * (size_t)j + 2];
-            c.kind = status == SLAQ_JOB_FITTED ? (int)fit.family[j] : 2;
+            c.p0 = kEager ? p[0] : fit.params[4 * (size_t)j];
+            c.p1 = kEager ? p[1] : fit.params[4 * (size_t)j + 1];
+            c.p2 = kEager ? p[2] : fit.params[4 * (size_t)j + 2];
+            c.kind = status == SLAQ_JOB_FITTED ? (kEager ? family : (int)fit.family[j]) : 2;
             c.step_scale = T * c.w * c.inv_span;
         }
     }

@@ -109,6 +109,7 @@ struct Scratch {
     SelectState* sel;
     long long* counters;             // [16] statistics accumulated by kernels during an epoch
     long long* published;            // [16] those of the last finished epoch
+    long long* stamps;               // [4] device clock (ns) when its first kernel, the gain kernel and the selection started, and at its end
     unsigned int* append_ticket;     // blocks of a reporting kernel that are done
     int32_t* load_flag;              // a bulk load brought a loss that is not finite
     size_t zero_bytes;
@@ -182,7 +183,12 @@ struct slaq_handle {
     bool mail_in_use = false;         // and whether it may still be reading them
     bool stats_published = true;      // the last epoch's statistics are in scratch.published (sharded steps: where they are counted)
     bool scratch_clean = false;       // the last epoch left its scratch cleared for the next one
-    cudaEvent_t ev[4] = {};
+    cudaEvent_t ev[4] = {};               // stage boundaries of the sharded steps and of replayed graphs
+    cudaEvent_t order_ev[2] = {};         // fork and join of fits that run beside one another
+    cudaEvent_t order_event(int i) {
+        if (!order_ev[i] && cudaEventCreateWithFlags(&order_ev[i], cudaEventDisableTiming) != cudaSuccess) order_ev[i] = nullptr;
+        return order_ev[i];
+    }
     bool have_epoch = false;
     int32_t last_launches = 0;            // kernels the last call launched
     int32_t last_steps = 0;               // its steps, as slaq_stats counts them
@@ -205,10 +211,47 @@ struct slaq_handle {
     cudaStream_t side_stream = nullptr;   // the fit of a handle that is scheduled together with others
     int32_t graph_launches = 0;
     bool last_epoch_was_graph = false;
+    bool last_epoch_stamped = false;      // its stage times are in scratch.stamps, not between the events
+    bool last_gain_launch = false;        // it had a gain kernel of its own
+    bool last_fit_launch = false;         // and a fit
     std::string err;
 };
 
 namespace slaq {
+
+// ---- launches of an epoch ----
+//
+// An epoch is two to five launches in a row, and at small sizes the gaps between them count: 8 us of a pass of 70 to 170 us were
+// four timing events between the launches, so the kernels note the device clock themselves, and a kernel that follows another
+// is launched while that one still runs (its blocks wait at after_previous() before they touch what it leaves).
+__device__ __forceinline__ void note_time(long long* stamp) {
+    if (stamp && blockIdx.x == 0 && threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        *stamp = (long long)t;
+    }
+}
+// Everything the kernels before this one wrote is visible behind this line; the kernel after this one may be launched.
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <bool kCooperative = false, class... Params, class... Args>
+cudaError_t launch_behind(void (*kernel)(Params...), int blocks, int threads, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = kCooperative ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 
 // kernel launchers: each returns the number of kernels it launched, or -1 after setting h->err
 int fit_setup();   // once per device before the first fit; 0 or -1

@@ -17,6 +17,8 @@
 //      and narrow the interval by another 2048 bins at a time first; candidates that are all equal are handed out
 //      in job order with a prefix sum over the blocks.
 //
+// Tables of up to a few thousand gains take a launch of one block instead (select_small_kernel).
+//
 // What bounds it: for up to a few thousand jobs the latency of its steps.  It replaces eleven launches (gain kernel,
 // six digits of a radix select over the whole table, counts, prefix sum, allocation) that took 90 to 110 us at every
 // size up to 33,000 jobs.
@@ -285,6 +287,7 @@ struct SelectArgs {
     Mailbox* mail;
     int32_t* mail_alloc;
     uint32_t seq;
+    long long* stamps;       // [2], [3]: when the launch started and ended
 };
 
 // One handle's jobs, or those of several handles on this GPU that share one cluster's cores: each owns a run of blocks, in
@@ -537,6 +540,11 @@ __device__ void finish_epoch(const Args& args) {
         if (a.published && tid < 16)
             a.published[tid] = tid == 15 ? (long long)__ldcg(&first.sel->prefix) : __ldcg(&a.counters[tid]);
     }
+    if (tid < args.shards() && args.of(tid).stamps) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        args.of(tid).stamps[3] = (long long)t;
+    }
     if (first.mail && tid == 0) {
         int32_t err = 0;
         for (int s = 0; s < args.shards(); ++s) err |= __ldcg(args.of(s).err_word);
@@ -563,6 +571,12 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     const int shard = args.mine(&block);
     const SelectArgs& a = args.of(shard);
     const int j0 = min(block * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
+    after_previous();
+    if (block == 0 && tid == 0 && a.stamps) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        a.stamps[2] = (long long)t;
+    }
     const bool resident = a.stride > 0;
     CurveTile tile;
     tile.v = dyn;
@@ -784,6 +798,236 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     finish_epoch(args);
 }
 
+// Few gains: one block does everything in shared memory, with no grid barrier and nothing but results in global memory.
+// The launch above takes 13 us for any small table, most of it round trips to global memory: flushing and
+// reading the histogram, arriving at two counters, listing and reading candidates.  This one takes 4.8 us for 128
+// gains, 7.3 for 2,048 and 10.5 for 160 rows of 32: one SM predicts about a thousand gains per microsecond, so the two
+// meet near 6,000.
+template <bool kCurves>
+__global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_constant__ OneHandle args) {
+    extern __shared__ double dyn[];
+    __shared__ Shared sh;
+    const SelectArgs& a = args.a;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    CurveTile tile;
+    tile.v = dyn;
+    tile.kind = reinterpret_cast<int*>(dyn + 7 * kThreads);
+    double* const rows = dyn + (kCurves ? 7 * kThreads + kThreads / 2 : 0);
+
+    for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
+    if (tid == 0) sh.count = 0;
+    after_previous();
+    if (a.stamps) note_time(a.stamps + 2);
+    if (kCurves && tid < a.J) {
+        bool no_time = false;
+        const bool active = a.count[tid] > 0;
+        const Curve c = load_curve<true>(a.job, a.fit, tid, a.J, a.T, &no_time);
+        if (no_time) a.fit.status[tid] = SLAQ_JOB_NO_TIME;
+        tile.put(tid, c, active);
+    }
+    __syncthreads();
+
+    // ---- A: all gains, and their histogram ----
+    unsigned int low = 0;
+    const int W = a.W, w = tid & (W - 1), groups = kThreads / W;
+    for (int r0 = 0; r0 < a.J; r0 += groups) {   // uniform trip count: the row steps use warp shuffles
+        const int r = r0 + tid / W;
+        const bool in = r < a.J;
+        Curve c;
+        c.kind = 3;
+        bool active = false;
+        if (in) {
+            if (kCurves) {
+                c = tile.get(r, a.T);
+                active = c.kind >= 0;
+                if (!active) c.kind = 3;
+            } else {
+                active = !a.count || a.count[r] > 0;
+            }
+        }
+        double* const row = a.gain + (size_t)(in ? r : 0) * a.cap;
+        double carry = CUDART_INF;
+        for (int n0 = 0; n0 < a.cap; n0 += W) {
+            const int i = n0 + w;
+            const bool has = in && i < a.cap && index_ok((long long)r * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+            double g = 0.0;
+            if (kCurves) {
+                if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
+                g = running_min(g, carry, w, W);
+                carry = __shfl_sync(kFull, g, W - 1, W);
+                if (has) row[i] = g;
+            } else if (has) {
+                g = row[i];
+            }
+            if (has) rows[r * a.stride + i] = g;
+            count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
+        }
+    }
+    low = __reduce_add_sync(kFull, low);
+    if (lane == 0 && low) atomicAdd(&sh.hist[0], low);
+    __syncthreads();
+    // ---- the bin of the want-th largest gain: the octave by one warp each, then its bins ----
+    const unsigned int octave = __reduce_add_sync(kFull, sh.hist[warp * kSub + lane] + sh.hist[warp * kSub + 32 + lane]);
+    if (lane == 0) sh.narrow[warp] = octave;
+    __syncthreads();
+    if (warp == 0) {
+        const u64 want = (u64)a.want;
+        const u64 c = sh.narrow[31 - lane], incl = warp_inclusive(c);
+        const unsigned hit = __ballot_sync(kFull, incl >= want);
+        if (a.want <= 0) {
+            if (lane == 0) sh.iv = Interval{~0ull, ~0ull, 0, 0};   // nothing wanted: a threshold above every gain
+        } else if (!hit) {
+            if (lane == 0) sh.iv = Interval{0, 0, want, 0};
+        } else {
+            const int at = __ffs(hit) - 1;
+            const u64 above = __shfl_sync(kFull, incl - c, at);
+            const int top = (31 - at) * kSub + kSub - 1 - 2 * lane;
+            const u64 first = sh.hist[top], sum = first + sh.hist[top - 1];
+            const u64 incl2 = warp_inclusive(sum);
+            const int at2 = __ffs(__ballot_sync(kFull, above + incl2 >= want)) - 1;
+            if (lane == at2) {
+                const u64 run = above + incl2 - sum;
+                const bool second = run + first < want;
+                const int b = second ? top - 1 : top;
+                sh.iv = Interval{bin_edge(b), bin_edge(b + 1), want - run - (second ? first : 0), second ? sum - first : first};
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- B: a thread per row, rows dealt out to the warps: what lies above the interval, and the row's candidates ----
+    const int j = warp + kWarps * lane;
+    const bool in = j < a.J, active = in && (!a.count || a.count[j] > 0);
+    const double* const row = rows + (size_t)j * a.stride;
+    int s = 0, c = 0;
+    double R = 0.0;
+    {
+        const u64 lo = sh.iv.lo, hi = sh.iv.hi;
+        bool more = false;
+        if (active) {
+            if (a.first_unit == 2) R = row[0], s = 1;
+            const int end = min(a.cap, kShortWalk);
+            more = s < a.cap;
+            while (more && s < end) {
+                const double g = row[s];
+                more = key_of(g) >= hi;
+                if (more) R += g, ++s;
+            }
+            more = more && s < a.cap;   // every gain so far is handed out
+        }
+        for (unsigned todo = __ballot_sync(kFull, more); todo; todo &= todo - 1) {   // the warp continues a long row
+            const int r = __ffs(todo) - 1;
+            const double* const far = rows + (size_t)(warp + kWarps * r) * a.stride;
+            int at = __shfl_sync(kFull, s, r);
+            double sum = __shfl_sync(kFull, R, r);
+            for (bool on = true; on && at < a.cap;) {
+                const double g = at + lane < a.cap ? far[at + lane] : 0.0;
+                const unsigned stop = __ballot_sync(kFull, at + lane >= a.cap || key_of(g) < hi);
+                const int n = stop ? __ffs(stop) - 1 : 32;
+                for (int k = 0; k < n; ++k) sum += __shfl_sync(kFull, g, k);   // in order, as the row's own thread adds
+                at += n;
+                on = n == 32;
+            }
+            if (lane == r) s = at, R = sum;
+        }
+        if (active)
+            while (s + c < a.cap && key_of(row[s + c]) >= lo) ++c;
+    }
+    // ---- the interval is narrowed until its candidates can be ranked, or are all equal ----
+    for (int step = 0; sh.iv.n > kRankDirect && sh.iv.hi - sh.iv.lo > 1 && step < kRadixPasses; ++step) {
+        const int shift = narrow_shift(sh.iv);
+        const u64 lo = sh.iv.lo;
+        for (int b = tid; b < kNarrowBins; b += kThreads) sh.narrow[b] = 0;
+        __syncthreads();
+        for (int k = 0; k < c; ++k) {
+            const u64 b = (key_of(row[s + k]) - lo) >> shift;
+            if (index_ok((long long)b, kNarrowBins, kErrBin, a.err_word)) atomicAdd(&sh.narrow[b], 1u);
+        }
+        __syncthreads();
+        pick_narrow([&](int b) { return (u64)sh.narrow[b]; }, sh);
+        const u64 lo2 = sh.iv.lo, hi2 = sh.iv.hi;
+        const int end = s + c;
+        while (s < end && key_of(row[s]) >= hi2) R += row[s++];
+        c = 0;
+        while (s + c < end && key_of(row[s + c]) >= lo2) ++c;
+    }
+    __syncthreads();   // every thread has read the interval and the histogram for the last time
+    // ---- C: how many of a row's candidates are handed out ----
+    const u64 want = sh.iv.want, n = sh.iv.n;
+    int take = 0;
+    u64 tau = ~0ull;
+    if (n > kRankDirect) {   // all equal: in job order
+        if (in) sh.idx[j] = (unsigned short)c;
+        __syncthreads();
+        u64 total;
+        const u64 mine = block_exclusive(tid < a.J ? sh.idx[tid] : 0, sh, &total);
+        if (tid < a.J) sh.cand.pos[tid] = mine;
+        __syncthreads();
+        const u64 before = in ? sh.cand.pos[j] : 0;
+        take = before >= want ? 0 : (int)min((u64)c, want - before);
+        tau = sh.iv.lo;
+    } else if (n > 0) {
+        for (int i = tid; i < a.J; i += kThreads) sh.narrow[i] = 0;
+        if (c) {
+            const int at = atomicAdd(&sh.count, c);
+            for (int k = 0; k < c; ++k) {
+                sh.cand.key[at + k] = key_of(row[s + k]);
+                sh.cand.pos[at + k] = ((u64)j << 10) | (u64)(s + k);
+            }
+        }
+        __syncthreads();
+        int share = kThreads / kRankDirect;   // threads per candidate
+        while (share < 32 && 2 * share * (int)n <= kThreads) share <<= 1;
+        const int i = tid / share;
+        const bool mine = i < (int)n;
+        const u64 key = mine ? sh.cand.key[i] : 0, pos = mine ? sh.cand.pos[i] : 0;
+        unsigned int rank = 0;
+        if (mine)
+            for (int k = tid & (share - 1); k < (int)n; k += share) {
+                const u64 other = sh.cand.key[k];
+                rank += (other > key || (other == key && sh.cand.pos[k] < pos)) ? 1 : 0;
+            }
+        for (int o = share >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(kFull, rank, o);
+        if (mine && (tid & (share - 1)) == 0) {
+            if (rank < want) atomicAdd(&sh.narrow[(int)(pos >> 10)], 1u);   // the taken ones of a row are its first
+            if (rank + 1 == want) sh.scan[0] = key;
+        }
+        __syncthreads();
+        if (in) take = (int)sh.narrow[j];
+        tau = sh.scan[0];
+    }
+    int ties = 0;
+    for (int k = 0; k < take; ++k) {
+        ties += key_of(row[s + k]) == tau;
+        R += row[s + k];
+    }
+    if (in) store_alloc(a, j, active ? s + take : 0, R, active);
+    // ---- totals of the statistics, the host's mailbox, a cleared scratch for the next epoch ----
+    const unsigned int cores = __reduce_add_sync(kFull, (unsigned int)(active ? s + take : 0));
+    ties = __reduce_add_sync(kFull, ties);
+    __syncthreads();   // and all results are stored
+    if (lane == 0) sh.hist[2 * warp] = cores, sh.hist[2 * warp + 1] = ties;
+    if (a.stamps) note_time(a.stamps + 3);
+    if (tid == 0 && a.mail) {
+        a.mail->err = __ldcg(a.err_word);
+        __threadfence_system();
+        a.mail->done = a.seq;
+    }
+    __syncthreads();
+    if (warp == 1) {
+        const unsigned int all = __reduce_add_sync(kFull, sh.hist[2 * lane]), tied = __reduce_add_sync(kFull, sh.hist[2 * lane + 1]);
+        if (lane == 0) a.sel->prefix = tau;
+        if (lane < 16) {
+            const long long v = lane == 6 ? all : lane == 7 ? tied : lane == 15 ? (long long)tau : __ldcg(&a.counters[lane]);
+            if (a.published) a.published[lane] = v;
+            else if (lane == 6 || lane == 7) a.counters[lane] = v;
+        }
+    }
+    __syncthreads();
+    if (a.zero)
+        for (int i = tid; i < a.zero_words; i += kThreads) static_cast<u64*>(a.zero)[i] = 0;
+}
+
 }  // namespace
 
 // Rule for the rows' home.  Up to kResidentGains gains per block (two evaluations per thread) all of them are predicted
@@ -792,6 +1036,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
 // cores handed out, at least 16, and only rows that need more are continued.
 constexpr int kResidentGains = 2048;
 constexpr int kKeepLast = 8192;
+constexpr int kSmallGains = 6144, kSmallRows = 256;   // one block up to here (see select_small_kernel)
 
 static size_t select_smem(bool curves, int rows, int stride) {
     return sizeof(double) * ((curves ? 7 * kThreads + kThreads / 2 : 0) + (size_t)rows * stride);
@@ -799,7 +1044,9 @@ static size_t select_smem(bool curves, int rows, int stride) {
 
 int select_setup(int* blocks_per_sm) {
     int per_sm = 1;
-    const size_t most = select_smem(true, kKeepLast, 1);
+    const size_t most = select_smem(true, kKeepLast, 1), most_small = select_smem(true, kSmallGains + kSmallRows, 1);
+    for (const void* k : {(const void*)select_small_kernel<true>, (const void*)select_small_kernel<false>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_small) != cudaSuccess) return -1;
     for (const void* k : {(const void*)select_kernel<true, OneHandle>, (const void*)select_kernel<false, OneHandle>,
                           (const void*)select_kernel<true, ManyHandles>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
@@ -851,13 +1098,18 @@ static void apply_plan(SelectArgs& a, const SelectPlan& p) {
     a.keep_last = p.keep_last;
 }
 
+static bool one_block(long long J, int cap) { return J <= kSmallRows && J * cap <= kSmallGains; }
+
 static cudaError_t launch_one(OneHandle& one, bool curves, int sm_count, int blocks_per_sm, cudaStream_t st) {
     SelectArgs& a = one.a;
     const SelectPlan p = plan_select(a.J, a.cap, a.want, curves, sm_count, blocks_per_sm);
     apply_plan(a, p);
-    void* args[] = {&one};
-    return cudaLaunchCooperativeKernel(curves ? (const void*)select_kernel<true, OneHandle> : (const void*)select_kernel<false, OneHandle>,
-                                       dim3((a.J + p.rows - 1) / p.rows), dim3(kThreads), args, p.smem, st);
+    if (one_block(a.J, a.cap)) {
+        const size_t smem = select_smem(curves, a.J, p.stride);
+        return launch_behind(curves ? select_small_kernel<true> : select_small_kernel<false>, 1, kThreads, smem, st, one);
+    }
+    return launch_behind<true>(curves ? select_kernel<true, OneHandle> : select_kernel<false, OneHandle>, (a.J + p.rows - 1) / p.rows,
+                               kThreads, p.smem, st, one);
 }
 
 static SelectArgs handle_args(slaq_handle* h, double epoch_seconds, long long want, int first_unit, int32_t* d_out_alloc, uint32_t seq) {
@@ -887,6 +1139,7 @@ static SelectArgs handle_args(slaq_handle* h, double epoch_seconds, long long wa
     a.mail = seq ? h->mailbox : nullptr;
     a.mail_alloc = seq && h->max_jobs <= h->mailbox_jobs ? h->mail_alloc() : nullptr;
     a.seq = seq;
+    a.stamps = h->scratch.stamps;
     return a;
 }
 
@@ -929,9 +1182,7 @@ int launch_select_group(slaq_handle* const* hs, int n, double epoch_seconds, lon
         }
         many.first_block[s + 1] = many.first_block[s] + (s < n ? (hs[s]->max_jobs + p.rows - 1) / p.rows : 0);
     }
-    void* args[] = {&many};
-    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)select_kernel<true, ManyHandles>, dim3(blocks), dim3(kThreads), args, p.smem,
-                                                      h->stream);
+    const cudaError_t e = launch_behind<true>(select_kernel<true, ManyHandles>, blocks, kThreads, p.smem, h->stream, many);
     if (e != cudaSuccess) {
         h->err = std::string("selection launch: ") + cudaGetErrorString(e);
         return -1;
@@ -1009,7 +1260,7 @@ extern "C" int slaq_allocate_static(const double* d_gain, int32_t n_jobs, int32_
     const int floor_units = total_cores >= J ? 1 : 0;
     const long long usable = total_cores < (long long)J * cap ? total_cores : (long long)J * cap;
     // the array keeps the previous call's contents: clear what the kernel accumulates into
-    if (cudaMemsetAsync(&dev.scratch->gl, 0, SelectGlobal::kZeroBytes, st) != cudaSuccess) return SLAQ_E_CUDA;
+    if (!one_block(J, cap) && cudaMemsetAsync(&dev.scratch->gl, 0, SelectGlobal::kZeroBytes, st) != cudaSuccess) return SLAQ_E_CUDA;
     OneHandle one = {};
     SelectArgs& a = one.a;
     a.gain = const_cast<double*>(d_gain);   // only read: no gains are predicted here
