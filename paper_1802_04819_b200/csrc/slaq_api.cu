@@ -564,14 +564,20 @@ bool strictly_increasing(const int32_t* ids, int32_t n) {
 
 // Device scratch for calls that move caller data of a size unknown at creation (a bulk load into
 // rings, the normalisation export): owned by the handle, grown when a call needs more, kept for
-// the next call, released by slaq_destroy.  The stream must be idle when it grows.
+// the next call, left to the next handle by slaq_destroy (see spare_take).  The stream must be idle when it grows.
 int ensure_call_buffer(slaq_handle* h, size_t bytes, void** out) {
     if (bytes > h->call_buf_bytes) {
         CK(cudaStreamSynchronize(h->stream), "sync before growing the call buffer");
-        if (h->call_buf) cudaFree(h->call_buf);
-        h->call_buf = nullptr;
+        if (h->call_buf) spare_give(h->device, h->call_buf, h->call_buf_bytes);
+        h->call_buf = spare_take(h->device, bytes, &h->call_buf_bytes);
+        if (h->call_buf) {
+            *out = h->call_buf;
+            return SLAQ_OK;
+        }
         h->call_buf_bytes = 0;
-        const size_t want = (bytes + kAlign - 1) / kAlign * kAlign;
+        size_t step = (size_t)64 << 10;   // steps of an eighth to a quarter of the size: the next handle of such a size can use it
+        while (step * 8 <= bytes) step *= 2;
+        const size_t want = (bytes + step - 1) / step * step;
         const cudaError_t e = cudaMalloc(&h->call_buf, want);
         if (e != cudaSuccess) {
             h->call_buf = nullptr;
@@ -1044,6 +1050,7 @@ int slaq_create(int32_t max_jobs, int32_t max_hist, slaq_t** out) {
 int slaq_destroy(slaq_t* h) {
     if (!h) return SLAQ_OK;
     if (h->ws) cudaStreamSynchronize(h->stream);
+    if (h->call_buf) spare_give(h->device, h->call_buf, h->call_buf_bytes);
     if (h->pipe_user) pipe_release();
     for (auto& ev : h->ev)
         if (ev) cudaEventDestroy(ev);
@@ -1054,7 +1061,6 @@ int slaq_destroy(slaq_t* h) {
     if (h->side_stream) cudaStreamDestroy(h->side_stream);
     page_locked_free(h->mailbox_mem);
     if (h->packed_pool) cudaFree(h->packed_pool);
-    if (h->call_buf) cudaFree(h->call_buf);
     if (h->owns_ws && h->ws) cudaFree(h->ws);
     delete h;
     return SLAQ_OK;

@@ -49,6 +49,13 @@ struct Pool {
     };
     std::map<const char*, Block> blocks;
     size_t block_bytes = 0;
+    // device memory that handles left behind, for the next ones' call buffers (guarded by count_lock)
+    struct Spare {
+        int device;
+        void* memory;
+        size_t bytes;
+    };
+    std::vector<Spare> spares;
 };
 
 Pool& pool() {
@@ -202,6 +209,8 @@ void pipe_release() {
     p.memory = nullptr;
     p.earned = 0;
     p.asked.clear();
+    for (const Pool::Spare& s : p.spares) cudaFree(s.memory);
+    p.spares.clear();
     for (auto it = p.blocks.begin(); it != p.blocks.end();) {
         if (it->second.taken) {
             ++it;   // freed when it is given back
@@ -211,6 +220,37 @@ void pipe_release() {
         page_locked_free(const_cast<char*>(it->first));
         it = p.blocks.erase(it);
     }
+}
+
+// A scheduler that takes over from another one makes its call buffer in the middle of its first call, and the driver takes 0.3
+// to 20 ms for that; the one it replaces has just given its own back.  At most kSpares buffers and kSpareBytes are kept.
+constexpr size_t kSpares = 4, kSpareBytes = 128 << 20;
+
+void* spare_take(int device, size_t bytes, size_t* got) {
+    Pool& p = pool();
+    std::lock_guard<std::mutex> hold(p.count_lock);
+    for (auto it = p.spares.begin(); it != p.spares.end(); ++it) {
+        if (it->device != device || it->bytes < bytes) continue;
+        void* const memory = it->memory;
+        *got = it->bytes;
+        p.spares.erase(it);
+        return memory;
+    }
+    return nullptr;
+}
+
+void spare_give(int device, void* memory, size_t bytes) {
+    Pool& p = pool();
+    {
+        std::lock_guard<std::mutex> hold(p.count_lock);
+        size_t kept = bytes;
+        for (const Pool::Spare& s : p.spares) kept += s.bytes;
+        if (p.handles > 0 && p.spares.size() < kSpares && kept <= kSpareBytes) {
+            p.spares.push_back({device, memory, bytes});
+            return;
+        }
+    }
+    cudaFree(memory);
 }
 
 bool in_result_block(const void* q, size_t bytes) {

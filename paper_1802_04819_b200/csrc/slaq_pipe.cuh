@@ -31,6 +31,10 @@ void page_locked_free(void* m);
 // Whether [p, p + bytes) lies in a block handed out by slaq_result_take.
 bool in_result_block(const void* p, size_t bytes);
 
+// Device memory that passes from one handle of a device to the next (its last work is done): null where none is large enough.
+void* spare_take(int device, size_t bytes, size_t* got);
+void spare_give(int device, void* memory, size_t bytes);
+
 }  // namespace slaq
 
 // Page-locked memory for results the binding hands to its caller: the device writes them where they are read, and memory
