@@ -321,9 +321,15 @@ namespace {
 __device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int cores, double R, bool active) {
     a.alloc[j] = cores;
     if (a.out_alloc) a.out_alloc[j] = cores;
-    if (a.mail_alloc) a.mail_alloc[j] = cores;
     if (active && a.last_alloc) a.last_alloc[j] = cores;
     a.reduction[j] = R;
+}
+
+// The block's share of the allocation goes to the host in whole lines: written row by row as the walk ends them, 20,000
+// entries were 20,000 transfers and the fence behind them took 12 to 20 us.  Every thread's stores lie before a block barrier.
+__device__ __forceinline__ void mail_rows(const SelectArgs& a, int j0, int j1) {
+    if (a.mail_alloc)
+        for (int j = j0 + threadIdx.x; j < j1; j += kThreads) a.mail_alloc[j] = a.alloc[j];
 }
 
 // A row's candidates, entries s .. s+c-1, for the block that ranks them.  The first of them carries the row's count.
@@ -337,12 +343,55 @@ __device__ __forceinline__ void list_candidates(const SelectArgs& a, int shard, 
 
 constexpr u64 kPosMask = (1ull << 48) - 1;
 
+// Up to 32 candidates, a lane for each.
+template <class Args>
+__device__ void rank_in_a_warp(const Args& args, u64 want, int n) {
+    const int lane = threadIdx.x;
+    const SelectGlobal* const gl = args.of(0).gl;
+    const bool has = lane < n;
+    const u64 key = has ? __ldcg(&gl->cand_key[lane]) : 0, pos = has ? __ldcg(&gl->cand_pos[lane]) : 0;
+    const int shard = (int)((pos >> 41) & 31), c = (int)(pos >> 48);   // c > 0: the first candidate of its row
+    const int j = (int)((pos >> 10) & 0x7fffffff), s = (int)(pos & 1023);
+    const SelectArgs& a = args.of(has ? shard : 0);
+    double R = c > 0 ? __ldcg(&a.reduction[j]) : 0.0;
+    unsigned int rank = 0;
+    for (int k = 0; k < n; ++k) {
+        const u64 other = __shfl_sync(kFull, key, k), other_pos = __shfl_sync(kFull, pos, k) & kPosMask;
+        rank += (other > key || (other == key && other_pos < (pos & kPosMask))) ? 1 : 0;
+    }
+    const unsigned taken = __ballot_sync(kFull, has && rank < want), last = __ballot_sync(kFull, has && rank + 1 == want);
+    const u64 tau = last ? __shfl_sync(kFull, key, __ffs(last) - 1) : 0;
+    const int t = c > 0 ? __popc(taken >> lane & (c >= 32 ? kFull : (1u << c) - 1u)) : 0;   // the taken ones of a row are its first
+    const int most = (int)__reduce_max_sync(kFull, (unsigned)t);
+    for (int k = 0; k < most; ++k) {
+        const u64 next = __shfl_sync(kFull, key, (lane + k) & 31);
+        if (k < t) R += __longlong_as_double((long long)next);
+    }
+    if (c > 0) {
+        store_alloc(a, j, s + t, R, true);
+        if (a.mail_alloc) a.mail_alloc[j] = s + t;
+    }
+    if (lane == 0) args.of(0).sel->prefix = tau;
+    for (int q = 0; q < args.shards(); ++q) {
+        const unsigned cores = __reduce_add_sync(kFull, c > 0 && shard == q ? (unsigned)(s + t) : 0u);
+        const unsigned ties = __ballot_sync(kFull, (taken >> lane & 1u) && key == tau && shard == q);
+        if (lane == 0) {
+            atomicAdd((u64*)&args.of(q).counters[6], (u64)cores);
+            args.of(q).counters[7] = __popc(ties);
+        }
+    }
+}
+
 // The last block: hand out `iv.want` of the n <= kFinal candidates, best first, and complete their rows.
 template <class Args>
 __device__ void finish_candidates(const Args& args, Shared& sh) {
     const int tid = threadIdx.x;
     const SelectGlobal* const gl = args.of(0).gl;
     const int all = min((int)__ldcg(&gl->n_cand), kFinal);
+    if (all <= 32) {   // one warp, without the block's barriers
+        if (tid < 32) rank_in_a_warp(args, sh.iv.want, all);
+        return;
+    }
     if (tid < 2 * kMaxShards) sh.handed[tid >> 1][tid & 1] = 0;
     for (int i = tid; i < all; i += kThreads) {
         sh.cand.key[i] = __ldcg(&gl->cand_key[i]);
@@ -406,19 +455,31 @@ __device__ void finish_candidates(const Args& args, Shared& sh) {
     }
     __syncthreads();
     const u64 tau = sh.scan[0];
-    for (int i = tid; i < all; i += kThreads) {
-        const u64 pos = sh.cand.pos[i];
+    for (int base = 0; base < all; base += kThreads) {   // uniform trip count: the totals are added up by warps
+        const int i = base + tid;
+        const u64 pos = i < all ? sh.cand.pos[i] : 0;
         const int shard = (int)((pos >> 41) & 31);
-        if (sh.taken[i] && sh.cand.key[i] == tau) atomicAdd(&sh.handed[shard][1], 1u);
-        const int c = (int)(pos >> 48);
-        if (c == 0) continue;          // not the first candidate of its row
-        const SelectArgs& a = args.of(shard);
-        const int j = (int)((pos >> 10) & 0x7fffffff), s = (int)(pos & 1023);
-        double R = __ldcg(&a.reduction[j]);
-        int t = 0;                     // the taken ones of a row are its first
-        while (t < c && sh.taken[i + t]) R += __longlong_as_double((long long)sh.cand.key[i + t++]);
-        store_alloc(a, j, s + t, R, true);
-        atomicAdd(&sh.handed[shard][0], (unsigned int)(s + t));
+        const int c = (int)(pos >> 48);   // 0: not the first candidate of its row
+        const bool tie = i < all && sh.taken[i] && sh.cand.key[i] == tau;
+        unsigned int cores = 0;
+        if (c > 0) {
+            const SelectArgs& a = args.of(shard);
+            const int j = (int)((pos >> 10) & 0x7fffffff), s = (int)(pos & 1023);
+            double R = __ldcg(&a.reduction[j]);
+            int t = 0;                     // the taken ones of a row are its first
+            while (t < c && sh.taken[i + t]) R += __longlong_as_double((long long)sh.cand.key[i + t++]);
+            store_alloc(a, j, s + t, R, true);
+            if (a.mail_alloc) a.mail_alloc[j] = s + t;
+            cores = (unsigned int)(s + t);
+        }
+        for (int q = 0; q < args.shards(); ++q) {
+            const unsigned int sum = __reduce_add_sync(kFull, shard == q ? cores : 0u);
+            const unsigned int ties = __popc(__ballot_sync(kFull, tie && shard == q));
+            if ((tid & 31) == 0) {
+                if (sum) atomicAdd(&sh.handed[q][0], sum);
+                if (ties) atomicAdd(&sh.handed[q][1], ties);
+            }
+        }
     }
     __syncthreads();
     if (tid == 0) args.of(0).sel->prefix = tau;
@@ -516,6 +577,20 @@ __device__ int narrow_on_the_grid(const SelectArgs& a, int shard, SelectState* s
     return equal ? 0 : 1;
 }
 
+// A tile's rows into sh.idx: those of family II from the end, the others from the front.
+__device__ __forceinline__ void place_by_kind(Shared& sh, bool in, bool expo, int n_rows) {
+    const int lane = threadIdx.x & 31;
+    const unsigned front = __ballot_sync(kFull, in && !expo), back = __ballot_sync(kFull, in && expo), below = (1u << lane) - 1u;
+    int f = 0, b = 0;
+    if (lane == 0) {
+        if (front) f = atomicAdd(&sh.count, __popc(front));
+        if (back) b = atomicAdd(&sh.n_more, __popc(back));
+    }
+    f = __shfl_sync(kFull, f, 0) + __popc(front & below);
+    b = __shfl_sync(kFull, b, 0) + __popc(back & below);
+    if (in) sh.idx[expo ? n_rows - 1 - b : f] = (unsigned short)threadIdx.x;
+}
+
 // Whether this is the last block to get here; it then sees what the others wrote.
 __device__ bool arrive_last(const SelectArgs& a, Shared& sh) {
     __syncthreads();
@@ -535,22 +610,25 @@ __device__ void finish_epoch(const Args& args) {
     const int tid = threadIdx.x;
     __syncthreads();
     const SelectArgs& first = args.of(0);
-    for (int s = 0; s < args.shards(); ++s) {
-        const SelectArgs& a = args.of(s);
-        if (a.published && tid < 16)
-            a.published[tid] = tid == 15 ? (long long)__ldcg(&first.sel->prefix) : __ldcg(&a.counters[tid]);
-    }
-    if (tid < args.shards() && args.of(tid).stamps) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-        args.of(tid).stamps[3] = (long long)t;
-    }
-    if (first.mail && tid == 0) {
-        int32_t err = 0;
-        for (int s = 0; s < args.shards(); ++s) err |= __ldcg(args.of(s).err_word);
-        first.mail->err = err;
-        __threadfence_system();
-        first.mail->done = first.seq;
+    if (tid < 32) {   // the host first; the others' statistics meanwhile
+        const bool mine = tid < args.shards();
+        if (mine && args.of(tid).stamps) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            args.of(tid).stamps[3] = (long long)t;
+        }
+        if (first.mail) {
+            const unsigned err = __reduce_or_sync(kFull, mine ? (unsigned)__ldcg(args.of(tid).err_word) : 0u);
+            if (tid == 0) {
+                first.mail->err = (int32_t)err;
+                __threadfence_system();
+                first.mail->done = first.seq;
+            }
+        }
+    } else if (tid < 32 + 16 * args.shards()) {
+        const int i = tid & 15;
+        const SelectArgs& a = args.of((tid - 32) >> 4);
+        if (a.published) a.published[i] = i == 15 ? (long long)__ldcg(&first.sel->prefix) : __ldcg(&a.counters[i]);
     }
     __syncthreads();
     for (int s = 0; s < args.shards(); ++s) {
@@ -588,6 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     // the narrowing histograms, should they be needed: cleared by all blocks before the first barrier
     for (int i = blockIdx.x * kThreads + tid; i < kRadixPasses * kNarrowBins; i += gridDim.x * kThreads)
         (&a.gl->narrow[0][0])[i] = 0;
+    if (tid == 0) sh.count = sh.n_more = 0;
     __syncthreads();
 
     // ---- A: the first `depth` gains of every row ----
@@ -596,6 +675,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     for (int base = j0; base < j1; base += kThreads) {
         const int n_rows = min(kThreads, j1 - base);
         if (kCurves) {
+            bool expo = false;
             if (tid < n_rows) {
                 const int j = base + tid;
                 bool no_time = false;
@@ -603,13 +683,18 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
                 const Curve c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
                 if (no_time) a.fit.status[j] = SLAQ_JOB_NO_TIME;
                 tile.put(tid, c, active);
+                expo = active && c.kind == 1;
             }
+            // Family II's rows last: the rows of a warp are then of one family, and only one of the two formulas is
+            // walked through (a gain costs 30 to 75 instructions of the fp64 pipe in one family, the sum in both).
+            place_by_kind(sh, tid < n_rows, expo, n_rows);
             __syncthreads();
         }
         for (int r0 = 0; r0 < n_rows; r0 += groups) {   // uniform trip count: the row steps use warp shuffles
-            const int r = r0 + tid / W;
-            const bool in = r < n_rows;
-            const int j = base + (in ? r : 0);
+            const int at = r0 + tid / W;
+            const bool in = at < n_rows;
+            const int r = in ? (kCurves ? sh.idx[at] : at) : 0;
+            const int j = base + r;
             Curve c;
             bool active = false;
             if (kCurves) {
@@ -640,6 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
                 count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
             }
         }
+        if (kCurves && tid == 0) sh.count = sh.n_more = 0;
         __syncthreads();
     }
     low = __reduce_add_sync(kFull, low);
@@ -661,18 +747,20 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
         low = 0;
         for (int base = j0; base < j1; base += kThreads) {
-            if (tid == 0) sh.n_more = 0;
+            if (tid == 0) sh.count = sh.n_more = 0;
             __syncthreads();
             const int mine = base + tid;
             if (mine < j1 && (!a.count || a.count[mine] > 0) &&
-                key_of(a.keep_last ? rows_sh[mine - j0] : a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound)
-                sh.narrow[atomicAdd(&sh.n_more, 1)] = (unsigned int)mine;
+                key_of(a.keep_last ? rows_sh[mine - j0] : a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound) {
+                const bool expo = kCurves && a.fit.status[mine] == SLAQ_JOB_FITTED && a.fit.family[mine] == 1;   // those last, as above
+                sh.narrow[expo ? kThreads - 1 - atomicAdd(&sh.n_more, 1) : atomicAdd(&sh.count, 1)] = (unsigned int)mine;
+            }
             __syncthreads();
-            const int n_more = sh.n_more;
+            const int n_front = sh.count, n_more = n_front + sh.n_more;
             for (int r0 = 0; r0 < n_more; r0 += groups) {
                 const int r = r0 + tid / W;
                 const bool in = r < n_more;
-                const int j = in ? (int)sh.narrow[r] : base;
+                const int j = in ? (int)sh.narrow[r < n_front ? r : kThreads - 1 - (r - n_front)] : base;
                 double* const row = a.gain + (size_t)j * a.cap;
                 Curve c;
                 c.kind = 3;
@@ -781,10 +869,12 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         u64 sum;
         block_exclusive((u64)handed, sh, &sum);
         if (tid == 0 && sum) atomicAdd((u64*)&a.counters[6], sum);
+        mail_rows(a, j0, j1);
     } else {
         __syncthreads();
         const int next = narrow_on_the_grid(a, shard, args.of(0).sel, sh, j0, j1, arrived);
         if (next < 0) return;
+        mail_rows(a, j0, j1);   // rows with candidates that are still to be ranked are written again after that
         if (next == 0) {
             if (arrive_last(a, sh)) finish_epoch(args);
             return;
@@ -1001,11 +1091,16 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
         ties += key_of(row[s + k]) == tau;
         R += row[s + k];
     }
-    if (in) store_alloc(a, j, active ? s + take : 0, R, active);
+    if (in) {
+        store_alloc(a, j, active ? s + take : 0, R, active);
+        sh.idx[j] = (unsigned short)(active ? s + take : 0);
+    }
     // ---- totals of the statistics, the host's mailbox, a cleared scratch for the next epoch ----
     const unsigned int cores = __reduce_add_sync(kFull, (unsigned int)(active ? s + take : 0));
     ties = __reduce_add_sync(kFull, ties);
     __syncthreads();   // and all results are stored
+    if (a.mail_alloc && tid < a.J) a.mail_alloc[tid] = sh.idx[tid];   // in whole lines
+    __syncthreads();
     if (lane == 0) sh.hist[2 * warp] = cores, sh.hist[2 * warp + 1] = ties;
     if (a.stamps) note_time(a.stamps + 3);
     if (tid == 0 && a.mail) {
