@@ -32,16 +32,19 @@ namespace {
 
 // Phase clocks (only in a library built with -DSLAQ_PHASE_CLOCKS): lane 0 of every warp adds up the
 // SM cycles it spends in each phase of the fit; the totals go to counters[8..13].
+struct Phases {
 #ifdef SLAQ_PHASE_CLOCKS
-#define SLAQ_PHASE_DECL long long ph_[6] = {0, 0, 0, 0, 0, 0}, ph_t_ = clock64()
-#define SLAQ_PHASE(i)                      \
-    do {                                   \
-        const long long now_ = clock64();  \
-        ph_[i] += now_ - ph_t_;            \
-        ph_t_ = now_;                      \
+    long long sum[6] = {0, 0, 0, 0, 0, 0}, since = clock64();
+#endif
+};
+#ifdef SLAQ_PHASE_CLOCKS
+#define SLAQ_PHASE(i)                        \
+    do {                                     \
+        const long long now_ = clock64();    \
+        phases.sum[i] += now_ - phases.since; \
+        phases.since = now_;                 \
     } while (0)
 #else
-#define SLAQ_PHASE_DECL
 #define SLAQ_PHASE(i)
 #endif
 
@@ -639,10 +642,223 @@ struct FitClasses {
     int slice;       // doubles of shared memory per warp: parked sums, window rows, one spare row
 };
 
-// kWarm: families may start from last epoch's parameters (a separate instantiation, so that the
-// plain one carries none of that code).  kL: lanes per job if the launch has one length class - every cluster with
-// windows of up to about 80 points, or with few jobs - as a constant, which takes branches and index arithmetic out of
-// every step of a trial; 0 where several classes share the launch.
+// One slot of the work queue: the place-th warp's worth of jobs of class c.  kWarm: families may start from last epoch's
+// parameters (a separate instantiation, so that the plain one carries none of that code).  kL: lanes per job, a
+// constant, which takes branches and index arithmetic out of every step of a trial.
+template <bool kWarm, int kL>
+__device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& fit, const int32_t* __restrict__ order,
+                                         const int32_t* __restrict__ start, const FitClasses& cls, int c, int place, int lm_trials,
+                                         int min_fit_points, const double* wtab, double* slice, unsigned long long* tally, int lane,
+                                         Phases& phases, int32_t* err_word) {
+    const int fam = lane & 1;             // even lanes solve family I, odd lanes family II
+    const int even = lane & ~1, oddl = lane | 1;
+    constexpr int L = kL;
+    const int h_hi = cls.h_hi[c];
+    LanesOf<kL> S;
+    S.wtab = wtab;
+    S.lane = lane;
+    S.slice = slice;
+    S.slice_len = cls.slice;
+    S.wtab_len = cls.h_max;
+    S.err_word = err_word;
+    S.any_L = L;
+    S.l = lane & (L - 1);
+    const int G = 32 / L, g = lane / L;
+    S.park = slice + 2 * g + (lane & 1);
+    S.y = slice + kParked * 2 * G;
+    const int last = order ? start[cls.h_lo[c]] : job.max_jobs;
+    const int base = (order ? start[h_hi] : 0) + place * G;
+    const int idx = base + g;
+    int j = idx < last && index_ok(idx, job.max_jobs, kErrJob, err_word) ? (order ? order[idx] : idx) : -1;
+    if (j >= 0 && !index_ok(j, job.max_jobs, kErrJob, err_word)) j = -1;
+    __syncwarp();
+    const int H = stage_window(job, j, h_hi, S, err_word);
+    const int k_all = warp_max_int((H + L - 1) / L);
+    __syncwarp();
+    const double m_seen = j >= 0 ? job.m_seen[j] : -CUDART_INF;
+    const Normalised nz = normalise_window(S, H, k_all, m_seen, min_fit_points, nullptr);
+    SLAQ_PHASE(0);   // staging and normalisation
+
+    int status = nz.status, family = -1;
+    double p_out[4] = {CUDART_NAN, CUDART_NAN, CUDART_NAN, CUDART_NAN};
+    double S_out[2] = {CUDART_INF, CUDART_INF};
+    int sweeps_out[2] = {0, 0};
+    int ended = 0;   // bit 0 / 1: family I / II ended with a finite residual
+    bool any_ended = false;
+    double both_out[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // both families' end points
+    const double span = (double)max(H - 1, 1);
+    const bool fits = status == SLAQ_JOB_FITTED && H >= min_fit_points;   // this lane's job gets curves fitted
+
+    if (__any_sync(kFull, fits)) {
+        const double inv_span = 1.0 / span;
+        Moments mom = {0.0, 0.0};
+        Family F = {};
+        double pI[4] = {0.0, 0.0, 0.0, 0.0}, pII[4] = {0.0, 0.0, 0.0, 0.0};   // the points the next sweep evaluates
+        // Starting points: the first guesses, or (kWarm) last epoch's parameters where the job
+        // has some; a carried-over point without a finite residual is dropped for the
+        // family's first guess in a second round.
+        int spent = 0;
+        SweepSums sums = {};
+        if (!kWarm) {
+            first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, fits, fits, mom, pI, pII);
+            sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
+        } else {
+            unsigned wmask = fits ? fit.warm_mask[j] : 0u;
+            if (wmask) carry_over(fit, job, j, span, nz.M, wmask, pI, pII);
+            {
+                double gI[4], gII[4];
+                const bool needI = fits && !(wmask & 1u), needII = fits && !(wmask & 2u);
+                first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, needI, needII, mom, gI, gII);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    if (needI) pI[a] = gI[a];
+                    if (needII) pII[a] = gII[a];
+                }
+            }
+            sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
+            const bool redo = fits && ((wmask >> fam) & 1u) && !sums.usable;
+            if (__any_sync(kFull, redo)) {   // rare: kept out of line, with its own copies of what it changes
+                double tI[4], tII[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) tI[a] = pI[a], tII[a] = pII[a];
+                SweepSums again = sums;
+                restart_from_first_guesses(S, fam, H, k_all, inv_span, nz.ymin, nz.ymax, fits, redo, tI, tII, &again);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) pI[a] = tI[a], pII[a] = tII[a];
+                sums = again;
+                spent = redo ? 1 : 0;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) F.p[a] = fam ? pII[a] : pI[a];
+        F.ok = fits && sums.usable;
+        F.S = sums.S;
+        F.lambda = kLambda0;
+        F.nu = 2.0;
+        F.was_frozen = 0;
+        F.sweeps = fits ? 1 + spent : 0;
+        F.done = !F.ok;
+        F.has_trial = false;
+        F.predicted = 0.0;
+        park(S, sums, true);
+        SLAQ_PHASE(1);   // first guesses and the sweep at the starting points
+        const double tiny_S = 1e-28 * mom.swy2;
+        for (int t = 0; t < lm_trials; ++t) {
+            if (!__any_sync(kFull, !F.done)) break;
+            {
+                Sym4 A;
+                double gr[4], trial[4] = {0.0, 0.0, 0.0, 0.0};
+                normal_equations(S, fam, mom.sw, A, gr);
+                prepare_trial(F, fam, A, gr, !F.done, tiny_S, trial);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
+                    pI[a] = __shfl_sync(kFull, trial[a], even);
+                    pII[a] = a < 3 ? __shfl_sync(kFull, trial[a], oddl) : 0.0;
+                }
+            }
+            const unsigned trying = __ballot_sync(kFull, F.has_trial);
+            SLAQ_PHASE(2);   // solver step of a trial
+            if (!trying) continue;
+            // the lane's own trial point is one of the two it swept: not kept a second time across the sweep
+#define SLAQ_OWN_TRIAL {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]}
+            if (t + 1 < lm_trials) {
+                sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
+                const double trial[4] = SLAQ_OWN_TRIAL;
+                park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
+            } else {   // no step follows: the objective decides, the normal equations are not needed
+                bool usable;
+                double objective;
+                sweep_objective(S, fam, H, k_all, inv_span, pI, pII, usable, objective);
+                const double trial[4] = SLAQ_OWN_TRIAL;
+                finish_trial(F, trial, usable, objective);
+            }
+#undef SLAQ_OWN_TRIAL
+            SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
+        }
+        // both results of the job, in every lane
+        const double S_I = __shfl_sync(kFull, F.S, even), S_II = __shfl_sync(kFull, F.S, oddl);
+        const bool ok_I = __shfl_sync(kFull, (int)F.ok, even), ok_II = __shfl_sync(kFull, (int)F.ok, oddl);
+        sweeps_out[0] = __shfl_sync(kFull, F.sweeps, even);
+        sweeps_out[1] = __shfl_sync(kFull, F.sweeps, oddl);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            pI[a] = __shfl_sync(kFull, F.p[a], even);
+            pII[a] = __shfl_sync(kFull, F.p[a], oddl);
+        }
+        if (fits) {
+            if (ok_I) S_out[0] = S_I;
+            if (ok_II) S_out[1] = S_II;
+            const bool okI = ok_I && finite_d(S_I), okII = ok_II && finite_d(S_II);
+            ended = (okI ? 1 : 0) | (okII ? 2 : 0);
+            // Kept as a flag of its own: a branch on `ended` placed here was compiled as never taken (nvcc 12.9,
+            // also with ptxas -O1) although the same value, stored below, is non-zero; a branch on okI || okII is taken.
+            any_ended = okI || okII;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) both_out[a] = pI[a], both_out[4 + a] = pII[a];
+            if (okI && (!okII || S_I <= S_II)) {   // a tie goes to family I
+                family = 0;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) p_out[a] = pI[a];
+            } else if (okII) {
+                family = 1;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) p_out[a] = pII[a];
+            }
+        } else {
+            sweeps_out[0] = sweeps_out[1] = 0;
+        }
+    }
+    const bool fit_failed = fits && family < 0;
+    double rho = nz.rho;
+    if (__any_sync(kFull, fit_failed)) {   // rare: the whole warp walks its windows once more
+        const double from_levels = mean_change_of_levels(S, H, k_all);
+        if (fit_failed) rho = from_levels;
+    }
+    if (status == SLAQ_JOB_NEW) {
+        p_out[0] = 1.0;   // one normalised unit per iteration
+        p_out[1] = 1.0;   // at most the whole normalised loss
+    } else if (status == SLAQ_JOB_FITTED && family < 0) {
+        status = H >= min_fit_points ? SLAQ_JOB_FIT_FAILED : SLAQ_JOB_SHORT;
+        const double y_new = S.holds(S.y + lane - S.l) ? S.y[lane - S.l] : 0.0;
+        p_out[0] = rho;
+        p_out[1] = y_new > 0.0 ? y_new : CUDART_INF;
+        p_out[2] = p_out[3] = CUDART_NAN;
+    }
+    {   // the slot's share of the statistics, one entry per lane
+        const bool own = S.l == 0 && H > 0, curve = own && status == SLAQ_JOB_FITTED;
+        const unsigned points = __reduce_add_sync(kFull, own ? (unsigned)H : 0u);
+        const unsigned swept = __reduce_add_sync(kFull, own ? (unsigned)H * (unsigned)(sweeps_out[0] + sweeps_out[1]) : 0u);
+        const unsigned sub = __ballot_sync(kFull, curve && family == 0), expo = __ballot_sync(kFull, curve && family == 1);
+        const unsigned other = __ballot_sync(kFull, own && (status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW || status == SLAQ_JOB_FIT_FAILED));
+        // 1/(a x^2 + b x + c) is convex for all x >= 0 exactly when b^2 >= a c
+        const unsigned bent = __ballot_sync(kFull, curve && family == 0 && p_out[1] * p_out[1] < p_out[0] * p_out[2]);
+        if (lane < 6)
+            tally[lane] += lane == 0 ? points : lane == 1 ? swept : __popc(lane == 2 ? sub : lane == 3 ? expo : lane == 4 ? other : bent);
+    }
+    if (S.l == 0 && H > 0) {
+        fit.status[j] = status;
+        fit.mask[j] = (uint8_t)ended;
+        if (any_ended) {   // what the next epoch may start from
+            fit.k_fit[j] = job.k_last[j];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) fit.both[8 * (size_t)j + a] = both_out[a];
+        }
+        fit.family[j] = (int8_t)family;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) fit.params[4 * (size_t)j + a] = p_out[a];
+        fit.residual[2 * (size_t)j] = S_out[0];
+        fit.residual[2 * (size_t)j + 1] = S_out[1];
+        fit.sweeps[2 * (size_t)j] = sweeps_out[0];
+        fit.sweeps[2 * (size_t)j + 1] = sweeps_out[1];
+        fit.largest[j] = nz.M;
+        fit.span[j] = span;
+    }
+    __syncwarp();
+    SLAQ_PHASE(4);   // winner, fallback, the job's record
+}
+
+// kL: lanes per job if the launch has one length class - every cluster with windows of up to about 80 points, or with
+// few jobs; 0 where several classes share the launch, each then runs its own instance of fit_slot.
 template <bool kWarm, int kL>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1)
 fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
@@ -654,13 +870,6 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     double* wtab = smem;                                   // [h_max]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* const slice = smem + cls.h_max + (size_t)warp * cls.slice;   // this warp's: parked sums, then the window rows
-    LanesOf<kL> S;
-    S.wtab = wtab;
-    S.lane = lane;
-    S.slice = slice;
-    S.slice_len = cls.slice;
-    S.wtab_len = cls.h_max;
-    S.err_word = err_word;
     for (int i = threadIdx.x; i < cls.h_max; i += blockDim.x) wtab[i] = g_wtab[i];
     if (lane < 6) tally[warp][lane] = 0;
     after_previous();
@@ -676,10 +885,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         for (int c = cls.n; c <= kMaxFitClasses; ++c) slot_base[c] = run;
     }
     __syncthreads();
-    const int fam = lane & 1;             // even lanes solve family I, odd lanes family II
-    const int even = lane & ~1, oddl = lane | 1;
-
-    SLAQ_PHASE_DECL;
+    Phases phases;
     // The first slots are dealt out to the SMs in turn: slots are sorted by length, and the warps of a block, which draw
     // together, would get neighbours - the longest windows all on one SM (4,000 windows of up to 200 at 16 lanes: 133 us
     // drawn, 113 dealt).  The rest are drawn.
@@ -694,201 +900,17 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         if (slot >= slot_base[cls.n]) break;
         int c = 0;
         while (slot >= slot_base[c + 1]) ++c;
-        const int L = kL ? kL : cls.L[c], h_hi = cls.h_hi[c];
-        S.any_L = L;
-        S.l = lane & (L - 1);
-        const int G = 32 / L, g = lane / L;
-        S.park = slice + 2 * g + (lane & 1);
-        S.y = slice + kParked * 2 * G;
-        const int last = order ? start[cls.h_lo[c]] : job.max_jobs;
-        const int base = (order ? start[h_hi] : 0) + (slot - slot_base[c]) * G;
-        const int idx = base + g;
-        int j = idx < last && index_ok(idx, job.max_jobs, kErrJob, err_word) ? (order ? order[idx] : idx) : -1;
-        if (j >= 0 && !index_ok(j, job.max_jobs, kErrJob, err_word)) j = -1;
-        __syncwarp();
-        const int H = stage_window(job, j, h_hi, S, err_word);
-        const int k_all = warp_max_int((H + L - 1) / L);
-        __syncwarp();
-        const double m_seen = j >= 0 ? job.m_seen[j] : -CUDART_INF;
-        const Normalised nz = normalise_window(S, H, k_all, m_seen, min_fit_points, nullptr);
-        SLAQ_PHASE(0);   // staging and normalisation
-
-        int status = nz.status, family = -1;
-        double p_out[4] = {CUDART_NAN, CUDART_NAN, CUDART_NAN, CUDART_NAN};
-        double S_out[2] = {CUDART_INF, CUDART_INF};
-        int sweeps_out[2] = {0, 0};
-        int ended = 0;   // bit 0 / 1: family I / II ended with a finite residual
-        bool any_ended = false;
-        double both_out[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // both families' end points
-        const double span = (double)max(H - 1, 1);
-        const bool fits = status == SLAQ_JOB_FITTED && H >= min_fit_points;   // this lane's job gets curves fitted
-
-        if (__any_sync(kFull, fits)) {
-            const double inv_span = 1.0 / span;
-            Moments mom = {0.0, 0.0};
-            Family F = {};
-            double pI[4] = {0.0, 0.0, 0.0, 0.0}, pII[4] = {0.0, 0.0, 0.0, 0.0};   // the points the next sweep evaluates
-            // Starting points: the first guesses, or (kWarm) last epoch's parameters where the job
-            // has some; a carried-over point without a finite residual is dropped for the
-            // family's first guess in a second round.
-            int spent = 0;
-            SweepSums sums = {};
-            if (!kWarm) {
-                first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, fits, fits, mom, pI, pII);
-                sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
-            } else {
-                unsigned wmask = fits ? fit.warm_mask[j] : 0u;
-                if (wmask) carry_over(fit, job, j, span, nz.M, wmask, pI, pII);
-                {
-                    double gI[4], gII[4];
-                    const bool needI = fits && !(wmask & 1u), needII = fits && !(wmask & 2u);
-                    first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, needI, needII, mom, gI, gII);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) {
-                        if (needI) pI[a] = gI[a];
-                        if (needII) pII[a] = gII[a];
-                    }
-                }
-                sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
-                const bool redo = fits && ((wmask >> fam) & 1u) && !sums.usable;
-                if (__any_sync(kFull, redo)) {   // rare: kept out of line, with its own copies of what it changes
-                    double tI[4], tII[4];
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) tI[a] = pI[a], tII[a] = pII[a];
-                    SweepSums again = sums;
-                    restart_from_first_guesses(S, fam, H, k_all, inv_span, nz.ymin, nz.ymax, fits, redo, tI, tII, &again);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) pI[a] = tI[a], pII[a] = tII[a];
-                    sums = again;
-                    spent = redo ? 1 : 0;
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < 4; ++a) F.p[a] = fam ? pII[a] : pI[a];
-            F.ok = fits && sums.usable;
-            F.S = sums.S;
-            F.lambda = kLambda0;
-            F.nu = 2.0;
-            F.was_frozen = 0;
-            F.sweeps = fits ? 1 + spent : 0;
-            F.done = !F.ok;
-            F.has_trial = false;
-            F.predicted = 0.0;
-            park(S, sums, true);
-            SLAQ_PHASE(1);   // first guesses and the sweep at the starting points
-            const double tiny_S = 1e-28 * mom.swy2;
-            for (int t = 0; t < lm_trials; ++t) {
-                if (!__any_sync(kFull, !F.done)) break;
-                {
-                    Sym4 A;
-                    double gr[4], trial[4] = {0.0, 0.0, 0.0, 0.0};
-                    normal_equations(S, fam, mom.sw, A, gr);
-                    prepare_trial(F, fam, A, gr, !F.done, tiny_S, trial);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
-                        pI[a] = __shfl_sync(kFull, trial[a], even);
-                        pII[a] = a < 3 ? __shfl_sync(kFull, trial[a], oddl) : 0.0;
-                    }
-                }
-                const unsigned trying = __ballot_sync(kFull, F.has_trial);
-                SLAQ_PHASE(2);   // solver step of a trial
-                if (!trying) continue;
-                // the lane's own trial point is one of the two it swept: not kept a second time across the sweep
-#define SLAQ_OWN_TRIAL {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]}
-                if (t + 1 < lm_trials) {
-                    sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
-                    const double trial[4] = SLAQ_OWN_TRIAL;
-                    park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
-                } else {   // no step follows: the objective decides, the normal equations are not needed
-                    bool usable;
-                    double objective;
-                    sweep_objective(S, fam, H, k_all, inv_span, pI, pII, usable, objective);
-                    const double trial[4] = SLAQ_OWN_TRIAL;
-                    finish_trial(F, trial, usable, objective);
-                }
-#undef SLAQ_OWN_TRIAL
-                SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
-            }
-            // both results of the job, in every lane
-            const double S_I = __shfl_sync(kFull, F.S, even), S_II = __shfl_sync(kFull, F.S, oddl);
-            const bool ok_I = __shfl_sync(kFull, (int)F.ok, even), ok_II = __shfl_sync(kFull, (int)F.ok, oddl);
-            sweeps_out[0] = __shfl_sync(kFull, F.sweeps, even);
-            sweeps_out[1] = __shfl_sync(kFull, F.sweeps, oddl);
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                pI[a] = __shfl_sync(kFull, F.p[a], even);
-                pII[a] = __shfl_sync(kFull, F.p[a], oddl);
-            }
-            if (fits) {
-                if (ok_I) S_out[0] = S_I;
-                if (ok_II) S_out[1] = S_II;
-                const bool okI = ok_I && finite_d(S_I), okII = ok_II && finite_d(S_II);
-                ended = (okI ? 1 : 0) | (okII ? 2 : 0);
-                // Kept as a flag of its own: a branch on `ended` placed here was compiled as never taken (nvcc 12.9,
-                // also with ptxas -O1) although the same value, stored below, is non-zero; a branch on okI || okII is taken.
-                any_ended = okI || okII;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) both_out[a] = pI[a], both_out[4 + a] = pII[a];
-                if (okI && (!okII || S_I <= S_II)) {   // a tie goes to family I
-                    family = 0;
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) p_out[a] = pI[a];
-                } else if (okII) {
-                    family = 1;
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) p_out[a] = pII[a];
-                }
-            } else {
-                sweeps_out[0] = sweeps_out[1] = 0;
-            }
+        const int place = slot - slot_base[c];
+        switch (kL ? kL : cls.L[c]) {
+#define SLAQ_SLOT(n)                                                                                                            \
+    case n:                                                                                                                     \
+        if constexpr (kL == 0 || kL == n)                                                                                       \
+            fit_slot<kWarm, n>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, slice, tally[warp], lane, \
+                               phases, err_word);                                                                               \
+        break;
+            SLAQ_SLOT(2) SLAQ_SLOT(4) SLAQ_SLOT(8) SLAQ_SLOT(16) SLAQ_SLOT(32)
+#undef SLAQ_SLOT
         }
-        const bool fit_failed = fits && family < 0;
-        double rho = nz.rho;
-        if (__any_sync(kFull, fit_failed)) {   // rare: the whole warp walks its windows once more
-            const double from_levels = mean_change_of_levels(S, H, k_all);
-            if (fit_failed) rho = from_levels;
-        }
-        if (status == SLAQ_JOB_NEW) {
-            p_out[0] = 1.0;   // one normalised unit per iteration
-            p_out[1] = 1.0;   // at most the whole normalised loss
-        } else if (status == SLAQ_JOB_FITTED && family < 0) {
-            status = H >= min_fit_points ? SLAQ_JOB_FIT_FAILED : SLAQ_JOB_SHORT;
-            const double y_new = S.holds(S.y + lane - S.l) ? S.y[lane - S.l] : 0.0;
-            p_out[0] = rho;
-            p_out[1] = y_new > 0.0 ? y_new : CUDART_INF;
-            p_out[2] = p_out[3] = CUDART_NAN;
-        }
-        {   // the slot's share of the statistics, one entry per lane
-            const bool own = S.l == 0 && H > 0, curve = own && status == SLAQ_JOB_FITTED;
-            const unsigned points = __reduce_add_sync(kFull, own ? (unsigned)H : 0u);
-            const unsigned swept = __reduce_add_sync(kFull, own ? (unsigned)H * (unsigned)(sweeps_out[0] + sweeps_out[1]) : 0u);
-            const unsigned sub = __ballot_sync(kFull, curve && family == 0), expo = __ballot_sync(kFull, curve && family == 1);
-            const unsigned other = __ballot_sync(kFull, own && (status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW || status == SLAQ_JOB_FIT_FAILED));
-            // 1/(a x^2 + b x + c) is convex for all x >= 0 exactly when b^2 >= a c
-            const unsigned bent = __ballot_sync(kFull, curve && family == 0 && p_out[1] * p_out[1] < p_out[0] * p_out[2]);
-            if (lane < 6)
-                tally[warp][lane] += lane == 0 ? points : lane == 1 ? swept : __popc(lane == 2 ? sub : lane == 3 ? expo : lane == 4 ? other : bent);
-        }
-        if (S.l == 0 && H > 0) {
-            fit.status[j] = status;
-            fit.mask[j] = (uint8_t)ended;
-            if (any_ended) {   // what the next epoch may start from
-                fit.k_fit[j] = job.k_last[j];
-#pragma unroll
-                for (int a = 0; a < 8; ++a) fit.both[8 * (size_t)j + a] = both_out[a];
-            }
-            fit.family[j] = (int8_t)family;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) fit.params[4 * (size_t)j + a] = p_out[a];
-            fit.residual[2 * (size_t)j] = S_out[0];
-            fit.residual[2 * (size_t)j + 1] = S_out[1];
-            fit.sweeps[2 * (size_t)j] = sweeps_out[0];
-            fit.sweeps[2 * (size_t)j + 1] = sweeps_out[1];
-            fit.largest[j] = nz.M;
-            fit.span[j] = span;
-        }
-        __syncwarp();
-        SLAQ_PHASE(4);   // winner, fallback, the job's record
     }
     // counters 0, 1: points, points swept; 2: fitted jobs; 3, 4: of family I, II; 5: jobs without a curve; 14: not convex ahead
     if (lane < 6) {
@@ -900,7 +922,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
     }
 #ifdef SLAQ_PHASE_CLOCKS
     if (lane == 0)
-        for (int i = 0; i < 6; ++i) atomicAdd((unsigned long long*)&counters[8 + i], (unsigned long long)ph_[i]);
+        for (int i = 0; i < 6; ++i) atomicAdd((unsigned long long*)&counters[8 + i], (unsigned long long)phases.sum[i]);
 #endif
 }
 
