@@ -860,7 +860,7 @@ int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32
     }
     const bool from_curves = gains_in_selection(h, only_allocate);
     if (!only_allocate && !from_curves) {
-        if ((k = launch_gain(h, T, floor_units + 1)) < 0) return -1;
+        if ((k = launch_gain(h, T, floor_units + 1, false)) < 0) return -1;
         launches += k;
     }
     if ((k = launch_select(h, T, want, floor_units + 1, from_curves, d_out, seq)) < 0) return -1;
@@ -1394,7 +1394,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     if ((k = launch_fit(h, st, h->sm_count)) < 0) return SLAQ_E_CUDA;
     launches += k;
     CK(cudaEventRecord(h->ev[1], st), "event");
-    if ((k = launch_gain(h, epoch_seconds, h->shard_first_unit)) < 0) return SLAQ_E_CUDA;
+    if ((k = launch_gain(h, epoch_seconds, h->shard_first_unit, true)) < 0) return SLAQ_E_CUDA;
     launches += k;
     CK(cudaEventRecord(h->ev[2], st), "event");
     CK(cudaEventRecord(h->ev[3], st), "event");
@@ -1490,7 +1490,7 @@ int slaq_get_predictions(slaq_t* h, double* out_reduction, double* out_gain, int
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     const size_t J = (size_t)h->max_jobs;
     if (out_gain && !h->gain_table_current) {   // the last epoch predicted rows only as far as it needed: write them now
-        if (launch_gain(h, h->last_T, h->last_first_unit) < 0) return SLAQ_E_CUDA;
+        if (launch_gain(h, h->last_T, h->last_first_unit, false) < 0) return SLAQ_E_CUDA;
         h->gain_table_current = true;
     }
     return results_to_host(h, {{out_gain, h->gain, 8 * J * h->max_cores},

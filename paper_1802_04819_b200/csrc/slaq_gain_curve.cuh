@@ -18,12 +18,12 @@ __device__ __forceinline__ bool finite_d(double v) { return fabs(v) <= 1.7976931
 // Iteration-time law of job j: the fixed one if set, else ordinary least squares of the
 // sampled seconds on u = 1/cores from the running sums.  s and w are left untouched if the
 // job has neither; returns whether the law can be used (s >= 0, w > 0, finite).
-// kEager: all loads are issued before any is used, for callers that wait for every one of them.
-template <bool kEager = false>
+// kSums: the sums of the samples are loaded with the rest, 64 bytes per job which only few jobs' callers can spare.
+template <bool kSums = false>
 __device__ inline bool time_law(const JobArrays& job, int j, int max_jobs, double& s, double& w) {
     const double s_fix = job.s_set[j], w_fix = job.w_set[j];
     double early[8];
-    if (kEager) {
+    if (kSums) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) early[k] = job.tm[k * (size_t)max_jobs + j];
     }
@@ -33,7 +33,7 @@ __device__ inline bool time_law(const JobArrays& job, int j, int max_jobs, doubl
     } else {
         const double* tm = job.tm + j;
         const size_t J = (size_t)max_jobs;
-        auto sum = [&](int k) { return kEager ? early[k] : tm[k * J]; };
+        auto sum = [&](int k) { return kSums ? early[k] : tm[k * J]; };
         const double cnt = sum(0), su = sum(1), suu = sum(2), st = sum(3), sut = sum(4), stn = sum(5);
         const double umin = sum(6), umax = sum(7);
         if (!(cnt > 0.0)) return false;
@@ -101,7 +101,8 @@ __device__ inline double raw_gain(const Curve& c, int n) {
 // The curve of job j for this epoch.  Sets kind 3 (no gain) for jobs that predict nothing; a job
 // that could predict but has no usable time law gets status SLAQ_JOB_NO_TIME, which the caller
 // records (*no_time).
-template <bool kEager = false>
+// kEager: all loads are issued before any is used, for callers that wait for every one of them.
+template <bool kEager = false, bool kSums = false>
 __device__ inline Curve load_curve(const JobArrays& job, const FitArrays& fit, int j, int max_jobs, double T,
                                    bool* no_time) {
     const int status = fit.status[j];
@@ -115,7 +116,7 @@ __device__ inline Curve load_curve(const JobArrays& job, const FitArrays& fit, i
 #pragma unroll
         for (int k = 0; k < 3; ++k) p[k] = fit.params[4 * (size_t)j + k];
         family = fit.family[j];
-        law = time_law<true>(job, j, max_jobs, c.s, c.w);
+        law = time_law<kSums>(job, j, max_jobs, c.s, c.w);
     }
     c.kind = 3;
     c.T = T;

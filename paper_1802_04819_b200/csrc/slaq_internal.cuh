@@ -258,7 +258,8 @@ int fit_setup();   // once per device before the first fit; 0 or -1
 // on `st`, with at most max_blocks blocks
 int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks);
 int fit_least_lanes(const slaq_handle* h);
-int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit);
+// histogram: the keys go into scratch.hist's first pass as well
+int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit, bool histogram);
 // seq != 0: the kernel reports to the handle's mailbox under that number, and writes the allocation there too if it fits
 int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
                   uint32_t seq);

@@ -911,7 +911,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
     if (kCurves && tid < a.J) {
         bool no_time = false;
         const bool active = a.count[tid] > 0;
-        const Curve c = load_curve<true>(a.job, a.fit, tid, a.J, a.T, &no_time);
+        const Curve c = load_curve<true, true>(a.job, a.fit, tid, a.J, a.T, &no_time);
         if (no_time) a.fit.status[tid] = SLAQ_JOB_NO_TIME;
         tile.put(tid, c, active);
     }
