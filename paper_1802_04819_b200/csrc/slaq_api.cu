@@ -279,12 +279,25 @@ __device__ __forceinline__ void append_one(const JobArrays& job, const FitArrays
     }
 }
 
+// flag: set if the call as a whole is to be refused (see append_check_kernel); reported and cleared.
 __global__ void append_kernel(JobArrays job, FitArrays fit, int max_jobs, int n, const int32_t* ids,
                               const double* losses, const double* times, const int32_t* cores, int checked,
-                              Mailbox* mail, uint32_t seq, unsigned int* ticket) {
+                              Mailbox* mail, uint32_t seq, unsigned int* ticket, int32_t* flag) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) append_one(job, fit, max_jobs, i, ids, losses, times, cores, checked);
-    if (mail) report(mail, seq, ticket, nullptr);
+    if (i < n && !(flag && *flag)) append_one(job, fit, max_jobs, i, ids, losses, times, cores, checked);
+    if (mail) report(mail, seq, ticket, flag);
+}
+
+// What the host checks of a small append, for a large one: sets *flag unless the ids rise and lie in range, losses and times are
+// finite and cores are at least 1.
+__global__ void append_check_kernel(int max_jobs, int n, const int32_t* ids, const double* losses, const double* times,
+                                    const int32_t* cores, int32_t* flag) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int j = ids[i], before = i > 0 ? ids[i - 1] : -1;
+    int top = __double2hiint(losses[i]) & 0x7ff00000;
+    if (times) top = max(top, __double2hiint(times[i]) & 0x7ff00000);
+    if (j <= before || j >= max_jobs || top == 0x7ff00000 || (cores && cores[i] < 1)) *flag = 1;
 }
 
 // Sets *flag if a value is not finite; with a mailbox the flag is reported (and cleared).
@@ -643,6 +656,16 @@ bool sizes_ok(int32_t max_jobs, int32_t max_hist, int32_t cap) {
     return max_jobs >= 1 && max_hist >= 4 && max_hist <= kMaxHistLimit && cap >= 1 && cap <= kMaxCoresLimit;
 }
 
+void note_active(slaq_handle* h, int32_t n, const int32_t* ids) {
+    if (h->n_active == h->max_jobs) return;   // every id is active
+    for (int32_t i = 0; i < n; ++i) {
+        if (!h->active[ids[i]]) {
+            h->active[ids[i]] = 1;
+            h->n_active += 1;
+        }
+    }
+}
+
 int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losses, const double* times,
               const int32_t* cores) {
     if (!h) return SLAQ_E_ARG;
@@ -656,9 +679,9 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
     const int threads = 256, blocks = (n + threads - 1) / threads;
     const int32_t *d_ids = h->stage.ids, *d_cores = times && cores ? h->stage.cores : nullptr;
     const double *d_losses = h->stage.losses, *d_times = times ? h->stage.times : nullptr;
-    // Small calls: the arrays are copied into the mailbox and the kernel reads them there.  Larger ones are copied to the
-    // device; from page-locked memory that runs while the host checks the arguments, so those copies go first.
-    // Nothing reads the staging arrays unless the checks pass.
+    // Small calls: the host checks the arrays and copies them into the mailbox, where the kernel reads them.  Larger ones are
+    // copied to the device and checked there: reading 100,000 entries once more on the host took 120 us, longer than the
+    // copies.  What the device refuses the host looks at again, to say why - or to accept ids that do not rise.
     bool mailed = n <= h->mailbox_jobs;
     if (mailed && n > kMailAlways) {
         cudaPointerAttributes attr;
@@ -670,6 +693,17 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
         CK(cudaMemcpyAsync(h->stage.losses, losses, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy losses");
         if (d_times) CK(cudaMemcpyAsync(h->stage.times, times, sizeof(double) * n, cudaMemcpyHostToDevice, st), "copy times");
         if (d_cores) CK(cudaMemcpyAsync(h->stage.cores, cores, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy cores");
+    }
+    if (!mailed && !(cores && !times)) {   // cores without times are checked although they are not used
+        append_check_kernel<<<blocks, threads, 0, st>>>(h->max_jobs, n, d_ids, d_losses, d_times, d_cores, h->scratch.load_flag);
+        append_kernel<<<blocks, threads, 0, st>>>(h->job, h->fit, h->max_jobs, n, d_ids, d_losses, d_times, d_cores, 0, h->mailbox,
+                                                  ++h->call_seq, h->scratch.append_ticket, h->scratch.load_flag);
+        CK(cudaGetLastError(), "append kernels");
+        if (const int rc = wait_mailbox(h, "append")) return rc;   // the caller may reuse its buffers
+        if (!h->mailbox->err) {
+            note_active(h, n, ids);
+            return SLAQ_OK;
+        }
     }
     int bad = check_ids(h, n, ids, true);
     if (!bad && !(all_finite(losses, n) && (!times || all_finite(times, n)))) {   // which comes first says the message
@@ -684,10 +718,7 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
         for (int32_t i = 0; i < n; ++i) least = cores[i] < least ? cores[i] : least;
         if (least < 1) bad = fail(h, SLAQ_E_ARG, "cores_used must be at least 1");
     }
-    if (bad) {
-        if (!mailed) cudaStreamSynchronize(st);   // the caller's buffers are free again; the state is untouched
-        return bad;
-    }
+    if (bad) return bad;   // the state is untouched
     if (mailed) {
         if (const int rc = mail_arrays_free(h)) return rc;
         std::memcpy(h->mail_ids(), ids, sizeof(int32_t) * n);
@@ -700,7 +731,7 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
         if (d_cores) d_cores = h->mail_cores();
     }
     append_kernel<<<blocks, threads, 0, st>>>(h->job, h->fit, h->max_jobs, n, d_ids, d_losses, d_times, d_cores, 0, h->mailbox,
-                                              ++h->call_seq, h->scratch.append_ticket);
+                                              ++h->call_seq, h->scratch.append_ticket, nullptr);
     CK(cudaGetLastError(), "append kernel");
     if (mailed) {
         h->mail_in_use = true;
@@ -708,14 +739,7 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
     } else if (const int rc = wait_mailbox(h, "append")) {   // the caller may reuse its buffers
         return rc;
     }
-    if (h->n_active < h->max_jobs) {   // nothing to do once every id is active
-        for (int32_t i = 0; i < n; ++i) {
-            if (!h->active[ids[i]]) {
-                h->active[ids[i]] = 1;
-                h->n_active += 1;
-            }
-        }
-    }
+    note_active(h, n, ids);
     return SLAQ_OK;
 }
 
@@ -1162,7 +1186,7 @@ int slaq_append_losses_device(slaq_t* h, int32_t n, const int32_t* d_job_ids, co
     if (n == 0) return SLAQ_OK;
     const int threads = 256;
     append_kernel<<<(n + threads - 1) / threads, threads, 0, h->stream>>>(h->job, h->fit, h->max_jobs, n, d_job_ids, d_losses,
-                                                                        d_iter_times, d_cores_used, 1, nullptr, 0, nullptr);
+                                                                        d_iter_times, d_cores_used, 1, nullptr, 0, nullptr, nullptr);
     CK(cudaGetLastError(), "append kernel");
     return SLAQ_OK;
 }
