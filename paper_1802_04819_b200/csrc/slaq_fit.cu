@@ -18,6 +18,7 @@
 // are reduced over the L lanes with shuffles; the even lanes of a group then run family I's
 // solver step for the job and the odd lanes family II's.  All per-job control flow is per
 // lane, so the jobs of a warp may be in different phases of the solver.
+// Clusters with fewer jobs than the GPU has sub-partitions take a block per job instead (fit_team_kernel).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -50,6 +51,8 @@ struct Phases {
 
 constexpr int kMaxWarpsPerBlock = 16;          // one block per SM: its warps share one copy of the weight table
 constexpr size_t kSmemLimit = 226 * 1024;   // shared memory one block may use on sm_100, less the static part
+constexpr int kTeamWarps = 8;               // warps of a block that works on one job
+constexpr size_t kTeamSmem = 220 * 1024;
 constexpr double kLambda0 = 1e-3, kLambdaMin = 1e-5, kLambdaMax = 1e12;
 
 // Reductions over the L lanes of a group (L a power of two); every lane of the warp takes part.
@@ -637,7 +640,6 @@ __device__ __noinline__ void restart_from_first_guesses(const Lanes& S, int fam,
 struct FitClasses {
     int n;
     int h_lo[kMaxFitClasses], h_hi[kMaxFitClasses], L[kMaxFitClasses];
-    int rows;        // sweeps a lane makes at most, over all classes
     int h_max;       // longest window
     int slice;       // doubles of shared memory per warp: parked sums, window rows, one spare row
 };
@@ -645,12 +647,13 @@ struct FitClasses {
 // One slot of the work queue: the place-th warp's worth of jobs of class c.  kWarm: families may start from last epoch's
 // parameters (a separate instantiation, so that the plain one carries none of that code).  kL: lanes per job, a
 // constant, which takes branches and index arithmetic out of every step of a trial.
-template <bool kWarm, int kL>
+template <bool kWarm, int kL, bool kTeam = false>
 __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& fit, const int32_t* __restrict__ order,
                                          const int32_t* __restrict__ start, const FitClasses& cls, int c, int place, int lm_trials,
                                          int min_fit_points, const double* wtab, double* slice, unsigned long long* tally, int lane,
-                                         Phases& phases, int32_t* err_word) {
-    const int fam = lane & 1;             // even lanes solve family I, odd lanes family II
+                                         Phases& phases, int32_t* err_word, Team team = {}) {
+    const int fam = kTeam ? team.fam : lane & 1;   // even lanes solve family I, odd lanes family II
+    const bool leader = !kTeam || (team.fam == 0 && team.part == 0);   // writes the job's record
     const int even = lane & ~1, oddl = lane | 1;
     constexpr int L = kL;
     const int h_hi = cls.h_hi[c];
@@ -664,7 +667,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
     S.any_L = L;
     S.l = lane & (L - 1);
     const int G = 32 / L, g = lane / L;
-    S.park = slice + 2 * g + (lane & 1);
+    S.park = slice + 2 * g + (kTeam ? 0 : lane & 1);
     S.y = slice + kParked * 2 * G;
     const int last = order ? start[cls.h_lo[c]] : job.max_jobs;
     const int base = (order ? start[h_hi] : 0) + place * G;
@@ -699,15 +702,32 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
         // family's first guess in a second round.
         int spent = 0;
         SweepSums sums = {};
+        const bool wantsI = fits && (!kTeam || fam == 0), wantsII = fits && (!kTeam || fam == 1);
+        auto sweep_at = [&](bool doI, bool doII) {
+            if constexpr (kTeam) {
+                if (fam == 0) sweep_team<0>(S, team, H, inv_span, pI, sums);
+                else sweep_team<1>(S, team, H, inv_span, pII, sums);
+            } else {
+                sweep(S, fam, H, k_all, inv_span, pI, doI, pII, doII, sums);
+            }
+        };
+        auto park_sums = [&](bool keep) {
+            if constexpr (kTeam) {
+                if (keep && team.index >= 0 && S.holds(S.park + 2 * team.index)) S.park[2 * team.index] = sums.v[0];
+                __syncwarp();
+            } else {
+                park(S, sums, keep);
+            }
+        };
         if (!kWarm) {
-            first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, fits, fits, mom, pI, pII);
-            sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
+            first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, wantsI, wantsII, mom, pI, pII);
+            sweep_at(fits, fits);
         } else {
             unsigned wmask = fits ? fit.warm_mask[j] : 0u;
             if (wmask) carry_over(fit, job, j, span, nz.M, wmask, pI, pII);
             {
                 double gI[4], gII[4];
-                const bool needI = fits && !(wmask & 1u), needII = fits && !(wmask & 2u);
+                const bool needI = wantsI && !(wmask & 1u), needII = wantsII && !(wmask & 2u);
                 first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, needI, needII, mom, gI, gII);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
@@ -715,9 +735,13 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
                     if (needII) pII[a] = gII[a];
                 }
             }
-            sweep(S, fam, H, k_all, inv_span, pI, fits, pII, fits, sums);
+            sweep_at(fits, fits);
             const bool redo = fits && ((wmask >> fam) & 1u) && !sums.usable;
-            if (__any_sync(kFull, redo)) {   // rare: kept out of line, with its own copies of what it changes
+            if (kTeam && redo) {   // the same in all lanes of the family's warps
+                first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, wantsI, wantsII, mom, pI, pII);
+                sweep_at(fits, fits);
+                spent = 1;
+            } else if (!kTeam && __any_sync(kFull, redo)) {   // rare: kept out of line, with its own copies of what it changes
                 double tI[4], tII[4];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) tI[a] = pI[a], tII[a] = pII[a];
@@ -740,7 +764,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
         F.done = !F.ok;
         F.has_trial = false;
         F.predicted = 0.0;
-        park(S, sums, true);
+        park_sums(true);
         SLAQ_PHASE(1);   // first guesses and the sweep at the starting points
         const double tiny_S = 1e-28 * mom.swy2;
         for (int t = 0; t < lm_trials; ++t) {
@@ -752,8 +776,8 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
                 prepare_trial(F, fam, A, gr, !F.done, tiny_S, trial);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
-                    pI[a] = __shfl_sync(kFull, trial[a], even);
-                    pII[a] = a < 3 ? __shfl_sync(kFull, trial[a], oddl) : 0.0;
+                    pI[a] = kTeam ? trial[a] : __shfl_sync(kFull, trial[a], even);
+                    pII[a] = kTeam ? trial[a] : a < 3 ? __shfl_sync(kFull, trial[a], oddl) : 0.0;
                 }
             }
             const unsigned trying = __ballot_sync(kFull, F.has_trial);
@@ -761,10 +785,10 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
             if (!trying) continue;
             // the lane's own trial point is one of the two it swept: not kept a second time across the sweep
 #define SLAQ_OWN_TRIAL {fam ? pII[0] : pI[0], fam ? pII[1] : pI[1], fam ? pII[2] : pI[2], fam ? 0.0 : pI[3]}
-            if (t + 1 < lm_trials) {
-                sweep(S, fam, H, k_all, inv_span, pI, (trying >> even) & 1u, pII, (trying >> oddl) & 1u, sums);
+            if (kTeam || t + 1 < lm_trials) {
+                sweep_at((trying >> even) & 1u, (trying >> oddl) & 1u);
                 const double trial[4] = SLAQ_OWN_TRIAL;
-                park(S, sums, finish_trial(F, trial, sums.usable, sums.S));
+                park_sums(finish_trial(F, trial, sums.usable, sums.S));
             } else {   // no step follows: the objective decides, the normal equations are not needed
                 bool usable;
                 double objective;
@@ -776,14 +800,35 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
             SLAQ_PHASE(3);   // sweep at the trial points, reduction, accept or reject
         }
         // both results of the job, in every lane
-        const double S_I = __shfl_sync(kFull, F.S, even), S_II = __shfl_sync(kFull, F.S, oddl);
-        const bool ok_I = __shfl_sync(kFull, (int)F.ok, even), ok_II = __shfl_sync(kFull, (int)F.ok, oddl);
-        sweeps_out[0] = __shfl_sync(kFull, F.sweeps, even);
-        sweeps_out[1] = __shfl_sync(kFull, F.sweeps, oddl);
+        double S_I, S_II;
+        bool ok_I, ok_II;
+        if constexpr (kTeam) {   // through shared memory; the whole block is on this job
+            __syncthreads();
+            if (lane == 0 && team.part == 0) {
+                double* const mine = team.exchange + 16 * fam;
+                mine[0] = F.S;
+                mine[1] = F.ok ? 1.0 : 0.0;
+                mine[2] = (double)F.sweeps;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            pI[a] = __shfl_sync(kFull, F.p[a], even);
-            pII[a] = __shfl_sync(kFull, F.p[a], oddl);
+                for (int a = 0; a < 4; ++a) mine[3 + a] = F.p[a];
+            }
+            __syncthreads();
+            const double *const one = team.exchange, *const two = team.exchange + 16;
+            S_I = one[0], S_II = two[0];
+            ok_I = one[1] > 0.0, ok_II = two[1] > 0.0;
+            sweeps_out[0] = (int)one[2], sweeps_out[1] = (int)two[2];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) pI[a] = one[3 + a], pII[a] = two[3 + a];
+        } else {
+            S_I = __shfl_sync(kFull, F.S, even), S_II = __shfl_sync(kFull, F.S, oddl);
+            ok_I = __shfl_sync(kFull, (int)F.ok, even), ok_II = __shfl_sync(kFull, (int)F.ok, oddl);
+            sweeps_out[0] = __shfl_sync(kFull, F.sweeps, even);
+            sweeps_out[1] = __shfl_sync(kFull, F.sweeps, oddl);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                pI[a] = __shfl_sync(kFull, F.p[a], even);
+                pII[a] = __shfl_sync(kFull, F.p[a], oddl);
+            }
         }
         if (fits) {
             if (ok_I) S_out[0] = S_I;
@@ -825,17 +870,17 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
         p_out[2] = p_out[3] = CUDART_NAN;
     }
     {   // the slot's share of the statistics, one entry per lane
-        const bool own = S.l == 0 && H > 0, curve = own && status == SLAQ_JOB_FITTED;
+        const bool own = leader && S.l == 0 && H > 0, curve = own && status == SLAQ_JOB_FITTED;
         const unsigned points = __reduce_add_sync(kFull, own ? (unsigned)H : 0u);
         const unsigned swept = __reduce_add_sync(kFull, own ? (unsigned)H * (unsigned)(sweeps_out[0] + sweeps_out[1]) : 0u);
         const unsigned sub = __ballot_sync(kFull, curve && family == 0), expo = __ballot_sync(kFull, curve && family == 1);
         const unsigned other = __ballot_sync(kFull, own && (status == SLAQ_JOB_SHORT || status == SLAQ_JOB_NEW || status == SLAQ_JOB_FIT_FAILED));
         // 1/(a x^2 + b x + c) is convex for all x >= 0 exactly when b^2 >= a c
         const unsigned bent = __ballot_sync(kFull, curve && family == 0 && p_out[1] * p_out[1] < p_out[0] * p_out[2]);
-        if (lane < 6)
+        if (leader && lane < 6)
             tally[lane] += lane == 0 ? points : lane == 1 ? swept : __popc(lane == 2 ? sub : lane == 3 ? expo : lane == 4 ? other : bent);
     }
-    if (S.l == 0 && H > 0) {
+    if (leader && S.l == 0 && H > 0) {
         fit.status[j] = status;
         fit.mask[j] = (uint8_t)ended;
         if (any_ended) {   // what the next epoch may start from
@@ -919,6 +964,44 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
             atomicAdd((unsigned long long*)&counters[lane < 2 ? lane : lane == 5 ? 14 : lane + 1], v);
             if (lane == 2 || lane == 3) atomicAdd((unsigned long long*)&counters[2], v);
         }
+    }
+#ifdef SLAQ_PHASE_CLOCKS
+    if (lane == 0)
+        for (int i = 0; i < 6; ++i) atomicAdd((unsigned long long*)&counters[8 + i], (unsigned long long)phases.sum[i]);
+#endif
+}
+
+// A block per job, for clusters with fewer jobs than the GPU has sub-partitions for: each family has warps of its own
+// (see Team).  The chain of a trial is shorter than in one warp that does both (fit of 8 windows of 20: 34 -> 28 us, of 160
+// of 40: 38 -> 32, of 8 of 1,000 with four warps per family: 82 -> 56).
+template <bool kWarm>
+__global__ void __launch_bounds__(kTeamWarps * 32)
+fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, FitClasses cls, int parts, int lm_trials,
+                int min_fit_points, long long* counters, long long* stamp, int32_t* err_word) {
+    extern __shared__ double smem[];
+    __shared__ double exchange[2 * 2 * 4 * 16];
+    __shared__ unsigned long long tally[6];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < cls.h_max; i += blockDim.x) smem[i] = g_wtab[i];
+    if (threadIdx.x < 6) tally[threadIdx.x] = 0;
+    after_previous();
+    note_time(stamp);
+    __syncthreads();
+    Team team;
+    team.parts = parts;
+    team.shift = 5 + (parts >> 1);   // 1, 2, 4 parts: 32, 64, 128 lanes
+    team.fam = warp & 1;
+    team.part = warp >> 1;
+    const int index = team_index(lane & 15);
+    team.index = lane < 16 && index < kParked ? index : -1;
+    team.turn = 0;
+    team.exchange = exchange;
+    Phases phases;
+    fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem,
+                              smem + cls.h_max + (size_t)warp * cls.slice, tally, lane, phases, err_word, team);
+    if (warp == 0 && lane < 6 && tally[lane]) {
+        atomicAdd((unsigned long long*)&counters[lane < 2 ? lane : lane == 5 ? 14 : lane + 1], tally[lane]);
+        if (lane == 2 || lane == 3) atomicAdd((unsigned long long*)&counters[2], tally[lane]);
     }
 #ifdef SLAQ_PHASE_CLOCKS
     if (lane == 0)
@@ -1163,12 +1246,18 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 }  // namespace
 
 using FitKernel = decltype(&fit_kernel<false, 0>);
+using FitTeamKernel = decltype(&fit_team_kernel<false>);
 static FitKernel const kFitKernels[2][6] = {
     {fit_kernel<false, 0>, fit_kernel<false, 2>, fit_kernel<false, 4>, fit_kernel<false, 8>, fit_kernel<false, 16>, fit_kernel<false, 32>},
     {fit_kernel<true, 0>, fit_kernel<true, 2>, fit_kernel<true, 4>, fit_kernel<true, 8>, fit_kernel<true, 16>, fit_kernel<true, 32>}};
 
+static FitTeamKernel const kFitTeamKernels[2] = {fit_team_kernel<false>, fit_team_kernel<true>};
+
 int fit_setup() {
     bool ok = true;
+    for (FitTeamKernel k : kFitTeamKernels)
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmem) == cudaSuccess &&
+             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
     for (const auto& row : kFitKernels)
         for (FitKernel k : row)
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
@@ -1187,6 +1276,10 @@ static long long jobs_for_lanes(const slaq_handle* h) {
 // does not fit at 32 lanes.
 static int fit_slice(const slaq_handle* h) {
     return std::max((int)(h->fit_slice_bytes / sizeof(double)), kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32);
+}
+static int team_slice(const slaq_handle* h) { return kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32; }
+static size_t team_smem(const slaq_handle* h, int parts) {
+    return sizeof(double) * ((size_t)h->max_hist + 2 * (size_t)parts * team_slice(h));
 }
 static int rows_at(int slice, int L) { return (slice - kParked * (64 / L)) / 32 - 1; }
 
@@ -1214,15 +1307,42 @@ int fit_least_lanes(const slaq_handle* h) {
     return best;
 }
 
+// Warps per family of a job's team; 0: no teams.  With a warp per sub-partition at most, a lane is left four rows of the longest
+// window; two warps share a sub-partition without loss where a lane would have twelve rows or more (140 windows of up to
+// 1,000: 61 -> 58 us, but 200 of up to 300: 44 -> 45), and teams of one warp per family up to sixteen rows (580 windows of 20: 38 ->
+// 35 us, but 300 of 1,000: 84 -> 87).
+static int fit_team_parts(const slaq_handle* h) {
+    const long long warps = 4LL * h->sm_count, jobs = std::max(1LL, jobs_for_lanes(h));
+    if (h->max_jobs > 4 * h->sm_count || 2 * jobs > (h->max_hist > 512 ? warps : 2 * warps)) return 0;
+    int parts = 1;
+    while (parts < kTeamWarps / 2 && ((4 * parts * jobs <= warps && h->max_hist > 128 * parts) ||
+                                      (4 * parts * jobs <= 2 * warps && h->max_hist > 384 * parts)))
+        parts *= 2;
+    while (parts > 0 && team_smem(h, parts) > kTeamSmem) parts >>= 1;
+    return parts;
+}
+
 int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     int launches = 0;
+    if (const int parts = fit_team_parts(h)) {
+        FitClasses all = {};
+        all.n = 1;
+        all.h_hi[0] = all.h_max = Hmax;
+        all.L[0] = 32;
+        all.slice = team_slice(h);
+        const cudaError_t e = launch_behind(kFitTeamKernels[h->warm_start ? 1 : 0], J, 64 * parts, team_smem(h, parts), st, h->job, h->fit,
+                                            h->wtab, all, parts, h->lm_trials, h->min_fit_points, h->scratch.counters, h->scratch.stamps,
+                                            h->err_word);
+        if (e == cudaSuccess) return 1;
+        h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
+        return -1;
+    }
     // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked doubles per job and
     // family), the window rows of 32 points and one spare row.  The class with L = 32, 16, .. lanes per job takes
     // the windows that do not fit at L/2 lanes; the last one has the fewest lanes and takes the rest.
     FitClasses cls;
     cls.n = 0;
-    cls.rows = 1;
     cls.h_max = Hmax;
     cls.slice = fit_slice(h);
     const int L_min = fit_least_lanes(h);
@@ -1233,7 +1353,6 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         cls.h_lo[cls.n] = h_lo;
         cls.h_hi[cls.n] = h_hi;
         cls.L[cls.n] = L;
-        cls.rows = std::max(cls.rows, (h_hi + L - 1) / L);
         ++cls.n;
         h_hi = h_lo;
     }

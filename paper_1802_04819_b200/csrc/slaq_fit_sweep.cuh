@@ -284,6 +284,78 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     out.usable = !(broken & group & (odd ? 0xaaaaaaaau : 0x55555555u)) && (odd || !(negative & group));
 }
 
+// A job's team of warps, where there are more warps than jobs: `parts` warps (1, 2 or 4) for each family, which share
+// its rows.  Every warp holds the whole window and runs its family's solver on the same sums, so they all decide alike.
+struct Team {
+    int fam, part, parts, shift;   // 32 parts = 1 << shift lanes in all
+    int index;                     // which sum the lane ends with (-1: none that is parked)
+    int turn;
+    double* exchange;              // [2][2][4][16] in shared memory
+};
+
+// Which of the 13 sums a lane holds after the steps of sweep_team (13: none).
+__device__ __forceinline__ int team_index(int lane) {
+    const int b0 = lane & 1, b1 = lane >> 1 & 1, b2 = lane >> 2 & 1, b3 = lane >> 3 & 1;
+    const int at = 4 * b1 + 2 * b2 + b3;
+    return b0 ? min(7 + at, 13) : (at < 7 ? at : 13);
+}
+
+// One sweep of one family by its team: half the arithmetic per point, no exchange between families, and a lane has
+// as few rows as the team has lanes.
+template <int kFam>
+__device__ __forceinline__ void sweep_team(const LanesOf<32>& S, Team& t, int H, double inv_span, const double (&p)[4], SweepSums& out) {
+    LaneSums a = {};
+    const int LT = 1 << t.shift, lt = S.lane + 32 * t.part;
+    const int k_last = H - 1 - lt >= 0 ? (H - 1 - lt) >> t.shift : -1;
+    const int k_all = (H + LT - 1) >> t.shift;
+    const int mi = lt + k_last * LT;
+    const double md = (double)mi, hx = (double)LT * inv_span;
+    double x = -md * inv_span, e = 0.0, ratio = 1.0;
+    if (kFam == 1) {
+        e = exp(fma(p[1], md * inv_span, p[0]));
+        ratio = exp(-p[1] * hx);
+    }
+    const double* yp = S.y + mi;   // point m lies at y[(m / 32) * 32 + lane], and mi is lane + 32 times something
+    const double* wp = S.wtab + mi;
+#pragma unroll 1
+    for (int i = 0; i < k_all; ++i, x += hx, yp -= LT, wp -= LT)
+        if (i <= k_last) add_point<kFam == 0, kFam == 1>(S, wp, yp, x, p, p, e, ratio, a);
+    const double x_l = -(double)lt * inv_span, g = -hx;
+    double v[13];
+    if (kFam == 0) {
+        chains_to_powers(a.m, x_l, g);
+        chains_to_powers(a.n, x_l, g);
+        chains_to_powers(a.h, x_l, g);
+        v[0] = a.m[0]; v[1] = a.m[1]; v[2] = a.m[2]; v[3] = a.m[3]; v[4] = a.m[4];
+        v[5] = a.n[0]; v[6] = a.n[1]; v[7] = a.n[2]; v[8] = a.h[0]; v[9] = a.h[1]; v[10] = a.h[2];
+        v[11] = a.gd; v[12] = a.sI;
+    } else {
+        chains_to_powers(a.ee, x_l, g);
+        chains_to_powers(a.f, x_l, g);
+        chains_to_powers(a.kk, x_l, g);
+        v[0] = 0.0; v[1] = -a.f[1]; v[2] = a.ee[2]; v[3] = -a.ee[1]; v[4] = a.ee[0]; v[5] = a.f[0]; v[6] = v[7] = 0.0;
+        v[8] = -a.gc; v[9] = a.kk[1]; v[10] = -a.kk[0]; v[11] = 0.0; v[12] = a.sII;
+    }
+    halve<7, 13>(v, 1, S.lane);
+    halve<4, 7>(v, 2, S.lane);
+    halve<2, 4>(v, 4, S.lane);
+    halve<1, 2>(v, 8, S.lane);
+    double own = v[0] + __shfl_xor_sync(kFull, v[0], 16);
+    bool negative = kFam == 0 && __any_sync(kFull, a.q_signs < 0);
+    if (t.parts > 1) {   // the parts' sums, in the same order in every warp
+        double* const at = t.exchange + ((t.turn * 2 + kFam) * 4) * 16;
+        t.turn ^= 1;   // the other half next time: a warp may still be reading this one then
+        if (S.lane < 16) at[t.part * 16 + S.lane] = S.lane == 15 ? (negative ? 1.0 : 0.0) : own;
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + kFam), "r"(LT) : "memory");
+        own = at[S.lane & 15];
+        for (int q = 1; q < t.parts; ++q) own += at[q * 16 + (S.lane & 15)];
+        negative = kFam == 0 && __shfl_sync(kFull, own, 15) > 0.0;
+    }
+    out.v[0] = own;
+    out.S = __shfl_sync(kFull, own, 11);   // where sum 12 ends
+    out.usable = __all_sync(kFull, finite_d(own)) && !negative;
+}
+
 // The objectives alone, for a trial after which no further step is taken: a third of the sweep's arithmetic per point, and
 // nothing to reduce but the objective.  Added up in the sweep's order, so the same to the bit.  A point at which the model
 // is not defined makes its objective non-finite or its denominator negative; the other sums are bounded by the
