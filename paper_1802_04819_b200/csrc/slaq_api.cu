@@ -39,7 +39,7 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     Bump b{base};
     const size_t Js = (size_t)J;
     double* ring = b.take<double>(Js * Hmax);
-    double* wtab = b.take<double>(Hmax);
+    double* wtab = b.take<double>(6 * (size_t)Hmax + 5);
     JobArrays job;
     job.row = b.take<double*>(Js);
     job.cap = b.take<int32_t>(Js);
@@ -497,8 +497,18 @@ int check_ids(slaq_handle* h, int32_t n, const int32_t* ids, bool forbid_dups) {
 
 int ensure_weights(slaq_handle* h) {
     if (h->wtab_gamma == h->gamma) return SLAQ_OK;
-    std::vector<double> tab((size_t)h->max_hist);
-    for (int m = 0; m < h->max_hist; ++m) tab[m] = std::pow(h->gamma, (double)m);
+    // gamma^m, then the sums over m < H of gamma^m m^p for H = 0..max_hist, p = 0..4
+    const size_t n = (size_t)h->max_hist;
+    std::vector<double> tab(n + 5 * (n + 1));
+    for (size_t m = 0; m < n; ++m) tab[m] = std::pow(h->gamma, (double)m);
+    long double sum[5] = {};
+    for (size_t m = 0; m <= n; ++m) {
+        long double term = m < n ? (long double)tab[m] : 0.0L;
+        for (int p = 0; p < 5; ++p, term *= (long double)m) {
+            tab[n + p * (n + 1) + m] = (double)sum[p];
+            sum[p] += term;
+        }
+    }
     CK(cudaMemcpyAsync(h->wtab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream),
        "upload weight table");
     CK(cudaStreamSynchronize(h->stream), "upload weight table");

@@ -449,8 +449,10 @@ struct Moments {
 // and log(y - d0) is a line in x (family II: weighted linear regression).  needI / needII: the
 // job wants that family's guess (a family that starts from last epoch's parameters does not);
 // the weight sums in `mom` are always produced.
+// The sums of the weights times powers of x depend on the window's length alone and come from a table: formed in the pass they
+// were 7 of its 50 fp64 instructions per point, and 5 of 11 reductions.
 struct GuessSums {
-    double sw, swx, swx2, swx3, swx4, swy2, r0, r1, r2, su, sxu;
+    double swy2, r0, r1, r2, su, sxu;
 };
 
 // One point of the first-guess pass.  kI / kII: the transformed values of family I (1 / (y - d0)) and of
@@ -461,15 +463,7 @@ __device__ __forceinline__ void guess_point(const Lanes& S, const double* wp, co
     const double x = -md * inv_span;
     const double w = S.weight(wp);
     const double y = S.holds(yp) ? *yp : 0.0;
-    g.sw += w;
     g.swy2 = fma(w * y, y, g.swy2);
-    if (kI || kII) {
-        const double wx = w * x, wx2 = wx * x;
-        g.swx += wx;
-        g.swx2 += wx2;
-        g.swx3 = fma(wx2, x, g.swx3);
-        g.swx4 = fma(wx2 * x, x, g.swx4);
-    }
     if (kI) {
         const double wz = w * fast_rcp(y - d0);
         g.r2 += wz;
@@ -516,12 +510,15 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
         else if (anyII) guess_rows<false, true>(S, own, k_all, inv_span, d0, g);
         else guess_rows<false, false>(S, own, k_all, inv_span, d0, g);
     }
-    double sw = g.sw, swx = g.swx, swx2 = g.swx2, swx3 = g.swx3, swx4 = g.swx4, swy2 = g.swy2;
+    double wm[5];
+#pragma unroll
+    for (int p = 0; p < 5; ++p) wm[p] = busy && index_ok(H, S.wtab_len + 1, kErrShared, S.err_word) ? S.wsum[p * (S.wtab_len + 1) + H] : 0.0;
+    const double inv2 = inv_span * inv_span;
+    const double sw = wm[0], swx = -wm[1] * inv_span, swx2 = wm[2] * inv2, swx3 = -wm[3] * (inv2 * inv_span), swx4 = wm[4] * (inv2 * inv2);
+    double swy2 = g.swy2;
     double r0 = g.r0, r1 = g.r1, r2 = g.r2, su = g.su, sxu = g.sxu;
     for (int o = S.L() >> 1; o > 0; o >>= 1) {
-        sw += __shfl_xor_sync(kFull, sw, o); swx += __shfl_xor_sync(kFull, swx, o);
-        swx2 += __shfl_xor_sync(kFull, swx2, o); swx3 += __shfl_xor_sync(kFull, swx3, o);
-        swx4 += __shfl_xor_sync(kFull, swx4, o); swy2 += __shfl_xor_sync(kFull, swy2, o);
+        swy2 += __shfl_xor_sync(kFull, swy2, o);
         r0 += __shfl_xor_sync(kFull, r0, o); r1 += __shfl_xor_sync(kFull, r1, o);
         r2 += __shfl_xor_sync(kFull, r2, o); su += __shfl_xor_sync(kFull, su, o);
         sxu += __shfl_xor_sync(kFull, sxu, o);
@@ -650,7 +647,8 @@ struct FitClasses {
 template <bool kWarm, int kL, bool kTeam = false>
 __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& fit, const int32_t* __restrict__ order,
                                          const int32_t* __restrict__ start, const FitClasses& cls, int c, int place, int lm_trials,
-                                         int min_fit_points, const double* wtab, double* slice, unsigned long long* tally, int lane,
+                                         int min_fit_points, const double* wtab, const double* wsum, double* slice, unsigned long long* tally,
+                                         int lane,
                                          Phases& phases, int32_t* err_word, Team team = {}) {
     const int fam = kTeam ? team.fam : lane & 1;   // even lanes solve family I, odd lanes family II
     const bool leader = !kTeam || (team.fam == 0 && team.part == 0);   // writes the job's record
@@ -659,6 +657,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
     const int h_hi = cls.h_hi[c];
     LanesOf<kL> S;
     S.wtab = wtab;
+    S.wsum = wsum;
     S.lane = lane;
     S.slice = slice;
     S.slice_len = cls.slice;
@@ -947,11 +946,11 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         while (slot >= slot_base[c + 1]) ++c;
         const int place = slot - slot_base[c];
         switch (kL ? kL : cls.L[c]) {
-#define SLAQ_SLOT(n)                                                                                                            \
-    case n:                                                                                                                     \
-        if constexpr (kL == 0 || kL == n)                                                                                       \
-            fit_slot<kWarm, n>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, slice, tally[warp], lane, \
-                               phases, err_word);                                                                               \
+#define SLAQ_SLOT(n)                                                                                                              \
+    case n:                                                                                                                       \
+        if constexpr (kL == 0 || kL == n)                                                                                         \
+            fit_slot<kWarm, n>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, g_wtab + cls.h_max, slice, \
+                               tally[warp], lane, phases, err_word);                                                              \
         break;
             SLAQ_SLOT(2) SLAQ_SLOT(4) SLAQ_SLOT(8) SLAQ_SLOT(16) SLAQ_SLOT(32)
 #undef SLAQ_SLOT
@@ -998,7 +997,7 @@ fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab,
     team.exchange = exchange;
     Phases phases;
     fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem,
-                              smem + cls.h_max + (size_t)warp * cls.slice, tally, lane, phases, err_word, team);
+                              g_wtab + cls.h_max, smem + cls.h_max + (size_t)warp * cls.slice, tally, lane, phases, err_word, team);
     if (warp == 0 && lane < 6 && tally[lane]) {
         atomicAdd((unsigned long long*)&counters[lane < 2 ? lane : lane == 5 ? 14 : lane + 1], tally[lane]);
         if (lane == 2 || lane == 3) atomicAdd((unsigned long long*)&counters[2], tally[lane]);

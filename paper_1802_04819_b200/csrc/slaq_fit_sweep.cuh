@@ -35,6 +35,7 @@ struct LanesOf {
     double* y;         // [k_cap + 1][32]
     double* park;      // this lane's family of its job in [kParked][2 * jobs per warp] (one column per job and family)
     const double* wtab;
+    const double* wsum;   // in global memory: [5][wtab_len + 1] sums over m < H of gamma^m m^p (first guesses only)
     int lane, l;
     int any_L;         // lanes per job (kL == 0)
     __device__ __forceinline__ int L() const { return kL ? kL : any_L; }

@@ -159,7 +159,7 @@ struct slaq_handle {
     size_t packed_len = 0;
     void* call_buf = nullptr;         // scratch of calls that move caller data of any size (grown on demand, kept)
     size_t call_buf_bytes = 0;
-    double* wtab = nullptr;           // gamma^m, m = 0..max_hist-1
+    double* wtab = nullptr;           // gamma^m, m = 0..max_hist-1, then the sums over m < H of gamma^m m^p: [5][max_hist + 1]
     double wtab_gamma = -1.0;
     slaq::JobArrays job;
     slaq::FitArrays fit;
