@@ -1284,11 +1284,11 @@ static int rows_at(int slice, int L) { return (slice - kParked * (64 / L)) / 32 
 
 // The fewest lanes a job gets.  Fewer lanes are less work - the solver's step and the reductions of a trial cost a warp
 // the same whatever it carries - and longer chains of rows.  Cycles per trial, fitted to clusters of 1,000 to 32,000 jobs
-// with windows of up to 12 to 1,000 points, full or ragged, at 2 to 32 lanes each: a warp alone takes 2500 + 142 per row,
-// and a sub-partition can issue 1500 + 106 per row for each of its warps; the longer of the two decides, over the lane
-// counts at which every window fits.  That choice is within 1 % of the best on average and 13 % at worst; filling
-// every warp of the GPU twice, the rule before, cost 36 % (fit of 8,000 windows of up to 100: 282 -> 118 us).  Beyond one
-// slot per warp of the GPU more lanes only add work, although the longest windows then get more lanes than
+// with windows of up to 12 to 1,000 points, full or ragged, at 2 to 32 lanes each: a warp alone takes 2300 + 170 per row,
+// and a sub-partition can issue 1300 + 106 per row for each of its warps, of which a part counts nearly as a whole one; the
+// longer of the two decides, over the lane counts at which every window fits.  That choice is within 1.3 % of the best on
+// average; filling every warp of the GPU twice, the rule before, cost 36 % (fit of 8,000 windows of up to 100: 282 -> 118 us).
+// Beyond one slot per warp of the GPU more lanes only add work, although the longest windows then get more lanes than
 // the others (100,000 windows of up to 1,000: 4.9 ms with 32 lanes for all, 4.0 with 2 and up).
 int fit_least_lanes(const slaq_handle* h) {
     const int slice = fit_slice(h), Hmax = h->max_hist;
@@ -1298,8 +1298,8 @@ int fit_least_lanes(const slaq_handle* h) {
     for (int L = 32; L >= 2 && rows_at(slice, L) * L >= Hmax; L >>= 1) {
         const int rows = (Hmax + L - 1) / L;
         double warps = std::ceil(jobs * L / 32.0) / (4.0 * h->sm_count);   // per sub-partition
-        if (warps < 4.0) warps = std::ceil(warps);
-        const double cycles = std::max(2500.0 + 142.0 * rows, warps * (1500.0 + 106.0 * rows));
+        if (warps < 4.0) warps = std::min(std::ceil(warps), warps + 0.3);
+        const double cycles = std::max(2300.0 + 170.0 * rows, warps * (1300.0 + 106.0 * rows));
         if (L == 32 || cycles <= least) best = L, least = cycles;
     }
     while (best > 2 && jobs * (best / 2) >= 32.0 * kMaxWarpsPerBlock * h->sm_count) best >>= 1;
