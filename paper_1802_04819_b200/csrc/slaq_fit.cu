@@ -35,7 +35,7 @@ namespace {
 // SM cycles it spends in each phase of the fit; the totals go to counters[8..13].
 struct Phases {
 #ifdef SLAQ_PHASE_CLOCKS
-    long long sum[6] = {0, 0, 0, 0, 0, 0}, since = clock64();
+    long long sum[6], since;
 #endif
 };
 #ifdef SLAQ_PHASE_CLOCKS
@@ -45,8 +45,10 @@ struct Phases {
         phases.sum[i] += now_ - phases.since; \
         phases.since = now_;                 \
     } while (0)
+#define SLAQ_PHASES_START(p) (p).since = clock64()
 #else
 #define SLAQ_PHASE(i)
+#define SLAQ_PHASES_START(p)
 #endif
 
 constexpr int kMaxWarpsPerBlock = 16;          // one block per SM: its warps share one copy of the weight table
@@ -929,7 +931,8 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
         for (int c = cls.n; c <= kMaxFitClasses; ++c) slot_base[c] = run;
     }
     __syncthreads();
-    Phases phases;
+    Phases phases = {};
+    SLAQ_PHASES_START(phases);
     // The first slots are dealt out to the SMs in turn: slots are sorted by length, and the warps of a block, which draw
     // together, would get neighbours - the longest windows all on one SM (4,000 windows of up to 200 at 16 lanes: 133 us
     // drawn, 113 dealt).  The rest are drawn.
@@ -995,7 +998,8 @@ fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab,
     team.index = lane < 16 && index < kParked ? index : -1;
     team.turn = 0;
     team.exchange = exchange;
-    Phases phases;
+    Phases phases = {};
+    SLAQ_PHASES_START(phases);
     fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem,
                               g_wtab + cls.h_max, smem + cls.h_max + (size_t)warp * cls.slice, tally, lane, phases, err_word, team);
     if (warp == 0 && lane < 6 && tally[lane]) {
