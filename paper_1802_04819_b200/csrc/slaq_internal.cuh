@@ -83,7 +83,10 @@ struct SelectGlobal {
     unsigned long long fine[kSelectFineBins];             // .. and its 64 bins each
     unsigned int barrier, ticket, n_cand, pad;            // blocks that arrived; blocks that finished; listed candidates
     static constexpr size_t kZeroBytes = sizeof(unsigned long long) * (32 + kSelectFineBins) + 16;
-    unsigned long long narrow[kRadixPasses][kRadixBins];  // cleared by the kernel itself
+    // cleared by the kernel itself: the counts of continued rows, apart from the first ones, which slower blocks may still
+    // be reading when the first of these arrive; the histograms of the narrowing steps
+    unsigned long long coarse_more[32], fine_more[kSelectFineBins];
+    unsigned long long narrow[kRadixPasses][kRadixBins];
     unsigned long long cand_key[kSelectCandidates];       // the candidates the last block ranks ..
     unsigned long long cand_pos[kSelectCandidates];       // .. and their (candidates of the row, job, n)
     long long block_eq[kSelectMaxGrid];                   // per block: candidates that equal the threshold

@@ -30,6 +30,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <cstddef>
 
 #include "slaq_gain_curve.cuh"
 #include "slaq_internal.cuh"
@@ -137,9 +138,12 @@ __device__ u64 block_exclusive(u64 v, Shared& sh, u64* total) {
 }
 
 // Warp 0: the bin of the want-th largest gain from the global histogram (octave totals first, then the bins of one octave).  Fewer gains than wanted: an interval below everything counted, n = 0.
+// kMore: the counts of continued rows are added to the first ones.  What is read here is complete: every block flushed it before the
+// grid barrier in front of the call, and no block adds to it behind that barrier.
+template <bool kMore>
 __device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
     const int lane = threadIdx.x & 31;
-    const u64 c = __ldcg(&gl->coarse[31 - lane]);
+    const u64 c = __ldcg(&gl->coarse[31 - lane]) + (kMore ? __ldcg(&gl->coarse_more[31 - lane]) : 0);
     const u64 incl = warp_inclusive(c);
     const unsigned hit = __ballot_sync(kFull, incl >= want);
     if (!hit) {
@@ -152,7 +156,7 @@ __device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
     const int top = (31 - at) * kSub + kSub - 1 - per * lane;
     u64 v[per], sum = 0;
 #pragma unroll
-    for (int k = 0; k < per; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]);
+    for (int k = 0; k < per; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]) + (kMore ? __ldcg(&gl->fine_more[top - k]) : 0);
     const u64 incl2 = warp_inclusive(sum);
     const int at2 = __ffs(__ballot_sync(kFull, above + incl2 >= want)) - 1;
     if (lane == at2) {
@@ -190,19 +194,19 @@ __device__ void pick_narrow(Counts counts, Shared& sh) {
     __syncthreads();
 }
 
-// Adds a block's shared counts to the global ones.
-__device__ void flush_first(Shared& sh, SelectGlobal* gl) {
+// Adds a block's shared counts to global ones.
+__device__ void flush_first(Shared& sh, u64* coarse, u64* fine) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int o = warp; o < 32; o += kWarps) {
         unsigned int sum = 0;
 #pragma unroll
         for (int k = 0; k < kSub / 32; ++k) {
             const unsigned int v = sh.hist[o * kSub + k * 32 + lane];
-            if (v) atomicAdd(&gl->fine[o * kSub + k * 32 + lane], (u64)v);
+            if (v) atomicAdd(&fine[o * kSub + k * 32 + lane], (u64)v);
             sum += v;
         }
         sum = __reduce_add_sync(kFull, sum);
-        if (lane == 0 && sum) atomicAdd(&gl->coarse[o], (u64)sum);
+        if (lane == 0 && sum) atomicAdd(&coarse[o], (u64)sum);
     }
 }
 
@@ -663,9 +667,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     unsigned int arrived = 0;
 
     for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
-    // the narrowing histograms, should they be needed: cleared by all blocks before the first barrier
-    for (int i = blockIdx.x * kThreads + tid; i < kRadixPasses * kNarrowBins; i += gridDim.x * kThreads)
-        (&a.gl->narrow[0][0])[i] = 0;
+    // the counts of continued rows and the narrowing histograms, should they be needed: cleared by all blocks before the first barrier
+    constexpr int kLater = (int)((offsetof(SelectGlobal, cand_key) - offsetof(SelectGlobal, coarse_more)) / sizeof(u64));
+    u64* const later = reinterpret_cast<u64*>(reinterpret_cast<char*>(a.gl) + offsetof(SelectGlobal, coarse_more));
+    for (int i = blockIdx.x * kThreads + tid; i < kLater; i += gridDim.x * kThreads) later[i] = 0;
     if (tid == 0) sh.count = sh.n_more = 0;
     __syncthreads();
 
@@ -731,11 +736,11 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     low = __reduce_add_sync(kFull, low);
     if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
     __syncthreads();
-    flush_first(sh, a.gl);
+    flush_first(sh, a.gl->coarse, a.gl->fine);
     arrived += gridDim.x;
     if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
     if (a.want > 0) {
-        if (tid < 32) pick_first(a.gl, (u64)a.want, &sh.iv);
+        if (tid < 32) pick_first<false>(a.gl, (u64)a.want, &sh.iv);
     } else if (tid == 0) {
         sh.iv = Interval{~0ull, ~0ull, 0, 0};   // nothing wanted: a threshold above every gain
     }
@@ -792,10 +797,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         low = __reduce_add_sync(kFull, low);
         if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
         __syncthreads();
-        flush_first(sh, a.gl);
+        flush_first(sh, a.gl->coarse_more, a.gl->fine_more);
         arrived += gridDim.x;
         if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
-        if (tid < 32) pick_first(a.gl, (u64)a.want, &sh.iv);
+        if (tid < 32) pick_first<true>(a.gl, (u64)a.want, &sh.iv);
         __syncthreads();
     }
 

@@ -51,3 +51,22 @@ def test_selection_equals_the_definition(J, cap, kind):
             R = sched.get_predictions(want_gain=False)["R"]
             ref = np.concatenate([np.zeros((J, 1)), np.cumsum(gain, 1)], 1)[np.arange(J), want]
             np.testing.assert_array_equal(R, ref)           # the same additions in the same order
+
+
+def test_rows_that_only_some_blocks_continue():
+    """A streamed table whose long rows lie in a tenth of the blocks: those are still counting while the others have long
+    reached the second barrier.  The same table over and over, as the blocks meet differently each time."""
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+    J, cap = 30000, 64
+    rng = np.random.default_rng(5)
+    gain = np.exp(rng.uniform(-30, -10, (J, 1))) * np.sort(rng.random((J, cap)), 1)[:, ::-1]
+    gain[J // 2: J // 2 + J // 10] *= np.exp(25.0)            # whole rows above everything else
+    with slaq.Scheduler(J, 4, cap) as sched:
+        sched.append_losses(np.arange(J), np.ones(J))
+        sched.set_gains(gain)
+        for C in (J + 1000, 3 * J, J + J // 10 * (cap - 1) - 1):
+            want = _expected(gain, C)
+            for _ in range(60):
+                alloc, _ = sched.allocate_only(C)
+                np.testing.assert_array_equal(alloc, want)
