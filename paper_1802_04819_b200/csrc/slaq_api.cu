@@ -68,6 +68,10 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     fit.warm_k = b.take<int64_t>(Js);
     fit.warm_span = b.take<double>(Js);
     fit.warm_scale = b.take<double>(Js);
+    GainBasis basis;
+    basis.v = b.take<double>(6 * Js);
+    basis.kind = b.take<int8_t>(Js);
+    basis.note = b.take<GainNote>(1);
     Scratch sc;
     sc.hist = b.take<unsigned long long>((size_t)kRadixPasses * kRadixBins);
     sc.ticket = b.take<unsigned int>(kTickets);
@@ -110,6 +114,7 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
         h->wtab = wtab;
         h->job = job;
         h->fit = fit;
+        h->basis = basis;
         h->scratch = sc;
         h->stage = st;
         h->gain = gain;
@@ -653,6 +658,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
     for (auto& ev : h->ev) CK(cudaEventCreate(&ev), "cudaEventCreate");
     CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, h->stream), "clear scratch");
     CK(cudaMemsetAsync(h->err_word, 0, 16, h->stream), "clear error word");
+    CK(cudaMemsetAsync(h->basis.note, 0, sizeof(GainNote), h->stream), "clear gain note");
     const int threads = 256;
     init_jobs_kernel<<<(max_jobs + threads - 1) / threads, threads, 0, h->stream>>>(
         h->job, h->fit, h->ring_pool, max_jobs, max_hist, nullptr, max_jobs, h->alloc, h->reduction);
@@ -885,6 +891,22 @@ bool gains_in_selection(const slaq_handle* h, bool only_allocate) {
     return !only_allocate && !h->gain_envelope && h->n_hinted == 0;
 }
 
+// Whether the caller captures the handle's stream into a graph (or the query fails: then it is treated as if).
+bool is_capturing(slaq_handle* h) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// h->gain holds the whole rows of the last epoch afterwards.
+int complete_gains(slaq_handle* h) {
+    if (!h->gain_partial && !h->epoch_captured) return SLAQ_OK;
+    if (launch_complete_gains(h) < 0) return SLAQ_E_CUDA;
+    h->gain_partial = false;
+    return SLAQ_OK;
+}
+
 // The launches of one epoch, put on h->stream in order.  Returns the number of kernels or -1.
 int enqueue_epoch(slaq_handle* h, double T, int64_t want, int floor_units, int32_t* d_out, bool only_allocate, uint32_t seq) {
     int launches = 0, k;
@@ -931,15 +953,10 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
 
     if (!h->scratch_clean) {
         CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
-        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone) h->scratch_clean = true;
+        if (!is_capturing(h)) h->scratch_clean = true;
     }
     bool graph_ok = h->epoch_graph == 1;
-    if (graph_ok) {   // not while the caller captures this stream into a graph of its own
-        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &status) != cudaSuccess || status != cudaStreamCaptureStatusNone) graph_ok = false;
-        if (!graph_ok) cudaGetLastError();
-    }
+    if (graph_ok && is_capturing(h)) graph_ok = false;   // not while the caller captures this stream into a graph of its own
     int launches = -1;
     h->last_epoch_was_graph = false;
     if (graph_ok) {
@@ -1000,11 +1017,8 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     h->last_launches = launches;
     h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
     h->last_cores = usable;
-    // whether h->gain holds this epoch's whole rows (plain launches and a replayed graph alike), and what a later
-    // request for them has to be predicted for
-    h->gain_table_current = !gains_in_selection(h, only_allocate) || select_writes_whole_table(h, want);
-    h->last_T = T;
-    h->last_first_unit = floor_units + 1;
+    h->gain_partial = gains_in_selection(h, only_allocate) && !select_writes_whole_table(h, want);
+    h->epoch_captured = h->epoch_captured || is_capturing(h);
     if (active > 0 && C < active) return SLAQ_W_OVERSUBSCRIBED;
     if (C > active * cap) return SLAQ_W_UNDERFILLED;
     return SLAQ_OK;
@@ -1379,9 +1393,7 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
         g->last_epoch_was_graph = false;
         g->last_launches += s == 0 ? k : 0;
         g->last_steps = kEpochSteps;
-        g->gain_table_current = whole_table;
-        g->last_T = epoch_seconds;
-        g->last_first_unit = floor_units + 1;
+        g->gain_partial = !whole_table;
     }
     bool copied = false;
     for (int32_t s = 0; s < n; ++s)
@@ -1434,9 +1446,8 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     CK(cudaEventRecord(h->ev[3], st), "event");
     h->have_epoch = true;
     h->last_launches = h->last_steps = launches;
-    h->gain_table_current = true;
-    h->last_T = epoch_seconds;
-    h->last_first_unit = h->shard_first_unit;
+    h->gain_partial = false;
+    h->epoch_captured = h->epoch_captured || is_capturing(h);
     return SLAQ_OK;
 }
 
@@ -1523,10 +1534,8 @@ int slaq_get_predictions(slaq_t* h, double* out_reduction, double* out_gain, int
     if (!h) return SLAQ_E_ARG;
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     const size_t J = (size_t)h->max_jobs;
-    if (out_gain && !h->gain_table_current) {   // the last epoch predicted rows only as far as it needed: write them now
-        if (launch_gain(h, h->last_T, h->last_first_unit, false) < 0) return SLAQ_E_CUDA;
-        h->gain_table_current = true;
-    }
+    if (out_gain)
+        if (const int rc = complete_gains(h)) return rc;
     return results_to_host(h, {{out_gain, h->gain, 8 * J * h->max_cores},
                                {out_reduction, h->reduction, 8 * J},
                                {out_family, h->fit.family, J},

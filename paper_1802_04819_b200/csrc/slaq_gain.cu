@@ -64,6 +64,7 @@ __device__ __forceinline__ void count_key(unsigned int* hist, double g, bool cou
     }
 }
 
+// kKept: the rows of the last epoch from the curves it kept (see GainBasis), where it has left them unfinished.
 // kOptions: the instantiation that knows the two options of the prediction (the plain one carries none of
 // their code).  envelope: rows become the slopes of the concave envelope of R(n) instead of a
 // running minimum; target-loss hints are read per job.  hist0: null where nobody reads the histogram.
@@ -71,14 +72,22 @@ __device__ __forceinline__ void count_key(unsigned int* hist, double g, bool cou
 // What bounds it is latency, of one row's steps (load the curve, predict, envelope, cap) where jobs are few, of all rows'
 // where they are many.  With a warp per job whatever its row's length, and the envelope walked in global memory, 4,000
 // rows of 64 took 35 us (now 31) and 542,000 rows of 5 took 370 (now 130).
-template <bool kOptions>
+template <bool kOptions, bool kKept>
 __global__ void __launch_bounds__(kThreads, 5)
-gain_kernel(JobArrays job, FitArrays fit, int max_jobs, int cap, int W, double T, int first_unit, double* __restrict__ gain, long long* stamp,
-            unsigned long long* __restrict__ hist0, bool envelope) {
+gain_kernel(JobArrays job, FitArrays fit, GainBasis basis, int max_jobs, int cap, int W, double T, int first_unit, double* __restrict__ gain,
+            long long* stamp, unsigned long long* __restrict__ hist0, bool envelope) {
     extern __shared__ double dyn[];      // kOptions: [groups][cap] rows, then [groups][cap + 1] vertices
     __shared__ unsigned int sh_hist[kRadixBins];
     after_previous();
-    note_time(stamp);
+    if (kKept) {
+        const GainNote note = *basis.note;
+        if (!note.partial) return;
+        cap = note.cap;
+        T = note.T;
+    } else {
+        note_time(stamp);
+        if (blockIdx.x == 0 && threadIdx.x == 0) *basis.note = GainNote{0, cap, T};
+    }
     if (hist0) {
         for (int i = threadIdx.x; i < kRadixBins; i += kThreads) sh_hist[i] = 0;
         __syncthreads();
@@ -91,7 +100,7 @@ gain_kernel(JobArrays job, FitArrays fit, int max_jobs, int cap, int W, double T
         bool no_time = false;
         Curve c = {};
         c.kind = 3;
-        if (in) c = load_curve<true>(job, fit, j, max_jobs, T, &no_time);
+        if (in) c = kKept ? kept_curve(basis, j, max_jobs, T) : load_curve<true>(job, fit, j, max_jobs, T, &no_time);
         if (no_time && w == 0) fit.status[j] = SLAQ_JOB_NO_TIME;
         double* const out = gain + (size_t)(in ? j : 0) * cap;
         double* const row = kOptions ? dyn + (size_t)group * cap : out;
@@ -187,7 +196,7 @@ int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit, bool histo
     const int groups = kThreads / W;
     const bool options = h->gain_envelope || h->n_hinted > 0;
     const size_t smem = options ? (size_t)groups * (sizeof(double) * cap + sizeof(unsigned short) * (cap + 1)) : 0;
-    const auto kernel = options ? gain_kernel<true> : gain_kernel<false>;
+    const auto kernel = options ? gain_kernel<true, false> : gain_kernel<false, false>;
     cudaError_t e = cudaSuccess;
     int per_sm = 5;
     if (smem > 32 * 1024) {
@@ -196,8 +205,22 @@ int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit, bool histo
     }
     const int blocks = std::min(h->sm_count * per_sm, (J + groups - 1) / groups);
     if (e == cudaSuccess)
-        e = launch_behind(kernel, blocks, kThreads, smem, h->stream, h->job, h->fit, J, cap, W, epoch_seconds, first_unit, h->gain,
-                          h->scratch.stamps + 1, histogram ? h->scratch.hist : nullptr, h->gain_envelope);
+        e = launch_behind(kernel, blocks, kThreads, smem, h->stream, h->job, h->fit, h->basis, J, cap, W, epoch_seconds, first_unit,
+                          h->gain, h->scratch.stamps + 1, histogram ? h->scratch.hist : nullptr, h->gain_envelope);
+    if (e != cudaSuccess) {
+        h->err = std::string("gain kernel launch: ") + cudaGetErrorString(e);
+        return -1;
+    }
+    return 1;
+}
+
+int launch_complete_gains(slaq_handle* h) {
+    const int J = h->max_jobs, cap = h->max_cores;   // the epoch's own cap is in its note; this one decides the lanes per row
+    int W = 1;
+    while (W < 32 && W < cap) W <<= 1;
+    const int groups = kThreads / W, blocks = std::min(h->sm_count * 5, (J + groups - 1) / groups);
+    gain_kernel<false, true><<<blocks, kThreads, 0, h->stream>>>(h->job, h->fit, h->basis, J, cap, W, 0.0, 2, h->gain, nullptr, nullptr, false);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         h->err = std::string("gain kernel launch: ") + cudaGetErrorString(e);
         return -1;

@@ -98,6 +98,37 @@ __device__ inline double raw_gain(const Curve& c, int n) {
     return (finite_d(gain) && gain > 0.0) ? gain : 0.0;
 }
 
+// T w / span, in one order of its two products wherever a curve is put together.
+__device__ __forceinline__ double step_scale_of(double T, double w, double inv_span) { return T * w * inv_span; }
+
+// A curve as it was when its epoch ran.
+__device__ __forceinline__ void keep_curve(const GainBasis& b, int j, int max_jobs, const Curve& c, int kind) {
+    double* const v = b.v + j;
+    const size_t J = (size_t)max_jobs;
+    v[0] = c.p0;
+    v[J] = c.p1;
+    v[2 * J] = c.p2;
+    v[3 * J] = c.inv_span;
+    v[4 * J] = c.s;
+    v[5 * J] = c.w;
+    b.kind[j] = (int8_t)kind;
+}
+__device__ __forceinline__ Curve kept_curve(const GainBasis& b, int j, int max_jobs, double T) {
+    const double* const v = b.v + j;
+    const size_t J = (size_t)max_jobs;
+    Curve c;
+    c.p0 = v[0];
+    c.p1 = v[J];
+    c.p2 = v[2 * J];
+    c.inv_span = v[3 * J];
+    c.s = v[4 * J];
+    c.w = v[5 * J];
+    c.kind = b.kind[j];
+    c.T = T;
+    c.step_scale = step_scale_of(T, c.w, c.inv_span);
+    return c;
+}
+
 // The curve of job j for this epoch.  Sets kind 3 (no gain) for jobs that predict nothing; a job
 // that could predict but has no usable time law gets status SLAQ_JOB_NO_TIME, which the caller
 // records (*no_time).
@@ -133,7 +164,7 @@ __device__ inline Curve load_curve(const JobArrays& job, const FitArrays& fit, i
             c.p1 = kEager ? p[1] : fit.params[4 * (size_t)j + 1];
             c.p2 = kEager ? p[2] : fit.params[4 * (size_t)j + 2];
             c.kind = status == SLAQ_JOB_FITTED ? (kEager ? family : (int)fit.family[j]) : 2;
-            c.step_scale = T * c.w * c.inv_span;
+            c.step_scale = step_scale_of(T, c.w, c.inv_span);
         }
     }
     return c;

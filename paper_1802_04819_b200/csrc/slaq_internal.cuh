@@ -66,6 +66,20 @@ struct FitArrays {
     double* warm_scale;
 };
 
+// What the last epoch's gain rows follow from.  An epoch writes rows of a large table only as far as its selection needs them;
+// asked for later they must still be that epoch's, whatever has happened to the time laws, the hints or the fits since.  So
+// such an epoch keeps its curves: 49 bytes per job, against 8 max_cores_per_job for the rows themselves.
+struct GainNote {
+    int32_t partial;     // the rows are written only in part, and the curves below are those they follow from
+    int32_t cap;         // entries of a row
+    double T;
+};
+struct GainBasis {
+    double* v;           // [6][max_jobs]: the curve's three parameters, 1 / span, s, w
+    int8_t* kind;        // [max_jobs]
+    GainNote* note;
+};
+
 // Running state of the radix select.
 struct SelectState {
     unsigned long long prefix;       // bits of the threshold key found so far
@@ -146,9 +160,8 @@ struct slaq_handle {
     size_t fit_slice_bytes = 13824;       // shared memory one warp of the fit kernel may use (parked sums, up to 52 rows of 32 points, a spare row)
     bool warm_start = false;              // fits start from the last epoch's parameters where there are some
     int selection = 0;                    // SLAQ_P_SELECTION: kept for callers that ask, the launches are the same
-    bool gain_table_current = false;      // h->gain holds the whole rows of the last epoch
-    double last_T = 0.0;                  // what the last epoch's gains were predicted for
-    int last_first_unit = 2;
+    bool gain_partial = false;            // h->gain holds the last epoch's rows only in part (see GainBasis)
+    bool epoch_captured = false;          // an epoch of the handle is part of a graph of the caller: only the device knows which was last
     std::vector<uint8_t> hinted;          // host mirror: job has a target-loss hint
     int32_t n_hinted = 0;
     bool gain_envelope = false;           // gain rows are slopes of the concave envelope of R(n), not a running minimum
@@ -166,6 +179,7 @@ struct slaq_handle {
     double wtab_gamma = -1.0;
     slaq::JobArrays job;
     slaq::FitArrays fit;
+    slaq::GainBasis basis;
     slaq::Scratch scratch;
     slaq::Staging stage;
     double* gain = nullptr;           // [max_jobs][max_cores]
@@ -263,6 +277,8 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks);
 int fit_least_lanes(const slaq_handle* h);
 // histogram: the keys go into scratch.hist's first pass as well
 int launch_gain(slaq_handle* h, double epoch_seconds, int first_unit, bool histogram);
+// the rest of the last epoch's rows, from the curves it kept; does nothing if the rows are whole
+int launch_complete_gains(slaq_handle* h);
 // seq != 0: the kernel reports to the handle's mailbox under that number, and writes the allocation there too if it fits
 int launch_select(slaq_handle* h, double epoch_seconds, long long want, int first_unit, bool from_curves, int32_t* d_out_alloc,
                   uint32_t seq);

@@ -284,6 +284,7 @@ struct SelectArgs {
     int32_t *alloc, *last_alloc, *out_alloc;
     double* reduction;
     int32_t* err_word;
+    GainBasis basis;         // where the curves of unfinished rows are kept (note null: nobody asks for rows)
     // after the last row: what the next epoch finds cleared, the published statistics, and the host's mailbox
     void* zero;
     int zero_words;
@@ -334,6 +335,12 @@ __device__ __forceinline__ void store_alloc(const SelectArgs& a, int j, int core
 __device__ __forceinline__ void mail_rows(const SelectArgs& a, int j0, int j1) {
     if (a.mail_alloc)
         for (int j = j0 + threadIdx.x; j < j1; j += kThreads) a.mail_alloc[j] = a.alloc[j];
+}
+
+// Whether the launch leaves rows unfinished.
+template <bool kCurves>
+__device__ __forceinline__ void note_rows(const SelectArgs& a) {
+    if (a.basis.note) *a.basis.note = GainNote{kCurves && a.depth < a.cap ? 1 : 0, a.cap, a.T};
 }
 
 // A row's candidates, entries s .. s+c-1, for the block that ranks them.  The first of them carries the row's count.
@@ -654,10 +661,13 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     const SelectArgs& a = args.of(shard);
     const int j0 = min(block * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
     after_previous();
-    if (block == 0 && tid == 0 && a.stamps) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-        a.stamps[2] = (long long)t;
+    if (block == 0 && tid == 0) {
+        note_rows<kCurves>(a);
+        if (a.stamps) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            a.stamps[2] = (long long)t;
+        }
     }
     const bool resident = a.stride > 0;
     CurveTile tile;
@@ -688,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
                 const Curve c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
                 if (no_time) a.fit.status[j] = SLAQ_JOB_NO_TIME;
                 tile.put(tid, c, active);
+                if (a.depth < a.cap) keep_curve(a.basis, j, a.J, c, active ? c.kind : 3);
                 expo = active && c.kind == 1;
             }
             // Family II's rows last: the rows of a warp are then of one family, and only one of the two formulas is
@@ -913,6 +924,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
     if (tid == 0) sh.count = 0;
     after_previous();
     if (a.stamps) note_time(a.stamps + 2);
+    if (tid == 0) note_rows<kCurves>(a);
     if (kCurves && tid < a.J) {
         bool no_time = false;
         const bool active = a.count[tid] > 0;
@@ -1233,6 +1245,7 @@ static SelectArgs handle_args(slaq_handle* h, double epoch_seconds, long long wa
     a.out_alloc = d_out_alloc;
     a.reduction = h->reduction;
     a.err_word = h->err_word;
+    a.basis = h->basis;
     a.zero = h->scratch.zero;
     a.zero_words = (int)(h->scratch.zero_bytes / sizeof(u64));
     a.published = h->scratch.published;
