@@ -945,6 +945,8 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     if (const int dc = check_device(h)) return dc;
     const int rc = ensure_weights(h);
     if (rc) return rc;
+    if (only_allocate)   // the rows it reads may be those of the last epoch
+        if (const int rows = complete_gains(h)) return rows;
     const int64_t active = h->n_active, cap = h->max_cores;
     const int floor_units = C >= active ? 1 : 0;
     const int64_t usable = std::min<int64_t>(C, active * cap);

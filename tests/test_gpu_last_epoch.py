@@ -101,3 +101,30 @@ def test_gain_rows_after_a_captured_epoch():
             np.testing.assert_array_equal(got[key], want[key])
     a.close()
     b.close()
+
+
+def _definition(gain, C):
+    J, cap = gain.shape
+    floor = 1 if C >= J else 0
+    want = min(C, J * cap) - floor * J
+    order = np.argsort(-gain[:, floor:].ravel(), kind="stable")[:want]
+    return (floor + np.bincount(order // (cap - floor), minlength=J)).astype(np.int32)
+
+
+@pytest.mark.parametrize("change", [False, True])
+def test_allocate_only_reads_the_whole_rows_of_the_epoch(change):
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+    wl = make_workload(4, n_jobs=JOBS)
+    twin, s = make_scheduler(wl), make_scheduler(wl)
+    for h in (twin, s):
+        h.schedule(wl.epoch_seconds, 2 * JOBS)
+    gain = twin.get_predictions()["gain"]
+    if change:
+        _change(slaq, s, wl, "time law")
+    for C in (20 * JOBS, 40 * JOBS, 2 * JOBS, JOBS // 2):
+        alloc, _ = s.allocate_only(C)
+        np.testing.assert_array_equal(alloc, _definition(gain, C))
+    np.testing.assert_array_equal(s.get_predictions()["gain"], gain)
+    twin.close()
+    s.close()
