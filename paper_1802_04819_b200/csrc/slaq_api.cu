@@ -1317,6 +1317,8 @@ int slaq_schedule(slaq_t* h, double epoch_seconds, int64_t total_cores, int32_t*
 
 int slaq_set_gains(slaq_t* h, const double* gain) {
     if (!h || !gain) return SLAQ_E_ARG;
+    h->gain_partial = false;   // from here on the rows are the caller's
+    CK(cudaMemsetAsync(h->basis.note, 0, sizeof(GainNote), h->stream), "clear gain note");
     if (const int rc = pipe_to_device(h, {{h->gain, gain, sizeof(double) * (size_t)h->max_jobs * h->max_cores}})) return rc;
     CK(cudaStreamSynchronize(h->stream), "copy gains");
     return SLAQ_OK;

@@ -99,6 +99,10 @@ def test_gain_rows_after_a_captured_epoch():
         got, want = a.get_predictions(), b.get_predictions()
         for key in ("gain", "R", "params", "status"):
             np.testing.assert_array_equal(got[key], want[key])
+    # a table the caller sets afterwards is the table
+    gain = np.sort(np.random.default_rng(1).random((J, wl.max_cores_per_job)), 1)[:, ::-1].copy()
+    a.set_gains(gain)
+    np.testing.assert_array_equal(a.get_predictions()["gain"], gain)
     a.close()
     b.close()
 
@@ -127,4 +131,18 @@ def test_allocate_only_reads_the_whole_rows_of_the_epoch(change):
         np.testing.assert_array_equal(alloc, _definition(gain, C))
     np.testing.assert_array_equal(s.get_predictions()["gain"], gain)
     twin.close()
+    s.close()
+
+
+def test_rows_the_caller_sets_stay_after_an_epoch():
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+    wl = make_workload(4, n_jobs=JOBS)
+    gain = np.sort(np.random.default_rng(7).random((JOBS, wl.max_cores_per_job)), 1)[:, ::-1].copy()
+    s = make_scheduler(wl)
+    s.schedule(wl.epoch_seconds, 2 * JOBS)
+    s.set_gains(gain)
+    np.testing.assert_array_equal(s.get_predictions()["gain"], gain)
+    for C in (3 * JOBS, 30 * JOBS):
+        np.testing.assert_array_equal(s.allocate_only(C)[0], _definition(gain, C))
     s.close()
