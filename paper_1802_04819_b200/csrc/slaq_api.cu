@@ -953,12 +953,13 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     const int64_t want = usable - active * floor_units;
     cudaStream_t st = h->stream;
 
-    if (!h->scratch_clean) {
+    // A captured epoch clears its scratch itself: its replays cannot know what the handle did before them.
+    const bool capturing = is_capturing(h);
+    if (!h->scratch_clean || capturing) {
         CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
-        if (!is_capturing(h)) h->scratch_clean = true;
+        if (!capturing) h->scratch_clean = true;
     }
-    bool graph_ok = h->epoch_graph == 1;
-    if (graph_ok && is_capturing(h)) graph_ok = false;   // not while the caller captures this stream into a graph of its own
+    const bool graph_ok = h->epoch_graph == 1 && !capturing;   // not while the caller captures this stream into a graph of its own
     int launches = -1;
     h->last_epoch_was_graph = false;
     if (graph_ok) {
@@ -1020,7 +1021,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
     h->last_cores = usable;
     h->gain_partial = gains_in_selection(h, only_allocate) && !select_writes_whole_table(h, want);
-    h->epoch_captured = h->epoch_captured || is_capturing(h);
+    h->epoch_captured = h->epoch_captured || capturing;
     if (active > 0 && C < active) return SLAQ_W_OVERSUBSCRIBED;
     if (C > active * cap) return SLAQ_W_UNDERFILLED;
     return SLAQ_OK;

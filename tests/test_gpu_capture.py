@@ -1,0 +1,42 @@
+"""Calls on a handle whose stream the caller captures into a graph of its own."""
+
+import numpy as np
+import pytest
+
+from gpu_common import make_scheduler
+from workloads import make_workload
+
+pytestmark = pytest.mark.gpu
+
+
+# one block sorts the windows and the queue hands out more slots than the GPU has warps; the counting sort of many jobs
+@pytest.mark.parametrize("cfg,jobs", [(3, 6000), (4, 60000)])
+def test_a_captured_epoch_clears_its_scratch_itself(cfg, jobs):
+    """Between two replays the handle makes calls that leave the scratch of an epoch as they used it."""
+    import torch
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+    wl = make_workload(cfg, n_jobs=jobs)
+    J, C = wl.n_jobs, wl.total_cores
+    last = wl.losses[wl.offsets[1:] - 1]
+    ids = np.arange(J, dtype=np.int32)
+    stream = torch.cuda.Stream()
+    a, b = make_scheduler(wl), make_scheduler(wl)
+    a.set_stream(stream)
+    out = torch.zeros(J, dtype=torch.int32, device="cuda")
+    a.schedule_device(wl.epoch_seconds, C, out)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        a.schedule_device(wl.epoch_seconds, C, out)
+    for step in range(3):
+        a.shard_predict(wl.epoch_seconds, True)
+        for s in (a, b):
+            s.append_losses(ids, (0.96 - 0.02 * step) * last)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        stream.synchronize()
+        ref, _ = b.schedule(wl.epoch_seconds, C)
+        np.testing.assert_array_equal(out.cpu().numpy(), ref)
+    a.close()
+    b.close()
