@@ -1013,8 +1013,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
             return SLAQ_E_CUDA;
         }
     }
-    h->have_epoch = h->stats_published = true;
-    h->last_epoch_stamped = !h->last_epoch_was_graph;
+    h->have_epoch = true;
     h->last_gain_launch = !only_allocate && !gains_in_selection(h, only_allocate);
     h->last_fit_launch = !only_allocate;
     h->last_launches = launches;
@@ -1393,7 +1392,7 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
     for (int32_t s = 0; s < n; ++s) {
         slaq_t* const g = handles[s];
         g->scratch_clean = true;
-        g->have_epoch = g->stats_published = g->last_epoch_stamped = g->last_fit_launch = true;
+        g->have_epoch = g->last_fit_launch = true;
         g->last_gain_launch = false;
         g->last_epoch_was_graph = false;
         g->last_launches += s == 0 ? k : 0;
@@ -1437,10 +1436,13 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     cudaStream_t st = h->stream;
     int launches = 0, k;
     h->shard_first_unit = with_floor ? 2 : 1;
-    h->last_epoch_was_graph = h->last_epoch_stamped = false;
+    h->last_epoch_was_graph = false;
     CK(cudaMemsetAsync(h->scratch.hist, 0, sizeof(unsigned long long) * kRadixPasses * kRadixBins, st), "clear scratch");
     CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
-    h->scratch_clean = h->stats_published = false;   // these steps leave their counts where they were added up
+    // These steps leave their counts where they were added up; an end time of zero says so, until an epoch publishes its own
+    // (one that the caller's graph replays too).
+    CK(cudaMemsetAsync(h->scratch.stamps + 3, 0, sizeof(long long), st), "clear end time");
+    h->scratch_clean = false;
     CK(cudaEventRecord(h->ev[0], st), "event");
     if ((k = launch_fit(h, st, h->sm_count)) < 0) return SLAQ_E_CUDA;
     launches += k;
@@ -1864,13 +1866,29 @@ int slaq_import_state(slaq_t* h, const void* blob_in, size_t bytes) {
     return SLAQ_OK;
 }
 
+namespace {
+
+// The last epoch's counts, in [15] the bits of its threshold, and from [16] on the times its launches noted; the latter
+// are zero at the end of the sharded steps, whose counts lie where they were added up.
+int read_counters(slaq_handle* h, long long (&counters)[20]) {
+    CK(cudaMemcpyAsync(counters, h->scratch.published, sizeof counters, cudaMemcpyDeviceToHost, h->stream), "copy counters");
+    CK(cudaStreamSynchronize(h->stream), "copy counters");
+    if (counters[19] != 0) return SLAQ_OK;
+    SelectState sel;
+    CK(cudaMemcpyAsync(counters, h->scratch.counters, sizeof(long long) * 16, cudaMemcpyDeviceToHost, h->stream), "copy counters");
+    CK(cudaMemcpyAsync(&sel, h->scratch.sel, sizeof sel, cudaMemcpyDeviceToHost, h->stream), "copy selection state");
+    CK(cudaStreamSynchronize(h->stream), "copy counters");
+    counters[15] = (long long)sel.prefix;
+    return SLAQ_OK;
+}
+
+}  // namespace
+
 int slaq_get_fit_phase_cycles(slaq_t* h, int64_t* out_cycles) {
     if (!h || !out_cycles) return SLAQ_E_ARG;
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
-    long long counters[16];
-    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters, sizeof counters,
-                       cudaMemcpyDeviceToHost, h->stream), "copy counters");
-    CK(cudaStreamSynchronize(h->stream), "copy phase cycles");
+    long long counters[20];
+    if (const int rc = read_counters(h, counters)) return rc;
     for (int i = 0; i < 6; ++i) out_cycles[i] = counters[8 + i];
     return SLAQ_OK;
 }
@@ -1880,13 +1898,8 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
     if (!h->have_epoch) return fail(h, SLAQ_E_ARG, "no epoch has been scheduled yet");
     std::memset(out, 0, sizeof *out);
     long long counters[20];
-    SelectState sel;
-    CK(cudaMemcpyAsync(counters, h->stats_published ? h->scratch.published : h->scratch.counters,
-                       sizeof(long long) * (h->stats_published ? 20 : 16), cudaMemcpyDeviceToHost, h->stream), "copy counters");
-    if (!h->stats_published) CK(cudaMemcpyAsync(&sel, h->scratch.sel, sizeof sel, cudaMemcpyDeviceToHost, h->stream), "copy selection state");
-    CK(cudaStreamSynchronize(h->stream), "copy statistics");
-    if (h->stats_published) sel.prefix = (unsigned long long)counters[15];
-    if (h->last_epoch_stamped) {
+    if (const int rc = read_counters(h, counters)) return rc;
+    if (counters[19] != 0 && !h->last_epoch_was_graph) {
         const long long* const at = counters + 16;
         auto ms = [](long long ns) { return (float)((double)(ns > 0 ? ns : 0) * 1e-6); };
         const long long first = h->last_fit_launch ? at[0] : at[2], gains = h->last_gain_launch ? at[1] : at[2];
@@ -1915,7 +1928,7 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
     out->cores_handed_out = counters[6];
     out->tie_units = counters[7];
     double tau = 0.0;
-    if (sel.prefix != ~0ull) std::memcpy(&tau, &sel.prefix, sizeof tau);
+    if ((unsigned long long)counters[15] != ~0ull) std::memcpy(&tau, &counters[15], sizeof tau);
     out->threshold = tau;
     return SLAQ_OK;
 }

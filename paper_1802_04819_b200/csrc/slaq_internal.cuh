@@ -126,7 +126,7 @@ struct Scratch {
     SelectState* sel;
     long long* counters;             // [16] statistics accumulated by kernels during an epoch
     long long* published;            // [16] those of the last finished epoch
-    long long* stamps;               // [4] device clock (ns) when its first kernel, the gain kernel and the selection started, and at its end
+    long long* stamps;               // [4] behind `published`: device clock (ns) when its first kernel, the gain kernel and the selection started, and at its end
     unsigned int* append_ticket;     // blocks of a reporting kernel that are done
     int32_t* load_flag;              // a bulk load brought a loss that is not finite
     size_t zero_bytes;
@@ -198,7 +198,6 @@ struct slaq_handle {
     uint32_t call_seq = 0;            // number of the last call that reports to the mailbox
     uint32_t mail_seq = 0;            // number of the append that reads its entries from the mailbox's arrays
     bool mail_in_use = false;         // and whether it may still be reading them
-    bool stats_published = true;      // the last epoch's statistics are in scratch.published (sharded steps: where they are counted)
     bool scratch_clean = false;       // the last epoch left its scratch cleared for the next one
     cudaEvent_t ev[4] = {};               // stage boundaries of the sharded steps and of replayed graphs
     cudaEvent_t order_ev[2] = {};         // fork and join of fits that run beside one another
@@ -228,7 +227,6 @@ struct slaq_handle {
     cudaStream_t side_stream = nullptr;   // the fit of a handle that is scheduled together with others
     int32_t graph_launches = 0;
     bool last_epoch_was_graph = false;
-    bool last_epoch_stamped = false;      // its stage times are in scratch.stamps, not between the events
     bool last_gain_launch = false;        // it had a gain kernel of its own
     bool last_fit_launch = false;         // and a fit
     std::string err;

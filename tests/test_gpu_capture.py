@@ -38,5 +38,9 @@ def test_a_captured_epoch_clears_its_scratch_itself(cfg, jobs):
         stream.synchronize()
         ref, _ = b.schedule(wl.epoch_seconds, C)
         np.testing.assert_array_equal(out.cpu().numpy(), ref)
+        mine, theirs = a.get_stats(), b.get_stats()       # the statistics are the replay's
+        for key in ("points", "model_sweeps", "fitted_jobs", "cores_handed_out", "tie_units", "threshold"):
+            assert getattr(mine, key) == getattr(theirs, key)
+        assert mine.ms_total > 0.0 and mine.ms_fit > 0.0
     a.close()
     b.close()
