@@ -975,11 +975,13 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
 
 // A block per job, for clusters with fewer jobs than the GPU has sub-partitions for: each family has warps of its own
 // (see Team).  The chain of a trial is shorter than in one warp that does both (fit of 8 windows of 20: 34 -> 28 us, of 160
-// of 40: 38 -> 32, of 8 of 1,000 with four warps per family: 82 -> 56).
-template <bool kWarm>
+// of 40: 38 -> 32, of 8 of 1,000 with four warps per family: 82 -> 56).  kListed: the blocks take the jobs of the work list, for
+// handles with many more ids (40 windows of up to 900 among 4,000 ids: 83 -> 61 with the sort).
+template <bool kWarm, bool kListed>
 __global__ void __launch_bounds__(kTeamWarps * 32)
-fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, FitClasses cls, int parts, int lm_trials,
-                int min_fit_points, long long* counters, long long* stamp, int32_t* err_word) {
+fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
+                const int32_t* __restrict__ start, FitClasses cls, int parts, int lm_trials, int min_fit_points,
+                long long* counters, long long* stamp, int32_t* err_word) {
     extern __shared__ double smem[];
     __shared__ double exchange[2 * 2 * 4 * 16];
     __shared__ unsigned long long tally[6];
@@ -1000,8 +1002,18 @@ fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab,
     team.exchange = exchange;
     Phases phases = {};
     SLAQ_PHASES_START(phases);
-    fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem,
-                              g_wtab + cls.h_max, smem + cls.h_max + (size_t)warp * cls.slice, tally, lane, phases, err_word, team);
+    double* const slice = smem + cls.h_max + (size_t)warp * cls.slice;
+    if constexpr (kListed) {
+        const int jobs = start[0];   // the active ones, at the front of the list
+        for (int place = blockIdx.x; place < jobs; place += gridDim.x) {
+            fit_slot<kWarm, 32, true>(job, fit, order, start, cls, 0, place, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+                                      tally, lane, phases, err_word, team);
+            __syncthreads();   // the exchanged results are read before the next job's are written
+        }
+    } else {
+        fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+                                  tally, lane, phases, err_word, team);
+    }
     if (warp == 0 && lane < 6 && tally[lane]) {
         atomicAdd((unsigned long long*)&counters[lane < 2 ? lane : lane == 5 ? 14 : lane + 1], tally[lane]);
         if (lane == 2 || lane == 3) atomicAdd((unsigned long long*)&counters[2], tally[lane]);
@@ -1249,18 +1261,20 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 }  // namespace
 
 using FitKernel = decltype(&fit_kernel<false, 0>);
-using FitTeamKernel = decltype(&fit_team_kernel<false>);
+using FitTeamKernel = decltype(&fit_team_kernel<false, false>);
 static FitKernel const kFitKernels[2][6] = {
     {fit_kernel<false, 0>, fit_kernel<false, 2>, fit_kernel<false, 4>, fit_kernel<false, 8>, fit_kernel<false, 16>, fit_kernel<false, 32>},
     {fit_kernel<true, 0>, fit_kernel<true, 2>, fit_kernel<true, 4>, fit_kernel<true, 8>, fit_kernel<true, 16>, fit_kernel<true, 32>}};
 
-static FitTeamKernel const kFitTeamKernels[2] = {fit_team_kernel<false>, fit_team_kernel<true>};
+static FitTeamKernel const kFitTeamKernels[2][2] = {{fit_team_kernel<false, false>, fit_team_kernel<false, true>},
+                                                    {fit_team_kernel<true, false>, fit_team_kernel<true, true>}};
 
 int fit_setup() {
     bool ok = true;
-    for (FitTeamKernel k : kFitTeamKernels)
-        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmem) == cudaSuccess &&
-             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    for (const auto& row : kFitTeamKernels)
+        for (FitTeamKernel k : row)
+            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmem) == cudaSuccess &&
+                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
     for (const auto& row : kFitKernels)
         for (FitKernel k : row)
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
@@ -1310,13 +1324,14 @@ int fit_least_lanes(const slaq_handle* h) {
     return best;
 }
 
-// Warps per family of a job's team; 0: no teams.  With a warp per sub-partition at most, a lane is left four rows of the longest
+// Warps per family of a job's team; 0: no teams.  A question of the cluster's active jobs and the windows alone, which every shard
+// answers alike, whatever its capacity: several warps add in another order than one, and one in another than a part of one.  With a warp per sub-partition at most, a lane is left four rows of the longest
 // window; two warps share a sub-partition without loss where a lane would have twelve rows or more (140 windows of up to
 // 1,000: 61 -> 58 us, but 200 of up to 300: 44 -> 45), and teams of one warp per family up to sixteen rows (580 windows of 20: 38 ->
 // 35 us, but 300 of 1,000: 84 -> 87).
 static int fit_team_parts(const slaq_handle* h) {
-    const long long warps = 4LL * h->sm_count, jobs = std::max(1LL, jobs_for_lanes(h));
-    if (h->max_jobs > 4 * h->sm_count || 2 * jobs > (h->max_hist > 512 ? warps : 2 * warps)) return 0;
+    const long long warps = 4LL * h->sm_count, jobs = std::max({1LL, jobs_for_lanes(h), (long long)h->n_active});
+    if (2 * jobs > (h->max_hist > 512 ? warps : 2 * warps)) return 0;
     int parts = 1;
     while (parts < kTeamWarps / 2 && ((4 * parts * jobs <= warps && h->max_hist > 128 * parts) ||
                                       (4 * parts * jobs <= 2 * warps && h->max_hist > 384 * parts)))
@@ -1325,19 +1340,48 @@ static int fit_team_parts(const slaq_handle* h) {
     return parts;
 }
 
+// The work list: job ids, longest window first.  Up to kOneBlockSort jobs one block sorts (one launch of about 5 us
+// instead of three of 3 to 4 us each), beyond that a block per 2048 jobs.
+static cudaError_t launch_sort(slaq_handle* h, cudaStream_t st, int* launches) {
+    const int J = h->max_jobs, Hmax = h->max_hist;
+    const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
+    long long* const stamp = h->scratch.stamps;
+    if (J <= kOneBlockSort) {
+        *launches += 1;
+        return launch_behind(length_sort_kernel, 1, 1024, 2 * bins, st, h->job.count, J, Hmax, h->scratch.start, h->scratch.order, stamp,
+                             h->err_word);
+    }
+    const int sort_blocks = (J + kSortJobsPerBlock - 1) / kSortJobsPerBlock;
+    *launches += 3;
+    cudaError_t e = launch_behind(length_count_kernel, sort_blocks, kSortThreads, bins, st, h->job.count, J, Hmax, h->scratch.bucket, stamp);
+    if (e == cudaSuccess) e = launch_behind(length_scan_kernel, 1, 1024, 0, st, h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
+    if (e == cudaSuccess)
+        e = launch_behind(length_scatter_kernel, sort_blocks, kSortThreads, 2 * bins, st, h->job.count, J, Hmax, h->scratch.cursor,
+                          h->scratch.order, h->err_word);
+    return e;
+}
+
 int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     int launches = 0;
-    if (const int parts = fit_team_parts(h)) {
+    const int parts = fit_team_parts(h);
+    // A block for each id is for handles with few of them: the empty ones cost 8 jobs among 592 ids 10 us.  A family with one
+    // warp adds its sums in the order in which one warp does both, so that teams of one are left to the other kernel there.
+    const bool many_ids = J > 4 * h->sm_count;
+    if (parts > 1 || (parts == 1 && !many_ids)) {
         FitClasses all = {};
         all.n = 1;
         all.h_hi[0] = all.h_max = Hmax;
         all.L[0] = 32;
         all.slice = team_slice(h);
-        const cudaError_t e = launch_behind(kFitTeamKernels[h->warm_start ? 1 : 0], J, 64 * parts, team_smem(h, parts), st, h->job, h->fit,
-                                            h->wtab, all, parts, h->lm_trials, h->min_fit_points, h->scratch.counters, h->scratch.stamps,
-                                            h->err_word);
-        if (e == cudaSuccess) return 1;
+        // the list's blocks: one per job that is active now (a graph of the caller's may meet more later)
+        const int blocks = many_ids ? std::max(1, h->n_active) : J;
+        cudaError_t e = many_ids ? launch_sort(h, st, &launches) : cudaSuccess;
+        if (e == cudaSuccess)
+            e = launch_behind(kFitTeamKernels[h->warm_start ? 1 : 0][many_ids ? 1 : 0], blocks, 64 * parts, team_smem(h, parts), st, h->job,
+                              h->fit, h->wtab, h->scratch.order, h->scratch.start, all, parts, h->lm_trials, h->min_fit_points,
+                              h->scratch.counters, many_ids ? nullptr : h->scratch.stamps, h->err_word);
+        if (e == cudaSuccess) return launches + 1;
         h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
         return -1;
     }
@@ -1348,7 +1392,7 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     cls.n = 0;
     cls.h_max = Hmax;
     cls.slice = fit_slice(h);
-    const int L_min = fit_least_lanes(h);
+    const int L_min = parts == 1 ? 32 : fit_least_lanes(h);
     int h_hi = Hmax;
     for (int L = 32; L >= L_min && h_hi > 0; L >>= 1) {
         const int h_lo = L > L_min ? std::max(rows_at(cls.slice, L / 2), 0) * (L / 2) : 0;
@@ -1360,26 +1404,9 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         h_hi = h_lo;
     }
     for (int c = cls.n; c < kMaxFitClasses; ++c) cls.h_lo[c] = cls.h_hi[c] = 0, cls.L[c] = 32;
-    // The work list: job ids, longest window first.  A job per warp of the GPU and no more: every job starts at once,
-    // so their order means nothing and none is made.  Up to kOneBlockSort jobs one block sorts (one launch of about 5 us
-    // instead of three of 3 to 4 us each), beyond that a block per 2048 jobs.
+    // A job per warp of the GPU and no more: every job starts at once, so their order means nothing and none is made.
     const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * kMaxWarpsPerBlock;
-    const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
-    long long* const stamp = h->scratch.stamps;
-    cudaError_t e = cudaSuccess;
-    if (in_order) {
-    } else if (J <= kOneBlockSort) {
-        e = launch_behind(length_sort_kernel, 1, 1024, 2 * bins, st, h->job.count, J, Hmax, h->scratch.start, h->scratch.order, stamp, h->err_word);
-        launches += 1;
-    } else {
-        const int sort_blocks = (J + kSortJobsPerBlock - 1) / kSortJobsPerBlock;
-        e = launch_behind(length_count_kernel, sort_blocks, kSortThreads, bins, st, h->job.count, J, Hmax, h->scratch.bucket, stamp);
-        if (e == cudaSuccess) e = launch_behind(length_scan_kernel, 1, 1024, 0, st, h->scratch.bucket, Hmax, h->scratch.start, h->scratch.cursor);
-        if (e == cudaSuccess)
-            e = launch_behind(length_scatter_kernel, sort_blocks, kSortThreads, 2 * bins, st, h->job.count, J, Hmax, h->scratch.cursor,
-                              h->scratch.order, h->err_word);
-        launches += 3;
-    }
+    cudaError_t e = in_order ? cudaSuccess : launch_sort(h, st, &launches);
     // One block per SM: its registers and shared memory fill one.  Where there are fewer slots than warps every SM gets
     // its share of them.
     const long long slots = ((long long)J * cls.L[0] + 31) / 32;   // at most
@@ -1397,7 +1424,7 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     if (e == cudaSuccess)
         e = launch_behind(kernel, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
                           h->scratch.start, cls, h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase, h->scratch.counters,
-                          in_order ? stamp : nullptr, h->err_word);
+                          in_order ? h->scratch.stamps : nullptr, h->err_word);
     ++launches;
     if (e != cudaSuccess) {
         h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
