@@ -954,11 +954,9 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     cudaStream_t st = h->stream;
 
     // A captured epoch clears its scratch itself: its replays cannot know what the handle did before them.
-    const bool capturing = is_capturing(h);
-    if (!h->scratch_clean || capturing) {
-        CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
-        if (!capturing) h->scratch_clean = true;
-    }
+    const bool capturing = is_capturing(h), was_clean = h->scratch_clean;
+    if (!was_clean || capturing) CK(cudaMemsetAsync(h->scratch.zero, 0, h->scratch.zero_bytes, st), "clear scratch");
+    h->scratch_clean = false;   // until the last launch, which leaves it cleared, is queued
     const bool graph_ok = h->epoch_graph == 1 && !capturing;   // not while the caller captures this stream into a graph of its own
     int launches = -1;
     h->last_epoch_was_graph = false;
@@ -1013,6 +1011,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
             return SLAQ_E_CUDA;
         }
     }
+    h->scratch_clean = capturing ? was_clean : true;
     h->have_epoch = true;
     h->last_gain_launch = !only_allocate && !gains_in_selection(h, only_allocate);
     h->last_fit_launch = !only_allocate;

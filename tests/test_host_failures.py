@@ -1,0 +1,55 @@
+"""Host code of the library where something fails: built against a CUDA runtime that only pretends (host_fakes/), so that launches
+and allocations fail when a test says so and no GPU is needed."""
+
+import ctypes
+import shutil
+import subprocess
+from ctypes import byref, c_double, c_int, c_int32, c_int64, c_long, c_size_t, c_void_p
+from pathlib import Path
+
+import pytest
+
+ROOT = Path(__file__).resolve().parent.parent
+CSRC = ROOT / "paper_1802_04819_b200" / "csrc"
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    where = tmp_path_factory.mktemp("fake")
+    inc = ["-I", str(ROOT / "include"), "-I", str(CSRC), "-I", str(Path(shutil.which("nvcc")).resolve().parent.parent / "include")]
+    fakes = ROOT / "tests" / "host_fakes"
+    objects = []
+    for source in (CSRC / "slaq_api.cu", CSRC / "slaq_pipe.cu", fakes / "fake_launches.cu", fakes / "fake_cuda.cpp"):
+        objects.append(str(where / (source.stem + ".o")))
+        cuda = ["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-cudart", "none", "-Xcompiler"]
+        compiler = cuda if source.suffix == ".cu" else ["g++"]
+        subprocess.run([*compiler, "-fPIC", "-O1", "-std=c++17", *inc, "-c", str(source), "-o", objects[-1]], check=True)
+    so = where / "libfake.so"
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", str(so), *objects, "-lpthread"], check=True)
+    return ctypes.CDLL(str(so))
+
+
+def _handle(lib, jobs=8):
+    h = c_void_p()
+    assert lib.slaq_create_in(None, c_size_t(0), c_int32(jobs), c_int32(16), c_int32(4), byref(h)) == 0
+    return h
+
+
+def _clears(lib):
+    return c_size_t.in_dll(lib, "fake_clears").value
+
+
+def _epoch(lib, h):
+    return lib.slaq_schedule_device(h, c_double(1.0), c_int64(8), None)
+
+
+def test_the_epoch_after_one_that_could_not_be_launched_clears_its_scratch(lib):
+    h = _handle(lib)
+    before = _clears(lib)
+    assert _epoch(lib, h) == 2 and _clears(lib) == before          # no active jobs: underfilled; nothing to clear
+    c_int.in_dll(lib, "fake_fail_select").value = 1
+    assert _epoch(lib, h) == -5                                    # the fit was queued, the selection was not
+    assert _epoch(lib, h) == 2
+    assert _clears(lib) == before + 1
+    assert _epoch(lib, h) == 2 and _clears(lib) == before + 1
+    lib.slaq_destroy(h)
