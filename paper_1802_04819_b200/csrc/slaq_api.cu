@@ -1358,7 +1358,7 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
         slaq_t* const g = handles[s];
         if (const int rc = ensure_weights(g)) return fail(h, rc, g->err);
         if (!g->scratch_clean) CK(cudaMemsetAsync(g->scratch.zero, 0, g->scratch.zero_bytes, st), "clear scratch");
-        g->scratch_clean = false;   // until the last launch is queued
+        g->scratch_clean = false;   // until the last launch has reported its end
     }
     if (n > 1) CK(cudaEventRecord(h->order_event(0), st), "event");
     // The fits run beside one another.  Few jobs: each gets SMs in proportion to its jobs, so that no fit waits for another's
@@ -1390,7 +1390,6 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
     if (k < 0) return SLAQ_E_CUDA;
     for (int32_t s = 0; s < n; ++s) {
         slaq_t* const g = handles[s];
-        g->scratch_clean = true;
         g->have_epoch = g->last_fit_launch = true;
         g->last_gain_launch = false;
         g->last_epoch_was_graph = false;
@@ -1410,9 +1409,15 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
     for (int32_t s = 0; s < n; ++s)
         if (handles[s]->max_jobs <= handles[s]->mailbox_jobs)
             std::memcpy(out_alloc[s], handles[s]->mail_alloc(), sizeof(int32_t) * (size_t)handles[s]->max_jobs);
-    if (h->mailbox->err)
-        for (int32_t s = 0; s < n; ++s)
-            if (const int ec = check_device_errors(handles[s])) return fail(h, ec, handles[s]->err);
+    if (h->mailbox->err) {   // one of the handles' words: the first says what, and all start their next epoch with a clear
+        int bad = SLAQ_OK;
+        for (int32_t s = 0; s < n; ++s) {
+            const int ec = check_device_errors(handles[s]);
+            if (ec && !bad) bad = fail(h, ec, std::string(handles[s]->err));
+        }
+        if (bad) return bad;
+    }
+    for (int32_t s = 0; s < n; ++s) handles[s]->scratch_clean = true;   // the launch left it cleared
     if (active > 0 && total_cores < active) return SLAQ_W_OVERSUBSCRIBED;
     if (total_cores > active * cap) return SLAQ_W_UNDERFILLED;
     return SLAQ_OK;

@@ -53,3 +53,28 @@ def test_the_epoch_after_one_that_could_not_be_launched_clears_its_scratch(lib):
     assert _clears(lib) == before + 1
     assert _epoch(lib, h) == 2 and _clears(lib) == before + 1
     lib.slaq_destroy(h)
+
+
+@pytest.mark.parametrize("failure", ["launch", "report"])
+def test_every_handle_of_a_group_that_failed_clears_its_scratch(lib, failure):
+    hs = [_handle(lib) for _ in range(3)]
+    rows = [(c_int32 * 8)() for _ in hs]
+    handles, out = (c_void_p * 3)(*[h.value for h in hs]), (c_void_p * 3)(*[ctypes.addressof(r) for r in rows])
+
+    def group():
+        return lib.slaq_schedule_group(handles, c_int32(3), c_double(1.0), c_int64(24), out)
+
+    assert group() == 2
+    before = _clears(lib)
+    assert group() == 2 and _clears(lib) == before
+    if failure == "launch":
+        c_int.in_dll(lib, "fake_fail_select").value = 1
+    else:
+        c_int.in_dll(lib, "fake_err_word").value = 1               # the launch ran, and some block found an inconsistency
+    assert group() == -5
+    before = _clears(lib)
+    for h in hs:                                                   # each member's next epoch, alone
+        assert _epoch(lib, h) == 2
+    assert _clears(lib) == before + 3
+    for h in hs:
+        lib.slaq_destroy(h)
