@@ -649,6 +649,14 @@ __device__ void finish_epoch(const Args& args) {
     }
 }
 
+// A block whose wait at a barrier ran out ends here (the error word says so already).  Blocks that were let through meet the next
+// barrier without it and end here too, so all of them arrive, and the last one leaves the scratch as the next epoch expects it:
+// nobody clears it between two epochs that are queued one behind the other.
+template <class Args>
+__device__ void give_up(const Args& args, const SelectArgs& a, Shared& sh) {
+    if (arrive_last(a, sh)) finish_epoch(args);
+}
+
 // kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
 // were continued); otherwise the table is read.
 template <bool kCurves, class Args>
@@ -749,7 +757,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     __syncthreads();
     flush_first(sh, a.gl->coarse, a.gl->fine);
     arrived += gridDim.x;
-    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
+    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
+        give_up(args, a, sh);
+        return;
+    }
     if (a.want > 0) {
         if (tid < 32) pick_first<false>(a.gl, (u64)a.want, &sh.iv);
     } else if (tid == 0) {
@@ -810,7 +821,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         __syncthreads();
         flush_first(sh, a.gl->coarse_more, a.gl->fine_more);
         arrived += gridDim.x;
-        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
+            give_up(args, a, sh);
+            return;
+        }
         if (tid < 32) pick_first<true>(a.gl, (u64)a.want, &sh.iv);
         __syncthreads();
     }
@@ -889,7 +903,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     } else {
         __syncthreads();
         const int next = narrow_on_the_grid(a, shard, args.of(0).sel, sh, j0, j1, arrived);
-        if (next < 0) return;
+        if (next < 0) {
+            give_up(args, a, sh);
+            return;
+        }
         mail_rows(a, j0, j1);   // rows with candidates that are still to be ranked are written again after that
         if (next == 0) {
             if (arrive_last(a, sh)) finish_epoch(args);
