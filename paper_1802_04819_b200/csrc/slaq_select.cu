@@ -337,7 +337,7 @@ __device__ __forceinline__ void mail_rows(const SelectArgs& a, int j0, int j1) {
         for (int j = j0 + threadIdx.x; j < j1; j += kThreads) a.mail_alloc[j] = a.alloc[j];
 }
 
-// Whether the launch leaves rows unfinished.
+// Whether the launch leaves rows unfinished: written at its end, behind the report to the host, which does not wait for it.
 template <bool kCurves>
 __device__ __forceinline__ void note_rows(const SelectArgs& a) {
     if (a.basis.note) *a.basis.note = GainNote{kCurves && a.depth < a.cap ? 1 : 0, a.cap, a.T};
@@ -616,7 +616,7 @@ __device__ bool arrive_last(const SelectArgs& a, Shared& sh) {
 }
 
 // The last block, after everything else: publish the statistics, tell the host, clear the scratch for the next epoch.
-template <class Args>
+template <bool kCurves, class Args>
 __device__ void finish_epoch(const Args& args) {
     const int tid = threadIdx.x;
     __syncthreads();
@@ -639,6 +639,7 @@ __device__ void finish_epoch(const Args& args) {
     } else if (tid < 32 + 16 * args.shards()) {
         const int i = tid & 15;
         const SelectArgs& a = args.of((tid - 32) >> 4);
+        if (i == 0) note_rows<kCurves>(a);
         if (a.published) a.published[i] = i == 15 ? (long long)__ldcg(&first.sel->prefix) : __ldcg(&a.counters[i]);
     }
     __syncthreads();
@@ -652,9 +653,9 @@ __device__ void finish_epoch(const Args& args) {
 // A block whose wait at a barrier ran out ends here (the error word says so already).  Blocks that were let through meet the next
 // barrier without it and end here too, so all of them arrive, and the last one leaves the scratch as the next epoch expects it:
 // nobody clears it between two epochs that are queued one behind the other.
-template <class Args>
+template <bool kCurves, class Args>
 __device__ void give_up(const Args& args, const SelectArgs& a, Shared& sh) {
-    if (arrive_last(a, sh)) finish_epoch(args);
+    if (arrive_last(a, sh)) finish_epoch<kCurves>(args);
 }
 
 // kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
@@ -669,13 +670,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     const SelectArgs& a = args.of(shard);
     const int j0 = min(block * a.rows, a.J), j1 = min(j0 + a.rows, a.J);
     after_previous();
-    if (block == 0 && tid == 0) {
-        note_rows<kCurves>(a);
-        if (a.stamps) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            a.stamps[2] = (long long)t;
-        }
+    if (block == 0 && tid == 0 && a.stamps) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        a.stamps[2] = (long long)t;
     }
     const bool resident = a.stride > 0;
     CurveTile tile;
@@ -758,7 +756,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     flush_first(sh, a.gl->coarse, a.gl->fine);
     arrived += gridDim.x;
     if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
-        give_up(args, a, sh);
+        give_up<kCurves>(args, a, sh);
         return;
     }
     if (a.want > 0) {
@@ -822,7 +820,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         flush_first(sh, a.gl->coarse_more, a.gl->fine_more);
         arrived += gridDim.x;
         if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
-            give_up(args, a, sh);
+            give_up<kCurves>(args, a, sh);
             return;
         }
         if (tid < 32) pick_first<true>(a.gl, (u64)a.want, &sh.iv);
@@ -904,12 +902,12 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         __syncthreads();
         const int next = narrow_on_the_grid(a, shard, args.of(0).sel, sh, j0, j1, arrived);
         if (next < 0) {
-            give_up(args, a, sh);
+            give_up<kCurves>(args, a, sh);
             return;
         }
         mail_rows(a, j0, j1);   // rows with candidates that are still to be ranked are written again after that
         if (next == 0) {
-            if (arrive_last(a, sh)) finish_epoch(args);
+            if (arrive_last(a, sh)) finish_epoch<kCurves>(args);
             return;
         }
     }
@@ -918,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     if (!arrive_last(a, sh)) return;
     if (sh.iv.n > 0) finish_candidates(args, sh);
     else if (tid == 0) args.of(0).sel->prefix = ~0ull;
-    finish_epoch(args);
+    finish_epoch<kCurves>(args);
 }
 
 // Few gains: one block does everything in shared memory, with no grid barrier and nothing but results in global memory.
@@ -941,7 +939,6 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
     if (tid == 0) sh.count = 0;
     after_previous();
     if (a.stamps) note_time(a.stamps + 2);
-    if (tid == 0) note_rows<kCurves>(a);
     if (kCurves && tid < a.J) {
         bool no_time = false;
         const bool active = a.count[tid] > 0;
@@ -1146,6 +1143,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
     if (warp == 1) {
         const unsigned int all = __reduce_add_sync(kFull, sh.hist[2 * lane]), tied = __reduce_add_sync(kFull, sh.hist[2 * lane + 1]);
         if (lane == 0) a.sel->prefix = tau;
+        if (lane == 16) note_rows<kCurves>(a);
         if (lane < 16) {
             const long long v = lane == 6 ? all : lane == 7 ? tied : lane == 15 ? (long long)tau : __ldcg(&a.counters[lane]);
             if (a.published) a.published[lane] = v;
