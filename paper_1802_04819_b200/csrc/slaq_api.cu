@@ -468,6 +468,14 @@ int check_device(slaq_handle* h) {
     return SLAQ_OK;
 }
 
+// Whether the caller captures the handle's stream into a graph (or the query fails: then it is treated as if).
+bool is_capturing(slaq_handle* h) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Mark the listed ids with a new stamp.
 void stamp_ids(slaq_handle* h, int32_t n, const int32_t* ids) {
     if (++h->stamp_epoch == 0) {
@@ -736,6 +744,8 @@ int do_append(slaq_handle* h, int32_t n, const int32_t* ids, const double* losse
     }
     if (bad) return bad;   // the state is untouched
     if (mailed) {
+        // nobody waits for this launch, so nothing else would notice that it is only recorded
+        if (is_capturing(h)) return fail(h, SLAQ_E_CUDA, "append: the handle's stream is being captured");
         if (const int rc = mail_arrays_free(h)) return rc;
         std::memcpy(h->mail_ids(), ids, sizeof(int32_t) * n);
         std::memcpy(h->mail_losses(), losses, sizeof(double) * n);
@@ -889,14 +899,6 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
 // whole rows, which the gain kernel writes first.
 bool gains_in_selection(const slaq_handle* h, bool only_allocate) {
     return !only_allocate && !h->gain_envelope && h->n_hinted == 0;
-}
-
-// Whether the caller captures the handle's stream into a graph (or the query fails: then it is treated as if).
-bool is_capturing(slaq_handle* h) {
-    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
-    cudaGetLastError();
-    return true;
 }
 
 // h->gain holds the whole rows of the last epoch afterwards.

@@ -44,3 +44,36 @@ def test_a_captured_epoch_clears_its_scratch_itself(cfg, jobs):
         assert mine.ms_total > 0.0 and mine.ms_fit > 0.0
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("jobs", [8, 5000])
+def test_an_append_from_host_arrays_is_refused_under_capture(jobs):
+    """It would be applied by the replays and not by the call, from arrays the caller may reuse."""
+    import torch
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+    wl = make_workload(2, n_jobs=jobs)
+    ids = np.arange(jobs, dtype=np.int32)
+    last = wl.losses[wl.offsets[1:] - 1]
+    stream = torch.cuda.Stream()
+    a, b = make_scheduler(wl), make_scheduler(wl)
+    a.set_stream(stream)
+    graph = torch.cuda.CUDAGraph()
+    refused = None
+    try:
+        with torch.cuda.graph(graph, stream=stream):
+            try:
+                a.append_losses(ids, 0.5 * last)
+            except slaq.SlaqError as e:
+                refused = e.code
+    except RuntimeError:
+        pass                      # the refused call may have ended the capture
+    assert refused == -5
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(a.schedule(wl.epoch_seconds, 2 * jobs)[0], b.schedule(wl.epoch_seconds, 2 * jobs)[0])
+    for s in (a, b):              # and the next one is taken
+        s.append_losses(ids, 0.9 * last)
+    np.testing.assert_array_equal(a.schedule(wl.epoch_seconds, 2 * jobs)[0], b.schedule(wl.epoch_seconds, 2 * jobs)[0])
+    assert a.export_state().tobytes() == b.export_state().tobytes()
+    a.close()
+    b.close()
