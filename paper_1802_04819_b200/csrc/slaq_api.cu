@@ -529,10 +529,13 @@ int ensure_weights(slaq_handle* h) {
     return SLAQ_OK;
 }
 
-int check_device_errors(slaq_handle* h) {
+// look_at: the bits that are reported (and cleared).
+int check_device_errors(slaq_handle* h, int32_t look_at = ~0) {
     int32_t word = 0;
     CK(cudaMemcpyAsync(&word, h->err_word, sizeof word, cudaMemcpyDeviceToHost, h->stream), "read error word");
     CK(cudaStreamSynchronize(h->stream), "read error word");
+    const int32_t rest = word & ~look_at;
+    word &= look_at;
     if (word != 0) {
         std::string what = "a kernel found an inconsistency:";
         if (word & kErrWindow) what += " a window longer than its ring;";
@@ -544,7 +547,8 @@ int check_device_errors(slaq_handle* h) {
         if (word & kErrJob) what += " a job id out of range;";
         if (word & kErrBarrier) what += " the blocks of the selection launch did not all arrive in time;";
         if (word & kErrInput) what += " slaq_append_losses_device was given an id out of range, a job without losses, a value that is not finite or a core count below 1 (those entries were skipped);";
-        cudaMemsetAsync(h->err_word, 0, sizeof word, h->stream);   // reported once: the next epoch starts clean
+        cudaMemcpyAsync(h->err_word, &rest, sizeof rest, cudaMemcpyHostToDevice, h->stream);   // reported once: the next epoch starts clean
+        cudaStreamSynchronize(h->stream);
         h->scratch_clean = false;
         return fail(h, SLAQ_E_CUDA, what);
     }
@@ -1049,11 +1053,12 @@ int results_to_host(slaq_handle* h, const std::vector<Segment>& segments) {
 int epoch_to_host(slaq_handle* h, double T, int64_t C, int32_t* out_alloc, bool only_allocate) {
     const int rc = run_epoch(h, T, C, nullptr, only_allocate, true);
     if (rc < 0) return rc;
+    const int32_t look_at = only_allocate ? ~kErrInput : ~0;   // what slaq_append_losses_device skipped is for slaq_schedule to report
     const size_t bytes = sizeof(int32_t) * (size_t)h->max_jobs;
     if (h->last_epoch_was_graph || h->max_jobs > h->mailbox_jobs) {
         CK(cudaMemcpyAsync(out_alloc, h->alloc, bytes, cudaMemcpyDeviceToHost, h->stream), "copy allocation");
         if (h->last_epoch_was_graph) {
-            const int ec = check_device_errors(h);   // its synchronisation also completes the copy above
+            const int ec = check_device_errors(h, look_at);   // its synchronisation also completes the copy above
             return ec ? ec : rc;
         }
         CK(cudaStreamSynchronize(h->stream), "epoch");
@@ -1062,8 +1067,8 @@ int epoch_to_host(slaq_handle* h, double T, int64_t C, int32_t* out_alloc, bool 
         if (const int wc = wait_mailbox(h, "epoch")) return wc;
         std::memcpy(out_alloc, h->mail_alloc(), bytes);
     }
-    if (h->mailbox->err) {
-        const int ec = check_device_errors(h);
+    if (h->mailbox->err & look_at) {
+        const int ec = check_device_errors(h, look_at);
         return ec ? ec : rc;
     }
     return rc;
