@@ -315,11 +315,29 @@ finalise_kernel(const double* __restrict__ gain, const int32_t* __restrict__ cou
         atomicAdd((unsigned long long*)&counters[6], (unsigned long long)(sh_pre[0] >> 20));
         atomicAdd((unsigned long long*)&counters[7], (unsigned long long)(sh_pre[0] & ((1ll << 20) - 1)));
     }
-    // predicted reduction at the allocation: the job's first a_j gains, in order (as the single launch adds them)
+    // Predicted reduction at the allocation: the job's first a_j gains, in order (as the single launch adds them).  Every thread walks
+    // a row of its own, and what bounds long rows is the number of requests: two gains per load where rows begin on 16 bytes.
+    // 4,000 rows with 512 of 1,024 cores on average, the copy of the allocation included: 133 us one gain per load (16 of them
+    // in flight change nothing), 187 in whole lines through shared memory, 93 so (94 with a warp per long row, in another order).
     if (jt < max_jobs) {
+        const double* const row = gain + (size_t)jt * cap;
         double R = 0.0;
-        const double* row = gain + (size_t)jt * cap;
-        for (int n = 0; n < a; ++n) R += row[n];
+        int n = 0;
+        if (cap % 2 == 0) {
+            constexpr int kAhead = 8;   // loads in flight
+            const double2* const pair = reinterpret_cast<const double2*>(row);
+            for (; n + 2 * kAhead <= a; n += 2 * kAhead) {
+                double2 g[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) g[k] = pair[n / 2 + k];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    R += g[k].x;
+                    R += g[k].y;
+                }
+            }
+        }
+        for (; n < a; ++n) R += row[n];
         reduction[jt] = R;
     }
 }

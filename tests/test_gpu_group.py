@@ -49,6 +49,36 @@ def test_handles_of_one_gpu(cfg, n_jobs, cuts):
         assert alloc.sum() == min(2, cap) * s.max_jobs
 
 
+# rows that end at and beside a multiple of the gains in flight together, and at the largest cap
+@pytest.mark.parametrize("cap,per_job", [(33, 30), (48, 44), (49, 47), (1024, 300), (1024, 900)])
+def test_steps_add_long_rows_as_one_handle_does(cap, per_job):
+    import paper_1802_04819_b200 as slaq
+    slaq.build()
+
+    class Steps(slaq.LocalExchange):
+        pass
+
+    wl = make_workload(4, n_jobs=700)
+    J = wl.n_jobs
+
+    def handle(lo, hi):
+        ids = np.arange(hi - lo, dtype=np.int32)
+        s = slaq.Scheduler(hi - lo, wl.max_hist, cap)
+        s.load_histories(ids, wl.offsets[lo:hi + 1] - wl.offsets[lo], wl.losses[wl.offsets[lo]:wl.offsets[hi]], wl.k_last[lo:hi],
+                         wl.m_seen[lo:hi])
+        s.set_time_model(ids, wl.s[lo:hi], wl.w[lo:hi])
+        return s
+
+    whole, shards = handle(0, J), [handle(0, 257), handle(257, J)]
+    for C in (per_job * J, J * cap - 1, J * cap):
+        ref, _ = whole.schedule(wl.epoch_seconds, C)
+        parts = slaq.schedule_sharded(shards, Steps(), wl.epoch_seconds, C)
+        np.testing.assert_array_equal(np.concatenate(parts), ref)
+        assert ref.max() > 32
+        got = np.concatenate([s.get_predictions(want_gain=False)["R"] for s in shards])
+        np.testing.assert_array_equal(got, whole.get_predictions(want_gain=False)["R"])
+
+
 def test_a_group_refuses_what_it_cannot_do():
     import paper_1802_04819_b200 as slaq
     from paper_1802_04819_b200.binding import P_GAIN_ENVELOPE, schedule_group
