@@ -115,10 +115,10 @@ enum {
 typedef struct slaq_stats {
     float ms_total;        /* device time of the whole epoch */
     float ms_fit;          /* normalise + fit kernel (the three stage times are 0 for an epoch replayed as a CUDA graph) */
-    float ms_gain;         /* marginal-gain kernel (with the first selection histogram) */
-    float ms_alloc;        /* threshold selection, per-job counts, allocation */
-    int32_t launches;      /* steps of the call, counted as if each were a kernel of its own (15 for an epoch: three of the
-                              work list, fit, gains, ten of the selection), however they are grouped into launches */
+    float ms_gain;         /* marginal-gain kernel (0 where the selection predicts the gains itself: all but the prediction
+                              options and the sharded steps) */
+    float ms_alloc;        /* selection: gains (unless a kernel of their own wrote them), threshold, allocation */
+    int32_t launches;      /* kernels the call launched (two to six for an epoch; the sharded steps: all since slaq_shard_predict) */
     int32_t active_jobs;
     int64_t cores_handed_out;
     int64_t points;        /* loss values read by the fit kernel */
@@ -131,7 +131,7 @@ typedef struct slaq_stats {
     int32_t fallback_jobs;
     int32_t nonconvex_fits;  /* fitted jobs whose winning curve is not convex ahead of the newest point (family I with
                                 b^2 < a c): their marginal gains rise before they fall, see SLAQ_P_GAIN_ENVELOPE */
-    int32_t kernel_launches; /* kernels the call launched */
+    int32_t kernel_launches; /* the same as `launches` */
 } slaq_stats;
 
 /*

@@ -20,7 +20,6 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int64_t kCheckOnHost = 32768;   // losses of a bulk load up to which the host checks them
 constexpr int32_t kMailAlways = 4096;   // entries of an append up to which asking where the arrays live costs more than it gives
-constexpr int32_t kEpochSteps = 15, kAllocateSteps = 11;   // slaq_stats.launches
 
 struct Bump {
     char* base;
@@ -1022,8 +1021,6 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
     h->last_gain_launch = !only_allocate && !gains_in_selection(h, only_allocate);
     h->last_fit_launch = !only_allocate;
     h->last_launches = launches;
-    h->last_steps = only_allocate ? kAllocateSteps : kEpochSteps;
-    h->last_cores = usable;
     h->gain_partial = gains_in_selection(h, only_allocate) && !select_writes_whole_table(h, want);
     h->epoch_captured = h->epoch_captured || capturing;
     if (active > 0 && C < active) return SLAQ_W_OVERSUBSCRIBED;
@@ -1401,7 +1398,6 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
         g->last_gain_launch = false;
         g->last_epoch_was_graph = false;
         g->last_launches += s == 0 ? k : 0;
-        g->last_steps = kEpochSteps;
         g->gain_partial = !whole_table;
     }
     bool copied = false;
@@ -1463,7 +1459,7 @@ int slaq_shard_predict(slaq_t* h, double epoch_seconds, int32_t with_floor) {
     CK(cudaEventRecord(h->ev[2], st), "event");
     CK(cudaEventRecord(h->ev[3], st), "event");
     h->have_epoch = true;
-    h->last_launches = h->last_steps = launches;
+    h->last_launches = launches;
     h->gain_partial = false;
     h->epoch_captured = h->epoch_captured || is_capturing(h);
     return SLAQ_OK;
@@ -1486,7 +1482,7 @@ int slaq_shard_pick(slaq_t* h, int32_t pass, int64_t want) {
     if (pass < 0 || pass >= kRadixPasses) return fail(h, SLAQ_E_ARG, "pass outside 0..5");
     const int k = launch_shard_pick(h, pass, want);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     return SLAQ_OK;
 }
 
@@ -1495,7 +1491,7 @@ int slaq_shard_pass(slaq_t* h, int32_t pass) {
     if (pass < 1 || pass >= kRadixPasses) return fail(h, SLAQ_E_ARG, "pass outside 1..5");
     const int k = launch_shard_pass(h, pass, h->shard_first_unit);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     return SLAQ_OK;
 }
 
@@ -1504,7 +1500,7 @@ int slaq_shard_count(slaq_t* h, int64_t* out_local_ties) {
     const long long* d_total = nullptr;
     const int k = launch_shard_count(h, h->shard_first_unit, &d_total);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     long long total = 0;
     CK(cudaMemcpyAsync(&total, d_total, sizeof total, cudaMemcpyDeviceToHost, h->stream), "read tie count");
     CK(cudaStreamSynchronize(h->stream), "read tie count");
@@ -1517,7 +1513,7 @@ int slaq_shard_count_device(slaq_t* h, int64_t* d_out_local_ties) {
     const long long* d_total = nullptr;
     const int k = launch_shard_count(h, h->shard_first_unit, &d_total);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     CK(cudaMemcpyAsync(d_out_local_ties, d_total, sizeof(long long), cudaMemcpyDeviceToDevice, h->stream), "export tie count");
     return SLAQ_OK;
 }
@@ -1527,7 +1523,7 @@ int slaq_shard_finalise_device(slaq_t* h, const int64_t* d_ties_before, int32_t*
     if (!out_alloc || !d_ties_before) return fail(h, SLAQ_E_ARG, "out_alloc or d_ties_before is null");
     const int k = launch_shard_finalise(h, h->shard_first_unit, 0, reinterpret_cast<const long long*>(d_ties_before), nullptr);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
        "copy allocation");
@@ -1540,7 +1536,7 @@ int slaq_shard_finalise(slaq_t* h, int64_t ties_before, int32_t* out_alloc) {
     if (ties_before < 0) return fail(h, SLAQ_E_ARG, "ties_before must not be negative");
     const int k = launch_shard_finalise(h, h->shard_first_unit, ties_before, nullptr, nullptr);
     if (k < 0) return SLAQ_E_CUDA;
-    h->last_launches += k, h->last_steps += k;
+    h->last_launches += k;
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(out_alloc, h->alloc, sizeof(int32_t) * (size_t)h->max_jobs, cudaMemcpyDeviceToHost, h->stream),
        "copy allocation");
@@ -1926,8 +1922,7 @@ int slaq_get_stats(slaq_t* h, slaq_stats* out) {
             CK(cudaEventElapsedTime(&out->ms_alloc, h->ev[2], h->ev[3]), "event time");
         }
     }
-    out->launches = h->last_steps;
-    out->kernel_launches = h->last_launches;
+    out->launches = out->kernel_launches = h->last_launches;
     out->active_jobs = h->n_active;
     out->points = counters[0];
     out->model_sweeps = counters[1];

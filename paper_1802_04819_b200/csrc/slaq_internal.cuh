@@ -207,9 +207,7 @@ struct slaq_handle {
     }
     bool have_epoch = false;
     int32_t last_launches = 0;            // kernels the last call launched
-    int32_t last_steps = 0;               // its steps, as slaq_stats counts them
     int select_blocks_per_sm = 1;         // resident blocks of the selection kernel
-    int64_t last_cores = 0;
     int sm_count = 148;
     std::vector<uint8_t> active;      // host mirror: job has at least one loss
     std::vector<uint32_t> stamp;      // host: duplicate detection
