@@ -865,12 +865,13 @@ int do_load(slaq_handle* h, int32_t n, const int32_t* ids, const int64_t* offset
             shifted.resize((size_t)n + 1);
             for (int32_t i = 0; i <= n; ++i) shifted[i] = offsets[i] - lo;
         }
-        std::vector<Segment> up = {{h->stage.ids, ids, sizeof(int32_t) * n},
-                                   {h->stage.offsets, lo != 0 ? shifted.data() : offsets, sizeof(int64_t) * ((size_t)n + 1)},
-                                   {h->stage.k_last, k_last, sizeof(int64_t) * n}};
-        if (m_seen) up.push_back({h->stage.m_seen, m_seen, sizeof(double) * n});
-        if (!packed) up.push_back({d_src, losses + lo, sizeof(double) * (size_t)total});
-        status = pipe_to_device(h, up);
+        Segment up[5] = {{h->stage.ids, ids, sizeof(int32_t) * n},
+                         {h->stage.offsets, lo != 0 ? shifted.data() : offsets, sizeof(int64_t) * ((size_t)n + 1)},
+                         {h->stage.k_last, k_last, sizeof(int64_t) * n}};
+        int pieces = 3;
+        if (m_seen) up[pieces++] = {h->stage.m_seen, m_seen, sizeof(double) * n};
+        if (!packed) up[pieces++] = {d_src, losses + lo, sizeof(double) * (size_t)total};
+        status = pipe_to_device(h, Segments(up, pieces));
         if (!status) {
             if (!packed && !check_here)
                 finite_kernel<<<h->sm_count * 4, 256, 0, st>>>(d_src, (size_t)total, h->scratch.load_flag, nullptr, 0, nullptr);
@@ -1030,7 +1031,7 @@ int run_epoch(slaq_handle* h, double T, int64_t C, int32_t* d_out, bool only_all
 
 // Results into host arrays.  Arrays in one of the binding's result blocks are written by one kernel, which reports to the
 // mailbox; anything else is copied.
-int results_to_host(slaq_handle* h, const std::vector<Segment>& segments) {
+int results_to_host(slaq_handle* h, Segments segments) {
     Pieces p;
     size_t bytes = 0;
     for (const Segment& s : segments) {

@@ -19,8 +19,9 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <system_error>
+#include <new>
 #include <thread>
+#include <vector>
 
 #include "slaq_internal.cuh"
 
@@ -107,7 +108,7 @@ void work(slaq_handle* h, const std::vector<Segment>& chunks, bool down, int thr
     if (e != cudaSuccess) error.store((int)e);
 }
 
-int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
+int copy(slaq_handle* h, Segments segments, bool down) {
     std::vector<Segment> pageable;
     size_t total = 0;
     for (const Segment& s : segments) {
@@ -152,7 +153,7 @@ int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
         for (; started < threads; ++started) {
             try {
                 helper[started] = std::thread(work, h, std::cref(chunks), down, started, threads, std::ref(error));
-            } catch (const std::system_error&) {
+            } catch (...) {   // no thread or no memory for one
                 break;
             }
         }
@@ -166,6 +167,17 @@ int copy(slaq_handle* h, const std::vector<Segment>& segments, bool down) {
         if (e != cudaSuccess) return failed(h, e);
     }
     return SLAQ_OK;
+}
+
+// The lists of a copy are its only allocations; without memory for them nothing of the caller's may still be in use on return.
+int copy_or_fail(slaq_handle* h, Segments segments, bool down) {
+    try {
+        return copy(h, segments, down);
+    } catch (const std::bad_alloc&) {
+        cudaStreamSynchronize(h->stream);
+        h->err = "out of memory";   // short enough to need none
+        return SLAQ_E_NOMEM;
+    }
 }
 
 }  // namespace
@@ -192,8 +204,8 @@ void page_locked_free(void* m) {
     std::free(m);
 }
 
-int pipe_to_device(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, false); }
-int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments) { return copy(h, segments, true); }
+int pipe_to_device(slaq_handle* h, Segments segments) { return copy_or_fail(h, segments, false); }
+int pipe_to_host(slaq_handle* h, Segments segments) { return copy_or_fail(h, segments, true); }
 
 void pipe_retain() {
     std::lock_guard<std::mutex> hold(pool().count_lock);
@@ -246,8 +258,11 @@ void spare_give(int device, void* memory, size_t bytes) {
         size_t kept = bytes;
         for (const Pool::Spare& s : p.spares) kept += s.bytes;
         if (p.handles > 0 && p.spares.size() < kSpares && kept <= kSpareBytes) {
-            p.spares.push_back({device, memory, bytes});
-            return;
+            try {
+                p.spares.push_back({device, memory, bytes});
+                return;
+            } catch (const std::bad_alloc&) {   // then it is not kept
+            }
         }
     }
     cudaFree(memory);
@@ -265,7 +280,7 @@ bool in_result_block(const void* q, size_t bytes) {
 
 }  // namespace slaq
 
-void* slaq_result_take(size_t bytes) {
+void* slaq_result_take(size_t bytes) try {
     using namespace slaq;
     size_t size = kResultLeast;
     while (size < bytes) size <<= 1;
@@ -289,9 +304,16 @@ void* slaq_result_take(size_t bytes) {
     if (p.block_bytes + size > kResultBytes) return nullptr;
     void* const m = page_locked_alloc(size);
     if (!m) return nullptr;
-    p.blocks[static_cast<char*>(m)] = {size, true};
+    try {
+        p.blocks[static_cast<char*>(m)] = {size, true};
+    } catch (const std::bad_alloc&) {
+        page_locked_free(m);
+        return nullptr;
+    }
     p.block_bytes += size;
     return m;
+} catch (const std::bad_alloc&) {
+    return nullptr;   // the binding takes ordinary memory
 }
 
 void slaq_result_give(void* block) {

@@ -2,7 +2,7 @@
 #pragma once
 
 #include <cstddef>
-#include <vector>
+#include <initializer_list>
 
 struct slaq_handle;
 
@@ -14,10 +14,19 @@ struct Segment {
     size_t bytes;
 };
 
-// Copy all segments, queued on the handle's stream.  to_device: returns once the sources have been read (the copies may
-// still run).  to_host: returns once everything has arrived.  Returns 0, or a status with the handle's message set.
-int pipe_to_device(slaq_handle* h, const std::vector<Segment>& segments);
-int pipe_to_host(slaq_handle* h, const std::vector<Segment>& segments);
+// Copy all segments, queued on the handle's stream.  to_device: the copies may still run on return, and page-locked sources of
+// kPipeFrom bytes and more may still be read by them: the caller waits for the stream before its own caller gets them back.
+// to_host: returns once everything has arrived.  Returns 0, or a status with the handle's message set.
+struct Segments {
+    const Segment* at;
+    size_t n;
+    Segments(std::initializer_list<Segment> list) : at(list.begin()), n(list.size()) {}
+    Segments(const Segment* first, size_t count) : at(first), n(count) {}
+    const Segment* begin() const { return at; }
+    const Segment* end() const { return at + n; }
+};
+int pipe_to_device(slaq_handle* h, Segments segments);
+int pipe_to_host(slaq_handle* h, Segments segments);
 
 // A handle begins / ends its life: the page-locked buffers behind the copies are shared by all handles of the process
 // and released with the last of them.

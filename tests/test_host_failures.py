@@ -78,3 +78,32 @@ def test_every_handle_of_a_group_that_failed_clears_its_scratch(lib, failure):
     assert _clears(lib) == before + 3
     for h in hs:
         lib.slaq_destroy(h)
+
+
+def test_a_bulk_copy_without_memory_for_its_lists_is_an_error(lib):
+    """No C entry throws: every allocation of a load and of its copies (threads among them) is let fail in turn."""
+    jobs, points = 8, 9_000_000                                    # enough for the page-locked buffers of the copies
+    h = c_void_p()
+    assert lib.slaq_create_in(None, c_size_t(0), c_int32(jobs), c_int32(16), c_int32(4), byref(h)) == 0
+    losses = (c_double * points)()
+    ids, k_last = (c_int32 * jobs)(*range(jobs)), (c_int64 * jobs)(*[points // jobs] * jobs)
+    offsets = (c_int64 * (jobs + 1))(*[points // jobs * j for j in range(jobs + 1)])
+    fails = c_long.in_dll(lib, "fake_new_fails_in")
+    kernels = c_int.in_dll(lib, "fake_device_kernels")
+    results = set()
+    for at in range(1, 25):
+        fails.value = at
+        before = kernels.value
+        rc = lib.slaq_load_histories(h, c_int32(jobs), ids, offsets, losses, k_last, None)
+        left, fails.value = fails.value, 0
+        results.add((rc, left > 0))
+        # the fake runs no kernel, so a load that got that far reports that its own did not come to an end
+        assert rc == (-5 if kernels.value > before else -4)
+    assert (-4, False) in results and (-5, False) in results and (-5, True) in results
+    lib.slaq_result_take.restype = c_void_p
+    for at in range(1, 12):
+        fails.value = 1
+        block = lib.slaq_result_take(c_size_t(70000 + 131072 * at))
+        assert block is None
+    fails.value = 0
+    lib.slaq_destroy(h)
