@@ -2,7 +2,9 @@
 // the scheduling epoch, and read-back of results.  The contract is in include/slaq.h.
 #include <math_constants.h>
 
+#if defined(__x86_64__)
 #include <immintrin.h>
+#endif
 
 #include <algorithm>
 #include <atomic>
@@ -554,12 +556,21 @@ int check_device_errors(slaq_handle* h, int32_t look_at = ~0) {
     return SLAQ_OK;
 }
 
+// One turn of a loop that watches memory: what the host's processor has for it.
+inline void spin_pause() {
+#if defined(__x86_64__)
+    _mm_pause();
+#elif defined(__aarch64__)
+    asm volatile("yield" ::: "memory");
+#endif
+}
+
 // Wait until the kernel that carries this call's number has reported to the mailbox.  Watching host memory sees the end of
 // a kernel a few microseconds before a stream synchronisation returns; the stream is asked now and then, for errors.
 int wait_mailbox_for(slaq_handle* h, uint32_t seq, const char* what) {
     // the number is written by kernels of one stream in order, so a later one says that this one is over too
     for (int spins = 0; (int32_t)(h->mailbox->done - seq) < 0;) {
-        _mm_pause();
+        spin_pause();
         if (++spins < 2000) continue;
         spins = 0;
         const cudaError_t e = cudaStreamQuery(h->stream);
