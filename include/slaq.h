@@ -27,7 +27,11 @@
  *     it passes and may release it when the call returns, unless stated otherwise.
  *   - The handle owns all scheduler state on the device.  Calls on one handle must not
  *     overlap; work is ordered on the handle's stream (slaq_set_stream).  Functions
- *     that take or fill host buffers return after the stream has finished that work.
+ *     that fill host buffers return when they are filled, functions that take host buffers
+ *     when they have been read; the stream may still be at work on what the call queued.
+ *   - The selection of an epoch (and of slaq_allocate_static) is a cooperative launch of up to a
+ *     block per SM, except for small tables: beside other work on the GPU it begins when every
+ *     SM it needs has room for its block.
  *   - Calls on a handle must be made with the handle's device current (SLAQ_E_ARG otherwise).
  *   - Job ids are 0 .. max_jobs-1.  A job is active from its first loss until removed.
  *   - The library needs a CUDA device: there is no CPU path.
@@ -83,7 +87,7 @@ enum {
     SLAQ_P_EPOCH_GRAPH = 8,       /* 1: slaq_schedule / slaq_schedule_device replay the epoch's launches as one
                                      CUDA graph once two calls in a row had the same arguments, parameters and
                                      number of active jobs; 0: always plain launches; -1 (default): what is faster,
-                                     which is plain launches at every size (an epoch is two to five of them).  Results
+                                     which is plain launches at every size (an epoch is two to six of them).  Results
                                      are the same either way.  Not used while the handle's stream is itself being
                                      captured. */
     SLAQ_P_GAIN_ENVELOPE = 9,     /* 0 (default) or 1.  The greedy loop is exact when every job's predicted reduction
@@ -94,9 +98,10 @@ enum {
                                      1: they are replaced by the slopes of the upper concave envelope of the points
                                      (n, R(n)), the smallest concave function nowhere below R, which keeps the curve's
                                      whole drop at max_cores_per_job.  Rows of convex fits are the same either way. */
-    SLAQ_P_SELECTION = 10         /* 0 or 1: whether a caller wants the whole table of gains written.  Both find the same
-                                  allocation with the same kernel, which predicts a row only as far as the selection
-                                  may need it; gain rows that slaq_get_predictions returns are completed on request. */
+    SLAQ_P_SELECTION = 10         /* 0 or 1, accepted and without effect: it once chose between a selection from a whole table of
+                                  gains and one without.  There is one selection, which predicts a row of a large
+                                  table only as far as it may need it; gain rows that slaq_get_predictions returns or
+                                  slaq_allocate_only reads are completed on request, as the epoch would have. */
 };
 
 /* per-job status written by slaq_schedule (slaq_get_predictions, out_status) */

@@ -175,11 +175,6 @@ __global__ void init_jobs_kernel(JobArrays job, FitArrays fit, double* ring, int
     reduction[j] = 0.0;
 }
 
-// One new iteration per listed job: ring write, iteration index, largest reduction seen,
-// and the sums of the iteration-time law (booked at the given or the current core count).
-// checked: the arrays come straight from the caller's device memory, unseen by the host - an id out of range,
-// a job without any loss yet, a loss or time that is not finite or a core count below 1 sets kErrInput and
-// that entry is skipped.
 // Called by every thread of a kernel at its end: the last block to get here tells the host.
 __device__ __forceinline__ void report(Mailbox* mail, uint32_t seq, unsigned int* ticket, int32_t* flag) {
     __syncthreads();
@@ -199,6 +194,11 @@ __device__ __forceinline__ void report(Mailbox* mail, uint32_t seq, unsigned int
     mail->done = seq;
 }
 
+// One new iteration per listed job: ring write, iteration index, largest reduction seen,
+// and the sums of the iteration-time law (booked at the given or the current core count).
+// checked: the arrays come straight from the caller's device memory, unseen by the host - an id out of range,
+// a job without any loss yet, a loss or time that is not finite or a core count below 1 sets kErrInput and
+// that entry is skipped.
 // All loads of an entry are issued before anything is stored: the chain is then three memory latencies long (entry, job,
 // newest loss) instead of one per array.
 __device__ __forceinline__ void append_one(const JobArrays& job, const FitArrays& fit, int max_jobs, int i, const int32_t* ids,

@@ -159,7 +159,7 @@ struct slaq_handle {
     int32_t lm_trials = 20, min_fit_points = 4;
     size_t fit_slice_bytes = 13824;       // shared memory one warp of the fit kernel may use (parked sums, up to 52 rows of 32 points, a spare row)
     bool warm_start = false;              // fits start from the last epoch's parameters where there are some
-    int selection = 0;                    // SLAQ_P_SELECTION: kept for callers that ask, the launches are the same
+    int selection = 0;                    // SLAQ_P_SELECTION: kept for callers that ask, read by nothing else
     bool gain_partial = false;            // h->gain holds the last epoch's rows only in part (see GainBasis)
     bool epoch_captured = false;          // an epoch of the handle is part of a graph of the caller: only the device knows which was last
     std::vector<uint8_t> hinted;          // host mirror: job has a target-loss hint

@@ -6,8 +6,9 @@ sharded over several GPUs"): per radix pass one sum of a 2048-entry histogram ov
 at the end one gather of each shard's number of threshold-equal gains.  Two ways to exchange:
 
 * ``ProcessGroupExchange``: one shard per process, ``torch.distributed`` (NCCL) does the sums;
-* ``LocalExchange``: several shards in one process on one GPU, summed directly - the same
-  steps in the same order, used to check the protocol where only one GPU is available.
+* ``LocalExchange``: several shards in one process on one GPU.  They are scheduled by one call
+  (``slaq_schedule_group``) where that is possible, to the same result; with a subclass, or with shards that call does not
+  take, the steps run in the protocol's order with the sums made directly, which checks the protocol on one GPU.
 """
 
 from __future__ import annotations

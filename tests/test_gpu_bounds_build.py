@@ -90,7 +90,10 @@ def test_appends_through_a_wrapping_ring_and_the_sharded_steps(slaq):
     alloc, rc = sched.schedule(wl.epoch_seconds, wl.total_cores)
     assert alloc[::5].sum() == 0
     sched.close()
-    # the step-by-step calls of a sharded cluster run the same kernels: two shards of the bounds build
+    # the step-by-step calls of a sharded cluster, and the one call for shards of one GPU: two shards of the bounds build
+    class Steps(LocalExchange):   # not the class itself: schedule_sharded goes through the steps
+        pass
+
     wl = make_workload(2, n_jobs=1200)
     cut = 500
     shards = []
@@ -102,5 +105,6 @@ def test_appends_through_a_wrapping_ring_and_the_sharded_steps(slaq):
                           wl.m_seen[lo:hi])
         sh.set_time_model(np.arange(n, dtype=np.int32), wl.s[lo:hi], wl.w[lo:hi])
         shards.append(sh)
-    allocs = schedule_sharded(shards, LocalExchange(), wl.epoch_seconds, wl.total_cores)
-    assert sum(int(a.sum()) for a in allocs) == wl.total_cores
+    for exchange in (Steps(), LocalExchange()):
+        allocs = schedule_sharded(shards, exchange, wl.epoch_seconds, wl.total_cores)
+        assert sum(int(a.sum()) for a in allocs) == wl.total_cores

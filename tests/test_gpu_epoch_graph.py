@@ -59,18 +59,18 @@ def test_graph_replay_equals_plain_launches(cfg, n_jobs):
 
 
 def test_graph_replay_without_a_gain_table():
-    """Selection without a table inside a replayed graph: the gain rows asked for after every epoch are written on
-    request and belong to that epoch, also after new losses arrived between two replays of the same graph."""
+    """Rows that a replayed graph leaves unfinished are completed on request and belong to that epoch, also after new losses
+    arrived between two replays of the same graph.  The last leg sets SLAQ_P_SELECTION, which is accepted and changes nothing."""
     import paper_1802_04819_b200 as slaq
-    wl = make_workload(1)
-    plain = _epochs(slaq, wl, 0, selection=1)
-    replay = _epochs(slaq, wl, 1, selection=1)
-    table = _epochs(slaq, wl, 0, selection=0)
+    wl = make_workload(4, n_jobs=6000)        # more than 2,048 gains per SM
+    plain = _epochs(slaq, wl, 0)
+    replay = _epochs(slaq, wl, 1)
+    table = _epochs(slaq, wl, 0, selection=1)
     for a, b, c in zip(plain, replay, table):
         np.testing.assert_array_equal(a[0], b[0])
         np.testing.assert_array_equal(a[1].view(np.int64), b[1].view(np.int64))
         np.testing.assert_array_equal(a[2].view(np.int64), b[2].view(np.int64))
-        np.testing.assert_array_equal(a[1].view(np.int64), c[1].view(np.int64))     # the rows are the table's rows
+        np.testing.assert_array_equal(a[1].view(np.int64), c[1].view(np.int64))
         assert a[0].sum() == c[0].sum()
 
 

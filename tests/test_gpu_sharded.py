@@ -1,8 +1,9 @@
 """One cluster split over several shards must be scheduled exactly like the same cluster on one handle.
 
 Only one GPU is available to these tests, so the shards live in one process on one GPU and their
-histograms are summed locally (``LocalExchange``): the calls, their order and the exchanged data are
-those of the multi-GPU protocol; with one shard per process only the transport differs."""
+histograms are summed locally.  With ``Steps`` the calls, their order and the exchanged data are those of the
+multi-GPU protocol; with one shard per process only the transport differs.  A plain ``LocalExchange`` schedules such
+shards by one call instead (``slaq_schedule_group``), which has to give the same."""
 
 import numpy as np
 import pytest
@@ -10,6 +11,13 @@ import pytest
 from workloads import make_workload
 
 pytestmark = pytest.mark.gpu
+
+
+def _exchanges(slaq):
+    class Steps(slaq.LocalExchange):   # not the class itself: schedule_sharded goes through the steps
+        pass
+
+    return Steps(), slaq.LocalExchange()
 
 
 def _build(slaq, wl, lo, hi):
@@ -31,12 +39,13 @@ def test_sharded_cluster_equals_one_handle(cfg, n_jobs, cuts):
     shards = [_build(slaq, wl, lo, hi) for lo, hi in zip(cuts[:-1], cuts[1:])]
     for C in (wl.total_cores, wl.n_jobs - 3, wl.n_jobs, 2 * wl.n_jobs + 1, wl.n_jobs * wl.max_cores_per_job + 5):
         ref, _ = whole.schedule(wl.epoch_seconds, C)
-        parts = slaq.schedule_sharded(shards, slaq.LocalExchange(), wl.epoch_seconds, C)
-        np.testing.assert_array_equal(np.concatenate(parts), ref)        # integer work: bit-exact
-        gains = np.concatenate([s.get_predictions()["gain"] for s in shards])
-        np.testing.assert_array_equal(gains, whole.get_predictions()["gain"])
-        R = np.concatenate([s.get_predictions(want_gain=False)["R"] for s in shards])
-        np.testing.assert_array_equal(R, whole.get_predictions(want_gain=False)["R"])
+        for exchange in _exchanges(slaq):
+            parts = slaq.schedule_sharded(shards, exchange, wl.epoch_seconds, C)
+            np.testing.assert_array_equal(np.concatenate(parts), ref)        # integer work: bit-exact
+            gains = np.concatenate([s.get_predictions()["gain"] for s in shards])
+            np.testing.assert_array_equal(gains, whole.get_predictions()["gain"])
+            R = np.concatenate([s.get_predictions(want_gain=False)["R"] for s in shards])
+            np.testing.assert_array_equal(R, whole.get_predictions(want_gain=False)["R"])
 
 
 def test_sharded_ties_cross_shard_boundaries():
@@ -62,6 +71,7 @@ def test_sharded_ties_cross_shard_boundaries():
     shards = [build(0, 100), build(100, 101), build(101, 300)]
     for C in (J + 1, J + 150, 2 * J + 7, 5 * J - 1):
         ref, _ = whole.schedule(3.0, C)
-        parts = np.concatenate(slaq.schedule_sharded(shards, slaq.LocalExchange(), 3.0, C))
-        np.testing.assert_array_equal(parts, ref)
+        for exchange in _exchanges(slaq):
+            parts = np.concatenate(slaq.schedule_sharded(shards, exchange, 3.0, C))
+            np.testing.assert_array_equal(parts, ref)
         assert (np.diff(ref) <= 0).all()          # identical jobs: extra units go to the lowest ids
