@@ -253,6 +253,12 @@ sweep_loop_kernel(const double* __restrict__ g_wtab, int L, int rows, int n_swee
                     (1e-3 * span * span + 0.2 * span + 1.0) / 40.0, 0.45};   // the same curve in window coordinates
     double pII[4] = {-0.2, 3.0, 0.4, 0.0};
     const int fam = lane & 1;
+    const double per_row = (double)L * inv_span;   // the library's sweep counts x in rows of a lane's points
+    if (kVariant == 0) {
+        pI[0] *= per_row * per_row;
+        pI[1] *= per_row;
+        pII[1] *= per_row;
+    }
     double check = 0.0;
     long long t0 = 0;
     if (threadIdx.x == 0) t0 = clock64();
@@ -268,13 +274,15 @@ sweep_loop_kernel(const double* __restrict__ g_wtab, int L, int rows, int n_swee
                     // where the alternatives have family II's sums, and the signs the library keeps them with (0: not one of its sums)
                     const int place[13] = {9, 4, 2, 1, 0, 3, 10, 11, 7, 6, 5, 12, 8};
                     const double sign[13] = {0, -1, 1, -1, 1, 1, 0, 0, -1, 1, -1, 0, 1};
+                    // the power of x in each sum, to bring it back to the window's unit
+                    const int power[2][13] = {{0, 1, 2, 3, 4, 0, 1, 2, 0, 1, 2, 0, 0}, {0, 1, 2, 1, 0, 0, 0, 0, 0, 1, 0, 0, 0}};
                     int from, own;
                     S.held(from, own);
                     for (int i = 0; i < 13; ++i)
                         if (i < own)
                             for (int q = fam; q < 32; q += 2)
                                 if ((S.group() >> q) & 1u)
-                                    last_sums[q * 13 + (fam ? place[from + i] : from + i)] = fam ? sign[from + i] * sums.v[i] : sums.v[i];
+                                    last_sums[q * 13 + (fam ? place[from + i] : from + i)] = (fam ? sign[from + i] : 1.0) * sums.v[i] * pow(per_row, (double)power[fam][from + i]);
                 } else {
                     for (int i = 0; i < 13; ++i) last_sums[lane * 13 + i] = (i < 9 || !fam) ? sums.v[i] : 0.0;
                 }

@@ -40,7 +40,7 @@ size_t layout(slaq_handle* h, char* base, int32_t J, int32_t Hmax, int32_t cap) 
     Bump b{base};
     const size_t Js = (size_t)J;
     double* ring = b.take<double>(Js * Hmax);
-    double* wtab = b.take<double>(6 * (size_t)Hmax + 5);
+    double* wtab = b.take<double>(6 * (size_t)Hmax + 6 + 3 * kLogBins);
     JobArrays job;
     job.row = b.take<double*>(Js);
     job.cap = b.take<int32_t>(Js);
@@ -511,9 +511,20 @@ int check_ids(slaq_handle* h, int32_t n, const int32_t* ids, bool forbid_dups) {
 
 int ensure_weights(slaq_handle* h) {
     if (h->wtab_gamma == h->gamma) return SLAQ_OK;
-    // gamma^m, then the sums over m < H of gamma^m m^p for H = 0..max_hist, p = 0..4
+    // gamma^m, then the sums over m < H of gamma^m m^p for H = 0..max_hist, p = 0..4, then 1 / c, the leading part of log c
+    // and its rest for the middles c of the logarithm's bins
     const size_t n = (size_t)h->max_hist;
-    std::vector<double> tab(n + 5 * (n + 1));
+    std::vector<double> tab(6 * n + 6 + 3 * kLogBins);
+    for (int i = 0; i < kLogBins; ++i) {
+        const uint64_t bits = (uint64_t)(kLogFrom + (i << kLogBinShift) + (1 << (kLogBinShift - 1))) << 32;
+        double c;
+        std::memcpy(&c, &bits, sizeof c);
+        const double inv = 1.0 / c;
+        tab[6 * n + 6 + 2 * i] = inv;
+        const long double log_c = -std::log((long double)inv), lead = std::nearbyint(log_c * 0x1p42L) * 0x1p-42L;
+        tab[6 * n + 6 + 2 * i + 1] = (double)lead;
+        tab[6 * n + 6 + 2 * kLogBins + i] = (double)(log_c - lead);
+    }
     for (size_t m = 0; m < n; ++m) tab[m] = std::pow(h->gamma, (double)m);
     long double sum[5] = {};
     for (size_t m = 0; m <= n; ++m) {

@@ -323,8 +323,10 @@ struct Family {
 // point and its denominator positive there; beta >= 0 of family II.  `busy` = this lane has a trial to prepare; the
 // re-solve loop runs while any lane of the warp needs another round (each freezes at least one more of the three
 // bounded parameters).  Family II has three parameters: the fourth row of its system is empty but for the diagonal.
+// kRows, rows: x counts rows, and the window's length in that unit.
+template <bool kRows>
 __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&g)[4], bool busy, double tiny_S,
-                              double (&trial)[4]) {
+                              double rows, double (&trial)[4]) {
     F.has_trial = false;
     if (busy && F.S <= tiny_S) {   // residual is zero to rounding
         F.done = true;
@@ -337,10 +339,23 @@ __device__ void prepare_trial(Family& F, int fam, const Sym4& A, const double (&
     if (at0 && (__double2hiint(g[0]) < 0 || (F.was_frozen & 1u))) frozen |= 1u;
     if (at1 && (__double2hiint(g[1]) < 0 || (F.was_frozen & 2u))) frozen |= 2u;
     if (at2 && (__double2hiint(g[2]) < 0 || (F.was_frozen & 4u))) frozen |= 4u;
-    // the damped diagonal; 0x01a56e1f is the high word of 1e-300
-    auto damped = [&](double d) { return fma(F.lambda, __double2hiint(d) < 0x01a56e1f ? 1e-300 : d, d); };
+    // The damped diagonal.  An entry below 1e-300 in the window's unit (a curve that has run off to infinity everywhere but at the
+    // newest point) is damped by that.
     Sym4 B = A;
-    B.a00 = damped(A.a00), B.a11 = damped(A.a11), B.a22 = damped(A.a22), B.a33 = damped(A.a33);
+    if constexpr (kRows) {
+        B.a00 = fma(F.lambda, A.a00, A.a00), B.a11 = fma(F.lambda, A.a11, A.a11);
+        B.a22 = fma(F.lambda, A.a22, A.a22), B.a33 = fma(F.lambda, A.a33, A.a33);
+        // 0x05000000 is the high word of some 1e-285, above 1e-300 in any unit
+        if (min(min(__double2hiint(A.a00), __double2hiint(A.a11)), min(__double2hiint(A.a22), __double2hiint(A.a33))) < 0x05000000) {
+            const double f = rows * rows;   // a power of x on either side of the product makes it rows times the window's value
+            auto damped = [&](double d, double least) { return fma(F.lambda, d < least ? least : d, d); };
+            B.a00 = damped(A.a00, one ? 1e-300 * f * f : 1e-300), B.a11 = damped(A.a11, 1e-300 * f);
+            B.a22 = damped(A.a22, 1e-300), B.a33 = damped(A.a33, 1e-300);
+        }
+    } else {   // 0x01a56e1f is the high word of 1e-300
+        auto damped = [&](double d) { return fma(F.lambda, __double2hiint(d) < 0x01a56e1f ? 1e-300 : d, d); };
+        B.a00 = damped(A.a00), B.a11 = damped(A.a11), B.a22 = damped(A.a22), B.a33 = damped(A.a33);
+    }
     double step[4] = {0.0, 0.0, 0.0, 0.0};
     bool solved = false, again = busy;
     while (__any_sync(kFull, again)) {
@@ -466,9 +481,30 @@ struct GuessSums {
     double swy2, r0, r1, r2, su, sxu;
 };
 
+// log of a positive normal number, to 1.2 ulp, by table lookup (Tang, "Table-driven implementation of the logarithm function", 1990):
+// x = 2^e z with z in about [0.71, 1.42) cut into 128 bins with middles c, log x = e log 2 + log c + log(1 + r) with
+// r = z / c - 1, |r| <= 2^-8, by its Taylor series.  log 2 and log c are split so that the leading parts add up exactly; the bin
+// around 1 has c = 1.  tab: 128 pairs of 1 / c and the leading part of log c, then the rests (written by ensure_weights).  Half the
+// instructions of log(), whose arguments may be anything (fit of 100,000 windows of up to 1,000, with x counted in rows: 3,615 ->
+// 3,511 us, of 1,000,000 of 64: 3,904 -> 3,803; about half of it each).
+__device__ __forceinline__ double log_of_normal(double x, const double* __restrict__ tab) {
+    const int hi = __double2hiint(x), t = hi - kLogFrom, e = t >> 20, bin = (t >> kLogBinShift) & (kLogBins - 1);
+    const double z = __hiloint2double(hi - (e << 20), __double2loint(x));
+    const double2 c = __ldg(reinterpret_cast<const double2*>(tab) + bin);
+    const double rest = __ldg(tab + 2 * kLogBins + bin);
+    const double r = fma(z, c.x, -1.0);
+    double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+    p = fma(r, p, 1.0 / 5.0);
+    p = fma(r, p, -1.0 / 4.0);
+    p = fma(r, p, 1.0 / 3.0);
+    p = fma(r, p, -1.0 / 2.0);
+    const double lead = fma((double)e, 0x1.62e42fefa3800p-1, c.y);   // log 2 to 42 bits behind the point
+    return lead + (r + fma(r * r, p, fma((double)e, 0x1.ef35793c76730p-45, rest)));
+}
+
 // One point of the first-guess pass.  kI / kII: the transformed values of family I (1 / (y - d0)) and of
-// family II (log(y - d0)) are wanted by some lane of the warp.
-template <bool kI, bool kII, class Lanes>
+// family II (log(y - d0)) are wanted by some lane of the warp.  kAny: y - d0 may be subnormal or not finite.
+template <bool kI, bool kII, bool kAny, class Lanes>
 __device__ __forceinline__ void guess_point(const Lanes& S, const double* wp, const double* yp, double md, double inv_span,
                                             double d0, GuessSums& g) {
     const double x = -md * inv_span;
@@ -482,14 +518,14 @@ __device__ __forceinline__ void guess_point(const Lanes& S, const double* wp, co
         g.r0 = fma(wz * x, x, g.r0);
     }
     if (kII) {
-        const double wu = w * log(y - d0);
+        const double wu = w * (kAny ? log(y - d0) : log_of_normal(y - d0, S.log_table()));
         g.su += wu;
         g.sxu = fma(wu, x, g.sxu);
     }
 }
 
 // The rows every lane of the warp has without a test per row, the ragged rest with one.
-template <bool kI, bool kII, class Lanes>
+template <bool kI, bool kII, bool kAny, class Lanes>
 __device__ __forceinline__ void guess_rows(const Lanes& S, int own, int k_all, double inv_span, double d0, GuessSums& g) {
     const int full = __reduce_min_sync(kFull, own);
     const double* yp = S.y + S.lane;
@@ -498,15 +534,16 @@ __device__ __forceinline__ void guess_rows(const Lanes& S, int own, int k_all, d
     const double dL = (double)S.L();
     int k = 0;
 #pragma unroll 1
-    for (; k < full; ++k, md += dL, yp += 32, wp += S.L()) guess_point<kI, kII>(S, wp, yp, md, inv_span, d0, g);
+    for (; k < full; ++k, md += dL, yp += 32, wp += S.L()) guess_point<kI, kII, kAny>(S, wp, yp, md, inv_span, d0, g);
 #pragma unroll 1
     for (; k < k_all; ++k, md += dL, yp += 32, wp += S.L())
-        if (k < own) guess_point<kI, kII>(S, wp, yp, md, inv_span, d0, g);
+        if (k < own) guess_point<kI, kII, kAny>(S, wp, yp, md, inv_span, d0, g);
 }
 
 template <class Lanes>
 __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span, double ymin, double ymax, bool busy,
                               bool needI, bool needII, Moments& mom, double (&pI)[4], double (&pII)[4]) {
+    constexpr bool kTable = Lanes::kRowUnit;   // log() for teams, where a lane takes one or two, and for warm starts, which take none
     const double d0 = ymax > ymin ? ymin - 0.1 * (ymax - ymin) : ymin - 1e-3 * fmax(fabs(ymin), 1.0);
     GuessSums g = {};
     const int shift = __ffs(S.L()) - 1;
@@ -514,12 +551,17 @@ __device__ void first_guesses(const Lanes& S, int H, int k_all, double inv_span,
     // a family that no lane of the warp wants a guess for is left out of the pass; a lane that does not want
     // what the warp computes gets sums it does not use
     const bool anyI = __any_sync(kFull, needI), anyII = __any_sync(kFull, needII);
-    if (anyI && anyII) {
-        guess_rows<true, true>(S, own, k_all, inv_span, d0, g);
+    // y - d0 lies between its values at the lowest and the highest level (rounding keeps the order)
+    const int least = __double2hiint(ymin - d0), most = __double2hiint(ymax - d0);
+    const bool odd_one = needII && (least < 0x00100000 || least >= 0x7ff00000 || most < 0x00100000 || most >= 0x7ff00000);
+    if (kTable && __any_sync(kFull, odd_one)) {
+        guess_rows<true, true, true>(S, own, k_all, inv_span, d0, g);
+    } else if (anyI && anyII) {
+        guess_rows<true, true, !kTable>(S, own, k_all, inv_span, d0, g);
     } else {
-        if (anyI) guess_rows<true, false>(S, own, k_all, inv_span, d0, g);
-        else if (anyII) guess_rows<false, true>(S, own, k_all, inv_span, d0, g);
-        else guess_rows<false, false>(S, own, k_all, inv_span, d0, g);
+        if (anyI) guess_rows<true, false, !kTable>(S, own, k_all, inv_span, d0, g);
+        else if (anyII) guess_rows<false, true, !kTable>(S, own, k_all, inv_span, d0, g);
+        else guess_rows<false, false, !kTable>(S, own, k_all, inv_span, d0, g);
     }
     double wm[5];
 #pragma unroll
@@ -605,6 +647,17 @@ __device__ void carry_over(const FitArrays& fit, const JobArrays& job, int j, do
     }
 }
 
+// Both families' parameters in another unit of x, f old ones long.  Cold fits count x in rows of a lane's points (x = -m / L): the row
+// pitch is then 1, so that x steps exactly, no power of it is multiplied into the sums, and four registers fewer are spilled (100,000
+// windows of up to 1,000, with the logarithm by table: 3,615 -> 3,511 us).  The damping scales with the diagonal, so the iteration is the same in every unit.
+// Warm starts stay in the window's unit (a curve that ran off to infinity is carried over to a double root at one of the window's points,
+// which only the window's unit meets exactly), and so do teams, whose lanes have a row or two.
+__device__ __forceinline__ void rescale(double (&pI)[4], double (&pII)[4], double f) {
+    pI[0] *= f * f;
+    pI[1] *= f;
+    pII[1] *= f;
+}
+
 // The second round of a warm start: the families whose carried-over point had no finite
 // residual (`redo`, per lane for its own family) take their first guesses and are swept again.
 template <class Lanes>
@@ -642,7 +695,7 @@ struct FitClasses {
 // One slot of the work queue: the place-th warp's worth of jobs of class c.  kWarm: families may start from last epoch's
 // parameters (a separate instantiation, so that the plain one carries none of that code).  kL: lanes per job, a
 // constant, which takes branches and index arithmetic out of every step of a trial.
-template <bool kWarm, int kL, bool kTeam = false>
+template <bool kWarm, int kL, bool kRows, bool kTeam = false>
 __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& fit, const int32_t* __restrict__ order,
                                          const int32_t* __restrict__ start, const FitClasses& cls, int c, int place, int lm_trials,
                                          int min_fit_points, const double* wtab, const double* wsum, double* slice, unsigned long long* tally,
@@ -653,7 +706,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
     const int even = lane & ~1, oddl = lane | 1;
     constexpr int L = kL;
     const int h_hi = cls.h_hi[c];
-    LanesOf<kL> S;
+    LanesOf<kL, kRows> S;
     S.wtab = wtab;
     S.wsum = wsum;
     S.lane = lane;
@@ -691,6 +744,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
 
     if (__any_sync(kFull, fits)) {
         const double inv_span = 1.0 / span;
+        const double pitch = kRows ? (double)L : span;   // points per unit of x
         Moments mom = {0.0, 0.0};
         Family F = {};
         double pI[4] = {0.0, 0.0, 0.0, 0.0}, pII[4] = {0.0, 0.0, 0.0, 0.0};   // the points the next sweep evaluates
@@ -718,6 +772,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
         };
         if (!kWarm) {
             first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, wantsI, wantsII, mom, pI, pII);
+            if (kRows) rescale(pI, pII, pitch / span);
             sweep_at(fits, fits);
         } else {
             unsigned wmask = fits ? fit.warm_mask[j] : 0u;
@@ -770,7 +825,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
                 Sym4 A;
                 double gr[4], trial[4] = {0.0, 0.0, 0.0, 0.0};
                 normal_equations(S, fam, mom.sw, A, gr);
-                prepare_trial(F, fam, A, gr, !F.done, tiny_S, trial);
+                prepare_trial<kRows>(F, fam, A, gr, !F.done, tiny_S, span / pitch, trial);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {   // each lane of a pair fetches the other family's trial point
                     pI[a] = kTeam ? trial[a] : __shfl_sync(kFull, trial[a], even);
@@ -827,6 +882,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
                 pII[a] = __shfl_sync(kFull, F.p[a], oddl);
             }
         }
+        if (kRows) rescale(pI, pII, span / pitch);   // back to the window's coordinates
         if (fits) {
             if (ok_I) S_out[0] = S_I;
             if (ok_II) S_out[1] = S_II;
@@ -901,7 +957,8 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
 
 // kL: lanes per job if the launch has one length class - every cluster with windows of up to about 80 points, or with
 // few jobs; 0 where several classes share the launch, each then runs its own instance of fit_slot.
-template <bool kWarm, int kL>
+// kRows: false for warm starts (see rescale), and where one warp takes the place of a team of one and has to add as it does.
+template <bool kWarm, int kL, bool kRows>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1)
 fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
            const int32_t* __restrict__ start, FitClasses cls, int lm_trials, int min_fit_points,
@@ -948,7 +1005,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
 #define SLAQ_SLOT(n)                                                                                                              \
     case n:                                                                                                                       \
         if constexpr (kL == 0 || kL == n)                                                                                         \
-            fit_slot<kWarm, n>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, g_wtab + cls.h_max, slice, \
+            fit_slot<kWarm, n, kRows>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, g_wtab + cls.h_max, slice, \
                                tally[warp], lane, phases, err_word);                                                              \
         break;
             SLAQ_SLOT(2) SLAQ_SLOT(4) SLAQ_SLOT(8) SLAQ_SLOT(16) SLAQ_SLOT(32)
@@ -1002,12 +1059,12 @@ fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab,
     if constexpr (kListed) {
         const int jobs = start[0];   // the active ones, at the front of the list
         for (int place = blockIdx.x; place < jobs; place += gridDim.x) {
-            fit_slot<kWarm, 32, true>(job, fit, order, start, cls, 0, place, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+            fit_slot<kWarm, 32, false, true>(job, fit, order, start, cls, 0, place, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
                                       tally, lane, phases, err_word, team);
             __syncthreads();   // the exchanged results are read before the next job's are written
         }
     } else {
-        fit_slot<kWarm, 32, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+        fit_slot<kWarm, 32, false, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
                                   tally, lane, phases, err_word, team);
     }
     if (warp == 0 && lane < 6 && tally[lane]) {
@@ -1256,11 +1313,13 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 
 }  // namespace
 
-using FitKernel = decltype(&fit_kernel<false, 0>);
+using FitKernel = decltype(&fit_kernel<false, 0, true>);
 using FitTeamKernel = decltype(&fit_team_kernel<false, false>);
-static FitKernel const kFitKernels[2][6] = {
-    {fit_kernel<false, 0>, fit_kernel<false, 2>, fit_kernel<false, 4>, fit_kernel<false, 8>, fit_kernel<false, 16>, fit_kernel<false, 32>},
-    {fit_kernel<true, 0>, fit_kernel<true, 2>, fit_kernel<true, 4>, fit_kernel<true, 8>, fit_kernel<true, 16>, fit_kernel<true, 32>}};
+#define SLAQ_ALL(warm) \
+    {fit_kernel<warm, 0, !warm>, fit_kernel<warm, 2, !warm>, fit_kernel<warm, 4, !warm>, fit_kernel<warm, 8, !warm>, fit_kernel<warm, 16, !warm>, fit_kernel<warm, 32, !warm>}
+static FitKernel const kFitKernels[2][6] = {SLAQ_ALL(false), SLAQ_ALL(true)};
+#undef SLAQ_ALL
+static FitKernel const kFitAsTeam[2] = {fit_kernel<false, 32, false>, fit_kernel<true, 32, false>};   // see fit_kernel
 
 static FitTeamKernel const kFitTeamKernels[2][2] = {{fit_team_kernel<false, false>, fit_team_kernel<false, true>},
                                                     {fit_team_kernel<true, false>, fit_team_kernel<true, true>}};
@@ -1274,6 +1333,9 @@ int fit_setup() {
     for (const auto& row : kFitKernels)
         for (FitKernel k : row)
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
+                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    for (FitKernel k : kFitAsTeam)
+        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
                  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
     for (const void* k : {(const void*)length_scatter_kernel, (const void*)length_sort_kernel})
         ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1416,7 +1478,8 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
-    const FitKernel kernel = kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
+    const FitKernel kernel = parts == 1 ? kFitAsTeam[h->warm_start ? 1 : 0]
+                                        : kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
     if (e == cudaSuccess)
         e = launch_behind(kernel, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
                           h->scratch.start, cls, h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase, h->scratch.counters,

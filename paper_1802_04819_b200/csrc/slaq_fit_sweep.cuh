@@ -30,8 +30,10 @@ __device__ __forceinline__ double fast_rcp(double q) {
 // point, m = l + L k for the lane with index l in its group) sits at y[k * 32 + lane]:
 // every access of the sweeps is lane-private and free of bank conflicts.
 // kL: the lanes per job where all jobs of a launch have the same (a constant for the compiler), else 0.
-template <int kL>
+// kRows: x counts rows of a lane's points (x = -m / L; see rescale), else windows (x = -m / (H - 1)).
+template <int kL, bool kRows = true>
 struct LanesOf {
+    static constexpr bool kRowUnit = kRows;
     double* y;         // [k_cap + 1][32]
     double* park;      // this lane's family of its job in [kParked][2 * jobs per warp] (one column per job and family)
     const double* wtab;
@@ -39,6 +41,7 @@ struct LanesOf {
     int lane, l;
     int any_L;         // lanes per job (kL == 0)
     __device__ __forceinline__ int L() const { return kL ? kL : any_L; }
+    __device__ __forceinline__ const double* log_table() const { return wsum + 5 * (wtab_len + 1) + 1; }   // see log_of_normal
     __device__ __forceinline__ int park_stride() const { return 64 >> (__ffs(L()) - 1); }   // 2 * (32 / L), L() a power of two
     // Which of its family's 13 sums the lane holds after a sweep's reduction (see halve): `n` of them from the `from`-th on.
     __device__ __forceinline__ void held(int& from, int& n) const {
@@ -93,14 +96,27 @@ struct SweepSums {
     bool usable;   // the model was defined at every point and all sums are finite
 };
 
-// Running sums to sums of powers of x.  A lane walks its points from the oldest to the newest and keeps, for a
-// weighted value a, the chain c0 += a, c1 += c0, c2 += c1, ... in which every link adds the value its
-// predecessor had one step earlier; after the walk c_p = sum a_k C(k, p), k = the row of the point counted from
+// Running sums to sums of powers of u.  A lane walks its points from the oldest to the newest and keeps, for a
+// weighted value a, the chain c0 += a, c1 -= c0, c2 -= c1, ... in which every link takes the value its
+// predecessor had one step earlier; after the walk c_p = (-1)^p sum a_k C(k, p), k = the row of the point counted from
 // the lane's newest.  Powers of k are fixed combinations with positive coefficients (k^2 = 2 C(k,2) + C(k,1),
-// k^3 = 6 C(k,3) + 6 C(k,2) + C(k,1), k^4 = 24 C(k,4) + 36 C(k,3) + 14 C(k,2) + C(k,1)); with x = x_l + g k
-// (x_l <= 0 the lane's newest point, g < 0 the row pitch) the powers of x follow from a scaling by g^p and a shift
-// of the origin, all of whose terms have the sign of (-1)^p: nothing cancels, the sums are as accurate as if the
-// powers had been multiplied out point by point.
+// k^3 = 6 C(k,3) + 6 C(k,2) + C(k,1), k^4 = 24 C(k,4) + 36 C(k,3) + 14 C(k,2) + C(k,1)); with u = u_l - k
+// (u_l <= 0 the lane's newest point) the powers of u follow from a shift of the origin, all of whose terms have the sign
+// of (-1)^p: nothing cancels, the sums are as accurate as if the powers had been multiplied out point by point.
+template <int P>
+__device__ __forceinline__ void chains_to_powers(double (&c)[P], double u_l) {
+    const double c1 = P > 1 ? c[1] : 0.0, c2 = P > 2 ? c[2] : 0.0, c3 = P > 3 ? c[3] : 0.0;
+    if (P > 2) c[2] = fma(2.0, c2, -c1);
+    if (P > 3) c[3] = fma(6.0, c3, fma(-6.0, c2, c1));
+    if (P > 4) c[4] = fma(24.0, c[4], fma(-36.0, c3, fma(14.0, c2, -c1)));
+#pragma unroll
+    for (int j = 1; j < P; ++j)
+#pragma unroll
+        for (int p = P - 1; p >= j; --p) c[p] = fma(u_l, c[p - 1], c[p]);
+}
+
+// The same in a unit in which a row is g long (g < 0), from chains that add: the powers of k are scaled by g^p first.  For warm starts and the
+// teams, whose lanes have a row or two: nothing is gained there by counting in rows.
 template <int P>
 __device__ __forceinline__ void chains_to_powers(double (&c)[P], double x_l, double g) {
     const double c1 = P > 1 ? c[1] : 0.0, c2 = P > 2 ? c[2] : 0.0, c3 = P > 3 ? c[3] : 0.0;
@@ -124,8 +140,14 @@ struct LaneSums {
     int q_signs;     // OR of the high words of family I's denominators: negative if one of them had its sign bit set
 };
 
-// One point of a lane's walk: both families' values at the point and their running sums.
-template <bool kI, bool kII, class Lanes>
+template <bool kRows>
+__device__ __forceinline__ void link(double& c, double before) {
+    if (kRows) c -= before;
+    else c += before;
+}
+
+// One point of a lane's walk: both families' values at the point and their running sums.  kRows: x counts rows (see chains_to_powers).
+template <bool kI, bool kII, bool kRows, class Lanes>
 __device__ __forceinline__ void add_point(const Lanes& S, const double* wp, const double* yp, double x,
                                           const double (&pI)[4], const double (&pII)[4], double& e, double ratio,
                                           LaneSums& a) {
@@ -138,18 +160,18 @@ __device__ __forceinline__ void add_point(const Lanes& S, const double* wp, cons
         const double r = y - (inv + pI[3]);
         const double u = inv * inv;
         const double wu = w * u, wuu = wu * u, wur = wu * r, wr = w * r;
-        a.m[4] += a.m[3]; a.m[3] += a.m[2]; a.m[2] += a.m[1]; a.m[1] += a.m[0]; a.m[0] += wuu;
-        a.n[2] += a.n[1]; a.n[1] += a.n[0]; a.n[0] += wu;
-        a.h[2] += a.h[1]; a.h[1] += a.h[0]; a.h[0] += wur;
+        link<kRows>(a.m[4], a.m[3]); link<kRows>(a.m[3], a.m[2]); link<kRows>(a.m[2], a.m[1]); link<kRows>(a.m[1], a.m[0]); a.m[0] += wuu;
+        link<kRows>(a.n[2], a.n[1]); link<kRows>(a.n[1], a.n[0]); a.n[0] += wu;
+        link<kRows>(a.h[2], a.h[1]); link<kRows>(a.h[1], a.h[0]); a.h[0] += wur;
         a.gd += wr;
         a.sI = fma(wr, r, a.sI);
     }
     if (kII) {
         const double r = y - (e + pII[2]);
         const double we = w * e, wee = we * e, wer = we * r, wr = w * r;
-        a.ee[2] += a.ee[1]; a.ee[1] += a.ee[0]; a.ee[0] += wee;
-        a.f[1] += a.f[0]; a.f[0] += we;
-        a.kk[1] += a.kk[0]; a.kk[0] += wer;
+        link<kRows>(a.ee[2], a.ee[1]); link<kRows>(a.ee[1], a.ee[0]); a.ee[0] += wee;
+        link<kRows>(a.f[1], a.f[0]); a.f[0] += we;
+        link<kRows>(a.kk[1], a.kk[0]); a.kk[0] += wer;
         a.gc += wr;
         a.sII = fma(wr, r, a.sII);
         e *= ratio;
@@ -161,33 +183,31 @@ __device__ __forceinline__ void add_point(const Lanes& S, const double* wp, cons
 // parameters nobody uses and its sums are discarded).  Branches inside the loop cost issue slots on every row:
 // the rows that every lane of the warp has are walked without a test, only the ragged rest with one.
 template <bool kI, bool kII, class Lanes>
-__device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all, double inv_span,
-                                          const double (&pI)[4], const double (&pII)[4], LaneSums& a) {
+__device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all, double inv_span, const double (&pI)[4],
+                                          const double (&pII)[4], LaneSums& a) {
     const int mi = S.l + k_last * S.L();
-    const double md = (double)mi;
-    const double dL = (double)S.L();
-    // x from the lane's oldest point by one addition per row (its rounding, at most a few 1e-15 absolute at the
-    // newest point, moves the predictions as little as the exponential's recurrence does: measured)
-    double x = -md * inv_span;
-    const double hx = dL * inv_span;
-    // e = exp(alpha - beta x) with x = -m / span falls geometrically towards the newest point: one
+    // in rows x and its steps are exact
+    constexpr bool kRows = Lanes::kRowUnit;
+    const double md = (double)mi, hx = kRows ? 1.0 : (double)S.L() * inv_span;
+    double x = kRows ? md * (-1.0 / (double)S.L()) : -md * inv_span;
+    // e = exp(alpha - beta x) falls geometrically towards the newest point: one
     // exact value at the lane's oldest point, then a constant ratio per step.  (Choosing the start such
     // that the recurrence lands on the exact value at the newest point was measured: the predictions stay
     // as close to the reference's either way, and the extra arithmetic costs 2 % of the kernel.)
     double e = 0.0, ratio = 1.0;
     if (kII) {
-        e = exp(fma(pII[1], md * inv_span, pII[0]));
-        ratio = exp(-pII[1] * (dL * inv_span));
+        e = exp(fma(-pII[1], x, pII[0]));
+        ratio = exp(-pII[1] * hx);
     }
     const double* yp = S.y + S.lane + k_last * 32;
     const double* wp = S.wtab + mi;
     const int k_min = __reduce_min_sync(kFull, k_last);
     int i = 0;
 #pragma unroll 1   // unrolling was measured (2 rows per step): slower, more spills
-    for (; i <= k_min; ++i, x += hx, yp -= 32, wp -= S.L()) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);
+    for (; i <= k_min; ++i, x += hx, yp -= 32, wp -= S.L()) add_point<kI, kII, kRows>(S, wp, yp, x, pI, pII, e, ratio, a);
 #pragma unroll 1
     for (; i < k_all; ++i, x += hx, yp -= 32, wp -= S.L())
-        if (i <= k_last) add_point<kI, kII>(S, wp, yp, x, pI, pII, e, ratio, a);   // row k_last - i >= 0
+        if (i <= k_last) add_point<kI, kII, kRows>(S, wp, yp, x, pI, pII, e, ratio, a);   // row k_last - i >= 0
 }
 
 // One step of the reduction over the lanes of a group: of N sums a lane keeps the lower K (bit `o` of its number clear) or
@@ -226,14 +246,15 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     }
     double (&m)[5] = a.m, (&n)[3] = a.n, (&h)[3] = a.h, (&ee)[3] = a.ee, (&f)[2] = a.f, (&kk)[2] = a.kk;
     const double gd = a.gd, sI = a.sI, gc = a.gc, sII = a.sII;
-    const double dL = (double)S.L();
-    const double x_l = -(double)S.l * inv_span, g = -dL * inv_span;
-    chains_to_powers(m, x_l, g);
-    chains_to_powers(n, x_l, g);
-    chains_to_powers(h, x_l, g);
-    chains_to_powers(ee, x_l, g);
-    chains_to_powers(f, x_l, g);
-    chains_to_powers(kk, x_l, g);
+    if constexpr (Lanes::kRowUnit) {
+        const double x_l = (double)S.l * (-1.0 / (double)S.L());
+        chains_to_powers(m, x_l), chains_to_powers(n, x_l), chains_to_powers(h, x_l);
+        chains_to_powers(ee, x_l), chains_to_powers(f, x_l), chains_to_powers(kk, x_l);
+    } else {
+        const double x_l = -(double)S.l * inv_span, g = -((double)S.L() * inv_span);
+        chains_to_powers(m, x_l, g), chains_to_powers(n, x_l, g), chains_to_powers(h, x_l, g);
+        chains_to_powers(ee, x_l, g), chains_to_powers(f, x_l, g), chains_to_powers(kk, x_l, g);
+    }
     // pair step: an even lane hands over its family-II partials and receives family-I ones, an odd lane the reverse
     const bool odd = fam != 0;
     double v[13];
@@ -304,7 +325,7 @@ __device__ __forceinline__ int team_index(int lane) {
 // One sweep of one family by its team: half the arithmetic per point, no exchange between families, and a lane has
 // as few rows as the team has lanes.
 template <int kFam>
-__device__ __forceinline__ void sweep_team(const LanesOf<32>& S, Team& t, int H, double inv_span, const double (&p)[4], SweepSums& out) {
+__device__ __forceinline__ void sweep_team(const LanesOf<32, false>& S, Team& t, int H, double inv_span, const double (&p)[4], SweepSums& out) {
     LaneSums a = {};
     const int LT = 1 << t.shift, lt = S.lane + 32 * t.part;
     const int k_last = H - 1 - lt >= 0 ? (H - 1 - lt) >> t.shift : -1;
@@ -320,7 +341,7 @@ __device__ __forceinline__ void sweep_team(const LanesOf<32>& S, Team& t, int H,
     const double* wp = S.wtab + mi;
 #pragma unroll 1
     for (int i = 0; i < k_all; ++i, x += hx, yp -= LT, wp -= LT)
-        if (i <= k_last) add_point<kFam == 0, kFam == 1>(S, wp, yp, x, p, p, e, ratio, a);
+        if (i <= k_last) add_point<kFam == 0, kFam == 1, false>(S, wp, yp, x, p, p, e, ratio, a);
     const double x_l = -(double)lt * inv_span, g = -hx;
     double v[13];
     if (kFam == 0) {
@@ -367,11 +388,10 @@ __device__ __forceinline__ void sweep_objective(const Lanes& S, int fam, int H, 
     const int shift = __ffs(S.L()) - 1;
     const int k_last = H - 1 - S.l >= 0 ? (H - 1 - S.l) >> shift : -1;
     const int mi = S.l + k_last * S.L();
-    const double md = (double)mi, dL = (double)S.L();
-    double x = -md * inv_span;
-    const double hx = dL * inv_span;
-    double e = exp(fma(pII[1], md * inv_span, pII[0]));
-    const double ratio = exp(-pII[1] * (dL * inv_span));
+    const double md = (double)mi, hx = Lanes::kRowUnit ? 1.0 : (double)S.L() * inv_span;
+    double x = Lanes::kRowUnit ? md * (-1.0 / (double)S.L()) : -md * inv_span;
+    double e = exp(fma(-pII[1], x, pII[0]));
+    const double ratio = exp(-pII[1] * hx);
     double sI = 0.0, sII = 0.0;
     int q_signs = 0;
     const double* yp = S.y + S.lane + k_last * 32;

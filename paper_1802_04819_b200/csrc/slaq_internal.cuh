@@ -18,6 +18,8 @@ constexpr int kRadixBits = 11;
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kRadixPasses = 6;       // 11 + 11 + 11 + 11 + 11 + 9 bits, most significant first
 constexpr int kMaxFitClasses = 8;     // window-length classes of the fit (one launch each)
+constexpr int kLogBins = 128;          // first guesses: the logarithm's table (see log_of_normal), its first bin and the width of a bin
+constexpr int kLogFrom = 0x3fe6b000, kLogBinShift = 13;   // in high words; 1 is the middle of bin 74
 constexpr int kFitQueueBase = 8;      // ticket[kFitQueueBase + c]: work queue head of class c
 constexpr int kTickets = 16;
 
@@ -175,7 +177,7 @@ struct slaq_handle {
     size_t packed_len = 0;
     void* call_buf = nullptr;         // scratch of calls that move caller data of any size (grown on demand, kept)
     size_t call_buf_bytes = 0;
-    double* wtab = nullptr;           // gamma^m, m = 0..max_hist-1, then the sums over m < H of gamma^m m^p: [5][max_hist + 1]
+    double* wtab = nullptr;           // gamma^m, m = 0..max_hist-1, then the sums over m < H of gamma^m m^p: [5][max_hist + 1], then (16-byte aligned) the logarithm's table
     double wtab_gamma = -1.0;
     slaq::JobArrays job;
     slaq::FitArrays fit;

@@ -1,5 +1,5 @@
-"""The fits' starting points (no trials at all) against the oracle's: the sign of family I's
-quadratic read off its lowest point are used nowhere else."""
+"""The fits' starting points (no trials at all) against the oracle's: the logarithm by table and the sign of family I's quadratic read off
+its lowest point are used nowhere else.  The second number of jobs is beyond what teams fit."""
 
 import numpy as np
 import pytest
@@ -29,11 +29,12 @@ def _windows():
     return out
 
 
-@pytest.mark.parametrize("warm", [0, 1])
-def test_first_guesses_match_the_oracle(oracle_mod, warm):
+@pytest.mark.parametrize("warm,copies", [(0, 1), (1, 1), (0, 8)])
+def test_first_guesses_match_the_oracle(oracle_mod, warm, copies):
     import paper_1802_04819_b200 as slaq
     rows = _windows()
-    J = len(rows)
+    n, J = len(rows), len(rows) * copies
+    rows = rows * copies
     sched = slaq.Scheduler(J, 200, 16)
     sched.set_param(slaq.binding.P_LM_TRIALS, 0)
     sched.set_param(slaq.binding.P_WARM_START, warm)
@@ -46,7 +47,11 @@ def test_first_guesses_match_the_oracle(oracle_mod, warm):
     sched.schedule(1.0, 4 * J)
     st = sched.get_fit_state()
     lines = 0
-    for j, (h, m_seen) in enumerate(rows):
+    for k in range(1, copies):
+        same = st["valid"][:n] != 0
+        np.testing.assert_array_equal(st["valid"][k * n: (k + 1) * n], st["valid"][:n])
+        np.testing.assert_array_equal(st["p"][k * n: (k + 1) * n][same], st["p"][:n][same])
+    for j, (h, m_seen) in enumerate(rows[:n]):
         for fam in (0, 1):
             ref = oracle_mod.fit_family(fam, h, m_seen, trials=0)
             got, p0 = st["p"][j, 4 * fam: 4 * fam + 4], ref["p0"]
@@ -58,4 +63,4 @@ def test_first_guesses_match_the_oracle(oracle_mod, warm):
                 lines += p0[0] == 0.0
             # weighted normal equations in x, x^2, 1 of up to 200 points: conditions up to some 1e6 times a few ulp
             np.testing.assert_allclose(got[:3 + (fam == 0)], p0[:3 + (fam == 0)], rtol=1e-7, atol=1e-9 * np.abs(p0).max())
-    assert 0 < lines < J
+    assert 0 < lines < n
