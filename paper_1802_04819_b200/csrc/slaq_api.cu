@@ -1390,7 +1390,7 @@ int slaq_schedule_group(slaq_t* const* handles, int32_t n, double epoch_seconds,
     if (n > 1) CK(cudaEventRecord(h->order_event(0), st), "event");
     // The fits run beside one another.  Few jobs: each gets SMs in proportion to its jobs, so that no fit waits for another's
     // last windows; many jobs: each may use the whole GPU and starts where the one before it runs out of work.
-    const bool split = active * fit_least_lanes(h) <= 4LL * 32 * 16 * h->sm_count;
+    const bool split = active * fit_least_lanes(h) <= 4LL * 32 * 12 * h->sm_count;
     int free_sms = h->sm_count;
     for (int32_t s = 0; s < n; ++s) {
         slaq_t* const g = handles[s];

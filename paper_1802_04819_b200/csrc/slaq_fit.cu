@@ -11,7 +11,7 @@
 // length classes.  In class c a group of L lanes (L = 2, 4, .. 32: the fewest lanes at which
 // the window fits the rows of a warp's shared-memory slice) owns one job (so a warp carries
 // 32/L jobs; with fewer jobs L is raised where a shorter chain of rows is worth the work, see
-// fit_least_lanes).  One persistent launch (one block of 16 warps per SM) serves all classes from one work queue,
+// fit_plan).  One persistent launch (one block of 8, 12 or 16 warps per SM, see fit_plan) serves all classes from one work queue,
 // longest windows first.  A lane walks its job's points m = l, l + L, l + 2L, ... counted
 // from the newest one; both families
 // are evaluated in the same sweep over the window; the partial sums of the normal equations
@@ -52,6 +52,11 @@ struct Phases {
 #endif
 
 constexpr int kMaxWarpsPerBlock = 16;          // one block per SM: its warps share one copy of the weight table
+// Warps of the fit kernel's block and shared memory of each.  Fewer warps have larger slices, so that a job needs fewer lanes, and more registers (128, 168, 255 a
+// thread at 16, 12, 8), which spill nothing and, at 8, let two rows overlap.
+constexpr int kFitWarps[3] = {16, 12, 8};
+constexpr size_t kFitSlices[3] = {kDefaultFitSlice, 18432, 27648};
+enum { kSixteen, kTwelve, kEight };
 constexpr size_t kSmemLimit = 226 * 1024;   // shared memory one block may use on sm_100, less the static part
 constexpr int kTeamWarps = 8;               // warps of a block that works on one job
 constexpr size_t kTeamSmem = 220 * 1024;
@@ -695,7 +700,7 @@ struct FitClasses {
 // One slot of the work queue: the place-th warp's worth of jobs of class c.  kWarm: families may start from last epoch's
 // parameters (a separate instantiation, so that the plain one carries none of that code).  kL: lanes per job, a
 // constant, which takes branches and index arithmetic out of every step of a trial.
-template <bool kWarm, int kL, bool kRows, bool kTeam = false>
+template <bool kWarm, int kL, bool kRows, int kStep, bool kTeam = false>
 __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& fit, const int32_t* __restrict__ order,
                                          const int32_t* __restrict__ start, const FitClasses& cls, int c, int place, int lm_trials,
                                          int min_fit_points, const double* wtab, const double* wsum, double* slice, unsigned long long* tally,
@@ -706,7 +711,7 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
     const int even = lane & ~1, oddl = lane | 1;
     constexpr int L = kL;
     const int h_hi = cls.h_hi[c];
-    LanesOf<kL, kRows> S;
+    LanesOf<kL, kRows, kStep> S;
     S.wtab = wtab;
     S.wsum = wsum;
     S.lane = lane;
@@ -958,14 +963,14 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
 // kL: lanes per job if the launch has one length class - every cluster with windows of up to about 80 points, or with
 // few jobs; 0 where several classes share the launch, each then runs its own instance of fit_slot.
 // kRows: false for warm starts (see rescale), and where one warp takes the place of a team of one and has to add as it does.
-template <bool kWarm, int kL, bool kRows>
-__global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1)
+template <bool kWarm, int kL, int kWarps, bool kRows = !kWarm>
+__global__ void __launch_bounds__(kWarps * 32, 1)
 fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, const int32_t* __restrict__ order,
            const int32_t* __restrict__ start, FitClasses cls, int lm_trials, int min_fit_points,
            unsigned int* queue, long long* counters, long long* stamp, int32_t* err_word) {
     extern __shared__ double smem[];
     __shared__ int slot_base[kMaxFitClasses + 1], dealt;
-    __shared__ unsigned long long tally[kMaxWarpsPerBlock][6];   // statistics of a warp's jobs, out of its registers
+    __shared__ unsigned long long tally[kWarps][6];   // statistics of a warp's jobs, out of its registers
     double* wtab = smem;                                   // [h_max]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* const slice = smem + cls.h_max + (size_t)warp * cls.slice;   // this warp's: parked sums, then the window rows
@@ -1005,7 +1010,7 @@ fit_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab, cons
 #define SLAQ_SLOT(n)                                                                                                              \
     case n:                                                                                                                       \
         if constexpr (kL == 0 || kL == n)                                                                                         \
-            fit_slot<kWarm, n, kRows>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, g_wtab + cls.h_max, slice, \
+            fit_slot<kWarm, n, kRows, kWarps == 8 ? 2 : 1>(job, fit, order, start, cls, c, place, lm_trials, min_fit_points, wtab, g_wtab + cls.h_max, slice, \
                                tally[warp], lane, phases, err_word);                                                              \
         break;
             SLAQ_SLOT(2) SLAQ_SLOT(4) SLAQ_SLOT(8) SLAQ_SLOT(16) SLAQ_SLOT(32)
@@ -1059,12 +1064,12 @@ fit_team_kernel(JobArrays job, FitArrays fit, const double* __restrict__ g_wtab,
     if constexpr (kListed) {
         const int jobs = start[0];   // the active ones, at the front of the list
         for (int place = blockIdx.x; place < jobs; place += gridDim.x) {
-            fit_slot<kWarm, 32, false, true>(job, fit, order, start, cls, 0, place, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+            fit_slot<kWarm, 32, false, 1, true>(job, fit, order, start, cls, 0, place, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
                                       tally, lane, phases, err_word, team);
             __syncthreads();   // the exchanged results are read before the next job's are written
         }
     } else {
-        fit_slot<kWarm, 32, false, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
+        fit_slot<kWarm, 32, false, 1, true>(job, fit, nullptr, nullptr, cls, 0, blockIdx.x, lm_trials, min_fit_points, smem, g_wtab + cls.h_max, slice,
                                   tally, lane, phases, err_word, team);
     }
     if (warp == 0 && lane < 6 && tally[lane]) {
@@ -1313,13 +1318,18 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 
 }  // namespace
 
-using FitKernel = decltype(&fit_kernel<false, 0, true>);
+using FitKernel = decltype(&fit_kernel<false, 0, 12>);
 using FitTeamKernel = decltype(&fit_team_kernel<false, false>);
-#define SLAQ_ALL(warm) \
-    {fit_kernel<warm, 0, !warm>, fit_kernel<warm, 2, !warm>, fit_kernel<warm, 4, !warm>, fit_kernel<warm, 8, !warm>, fit_kernel<warm, 16, !warm>, fit_kernel<warm, 32, !warm>}
-static FitKernel const kFitKernels[2][6] = {SLAQ_ALL(false), SLAQ_ALL(true)};
+// [warps][warm start][lanes: 0 for several, 2, 4, .. 32]; null: never chosen
+#define SLAQ_ALL(warm, w, two) \
+    {fit_kernel<warm, 0, w>, two, fit_kernel<warm, 4, w>, fit_kernel<warm, 8, w>, fit_kernel<warm, 16, w>, fit_kernel<warm, 32, w>}
+static FitKernel const kFitKernels[3][2][6] = {
+    {{nullptr, fit_kernel<false, 2, 16>}, {nullptr, fit_kernel<true, 2, 16>}},
+    {SLAQ_ALL(false, 12, (fit_kernel<false, 2, 12>)), SLAQ_ALL(true, 12, (fit_kernel<true, 2, 12>))},
+    {{nullptr, fit_kernel<false, 2, 8>, fit_kernel<false, 4, 8>, fit_kernel<false, 8, 8>, fit_kernel<false, 16, 8>, fit_kernel<false, 32, 8>},
+     {nullptr, fit_kernel<true, 2, 8>, fit_kernel<true, 4, 8>, fit_kernel<true, 8, 8>, fit_kernel<true, 16, 8>, fit_kernel<true, 32, 8>}}};
 #undef SLAQ_ALL
-static FitKernel const kFitAsTeam[2] = {fit_kernel<false, 32, false>, fit_kernel<true, 32, false>};   // see fit_kernel
+static FitKernel const kFitAsTeam[2] = {fit_kernel<false, 32, 8, false>, fit_kernel<true, 32, 8, false>};   // see fit_kernel
 
 static FitTeamKernel const kFitTeamKernels[2][2] = {{fit_team_kernel<false, false>, fit_team_kernel<false, true>},
                                                     {fit_team_kernel<true, false>, fit_team_kernel<true, true>}};
@@ -1330,10 +1340,11 @@ int fit_setup() {
         for (FitTeamKernel k : row)
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmem) == cudaSuccess &&
                  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-    for (const auto& row : kFitKernels)
-        for (FitKernel k : row)
-            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
-                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    for (const auto& warps : kFitKernels)
+        for (const auto& row : warps)
+            for (FitKernel k : row)
+                ok = ok && (!k || (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
+                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess));
     for (FitKernel k : kFitAsTeam)
         ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
                  cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
@@ -1349,8 +1360,8 @@ static long long jobs_for_lanes(const slaq_handle* h) {
 
 // Doubles of shared memory per warp: the parked sums, the window rows and one spare row.  It grows if the longest window
 // does not fit at 32 lanes.
-static int fit_slice(const slaq_handle* h) {
-    return std::max((int)(h->fit_slice_bytes / sizeof(double)), kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32);
+static int fit_slice(const slaq_handle* h, size_t bytes) {
+    return std::max((int)(bytes / sizeof(double)), kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32);
 }
 static int team_slice(const slaq_handle* h) { return kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32; }
 static size_t team_smem(const slaq_handle* h, int parts) {
@@ -1358,29 +1369,52 @@ static size_t team_smem(const slaq_handle* h, int parts) {
 }
 static int rows_at(int slice, int L) { return (slice - kParked * (64 / L)) / 32 - 1; }
 
-// The fewest lanes a job gets.  Fewer lanes are less work - the solver's step and the reductions of a trial cost a warp
-// the same whatever it carries - and longer chains of rows.  Cycles per trial, fitted to clusters of 1,000 to 32,000 jobs
-// with windows of up to 12 to 1,000 points, full or ragged, at 2 to 32 lanes each: a warp alone takes 2300 + 170 per row,
-// and a sub-partition can issue 1300 + 106 per row for each of its warps, of which a part counts nearly as a whole one; the
-// longer of the two decides, over the lane counts at which every window fits.  That choice is within 1.3 % of the best on
-// average; filling every warp of the GPU twice, the rule before, cost 36 % (fit of 8,000 windows of up to 100: 282 -> 118 us).
-// Beyond one slot per warp of the GPU more lanes only add work, although the longest windows then get more lanes than
-// the others (100,000 windows of up to 1,000: 4.9 ms with 32 lanes for all, 4.0 with 2 and up).
-int fit_least_lanes(const slaq_handle* h) {
-    const int slice = fit_slice(h), Hmax = h->max_hist;
-    const double jobs = (double)std::max(1LL, jobs_for_lanes(h));
-    int best = 32;
-    double least = 0.0;
-    for (int L = 32; L >= 2 && rows_at(slice, L) * L >= Hmax; L >>= 1) {
-        const int rows = (Hmax + L - 1) / L;
-        double warps = std::ceil(jobs * L / 32.0) / (4.0 * h->sm_count);   // per sub-partition
-        if (warps < 4.0) warps = std::min(std::ceil(warps), warps + 0.3);
-        const double cycles = std::max(2300.0 + 170.0 * rows, warps * (1300.0 + 106.0 * rows));
-        if (L == 32 || cycles <= least) best = L, least = cycles;
+// The warps of a block and the fewest lanes a job gets, from the cluster's jobs and the longest window alone.  Fewer lanes are less
+// work - the solver's step and the reductions of a trial cost a warp the same whatever it carries - and longer chains of rows.  Fewer
+// warps have room for fewer lanes, and leave issue slots empty.  Costs in cycles per trial: a warp alone takes `chain` + `chain_row` per row, a
+// sub-partition issues `issue` + `issue_row` per row for each of its warps, of which a part counts `part` more; slots beyond what is
+// resident are another wave, of which `mixed` is hidden behind the one before.  Every window is taken for full, and a fifth of the jobs,
+// half the time, for new ones of a few points.  Fitted to the fits of 700 to 200,000 windows of 20 to 1,000 points at 8, 12 and 16 warps and
+// 2 to 32 lanes: full ones 2.4 % from the best choice on average, ragged ones 2.9 %, a fifth of them new 6.3 %.  Sixteen warps for
+// all with the lanes they have room for, the rule before, were 7.4, 9.6 and 11.2 % from it.
+struct FitPlan {
+    int kind, lanes;   // index into kFitWarps; least lanes
+    size_t slice_bytes;
+};
+static FitPlan fit_plan(const slaq_handle* h) {
+    constexpr struct {
+        double chain, chain_row, issue, issue_row, part, mixed;
+    } cost_of[3] = {{4600, 315, 1230, 95, 0.5, 0.55}, {3600, 220, 1250, 97, 0.9, 0.4}, {3300, 190, 1340, 106, 0.1, 0.4}};
+    const int Hmax = h->max_hist;
+    const double jobs = (double)std::max(1LL, jobs_for_lanes(h)), sub = 4.0 * h->sm_count;
+    const bool by_size = h->fit_slice_bytes == kDefaultFitSlice;
+    FitPlan best = {kTwelve, 32, by_size ? kFitSlices[kTwelve] : h->fit_slice_bytes};
+    double least = -1.0;
+    for (int L = 32; L >= 2; L >>= 1) {
+        for (int kind : {kTwelve, kEight, kSixteen}) {
+            const size_t bytes = by_size ? kFitSlices[kind] : h->fit_slice_bytes;
+            if (rows_at(fit_slice(h, bytes), L) * L < Hmax) continue;
+            if (kind != kTwelve && !by_size) continue;
+            if (kind == kSixteen && L > 2) continue;   // more lanes are always better off with more registers
+            const auto& c = cost_of[kind];
+            const double rows = (Hmax + L - 1) / L, chain = c.chain + c.chain_row * rows, each = c.issue + c.issue_row * rows;
+            const double resident = kFitWarps[kind] / 4;
+            auto wave = [&](double n) { return n > 0.02 ? std::max(chain, std::min(std::ceil(n), n + c.part) * each) : 0.0; };
+            auto cycles = [&](double n) {   // n slots per sub-partition
+                const double full = std::floor(n / resident);
+                const double stepped = full * wave(resident) + wave(n - full * resident);
+                return c.mixed * n * std::max(each, chain / resident) + (1.0 - c.mixed) * stepped;
+            };
+            const double slots = jobs * L / 32.0 / sub, cost = cycles(slots) + cycles(0.8 * slots);
+            if (least < 0.0 || cost <= least) best = {kind, L, bytes}, least = cost;
+        }
     }
-    while (best > 2 && jobs * (best / 2) >= 32.0 * kMaxWarpsPerBlock * h->sm_count) best >>= 1;
+    // Beyond a wave and a half more lanes only add work, although the longest windows then get more lanes than the others.
+    if (best.kind == kTwelve)
+        while (best.lanes > 2 && jobs * (best.lanes / 2) >= 1.5 * 32.0 * kFitWarps[kTwelve] * h->sm_count) best.lanes >>= 1;
     return best;
 }
+int fit_least_lanes(const slaq_handle* h) { return fit_plan(h).lanes; }
 
 // Warps per family of a job's team; 0: no teams.  A question of the cluster's active jobs and the windows alone, which every shard
 // answers alike, whatever its capacity: several warps add in another order than one, and one in another than a part of one.  With a warp per sub-partition at most, a lane is left four rows of the longest
@@ -1449,8 +1483,10 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     FitClasses cls;
     cls.n = 0;
     cls.h_max = Hmax;
-    cls.slice = fit_slice(h);
-    const int L_min = parts == 1 ? 32 : fit_least_lanes(h);
+    const FitPlan plan = parts == 1 ? FitPlan{kEight, 32, kFitSlices[kEight]} : fit_plan(h);
+    const int max_warps = kFitWarps[plan.kind];
+    cls.slice = fit_slice(h, plan.slice_bytes);
+    const int L_min = plan.lanes;
     int h_hi = Hmax;
     for (int L = 32; L >= L_min && h_hi > 0; L >>= 1) {
         const int h_lo = L > L_min ? std::max(rows_at(cls.slice, L / 2), 0) * (L / 2) : 0;
@@ -1463,13 +1499,13 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
     }
     for (int c = cls.n; c < kMaxFitClasses; ++c) cls.h_lo[c] = cls.h_hi[c] = 0, cls.L[c] = 32;
     // A job per warp of the GPU and no more: every job starts at once, so their order means nothing and none is made.
-    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * kMaxWarpsPerBlock;
+    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * max_warps;
     cudaError_t e = in_order ? cudaSuccess : launch_sort(h, st, &launches);
     // One block per SM: its registers and shared memory fill one.  Where there are fewer slots than warps every SM gets
     // its share of them.
     const long long slots = ((long long)J * cls.L[0] + 31) / 32;   // at most
     const int blocks = (int)std::max(1LL, std::min((long long)max_blocks, slots));
-    int warps = kMaxWarpsPerBlock;
+    int warps = max_warps;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
     warps = (int)std::min((long long)warps, (slots + blocks - 1) / blocks);
     // more than half of an SM's shared memory: no SM gets two blocks while another one still holds the kernel before
@@ -1479,7 +1515,7 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         return -1;
     }
     const FitKernel kernel = parts == 1 ? kFitAsTeam[h->warm_start ? 1 : 0]
-                                        : kFitKernels[h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
+                                        : kFitKernels[plan.kind][h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
     if (e == cudaSuccess)
         e = launch_behind(kernel, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
                           h->scratch.start, cls, h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase, h->scratch.counters,

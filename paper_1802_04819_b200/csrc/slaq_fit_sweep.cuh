@@ -31,8 +31,10 @@ __device__ __forceinline__ double fast_rcp(double q) {
 // every access of the sweeps is lane-private and free of bank conflicts.
 // kL: the lanes per job where all jobs of a launch have the same (a constant for the compiler), else 0.
 // kRows: x counts rows of a lane's points (x = -m / L; see rescale), else windows (x = -m / (H - 1)).
-template <int kL, bool kRows = true>
+// kStep: rows a sweep's walk takes at once, where registers are there for two.
+template <int kL, bool kRows = true, int kStep = 1>
 struct LanesOf {
+    static constexpr int kRowsAtOnce = kStep;
     static constexpr bool kRowUnit = kRows;
     double* y;         // [k_cap + 1][32]
     double* park;      // this lane's family of its job in [kParked][2 * jobs per warp] (one column per job and family)
@@ -203,7 +205,7 @@ __device__ __forceinline__ void walk_rows(const Lanes& S, int k_last, int k_all,
     const double* wp = S.wtab + mi;
     const int k_min = __reduce_min_sync(kFull, k_last);
     int i = 0;
-#pragma unroll 1   // unrolling was measured (2 rows per step): slower, more spills
+#pragma unroll Lanes::kRowsAtOnce
     for (; i <= k_min; ++i, x += hx, yp -= 32, wp -= S.L()) add_point<kI, kII, kRows>(S, wp, yp, x, pI, pII, e, ratio, a);
 #pragma unroll 1
     for (; i < k_all; ++i, x += hx, yp -= 32, wp -= S.L())

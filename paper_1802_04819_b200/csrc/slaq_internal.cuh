@@ -20,6 +20,7 @@ constexpr int kRadixPasses = 6;       // 11 + 11 + 11 + 11 + 11 + 9 bits, most s
 constexpr int kMaxFitClasses = 8;     // window-length classes of the fit (one launch each)
 constexpr int kLogBins = 128;          // first guesses: the logarithm's table (see log_of_normal), its first bin and the width of a bin
 constexpr int kLogFrom = 0x3fe6b000, kLogBinShift = 13;   // in high words; 1 is the middle of bin 74
+constexpr size_t kDefaultFitSlice = 13824;
 constexpr int kFitQueueBase = 8;      // ticket[kFitQueueBase + c]: work queue head of class c
 constexpr int kTickets = 16;
 
@@ -159,7 +160,7 @@ struct slaq_handle {
     int32_t max_cores = 64;
     double gamma = 0.9;
     int32_t lm_trials = 20, min_fit_points = 4;
-    size_t fit_slice_bytes = 13824;       // shared memory one warp of the fit kernel may use (parked sums, up to 52 rows of 32 points, a spare row)
+    size_t fit_slice_bytes = slaq::kDefaultFitSlice;   // shared memory one warp of the fit kernel may use (parked sums, rows of 32 points, a spare row); the default: by size
     bool warm_start = false;              // fits start from the last epoch's parameters where there are some
     int selection = 0;                    // SLAQ_P_SELECTION: kept for callers that ask, read by nothing else
     bool gain_partial = false;            // h->gain holds the last epoch's rows only in part (see GainBasis)
