@@ -96,13 +96,12 @@ constexpr int kSelectMaxGrid = 4096;
 
 // Global memory of the selection launch.  The leading part is cleared before every launch.
 struct SelectGlobal {
-    unsigned long long coarse[32];                        // first histogram: one total per power of two ..
-    unsigned long long fine[kSelectFineBins];             // .. and its 64 bins each
-    unsigned int barrier, ticket, n_cand, pad;            // blocks that arrived; blocks that finished; listed candidates
-    static constexpr size_t kZeroBytes = sizeof(unsigned long long) * (32 + kSelectFineBins) + 16;
-    // cleared by the kernel itself: the counts of continued rows, apart from the first ones, which slower blocks may still
-    // be reading when the first of these arrive; the histograms of the narrowing steps
-    unsigned long long coarse_more[32], fine_more[kSelectFineBins];
+    unsigned long long fine[kSelectFineBins];             // first histogram: 64 bins per power of two
+    unsigned int barrier, ticket, n_cand, sampled;        // blocks that arrived; blocks that finished; listed candidates; rows in the sample
+    static constexpr size_t kZeroBytes = sizeof(unsigned long long) * kSelectFineBins + 16;
+    // cleared by the kernel itself: later histograms, apart from the first one, which slower blocks may still be reading when
+    // the first of these counts arrive; the histograms of the narrowing steps
+    unsigned long long fine_more[kSelectFineBins], fine_rest[kSelectFineBins];
     unsigned long long narrow[kRadixPasses][kRadixBins];
     unsigned long long cand_key[kSelectCandidates];       // the candidates the last block ranks ..
     unsigned long long cand_pos[kSelectCandidates];       // .. and their (candidates of the row, job, n)

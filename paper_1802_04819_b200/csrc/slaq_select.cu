@@ -26,7 +26,8 @@
 // How much of a row is looked at.  Jobs get few cores on average, so of a large table only the first `depth` cores
 // of each row enter the histogram; their bin bounds the threshold from below, and only the rows whose last gain
 // still reaches that bound are continued (once, until they fall below it) before the interval is taken again.  Gains
-// behind a row's first gain below the bound are below it too and can never be handed out.
+// behind a row's first gain below the bound are below it too and can never be handed out.  Of 60,000 rows and
+// more the bound comes from a sample of them, before any other is looked at (predict_to_bound).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -54,6 +55,7 @@ constexpr int kNarrowBins = kRadixBins;              // a narrowing step divides
 constexpr int kFinal = kSelectCandidates;            // candidates one block ranks
 constexpr int kRankDirect = 256;                     // ranked against each other; more are narrowed in the block first
 constexpr int kShortWalk = 16;                       // gains of a row its own thread walks; its warp continues
+constexpr int kListWalk = 64;                        // the same where most rows are long
 constexpr u64 kTopKey = 1ull << 63;                  // above every key
 constexpr int kSpinLimit = 1 << 22;                  // polls of a barrier before it gives up (seconds)
 
@@ -137,33 +139,40 @@ __device__ u64 block_exclusive(u64 v, Shared& sh, u64* total) {
     return out;
 }
 
-// Warp 0: the bin of the want-th largest gain from the global histogram (octave totals first, then the bins of one octave).  Fewer gains than wanted: an interval below everything counted, n = 0.
-// kMore: the counts of continued rows are added to the first ones.  What is read here is complete: every block flushed it before the
+// The bin of the want-th largest gain from the global histogram: every warp reads one octave, and the one whose octave it is finds
+// the bin.  One round trip to global memory (octave totals of their own, read first, make it two).  Fewer gains than
+// wanted: an interval below everything counted, n = 0.
+// kOf: which of fine (1), fine_more (2) and fine_rest (4) are added up.  What is read here is complete: every block flushed it before the
 // grid barrier in front of the call, and no block adds to it behind that barrier.
-template <bool kMore>
-__device__ void pick_first(const SelectGlobal* gl, u64 want, Interval* iv) {
-    const int lane = threadIdx.x & 31;
-    const u64 c = __ldcg(&gl->coarse[31 - lane]) + (kMore ? __ldcg(&gl->coarse_more[31 - lane]) : 0);
-    const u64 incl = warp_inclusive(c);
-    const unsigned hit = __ballot_sync(kFull, incl >= want);
-    if (!hit) {
-        if (lane == 0) *iv = Interval{0, 0, want, 0};
-        return;
-    }
-    const int at = __ffs(hit) - 1;
-    const u64 above = __shfl_sync(kFull, incl - c, at);
-    constexpr int per = kSub / 32;
-    const int top = (31 - at) * kSub + kSub - 1 - per * lane;
-    u64 v[per], sum = 0;
+template <int kOf>
+__device__ void pick_first(const SelectGlobal* gl, u64 want, Shared& sh) {
+    static_assert(kSub == 64 && kFine == kWarps * kSub, "a warp per octave, two bins per lane");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int top = warp * kSub + kSub - 1 - 2 * lane;   // from the octave's last bin down
+    u64 v[2];
 #pragma unroll
-    for (int k = 0; k < per; ++k) sum += v[k] = __ldcg(&gl->fine[top - k]) + (kMore ? __ldcg(&gl->fine_more[top - k]) : 0);
-    const u64 incl2 = warp_inclusive(sum);
-    const int at2 = __ffs(__ballot_sync(kFull, above + incl2 >= want)) - 1;
-    if (lane == at2) {
-        u64 run = above + incl2 - sum;
-        int k = 0;
-        while (k < per - 1 && run + v[k] < want) run += v[k++];
-        *iv = Interval{bin_edge(top - k), bin_edge(top - k + 1), want - run, v[k]};
+    for (int k = 0; k < 2; ++k) {
+        v[k] = 0;
+        if (kOf & 1) v[k] += __ldcg(&gl->fine[top - k]);
+        if (kOf & 2) v[k] += __ldcg(&gl->fine_more[top - k]);
+        if (kOf & 4) v[k] += __ldcg(&gl->fine_rest[top - k]);
+    }
+    const u64 sum = v[0] + v[1], incl = warp_inclusive(sum);
+    if (lane == 31) sh.scan[warp] = incl;
+    __syncthreads();
+    const u64 octave = sh.scan[31 - lane], above = warp_inclusive(octave);
+    const unsigned hit = __ballot_sync(kFull, above >= want);
+    if (!hit) {
+        if (threadIdx.x == 0) sh.iv = Interval{0, 0, want, 0};
+    } else if (warp == 32 - __ffs(hit)) {
+        const u64 before = __shfl_sync(kFull, above - octave, 31 - warp);
+        const int at = __ffs(__ballot_sync(kFull, before + incl >= want)) - 1;
+        if (lane == at) {
+            const u64 run = before + incl - sum;
+            const bool second = run + v[0] < want;
+            const int b = second ? top - 1 : top;
+            sh.iv = Interval{bin_edge(b), bin_edge(b + 1), want - run - (second ? v[0] : 0), second ? v[1] : v[0]};
+        }
     }
 }
 
@@ -195,18 +204,10 @@ __device__ void pick_narrow(Counts counts, Shared& sh) {
 }
 
 // Adds a block's shared counts to global ones.
-__device__ void flush_first(Shared& sh, u64* coarse, u64* fine) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int o = warp; o < 32; o += kWarps) {
-        unsigned int sum = 0;
-#pragma unroll
-        for (int k = 0; k < kSub / 32; ++k) {
-            const unsigned int v = sh.hist[o * kSub + k * 32 + lane];
-            if (v) atomicAdd(&fine[o * kSub + k * 32 + lane], (u64)v);
-            sum += v;
-        }
-        sum = __reduce_add_sync(kFull, sum);
-        if (lane == 0 && sum) atomicAdd(&coarse[o], (u64)sum);
+__device__ void flush_first(Shared& sh, u64* fine) {
+    for (int b = threadIdx.x; b < kFine; b += kThreads) {
+        const unsigned int v = sh.hist[b];
+        if (v) atomicAdd(&fine[b], (u64)v);
     }
 }
 
@@ -274,13 +275,14 @@ struct SelectArgs {
     int W;                   // lanes per row (power of two)
     int rows;                // rows per block
     int stride;              // resident rows in shared memory: entries per row (0: rows stay in global memory)
-    int keep_last;           // rows in global memory: the last gain of each row is kept in shared memory
+    int keep_last;           // rows in global memory: the last of each row's first gains is kept in shared memory
     double T;
     long long want;
     SelectGlobal* gl;
     SelectState* sel;
     long long* counters;
     int32_t *gt, *eq;
+    int32_t* list;           // [J], for rows with gains at or above the bound (see predict_to_bound)
     int32_t *alloc, *last_alloc, *out_alloc;
     double* reduction;
     int32_t* err_word;
@@ -658,9 +660,208 @@ __device__ void give_up(const Args& args, const SelectArgs& a, Shared& sh) {
     if (arrive_last(a, sh)) finish_epoch<kCurves>(args);
 }
 
+// A tile's curves into shared memory, and its rows into sh.idx, family II's last: the rows of a warp are then of one family, and
+// only one of the two formulas is walked through (a gain costs 30 to 75 instructions of the fp64 pipe in one family, the sum in
+// both).  keep: the curves are also kept for rows that are asked for later.
+__device__ __forceinline__ void load_tile(const SelectArgs& a, Shared& sh, CurveTile& tile, int base, int n_rows, bool keep) {
+    const int tid = threadIdx.x;
+    bool expo = false;
+    if (tid < n_rows) {
+        const int j = base + tid;
+        bool no_time = false;
+        const bool active = a.count[j] > 0;
+        const Curve c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
+        if (no_time) a.fit.status[j] = SLAQ_JOB_NO_TIME;
+        tile.put(tid, c, active);
+        if (keep) keep_curve(a.basis, j, a.J, c, active ? c.kind : 3);
+        expo = active && c.kind == 1;
+    }
+    place_by_kind(sh, tid < n_rows, expo, n_rows);
+    __syncthreads();
+}
+
+// The counts of bin 0 that threads kept in a register join the others; every thread's counts lie before the block barrier.
+__device__ __forceinline__ void add_low(Shared& sh, unsigned int low) {
+    low = __reduce_add_sync(kFull, low);
+    if ((threadIdx.x & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
+    __syncthreads();
+}
+
+// Half a warp's row from gain `from` on, predicted, written and counted where the key lies in [lo, hi), until it falls below `until`.
+__device__ __forceinline__ void predict_row(const SelectArgs& a, Shared& sh, bool in, int j, int from, u64 lo, u64 hi, u64 until, bool store,
+                                            unsigned int& low) {
+    constexpr int W = 16;
+    const int w = threadIdx.x & (W - 1);
+    double* const row = a.gain + (size_t)j * a.cap;
+    Curve c;
+    c.kind = 3;
+    double carry = CUDART_INF;
+    bool active = false;
+    if (in) {
+        bool no_time = false;
+        c = load_curve<true>(a.job, a.fit, j, a.J, a.T, &no_time);
+        active = a.count[j] > 0;
+        if (from > 0) carry = row[from - 1];
+    }
+    bool on = in;
+    for (int n0 = from; n0 < a.cap && __any_sync(kFull, on); n0 += W) {
+        const int i = n0 + w;
+        const bool has = on && i < a.cap && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+        double g = 0.0;
+        if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
+        g = running_min(g, carry, w, W);
+        if (has && store) row[i] = g;
+        count_gain(g, has && active && i + 1 >= a.first_unit && key_of(g) >= lo && key_of(g) < hi, sh, low, a.err_word);
+        carry = __shfl_sync(kFull, g, W - 1, W);
+        on = on && key_of(carry) >= until;
+    }
+}
+
+// Large tables are not predicted as a whole: few jobs get more than their first core (of 1,000,000 jobs one in ten), so gains are
+// predicted down to a bound that lies just below the threshold.  Where that is, a sample of the rows tells - every block takes some of its
+// own, predicts them to the end and adds them to a histogram; the bound is the bin at the rank that the gains wanted have in the
+// sample, and five times the deviation such a rank can have at most (sqrt(cap x rank): a row counts for up to cap) beyond.  Then every row is predicted
+// four gains at a time until it falls below the bound.  Rows without a gain at or above it keep their floor and are done; the others are
+// listed, those that need more than four gains from the front, and their gains make the histogram the interval is taken from.
+// Should the sample have misled (fewer gains than wanted at or above the bound), every row is predicted to its end: slow, and the same result.
+// Predicting the first 16 gains of every row and taking the bound from those instead continued rows for a bound far below the
+// threshold, since they hold too few of the gains of the rows that get many (launch for 1,000,000 rows of 128: 438 -> 204 us, first gains
+// 142 -> 60 of them, continued rows 151 -> 50, walk 106 -> 30).
+// Returns false after a barrier that was not reached.
+constexpr int kSampleLeast = 32, kSampleShare = 64;   // rows a block samples: at least, and one in so many
+constexpr int kFirstGains = 4;
+template <class Args>
+__device__ bool predict_to_bound(const Args& args, const SelectArgs& a, Shared& sh, CurveTile& tile, int j0, int j1, unsigned int& arrived,
+                                 bool* listed, int* n_more, int* n_some, long long* handed) {
+    const int tid = threadIdx.x, lane = tid & 31, n = j1 - j0;
+    const int floor_cores = a.first_unit - 1;
+    int32_t* const list = a.list + j0;
+    unsigned int low = 0;
+    // the next two rows of n for the calling warp: a row for each half of it
+    auto draw = [&](int limit, bool* in) {
+        int r = lane == 0 ? (int)atomicAdd(&sh.narrow[2], 2u) : 0;
+        r = __shfl_sync(kFull, r, 0) + (lane >> 4);
+        *in = r < limit;
+        return r;
+    };
+    auto reset = [&]() {   // counters and the histogram
+        __syncthreads();
+        for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
+        if (tid < 3) sh.narrow[tid] = 0;
+        low = 0;
+        __syncthreads();
+    };
+    u64 bound = ~0ull;   // nothing wanted: above every gain
+    if (a.want > 0) {
+        const int n_sample = min(n, max(kSampleLeast, n / kSampleShare));
+        if (tid == 0) {
+            sh.narrow[2] = 0;
+            atomicAdd(&a.gl->sampled, (unsigned int)n_sample);
+        }
+        __syncthreads();
+        for (;;) {
+            bool in;
+            const int r = draw(n_sample, &in);
+            if (__all_sync(kFull, !in)) break;
+            // one row of each of n_sample equal parts
+            const int j = in ? j0 + (int)(((long long)r * n + (unsigned int)(r * 2654435761u + blockIdx.x * 40503u) % (unsigned int)n) / n_sample) : j0;
+            predict_row(a, sh, in, j, 0, bin_edge(1), kTopKey, bin_edge(1), false, low);
+        }
+        __syncthreads();
+        flush_first(sh, a.gl->fine);
+        arrived += gridDim.x;
+        if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+        long long J = 0;
+        for (int q = 0; q < args.shards(); ++q) J += args.of(q).J;
+        const double rank = (double)a.want * ((double)__ldcg(&a.gl->sampled) / (double)J);
+        pick_first<1>(a.gl, (u64)(rank + 5.0 * sqrt((double)a.cap * rank) + 8.0), sh);
+        __syncthreads();
+        bound = sh.iv.lo;
+    }
+    reset();
+    for (int base = j0; base < j1; base += kThreads) {
+        const int n_rows = min(kThreads, j1 - base);
+        if (tid == 0) sh.count = sh.n_more = 0;
+        __syncthreads();
+        load_tile(a, sh, tile, base, n_rows, true);
+        const int w = tid & (kFirstGains - 1);
+        for (int r0 = 0; r0 < n_rows; r0 += kThreads / kFirstGains) {   // uniform trip count: the row steps use warp shuffles
+            const int at = r0 + tid / kFirstGains;
+            const bool in = at < n_rows;
+            const int r = in ? sh.idx[at] : 0, j = base + r;
+            Curve c;
+            c.kind = -1;
+            if (in) c = tile.get(r, a.T);
+            const bool active = c.kind >= 0;
+            const bool has = in && index_ok((long long)j * a.cap + w, (long long)a.J * a.cap, kErrGain, a.err_word);
+            const double g = running_min(has && active && c.kind != 3 ? raw_gain(c, w + 1) : 0.0, CUDART_INF, w, kFirstGains);
+            const double first = __shfl_sync(kFull, g, floor_cores, kFirstGains), last = __shfl_sync(kFull, g, kFirstGains - 1, kFirstGains);
+            const bool some = active && key_of(first) >= bound, more = some && key_of(last) >= bound;
+            if (has && some) a.gain[(size_t)j * a.cap + w] = g;
+            count_gain(g, has && some && w + 1 >= a.first_unit && key_of(g) >= bound, sh, low, a.err_word);
+            if (in && w == 0) {   // the row's curve is in its lanes' registers: its place holds the first gain now
+                tile.v[r] = g;
+                sh.taken[r] = some ? (more ? 2 : 1) : 0;
+            }
+        }
+        __syncthreads();
+        if (tid < n_rows) {
+            const int j = base + tid, state = sh.taken[tid];
+            const bool active = tile.kind[tid] >= 0;
+            if (state == 0) {
+                store_alloc(a, j, active ? floor_cores : 0, active && floor_cores ? tile.v[tid] : 0.0, active);
+                *handed += active ? floor_cores : 0;
+            } else if (state == 2) {
+                list[atomicAdd(&sh.narrow[0], 1u)] = j;
+            } else {
+                list[n - 1 - (int)atomicAdd(&sh.narrow[1], 1u)] = j;
+            }
+        }
+        __syncthreads();
+    }
+    *listed = true;
+    *n_more = (int)sh.narrow[0];
+    *n_some = (int)sh.narrow[1];
+    for (;;) {
+        bool in;
+        const int r = draw(*n_more, &in);
+        if (__all_sync(kFull, !in)) break;
+        predict_row(a, sh, in, in ? list[r] : j0, kFirstGains, bound, kTopKey, bound, true, low);
+    }
+    add_low(sh, low);
+    flush_first(sh, a.gl->fine_more);
+    arrived += gridDim.x;
+    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+    if (a.want > 0) {
+        pick_first<2>(a.gl, (u64)a.want, sh);
+    } else if (tid == 0) {
+        sh.iv = Interval{~0ull, ~0ull, 0, 0};
+    }
+    __syncthreads();
+    if (sh.iv.hi > 0 || bound == 0) return true;
+    // the sample has misled: all gains below the bound as well, and all rows to be walked
+    reset();
+    *listed = false;
+    *handed = 0;
+    for (;;) {
+        bool in;
+        const int r = draw(n, &in);
+        if (__all_sync(kFull, !in)) break;
+        predict_row(a, sh, in, in ? j0 + r : j0, 0, 0, bound, 0, true, low);
+    }
+    add_low(sh, low);
+    flush_first(sh, a.gl->fine_rest);
+    arrived += gridDim.x;
+    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) return false;
+    pick_first<6>(a.gl, (u64)a.want, sh);
+    __syncthreads();
+    return true;
+}
+
 // kCurves: gains are predicted from the fitted curves and written to the table (rows beyond `depth` only as far as they
 // were continued); otherwise the table is read.
-template <bool kCurves, class Args>
+// kBounded: see predict_to_bound; a kernel of its own, since the two ways in one cost the smaller tables 2 to 5 us.
+template <bool kCurves, bool kBounded, class Args>
 __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_constant__ Args args) {
     extern __shared__ double dyn[];
     __shared__ Shared sh;
@@ -684,167 +885,167 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
 
     for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
     // the counts of continued rows and the narrowing histograms, should they be needed: cleared by all blocks before the first barrier
-    constexpr int kLater = (int)((offsetof(SelectGlobal, cand_key) - offsetof(SelectGlobal, coarse_more)) / sizeof(u64));
-    u64* const later = reinterpret_cast<u64*>(reinterpret_cast<char*>(a.gl) + offsetof(SelectGlobal, coarse_more));
+    constexpr int kLater = (int)((offsetof(SelectGlobal, cand_key) - offsetof(SelectGlobal, fine_more)) / sizeof(u64));
+    u64* const later = reinterpret_cast<u64*>(reinterpret_cast<char*>(a.gl) + offsetof(SelectGlobal, fine_more));
     for (int i = blockIdx.x * kThreads + tid; i < kLater; i += gridDim.x * kThreads) later[i] = 0;
     if (tid == 0) sh.count = sh.n_more = 0;
     __syncthreads();
 
-    // ---- A: the first `depth` gains of every row ----
-    unsigned int low = 0;
-    const int W = a.W, w = tid & (W - 1), groups = kThreads / W;
-    for (int base = j0; base < j1; base += kThreads) {
-        const int n_rows = min(kThreads, j1 - base);
-        if (kCurves) {
-            bool expo = false;
-            if (tid < n_rows) {
-                const int j = base + tid;
-                bool no_time = false;
-                const bool active = a.count[j] > 0;
-                const Curve c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
-                if (no_time) a.fit.status[j] = SLAQ_JOB_NO_TIME;
-                tile.put(tid, c, active);
-                if (a.depth < a.cap) keep_curve(a.basis, j, a.J, c, active ? c.kind : 3);
-                expo = active && c.kind == 1;
-            }
-            // Family II's rows last: the rows of a warp are then of one family, and only one of the two formulas is
-            // walked through (a gain costs 30 to 75 instructions of the fp64 pipe in one family, the sum in both).
-            place_by_kind(sh, tid < n_rows, expo, n_rows);
-            __syncthreads();
+    long long handed = 0;
+    bool listed = false;             // B walks the rows of `list`: n_more from the front of the block's part, n_some from its end
+    int n_more = 0, n_some = 0;
+    const int32_t* const list = kBounded ? a.list + j0 : nullptr;
+    if constexpr (kBounded) {
+        if (!predict_to_bound(args, a, sh, tile, j0, j1, arrived, &listed, &n_more, &n_some, &handed)) {
+            give_up<kCurves>(args, a, sh);
+            return;
         }
-        for (int r0 = 0; r0 < n_rows; r0 += groups) {   // uniform trip count: the row steps use warp shuffles
-            const int at = r0 + tid / W;
-            const bool in = at < n_rows;
-            const int r = in ? (kCurves ? sh.idx[at] : at) : 0;
-            const int j = base + r;
-            Curve c;
-            bool active = false;
-            if (kCurves) {
-                if (in) {
-                    c = tile.get(r, a.T);
-                    active = c.kind >= 0;
-                    if (!active) c.kind = 3;
-                }
-            } else if (in) {
-                active = !a.count || a.count[j] > 0;
-            }
-            double* const row = a.gain + (size_t)j * a.cap;
-            double carry = CUDART_INF;
-            for (int n0 = 0; n0 < a.depth; n0 += W) {
-                const int i = n0 + w;
-                const bool has = in && i < a.depth && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
-                double g = 0.0;
-                if (kCurves) {
-                    if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
-                    g = running_min(has ? g : 0.0, carry, w, W);
-                    carry = __shfl_sync(kFull, g, W - 1, W);
-                    if (has) row[i] = g;
-                } else if (has) {
-                    g = row[i];
-                }
-                if (has && resident) rows_sh[(base - j0 + r) * a.stride + i] = g;
-                else if (has && a.keep_last && i == a.depth - 1) rows_sh[base - j0 + r] = g;
-                count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
-            }
-        }
-        if (kCurves && tid == 0) sh.count = sh.n_more = 0;
-        __syncthreads();
-    }
-    low = __reduce_add_sync(kFull, low);
-    if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
-    __syncthreads();
-    flush_first(sh, a.gl->coarse, a.gl->fine);
-    arrived += gridDim.x;
-    if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
-        give_up<kCurves>(args, a, sh);
-        return;
-    }
-    if (a.want > 0) {
-        if (tid < 32) pick_first<false>(a.gl, (u64)a.want, &sh.iv);
-    } else if (tid == 0) {
-        sh.iv = Interval{~0ull, ~0ull, 0, 0};   // nothing wanted: a threshold above every gain
-    }
-    __syncthreads();
-
-    // ---- rows that may reach the threshold beyond `depth` are continued ----
-    if (a.depth < a.cap && a.want > 0) {
-        const u64 bound = sh.iv.lo;
-        for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
-        low = 0;
+    } else {
+        // ---- A: the first `depth` gains of every row ----
+        unsigned int low = 0;
+        const int W = a.W, w = tid & (W - 1), groups = kThreads / W;
         for (int base = j0; base < j1; base += kThreads) {
-            if (tid == 0) sh.count = sh.n_more = 0;
-            __syncthreads();
-            const int mine = base + tid;
-            if (mine < j1 && (!a.count || a.count[mine] > 0) &&
-                key_of(a.keep_last ? rows_sh[mine - j0] : a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound) {
-                const bool expo = kCurves && a.fit.status[mine] == SLAQ_JOB_FITTED && a.fit.family[mine] == 1;   // those last, as above
-                sh.narrow[expo ? kThreads - 1 - atomicAdd(&sh.n_more, 1) : atomicAdd(&sh.count, 1)] = (unsigned int)mine;
-            }
-            __syncthreads();
-            const int n_front = sh.count, n_more = n_front + sh.n_more;
-            for (int r0 = 0; r0 < n_more; r0 += groups) {
-                const int r = r0 + tid / W;
-                const bool in = r < n_more;
-                const int j = in ? (int)sh.narrow[r < n_front ? r : kThreads - 1 - (r - n_front)] : base;
-                double* const row = a.gain + (size_t)j * a.cap;
+            const int n_rows = min(kThreads, j1 - base);
+            if constexpr (kCurves) load_tile(a, sh, tile, base, n_rows, a.depth < a.cap);
+            for (int r0 = 0; r0 < n_rows; r0 += groups) {   // uniform trip count: the row steps use warp shuffles
+                const int at = r0 + tid / W;
+                const bool in = at < n_rows;
+                const int r = in ? (kCurves ? sh.idx[at] : at) : 0;
+                const int j = base + r;
                 Curve c;
-                c.kind = 3;
-                double carry = CUDART_INF;
-                if (kCurves && in) {
-                    bool no_time = false;
-                    c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
-                    carry = row[a.depth - 1];
+                bool active = false;
+                if (kCurves) {
+                    if (in) {
+                        c = tile.get(r, a.T);
+                        active = c.kind >= 0;
+                        if (!active) c.kind = 3;
+                    }
+                } else if (in) {
+                    active = !a.count || a.count[j] > 0;
                 }
-                bool on = in;
-                for (int n0 = a.depth; n0 < a.cap && __any_sync(kFull, on); n0 += W) {
+                double* const row = a.gain + (size_t)j * a.cap;
+                double carry = CUDART_INF;
+                for (int n0 = 0; n0 < a.depth; n0 += W) {
                     const int i = n0 + w;
-                    const bool has = on && i < a.cap && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+                    const bool has = in && i < a.depth && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
                     double g = 0.0;
                     if (kCurves) {
                         if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
-                        g = running_min(g, carry, w, W);
+                        g = running_min(has ? g : 0.0, carry, w, W);
+                        carry = __shfl_sync(kFull, g, W - 1, W);
                         if (has) row[i] = g;
                     } else if (has) {
                         g = row[i];
                     }
-                    count_gain(g, has && i + 1 >= a.first_unit, sh, low, a.err_word);
-                    carry = __shfl_sync(kFull, g, W - 1, W);
-                    on = on && key_of(carry) >= bound;
+                    if (has && resident) rows_sh[(base - j0 + r) * a.stride + i] = g;
+                    else if (has && a.keep_last && i == a.depth - 1) rows_sh[base - j0 + r] = g;
+                    count_gain(g, has && active && i + 1 >= a.first_unit, sh, low, a.err_word);
                 }
             }
+            if (kCurves && tid == 0) sh.count = sh.n_more = 0;
             __syncthreads();
         }
-        low = __reduce_add_sync(kFull, low);
-        if ((tid & 31) == 0 && low) atomicAdd(&sh.hist[0], low);
-        __syncthreads();
-        flush_first(sh, a.gl->coarse_more, a.gl->fine_more);
+        add_low(sh, low);
+        flush_first(sh, a.gl->fine);
         arrived += gridDim.x;
         if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
             give_up<kCurves>(args, a, sh);
             return;
         }
-        if (tid < 32) pick_first<true>(a.gl, (u64)a.want, &sh.iv);
+        if (a.want > 0) {
+            pick_first<1>(a.gl, (u64)a.want, sh);
+        } else if (tid == 0) {
+            sh.iv = Interval{~0ull, ~0ull, 0, 0};   // nothing wanted: a threshold above every gain
+        }
         __syncthreads();
+
+        // ---- rows that may reach the threshold beyond `depth` are continued ----
+        if (a.depth < a.cap && a.want > 0) {
+            const u64 bound = sh.iv.lo;
+            for (int i = tid; i < kFine; i += kThreads) sh.hist[i] = 0;
+            low = 0;
+            for (int base = j0; base < j1; base += kThreads) {
+                if (tid == 0) sh.count = sh.n_more = 0;
+                __syncthreads();
+                const int mine = base + tid;
+                if (mine < j1 && (!a.count || a.count[mine] > 0) &&
+                    key_of(a.keep_last ? rows_sh[mine - j0] : a.gain[(size_t)mine * a.cap + a.depth - 1]) >= bound) {
+                    const bool expo = kCurves && a.fit.status[mine] == SLAQ_JOB_FITTED && a.fit.family[mine] == 1;   // those last, as above
+                    sh.narrow[expo ? kThreads - 1 - atomicAdd(&sh.n_more, 1) : atomicAdd(&sh.count, 1)] = (unsigned int)mine;
+                }
+                __syncthreads();
+                const int n_front = sh.count, n_all = n_front + sh.n_more;
+                for (int r0 = 0; r0 < n_all; r0 += groups) {
+                    const int r = r0 + tid / W;
+                    const bool in = r < n_all;
+                    const int j = in ? (int)sh.narrow[r < n_front ? r : kThreads - 1 - (r - n_front)] : base;
+                    double* const row = a.gain + (size_t)j * a.cap;
+                    Curve c;
+                    c.kind = 3;
+                    double carry = CUDART_INF;
+                    if (kCurves && in) {
+                        bool no_time = false;
+                        c = load_curve(a.job, a.fit, j, a.J, a.T, &no_time);
+                        carry = row[a.depth - 1];
+                    }
+                    bool on = in;
+                    for (int n0 = a.depth; n0 < a.cap && __any_sync(kFull, on); n0 += W) {
+                        const int i = n0 + w;
+                        const bool has = on && i < a.cap && index_ok((long long)j * a.cap + i, (long long)a.J * a.cap, kErrGain, a.err_word);
+                        double g = 0.0;
+                        if (kCurves) {
+                            if (has) g = c.kind == 3 ? 0.0 : raw_gain(c, i + 1);
+                            g = running_min(g, carry, w, W);
+                            if (has) row[i] = g;
+                        } else if (has) {
+                            g = row[i];
+                        }
+                        count_gain(g, has && i + 1 >= a.first_unit, sh, low, a.err_word);
+                        carry = __shfl_sync(kFull, g, W - 1, W);
+                        on = on && key_of(carry) >= bound;
+                    }
+                }
+                __syncthreads();
+            }
+            add_low(sh, low);
+            flush_first(sh, a.gl->fine_more);
+            arrived += gridDim.x;
+            if (!grid_barrier(&a.gl->barrier, arrived, &sh.flag, a.err_word)) {
+                give_up<kCurves>(args, a, sh);
+                return;
+            }
+            pick_first<3>(a.gl, (u64)a.want, sh);
+            __syncthreads();
+        }
     }
 
-    // ---- B: every row up to the interval ----
+    // ---- B: every row that may have gains at or above the interval, up to it ----
     const Interval iv = sh.iv;
     const bool few = iv.n <= kFinal;
-    long long handed = 0;
     const int lane = tid & 31;
-    // a few rows per block are spread over its warps, one per warp at first
-    const int pitch = j1 - j0 <= kThreads / 4 ? kWarps : 1;
+    const int n_walk = listed ? n_more + n_some : j1 - j0;
+    if (listed && !few) {   // the others have no candidates
+        for (int j = j0 + tid; j < j1; j += kThreads) {
+            a.gt[j] = a.count[j] > 0 ? a.first_unit - 1 : 0;
+            a.eq[j] = 0;
+        }
+        __syncthreads();
+    }
+    // few rows per block, or long ones, are spread over its warps, one per warp at first
+    const int pitch = n_walk <= (listed ? kThreads : kThreads / 4) ? kWarps : 1;
     const int slot0 = pitch == 1 ? tid & ~31 : tid >> 5, slot = slot0 + pitch * lane;
-    for (int base = j0; base < j1; base += kThreads) {   // uniform trip count: a warp finishes its long rows together
-        const int j = base + slot;
-        const bool in = j < j1, active = in && (!a.count || a.count[j] > 0);
+    for (int base = 0; base < n_walk; base += kThreads) {   // uniform trip count: a warp finishes its long rows together
+        const int at = base + slot;
+        const bool in = at < n_walk;
+        const int j = !in ? j0 : !listed ? j0 + at : list[at < n_more ? at : j1 - j0 - 1 - (at - n_more)];
+        const bool active = in && (!a.count || a.count[j] > 0);
         const double* row = resident ? rows_sh + (size_t)(j - j0) * a.stride : a.gain + (size_t)j * a.cap;
         int s = 0, c = 0;
         double R = 0.0;
         bool more = false;
         if (active) {
             if (a.first_unit == 2) R = row[0], s = 1;
-            const int end = min(a.cap, kShortWalk);
+            const int end = min(a.cap, listed ? kListWalk : kShortWalk);
             more = s < a.cap;
             while (more && s < end) {
                 double g[4];   // four loads in flight; entries behind a row's first gain below the interval mean nothing
@@ -862,19 +1063,19 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
         }
         for (unsigned todo = __ballot_sync(kFull, more); todo; todo &= todo - 1) {
             const int r = __ffs(todo) - 1;
-            const int jr = base + slot0 + pitch * r;
+            const int jr = __shfl_sync(kFull, j, r);
             const double* far = resident ? rows_sh + (size_t)(jr - j0) * a.stride : a.gain + (size_t)jr * a.cap;
-            int at = __shfl_sync(kFull, s, r);
+            int at_n = __shfl_sync(kFull, s, r);
             double sum = __shfl_sync(kFull, R, r);
-            for (bool on = true; on && at < a.cap;) {
-                const double g = at + lane < a.cap ? far[at + lane] : 0.0;
-                const unsigned stop = __ballot_sync(kFull, at + lane >= a.cap || key_of(g) < iv.hi);
+            for (bool on = true; on && at_n < a.cap;) {
+                const double g = at_n + lane < a.cap ? far[at_n + lane] : 0.0;
+                const unsigned stop = __ballot_sync(kFull, at_n + lane >= a.cap || key_of(g) < iv.hi);
                 const int n = stop ? __ffs(stop) - 1 : 32;
                 for (int k = 0; k < n; ++k) sum += __shfl_sync(kFull, g, k);   // in order, as the row's own thread adds
-                at += n;
+                at_n += n;
                 on = n == 32;
             }
-            if (lane == r) s = at, R = sum;
+            if (lane == r) s = at_n, R = sum;
         }
         if (!in) continue;
         if (active)
@@ -1160,8 +1361,11 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
 // Rule for the rows' home.  Up to kResidentGains gains per block (two evaluations per thread) all of them are predicted
 // at once, kept in shared memory and walked there; the whole table is written as well.  Beyond that prediction is what
 // costs (910 us for 128 gains of a million jobs each), so rows start with four times the average number of
-// cores handed out, at least 16, and only rows that need more are continued.
+// cores handed out, at least 16, and only rows that need more are continued.  From kBoundedRows rows on gains are predicted down to a bound
+// from a sample instead, whose barrier and long rows cost the smaller ones 3 to 6 us more than it gives (launch of 33,000 rows: 34 -> 37
+// us, of 100,000: 55 -> 47).
 constexpr int kResidentGains = 2048;
+constexpr int kBoundedRows = 60000;
 constexpr int kKeepLast = 8192;
 constexpr int kSmallGains = 6144, kSmallRows = 256;   // one block up to here (see select_small_kernel)
 
@@ -1174,10 +1378,11 @@ int select_setup(int* blocks_per_sm) {
     const size_t most = select_smem(true, kKeepLast, 1), most_small = select_smem(true, kSmallGains + kSmallRows, 1);
     for (const void* k : {(const void*)select_small_kernel<true>, (const void*)select_small_kernel<false>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_small) != cudaSuccess) return -1;
-    for (const void* k : {(const void*)select_kernel<true, OneHandle>, (const void*)select_kernel<false, OneHandle>,
-                          (const void*)select_kernel<true, ManyHandles>})
+    for (const void* k : {(const void*)select_kernel<true, false, OneHandle>, (const void*)select_kernel<true, true, OneHandle>,
+                          (const void*)select_kernel<false, false, OneHandle>, (const void*)select_kernel<true, false, ManyHandles>,
+                          (const void*)select_kernel<true, true, ManyHandles>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true, ManyHandles>, kThreads, most) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<true, true, ManyHandles>, kThreads, most) != cudaSuccess) return -1;
     *blocks_per_sm = per_sm < 1 ? 1 : per_sm;
     return 0;
 }
@@ -1191,18 +1396,19 @@ static int select_depth(long long J, int cap, long long want, int sm_count) {
 
 // The part of the arguments that depends on the sizes, the same for all handles of a launch (J: their rows in all).
 struct SelectPlan {
-    int depth, W, rows, stride, keep_last;
+    int depth, W, rows, stride, keep_last, bounded;
     size_t smem;
 };
 static void set_rows(SelectPlan& p, int rows, int cap, bool curves) {
     p.rows = rows;
-    p.keep_last = p.stride == 0 && p.depth < cap && rows <= kKeepLast;
+    p.keep_last = !p.bounded && p.stride == 0 && p.depth < cap && rows <= kKeepLast;
     p.smem = select_smem(curves, p.stride > 0 || p.keep_last ? rows : 0, p.stride > 0 ? p.stride : 1);
 }
 static SelectPlan plan_select(long long J, int cap, long long want, bool curves, int sm_count, int blocks_per_sm) {
     SelectPlan p;
     const long long gains = J * cap;
     p.depth = select_depth(J, cap, want, sm_count);
+    p.bounded = curves && p.depth < cap && J >= kBoundedRows;
     p.W = 1;
     long long grid;
     if (gains <= (long long)kResidentGains * sm_count) {
@@ -1235,7 +1441,7 @@ static cudaError_t launch_one(OneHandle& one, bool curves, int sm_count, int blo
         const size_t smem = select_smem(curves, a.J, p.stride);
         return launch_behind(curves ? select_small_kernel<true> : select_small_kernel<false>, 1, kThreads, smem, st, one);
     }
-    return launch_behind<true>(curves ? select_kernel<true, OneHandle> : select_kernel<false, OneHandle>, (a.J + p.rows - 1) / p.rows,
+    return launch_behind<true>(p.bounded ? select_kernel<true, true, OneHandle> : curves ? select_kernel<true, false, OneHandle> : select_kernel<false, false, OneHandle>, (a.J + p.rows - 1) / p.rows,
                                kThreads, p.smem, st, one);
 }
 
@@ -1255,6 +1461,7 @@ static SelectArgs handle_args(slaq_handle* h, double epoch_seconds, long long wa
     a.counters = h->scratch.counters;
     a.gt = h->scratch.gt;
     a.eq = h->scratch.eq;
+    a.list = h->scratch.order;   // the fits are done with it
     a.alloc = h->alloc;
     a.last_alloc = h->job.last_alloc;
     a.out_alloc = d_out_alloc;
@@ -1310,7 +1517,7 @@ int launch_select_group(slaq_handle* const* hs, int n, double epoch_seconds, lon
         }
         many.first_block[s + 1] = many.first_block[s] + (s < n ? (hs[s]->max_jobs + p.rows - 1) / p.rows : 0);
     }
-    const cudaError_t e = launch_behind<true>(select_kernel<true, ManyHandles>, blocks, kThreads, p.smem, h->stream, many);
+    const cudaError_t e = launch_behind<true>(p.bounded ? select_kernel<true, true, ManyHandles> : select_kernel<true, false, ManyHandles>, blocks, kThreads, p.smem, h->stream, many);
     if (e != cudaSuccess) {
         h->err = std::string("selection launch: ") + cudaGetErrorString(e);
         return -1;
