@@ -7,6 +7,7 @@
 #endif
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -509,22 +510,32 @@ int check_ids(slaq_handle* h, int32_t n, const int32_t* ids, bool forbid_dups) {
     return SLAQ_OK;
 }
 
+// The logarithm's table (see log_of_normal): pairs of 1 / c and the leading part of log c for the middles c of the bins, then the rests of
+// log c.  Made once: it took 18 us of a new handle's first pass.
+const std::array<double, 3 * kLogBins>& log_table() {
+    static const std::array<double, 3 * kLogBins> table = [] {
+        std::array<double, 3 * kLogBins> t;
+        for (int i = 0; i < kLogBins; ++i) {
+            const uint64_t bits = (uint64_t)(kLogFrom + (i << kLogBinShift) + (1 << (kLogBinShift - 1))) << 32;
+            double c;
+            std::memcpy(&c, &bits, sizeof c);
+            const double inv = 1.0 / c;
+            const long double log_c = -std::log((long double)inv), lead = std::nearbyint(log_c * 0x1p42L) * 0x1p-42L;
+            t[2 * i] = inv;
+            t[2 * i + 1] = (double)lead;
+            t[2 * kLogBins + i] = (double)(log_c - lead);
+        }
+        return t;
+    }();
+    return table;
+}
+
 int ensure_weights(slaq_handle* h) {
     if (h->wtab_gamma == h->gamma) return SLAQ_OK;
-    // gamma^m, then the sums over m < H of gamma^m m^p for H = 0..max_hist, p = 0..4, then 1 / c, the leading part of log c
-    // and its rest for the middles c of the logarithm's bins
+    // gamma^m, then the sums over m < H of gamma^m m^p for H = 0..max_hist, p = 0..4, then the logarithm's table
     const size_t n = (size_t)h->max_hist;
     std::vector<double> tab(6 * n + 6 + 3 * kLogBins);
-    for (int i = 0; i < kLogBins; ++i) {
-        const uint64_t bits = (uint64_t)(kLogFrom + (i << kLogBinShift) + (1 << (kLogBinShift - 1))) << 32;
-        double c;
-        std::memcpy(&c, &bits, sizeof c);
-        const double inv = 1.0 / c;
-        tab[6 * n + 6 + 2 * i] = inv;
-        const long double log_c = -std::log((long double)inv), lead = std::nearbyint(log_c * 0x1p42L) * 0x1p-42L;
-        tab[6 * n + 6 + 2 * i + 1] = (double)lead;
-        tab[6 * n + 6 + 2 * kLogBins + i] = (double)(log_c - lead);
-    }
+    std::memcpy(&tab[6 * n + 6], log_table().data(), 3 * kLogBins * sizeof(double));
     for (size_t m = 0; m < n; ++m) tab[m] = std::pow(h->gamma, (double)m);
     long double sum[5] = {};
     for (size_t m = 0; m <= n; ++m) {
