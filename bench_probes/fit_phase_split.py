@@ -7,12 +7,14 @@ every warp reads clock64() at the phase boundaries, nothing is skipped), schedul
 with it and with the ordinary library, and prints per phase the share of the warps' cycles and
 that share of the ordinary library's fit time.  Also prints the cycles a sub-partition spends per
 warp row of a trial sweep inside the kernel: (cycles in phase 3 / warps per sub-partition) / rows
-swept, to set beside fit_sweep_probe's figure for the sweep alone.
+swept, to set beside fit_sweep_probe's figure for the sweep alone.  How many warps a sub-partition had (the library runs two,
+three or four) follows from all cycles over the stage's duration.
 """
 
 from __future__ import annotations
 
 import argparse
+import subprocess
 import sys
 from pathlib import Path
 
@@ -61,8 +63,12 @@ def main():
     fitted = pred["status"] == 0
     H = wl.hist_len[fitted].astype(np.float64)
     trial_rows = float((H * (pred["evals"][fitted].max(axis=1) - 1)).sum()) / 32.0   # rows of 32 points, both families in one sweep
-    print(f"trial sweeps: about {trial_rows:.3e} warp rows; phase 3 = {cycles[3] / 4.0 / trial_rows:.1f} cycles per "
-          f"warp row and sub-partition (4 warps per sub-partition share it)")
+    sub = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    mhz = float(subprocess.run(["nvidia-smi", "--query-gpu=clocks.max.sm", "--format=csv,noheader,nounits", "-i", "0"],
+                               capture_output=True, text=True, check=True).stdout)
+    warps = max(1, round(total / (ms_clocked * 1e3 * mhz * sub)))
+    print(f"trial sweeps: about {trial_rows:.3e} warp rows; phase 3 = {cycles[3] / warps / trial_rows:.1f} cycles per "
+          f"warp row and sub-partition ({warps} warps per sub-partition share it)")
 
 
 if __name__ == "__main__":
