@@ -143,8 +143,7 @@ struct Normalised {
 //
 // A level is l / M correctly rounded.  Where all magnitudes lie between 2^-400 and 2^400 it is formed from the correctly rounded r = 1 / M
 // by q = l r, q += (l - q M) r twice: the first correction brings q to within an ulp, the second rounds correctly (Markstein, "Computation
-// of elementary functions on the IBM RISC System/6000 processor", 1990), 5 operations instead of a division's 9 and its test for
-// special cases (fit of 100,000 windows of up to 1,000: 3,483 -> 3,448 us; warm started, without the range as well, 1,354 -> 1,307).
+// of elementary functions on the IBM RISC System/6000 processor", 1990), five operations and no test for special cases per row (fit of 100,000 windows of up to 1,000: 3,483 -> 3,448 us; warm started, without the range as well, 1,354 -> 1,307).
 // kRange: the lowest and the highest level are wanted (first guesses).
 template <bool kRange, class Lanes>
 __device__ Normalised normalise_window(const Lanes& S, int H, int k_all, double m_seen, int min_fit_points,
@@ -527,8 +526,8 @@ struct GuessSums {
 // log of a positive normal number, to 1.2 ulp, by table lookup (Tang, "Table-driven implementation of the logarithm function", 1990):
 // x = 2^e z with z in about [0.71, 1.42) cut into 128 bins with middles c, log x = e log 2 + log c + log(1 + r) with
 // r = z / c - 1, |r| <= 2^-8, by its Taylor series.  log 2 and log c are split so that the leading parts add up exactly; the bin
-// around 1 has c = 1.  tab: 128 pairs of 1 / c and the leading part of log c, then the rests (written by ensure_weights).  Half the
-// instructions of log(), whose arguments may be anything (fit of 100,000 windows of up to 1,000, with x counted in rows: 3,615 ->
+// around 1 has c = 1.  tab: 128 pairs of 1 / c and the leading part of log c, then the rests (written by ensure_weights).  Shorter
+// than log(), whose arguments may be anything (fit of 100,000 windows of up to 1,000, with x counted in rows: 3,615 ->
 // 3,511 us, of 1,000,000 of 64: 3,904 -> 3,803; about half of it each).
 __device__ __forceinline__ double log_of_normal(double x, const double* __restrict__ tab) {
     const int hi = __double2hiint(x), t = hi - kLogFrom, e = t >> 20, bin = (t >> kLogBinShift) & (kLogBins - 1);
@@ -701,6 +700,32 @@ __device__ __forceinline__ void rescale(double (&pI)[4], double (&pII)[4], doubl
     pII[1] *= f;
 }
 
+// A warm start's first guesses, out of line: most warps of a loop need none, and in line they cost the others registers (944 bytes
+// spilled instead of 200; fit of 100,000 windows of up to 1,000: 1,307 against 1,278 us).
+template <class Lanes>
+__device__ __noinline__ void warm_first_guesses(const Lanes& S, int H, int k_all, double inv_span, bool fits, bool needI, bool needII,
+                                                Moments* mom, double* gI, double* gII) {
+    Normalised nz;
+    level_range(S, H, k_all, nz);
+    Moments found;
+    double one[4] = {0.0, 0.0, 0.0, 0.0}, two[4] = {0.0, 0.0, 0.0, 0.0};
+    first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, needI, needII, found, one, two);
+    *mom = found;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) gI[a] = one[a], gII[a] = two[a];
+}
+
+// The sums of first_guesses that do not depend on a guess.
+template <class Lanes>
+__device__ __forceinline__ void weight_moments(const Lanes& S, int H, int k_all, double inv_span, bool busy, Moments& mom) {
+    GuessSums g = {};
+    const int shift = __ffs(S.L()) - 1;
+    const int own = busy && H - 1 - S.l >= 0 ? ((H - 1 - S.l) >> shift) + 1 : 0;
+    guess_rows<false, false, false>(S, own, k_all, inv_span, 0.0, g);
+    mom.sw = busy && index_ok(H, S.wtab_len + 1, kErrShared, S.err_word) ? S.wsum[H] : 0.0;
+    mom.swy2 = group_sum(g.swy2, S.L());
+}
+
 // The second round of a warm start: the families whose carried-over point had no finite
 // residual (`redo`, per lane for its own family) take their first guesses and are swept again.
 template <class Lanes>
@@ -823,12 +848,17 @@ __device__ __forceinline__ void fit_slot(const JobArrays& job, const FitArrays& 
             {
                 double gI[4], gII[4];
                 const bool needI = wantsI && !(wmask & 1u), needII = wantsII && !(wmask & 2u);
-                if (__any_sync(kFull, needI || needII)) level_range(S, H, k_all, nz);
-                first_guesses(S, H, k_all, inv_span, nz.ymin, nz.ymax, fits, needI, needII, mom, gI, gII);
+                if (__any_sync(kFull, needI || needII)) {
+                    Moments found;
+                    warm_first_guesses(S, H, k_all, inv_span, fits, needI, needII, &found, gI, gII);
+                    mom = found;
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    if (needI) pI[a] = gI[a];
-                    if (needII) pII[a] = gII[a];
+                    for (int a = 0; a < 4; ++a) {
+                        if (needI) pI[a] = gI[a];
+                        if (needII) pII[a] = gII[a];
+                    }
+                } else {
+                    weight_moments(S, H, k_all, inv_span, fits, mom);
                 }
             }
             sweep_at(fits, fits);
