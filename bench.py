@@ -41,9 +41,9 @@ SWEEP_FLOP_PER_POINT, SWEEP_ISSUE_CYCLES_PER_ROW = FLOP_SWEEP_I + FLOP_SWEEP_II,
 SUBPARTITIONS_PER_SM = 4
 MIN_TIMED_SECONDS = 1.0   # the block of --steps steps is repeated until the timed region is at least this long
 # DRAM bytes per stored loss moved by the fit kernel (ncu: dram__bytes_read.sum + dram__bytes_write.sum =
-# 165.46 MB + 10.47 MB on a 20,068,408-loss cut of this workload, profiles/fit_kernel_40k_jobs.md; traffic grows
+# 165.28 MB + 11.00 MB on a 20,068,408-loss cut of this workload, profiles/fit_kernel_40k_jobs.md; traffic grows
 # with the stored losses)
-NCU_FIT_DRAM_BYTES_PER_LOSS = (165.46e6 + 10.47e6) / 20_068_408
+NCU_FIT_DRAM_BYTES_PER_LOSS = (165.28e6 + 11.00e6) / 20_068_408
 
 
 from paper_1802_04819_b200.partition import max_over_ranks, partition_seed_offset, rank_info, whole_job_rate  # noqa: E402
