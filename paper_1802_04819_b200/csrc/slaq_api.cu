@@ -694,7 +694,7 @@ int create_common(slaq_handle* h, int32_t max_jobs, int32_t max_hist, int32_t ca
         if (!h->mailbox_mem) return fail(h, SLAQ_E_NOMEM, "page-locked memory of the mailbox");
         h->mailbox = new (h->mailbox_mem) Mailbox();
     }
-    if (fit_setup()) return fail(h, SLAQ_E_CUDA, "fit kernel setup failed");
+    if (fit_prepare(h)) return fail(h, SLAQ_E_CUDA, "fit kernel setup failed");
     h->active.assign((size_t)max_jobs, 0);
     h->stamp.assign((size_t)max_jobs, 0u);
     h->in_packed.assign((size_t)max_jobs, 0);

@@ -1404,28 +1404,20 @@ static FitKernel const kFitAsTeam[2] = {fit_kernel<false, 32, 8, false>, fit_ker
 static FitTeamKernel const kFitTeamKernels[2][2] = {{fit_team_kernel<false, false>, fit_team_kernel<false, true>},
                                                     {fit_team_kernel<true, false>, fit_team_kernel<true, true>}};
 
-int fit_setup() {
-    bool ok = true;
-    for (const auto& row : kFitTeamKernels)
-        for (FitTeamKernel k : row)
-            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmem) == cudaSuccess &&
-                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-    for (const auto& warps : kFitKernels)
-        for (const auto& row : warps)
-            for (FitKernel k : row)
-                ok = ok && (!k || (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
-                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess));
-    for (FitKernel k : kFitAsTeam)
-        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
-                 cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-    for (const void* k : {(const void*)length_scatter_kernel, (const void*)length_sort_kernel})
-        ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(2 * sizeof(int) * (kMaxHistLimit + 1))) == cudaSuccess;
-    return ok ? 0 : -1;
+// Shared memory beyond the default is allowed to a kernel when a handle is about to use it, which also loads the kernel.  Doing all 26
+// in every new handle cost the first one of a process 3 ms more and the later ones 5 us.  The handle remembers the last one: a context
+// that is gone takes its handles along.
+static cudaError_t allow_shared(slaq_handle* h, const void* kernel, size_t bytes) {
+    if (h->fit_ready == kernel) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) h->fit_ready = kernel;
+    return e;
 }
 
-static long long jobs_for_lanes(const slaq_handle* h) {
-    return h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : (long long)h->n_active;
+// active: the handle's active jobs, or as many as it may come to have
+static long long jobs_for_lanes(const slaq_handle* h, long long active) {
+    return h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : active;
 }
 
 // Doubles of shared memory per warp: the parked sums, the window rows and one spare row.  It grows if the longest window
@@ -1451,12 +1443,12 @@ struct FitPlan {
     int kind, lanes;   // index into kFitWarps; least lanes
     size_t slice_bytes;
 };
-static FitPlan fit_plan(const slaq_handle* h) {
+static FitPlan fit_plan(const slaq_handle* h, long long active) {
     constexpr struct {
         double chain, chain_row, issue, issue_row, part, mixed;
     } cost_of[3] = {{4600, 315, 1230, 95, 0.5, 0.55}, {3600, 220, 1250, 97, 0.9, 0.4}, {3300, 190, 1340, 106, 0.1, 0.4}};
     const int Hmax = h->max_hist;
-    const double jobs = (double)std::max(1LL, jobs_for_lanes(h)), sub = 4.0 * h->sm_count;
+    const double jobs = (double)std::max(1LL, jobs_for_lanes(h, active)), sub = 4.0 * h->sm_count;
     const bool by_size = h->fit_slice_bytes == kDefaultFitSlice;
     FitPlan best = {kTwelve, 32, by_size ? kFitSlices[kTwelve] : h->fit_slice_bytes};
     double least = -1.0;
@@ -1484,15 +1476,15 @@ static FitPlan fit_plan(const slaq_handle* h) {
         while (best.lanes > 2 && jobs * (best.lanes / 2) >= 1.5 * 32.0 * kFitWarps[kTwelve] * h->sm_count) best.lanes >>= 1;
     return best;
 }
-int fit_least_lanes(const slaq_handle* h) { return fit_plan(h).lanes; }
+int fit_least_lanes(const slaq_handle* h) { return fit_plan(h, h->n_active).lanes; }
 
 // Warps per family of a job's team; 0: no teams.  A question of the cluster's active jobs and the windows alone, which every shard
 // answers alike, whatever its capacity: several warps add in another order than one, and one in another than a part of one.  With a warp per sub-partition at most, a lane is left four rows of the longest
 // window; two warps share a sub-partition without loss where a lane would have twelve rows or more (140 windows of up to
 // 1,000: 61 -> 58 us, but 200 of up to 300: 44 -> 45), and teams of one warp per family up to sixteen rows (580 windows of 20: 38 ->
 // 35 us, but 300 of 1,000: 84 -> 87).
-static int fit_team_parts(const slaq_handle* h) {
-    const long long warps = 4LL * h->sm_count, jobs = std::max({1LL, jobs_for_lanes(h), (long long)h->n_active});
+static int fit_team_parts(const slaq_handle* h, long long active) {
+    const long long warps = 4LL * h->sm_count, jobs = std::max({1LL, jobs_for_lanes(h, active), active});
     if (2 * jobs > (h->max_hist > 512 ? warps : 2 * warps)) return 0;
     int parts = 1;
     while (parts < kTeamWarps / 2 && ((4 * parts * jobs <= warps && h->max_hist > 128 * parts) ||
@@ -1508,6 +1500,9 @@ static cudaError_t launch_sort(slaq_handle* h, cudaStream_t st, int* launches) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
     long long* const stamp = h->scratch.stamps;
+    const auto sorter = J <= kOneBlockSort ? (const void*)length_sort_kernel : (const void*)length_scatter_kernel;
+    if (2 * bins > 48 * 1024)
+        if (const cudaError_t no = cudaFuncSetAttribute(sorter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * bins))) return no;
     if (J <= kOneBlockSort) {
         *launches += 1;
         return launch_behind(length_sort_kernel, 1, 1024, 2 * bins, st, h->job.count, J, Hmax, h->scratch.start, h->scratch.order, stamp,
@@ -1523,38 +1518,40 @@ static cudaError_t launch_sort(slaq_handle* h, cudaStream_t st, int* launches) {
     return e;
 }
 
-int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
-    const int J = h->max_jobs, Hmax = h->max_hist;
-    int launches = 0;
-    const int parts = fit_team_parts(h);
+// What a launch of so many active jobs is made of.
+struct FitChoice {
+    FitClasses cls;
+    int parts;      // warps per family of a job's team; 0: fit_kernel
+    bool listed;    // the teams take their jobs from the work list
+    int warps;      // of a block, at most
+    const void* kernel;
+    FitKernel fit;
+    FitTeamKernel team;
+};
+static FitChoice fit_choice(const slaq_handle* h, long long active) {
+    const int J = h->max_jobs, Hmax = h->max_hist, warm = h->warm_start ? 1 : 0;
+    FitChoice c = {};
+    c.cls.h_max = Hmax;
+    const int parts = fit_team_parts(h, active);
     // A block for each id is for handles with few of them: the empty ones cost 8 jobs among 592 ids 10 us.  A family with one
     // warp adds its sums in the order in which one warp does both, so that teams of one are left to the other kernel there.
-    const bool many_ids = J > 4 * h->sm_count;
-    if (parts > 1 || (parts == 1 && !many_ids)) {
-        FitClasses all = {};
-        all.n = 1;
-        all.h_hi[0] = all.h_max = Hmax;
-        all.L[0] = 32;
-        all.slice = team_slice(h);
-        // the list's blocks: one per job that is active now (a graph of the caller's may meet more later)
-        const int blocks = many_ids ? std::max(1, h->n_active) : J;
-        cudaError_t e = many_ids ? launch_sort(h, st, &launches) : cudaSuccess;
-        if (e == cudaSuccess)
-            e = launch_behind(kFitTeamKernels[h->warm_start ? 1 : 0][many_ids ? 1 : 0], blocks, 64 * parts, team_smem(h, parts), st, h->job,
-                              h->fit, h->wtab, h->scratch.order, h->scratch.start, all, parts, h->lm_trials, h->min_fit_points,
-                              h->scratch.counters, many_ids ? nullptr : h->scratch.stamps, h->err_word);
-        if (e == cudaSuccess) return launches + 1;
-        h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
-        return -1;
+    c.listed = J > 4 * h->sm_count;
+    if (parts > 1 || (parts == 1 && !c.listed)) {
+        c.parts = parts;
+        c.cls.n = 1;
+        c.cls.h_hi[0] = Hmax;
+        c.cls.L[0] = 32;
+        c.cls.slice = team_slice(h);
+        c.team = kFitTeamKernels[warm][c.listed ? 1 : 0];
+        c.kernel = (const void*)c.team;
+        return c;
     }
     // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked doubles per job and
     // family), the window rows of 32 points and one spare row.  The class with L = 32, 16, .. lanes per job takes
     // the windows that do not fit at L/2 lanes; the last one has the fewest lanes and takes the rest.
-    FitClasses cls;
-    cls.n = 0;
-    cls.h_max = Hmax;
-    const FitPlan plan = parts == 1 ? FitPlan{kEight, 32, kFitSlices[kEight]} : fit_plan(h);
-    const int max_warps = kFitWarps[plan.kind];
+    FitClasses& cls = c.cls;
+    const FitPlan plan = parts == 1 ? FitPlan{kEight, 32, kFitSlices[kEight]} : fit_plan(h, active);
+    c.warps = kFitWarps[plan.kind];
     cls.slice = fit_slice(h, plan.slice_bytes);
     const int L_min = plan.lanes;
     int h_hi = Hmax;
@@ -1567,15 +1564,43 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         ++cls.n;
         h_hi = h_lo;
     }
-    for (int c = cls.n; c < kMaxFitClasses; ++c) cls.h_lo[c] = cls.h_hi[c] = 0, cls.L[c] = 32;
+    for (int k = cls.n; k < kMaxFitClasses; ++k) cls.h_lo[k] = cls.h_hi[k] = 0, cls.L[k] = 32;
+    c.fit = parts == 1 ? kFitAsTeam[warm] : kFitKernels[plan.kind][warm][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
+    c.kernel = (const void*)c.fit;
+    return c;
+}
+
+int fit_prepare(slaq_handle* h) {
+    const FitChoice c = fit_choice(h, h->max_jobs);
+    return allow_shared(h, c.kernel, c.parts ? kTeamSmem : kSmemLimit) == cudaSuccess ? 0 : -1;
+}
+
+int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
+    const int J = h->max_jobs;
+    int launches = 0;
+    const FitChoice c = fit_choice(h, h->n_active);
+    const FitClasses& cls = c.cls;
+    cudaError_t e = allow_shared(h, c.kernel, c.parts ? kTeamSmem : kSmemLimit);
+    if (c.parts) {
+        // the list's blocks: one per job that is active now (a graph of the caller's may meet more later)
+        const int blocks = c.listed ? std::max(1, h->n_active) : J;
+        if (e == cudaSuccess && c.listed) e = launch_sort(h, st, &launches);
+        if (e == cudaSuccess)
+            e = launch_behind(c.team, blocks, 64 * c.parts, team_smem(h, c.parts), st, h->job, h->fit, h->wtab, h->scratch.order,
+                              h->scratch.start, cls, c.parts, h->lm_trials, h->min_fit_points, h->scratch.counters,
+                              c.listed ? nullptr : h->scratch.stamps, h->err_word);
+        if (e == cudaSuccess) return launches + 1;
+        h->err = std::string("fit kernel launch: ") + cudaGetErrorString(e);
+        return -1;
+    }
     // A job per warp of the GPU and no more: every job starts at once, so their order means nothing and none is made.
-    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * max_warps;
-    cudaError_t e = in_order ? cudaSuccess : launch_sort(h, st, &launches);
+    const bool in_order = cls.n == 1 && cls.L[0] == 32 && J <= max_blocks * c.warps;
+    if (e == cudaSuccess && !in_order) e = launch_sort(h, st, &launches);
     // One block per SM: its registers and shared memory fill one.  Where there are fewer slots than warps every SM gets
     // its share of them.
     const long long slots = ((long long)J * cls.L[0] + 31) / 32;   // at most
     const int blocks = (int)std::max(1LL, std::min((long long)max_blocks, slots));
-    int warps = max_warps;
+    int warps = c.warps;
     while (warps > 1 && fit_smem_bytes(cls, warps) > kSmemLimit) --warps;
     warps = (int)std::min((long long)warps, (slots + blocks - 1) / blocks);
     // more than half of an SM's shared memory: no SM gets two blocks while another one still holds the kernel before
@@ -1584,10 +1609,8 @@ int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks) {
         h->err = "fit kernel: a window does not fit in shared memory";
         return -1;
     }
-    const FitKernel kernel = parts == 1 ? kFitAsTeam[h->warm_start ? 1 : 0]
-                                        : kFitKernels[plan.kind][h->warm_start ? 1 : 0][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
     if (e == cudaSuccess)
-        e = launch_behind(kernel, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
+        e = launch_behind(c.fit, blocks, warps * 32, smem, st, h->job, h->fit, h->wtab, in_order ? nullptr : h->scratch.order,
                           h->scratch.start, cls, h->lm_trials, h->min_fit_points, h->scratch.ticket + kFitQueueBase, h->scratch.counters,
                           in_order ? h->scratch.stamps : nullptr, h->err_word);
     ++launches;

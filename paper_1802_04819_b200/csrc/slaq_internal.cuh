@@ -210,6 +210,7 @@ struct slaq_handle {
     bool have_epoch = false;
     int32_t last_launches = 0;            // kernels the last call launched
     int select_blocks_per_sm = 1;         // resident blocks of the selection kernel
+    const void* fit_ready = nullptr;      // the fit kernel whose shared memory was allowed last
     int sm_count = 148;
     std::vector<uint8_t> active;      // host mirror: job has at least one loss
     std::vector<uint32_t> stamp;      // host: duplicate detection
@@ -269,7 +270,7 @@ cudaError_t launch_behind(void (*kernel)(Params...), int blocks, int threads, si
 }
 
 // kernel launchers: each returns the number of kernels it launched, or -1 after setting h->err
-int fit_setup();   // once per device before the first fit; 0 or -1
+int fit_prepare(slaq_handle* h);   // loads what a fit of all the handle's ids launches; 0 or -1
 // on `st`, with at most max_blocks blocks
 int launch_fit(slaq_handle* h, cudaStream_t st, int max_blocks);
 int fit_least_lanes(const slaq_handle* h);
@@ -285,7 +286,7 @@ constexpr int kMaxGroup = 8;
 int launch_select_group(slaq_handle* const* hs, int n, double epoch_seconds, long long want, int first_unit, uint32_t seq,
                         bool* whole_table);
 bool select_writes_whole_table(const slaq_handle* h, long long want);
-int select_setup(int* blocks_per_sm);   // once per device before the first selection launch; 0 or -1
+int select_setup(int* blocks_per_sm);   // before a handle's first selection launch; 0 or -1
 int launch_normalise_export(slaq_handle* h, int32_t n, const int64_t* d_offsets, double* d_changes,
                             double* d_levels, double* d_largest);
 int launch_time_model(slaq_handle* h, double* d_s, double* d_w);

@@ -7,7 +7,7 @@ int fake_err_word = 0;             // what the next selection that reports finds
 }
 
 namespace slaq {
-int fit_setup() { return 0; }
+int fit_prepare(slaq_handle*) { return 0; }
 int select_setup(int* per_sm) { *per_sm = 1; return 0; }
 int fit_least_lanes(const slaq_handle*) { return 2; }
 int launch_fit(slaq_handle*, cudaStream_t, int) { return 1; }
