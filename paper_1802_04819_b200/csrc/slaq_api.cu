@@ -7,13 +7,13 @@
 #endif
 
 #include <algorithm>
-#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstring>
 #include <new>
 
 #include "slaq_internal.cuh"
+#include "slaq_log.cuh"
 #include "slaq_pipe.cuh"
 
 using namespace slaq;
@@ -508,26 +508,6 @@ int check_ids(slaq_handle* h, int32_t n, const int32_t* ids, bool forbid_dups) {
         }
     }
     return SLAQ_OK;
-}
-
-// The logarithm's table (see log_of_normal): pairs of 1 / c and the leading part of log c for the middles c of the bins, then the rests of
-// log c.  Made once: it took 18 us of a new handle's first pass.
-const std::array<double, 3 * kLogBins>& log_table() {
-    static const std::array<double, 3 * kLogBins> table = [] {
-        std::array<double, 3 * kLogBins> t;
-        for (int i = 0; i < kLogBins; ++i) {
-            const uint64_t bits = (uint64_t)(kLogFrom + (i << kLogBinShift) + (1 << (kLogBinShift - 1))) << 32;
-            double c;
-            std::memcpy(&c, &bits, sizeof c);
-            const double inv = 1.0 / c;
-            const long double log_c = -std::log((long double)inv), lead = std::nearbyint(log_c * 0x1p42L) * 0x1p-42L;
-            t[2 * i] = inv;
-            t[2 * i + 1] = (double)lead;
-            t[2 * kLogBins + i] = (double)(log_c - lead);
-        }
-        return t;
-    }();
-    return table;
 }
 
 int ensure_weights(slaq_handle* h) {

@@ -26,6 +26,7 @@
 
 #include "slaq_internal.cuh"
 #include "slaq_fit_sweep.cuh"
+#include "slaq_log.cuh"
 
 namespace slaq {
 
@@ -522,27 +523,6 @@ struct Moments {
 struct GuessSums {
     double swy2, r0, r1, r2, su, sxu;
 };
-
-// log of a positive normal number, to 1.2 ulp, by table lookup (Tang, "Table-driven implementation of the logarithm function", 1990):
-// x = 2^e z with z in about [0.71, 1.42) cut into 128 bins with middles c, log x = e log 2 + log c + log(1 + r) with
-// r = z / c - 1, |r| <= 2^-8, by its Taylor series.  log 2 and log c are split so that the leading parts add up exactly; the bin
-// around 1 has c = 1.  tab: 128 pairs of 1 / c and the leading part of log c, then the rests (written by ensure_weights).  Shorter
-// than log(), whose arguments may be anything (fit of 100,000 windows of up to 1,000, with x counted in rows: 3,615 ->
-// 3,511 us, of 1,000,000 of 64: 3,904 -> 3,803; about half of it each).
-__device__ __forceinline__ double log_of_normal(double x, const double* __restrict__ tab) {
-    const int hi = __double2hiint(x), t = hi - kLogFrom, e = t >> 20, bin = (t >> kLogBinShift) & (kLogBins - 1);
-    const double z = __hiloint2double(hi - (e << 20), __double2loint(x));
-    const double2 c = __ldg(reinterpret_cast<const double2*>(tab) + bin);
-    const double rest = __ldg(tab + 2 * kLogBins + bin);
-    const double r = fma(z, c.x, -1.0);
-    double p = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-    p = fma(r, p, 1.0 / 5.0);
-    p = fma(r, p, -1.0 / 4.0);
-    p = fma(r, p, 1.0 / 3.0);
-    p = fma(r, p, -1.0 / 2.0);
-    const double lead = fma((double)e, 0x1.62e42fefa3800p-1, c.y);   // log 2 to 42 bits behind the point
-    return lead + (r + fma(r * r, p, fma((double)e, 0x1.ef35793c76730p-45, rest)));
-}
 
 // One point of the first-guess pass.  kI / kII: the transformed values of family I (1 / (y - d0)) and of
 // family II (log(y - d0)) are wanted by some lane of the warp.  kAny: y - d0 may be subnormal or not finite.

@@ -18,8 +18,6 @@ constexpr int kRadixBits = 11;
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kRadixPasses = 6;       // 11 + 11 + 11 + 11 + 11 + 9 bits, most significant first
 constexpr int kMaxFitClasses = 8;     // window-length classes of the fit (one launch each)
-constexpr int kLogBins = 128;          // first guesses: the logarithm's table (see log_of_normal), its first bin and the width of a bin
-constexpr int kLogFrom = 0x3fe6b000, kLogBinShift = 13;   // in high words; 1 is the middle of bin 74
 constexpr size_t kDefaultFitSlice = 13824;
 constexpr int kFitQueueBase = 8;      // ticket[kFitQueueBase + c]: work queue head of class c
 constexpr int kTickets = 16;
