@@ -18,6 +18,7 @@
 
 #include <cuda_runtime.h>
 
+#include "slaq_fit_plan.cuh"
 #include "slaq_fit_sweep.cuh"
 
 namespace {

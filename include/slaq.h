@@ -69,7 +69,9 @@ enum {
     SLAQ_P_FIT_SLICE_BYTES = 5,   /* tuning: shared memory one warp of the fit kernel may use (8 KB..200 KB;
                                      the default, 13,824, lets the library choose 13.5, 18 or 27 KB for
                                      sixteen, twelve or eight warps per SM by the number and length of the
-                                     windows); decides how many lanes share a job; results stay within rounding */
+                                     windows).  With another value twelve warps run per SM where so many have
+                                     room, or sixteen where all windows fit at two lanes; it then decides how
+                                     many lanes share a job.  Results stay within rounding */
     SLAQ_P_WARM_START = 6,        /* 0 (default) or 1.  The scheduler refits every job at short intervals
                                      (Evaluation, "Scalability and efficiency"); with 1, a family starts from the
                                      parameters the job's last epoch ended with, carried into this epoch's window

@@ -53,12 +53,6 @@ struct Phases {
 #endif
 
 constexpr int kMaxWarpsPerBlock = 16;          // one block per SM: its warps share one copy of the weight table
-// Warps of the fit kernel's block and shared memory of each.  Fewer warps have larger slices, so that a job needs fewer lanes, and more registers (128, 168, 255 a
-// thread at 16, 12, 8), which spill nothing and, at 8, let two rows overlap.
-constexpr int kFitWarps[3] = {16, 12, 8};
-constexpr size_t kFitSlices[3] = {kDefaultFitSlice, 18432, 27648};
-enum { kSixteen, kTwelve, kEight };
-constexpr size_t kSmemLimit = 226 * 1024;   // shared memory one block may use on sm_100, less the static part
 constexpr int kTeamWarps = 8;               // warps of a block that works on one job
 constexpr size_t kTeamSmem = 220 * 1024;
 constexpr double kLambda0 = 1e-3, kLambdaMin = 1e-5, kLambdaMax = 1e12;
@@ -730,16 +724,6 @@ __device__ __noinline__ void restart_from_first_guesses(const Lanes& S, int fam,
     if (redo) *sums = again;
 }
 
-// Window-length classes, longest first: class c holds the jobs with h_lo[c] < H <= h_hi[c] and
-// gives each of them L[c] lanes.  All classes are served by one launch from one work queue
-// whose slots are numbered class by class, so the longest windows start first.
-struct FitClasses {
-    int n;
-    int h_lo[kMaxFitClasses], h_hi[kMaxFitClasses], L[kMaxFitClasses];
-    int h_max;       // longest window
-    int slice;       // doubles of shared memory per warp: parked sums, window rows, one spare row
-};
-
 // One slot of the work queue: the place-th warp's worth of jobs of class c.  kWarm: families may start from last epoch's
 // parameters (a separate instantiation, so that the plain one carries none of that code).  kL: lanes per job, a
 // constant, which takes branches and index arithmetic out of every step of a trial.
@@ -1371,14 +1355,12 @@ size_t fit_smem_bytes(const FitClasses& c, int warps) {
 using FitKernel = decltype(&fit_kernel<false, 0, 12>);
 using FitTeamKernel = decltype(&fit_team_kernel<false, false>);
 // [warps][warm start][lanes: 0 for several, 2, 4, .. 32]; null: never chosen
-#define SLAQ_ALL(warm, w, two) \
-    {fit_kernel<warm, 0, w>, two, fit_kernel<warm, 4, w>, fit_kernel<warm, 8, w>, fit_kernel<warm, 16, w>, fit_kernel<warm, 32, w>}
+#define SLAQ_SOME(warm, w) fit_kernel<warm, 2, w>, fit_kernel<warm, 4, w>, fit_kernel<warm, 8, w>, fit_kernel<warm, 16, w>, fit_kernel<warm, 32, w>
 static FitKernel const kFitKernels[3][2][6] = {
     {{nullptr, fit_kernel<false, 2, 16>}, {nullptr, fit_kernel<true, 2, 16>}},
-    {SLAQ_ALL(false, 12, (fit_kernel<false, 2, 12>)), SLAQ_ALL(true, 12, (fit_kernel<true, 2, 12>))},
-    {{nullptr, fit_kernel<false, 2, 8>, fit_kernel<false, 4, 8>, fit_kernel<false, 8, 8>, fit_kernel<false, 16, 8>, fit_kernel<false, 32, 8>},
-     {nullptr, fit_kernel<true, 2, 8>, fit_kernel<true, 4, 8>, fit_kernel<true, 8, 8>, fit_kernel<true, 16, 8>, fit_kernel<true, 32, 8>}}};
-#undef SLAQ_ALL
+    {{fit_kernel<false, 0, 12>, SLAQ_SOME(false, 12)}, {fit_kernel<true, 0, 12>, SLAQ_SOME(true, 12)}},
+    {{nullptr, SLAQ_SOME(false, 8)}, {nullptr, SLAQ_SOME(true, 8)}}};
+#undef SLAQ_SOME
 static FitKernel const kFitAsTeam[2] = {fit_kernel<false, 32, 8, false>, fit_kernel<true, 32, 8, false>};   // see fit_kernel
 
 static FitTeamKernel const kFitTeamKernels[2][2] = {{fit_team_kernel<false, false>, fit_team_kernel<false, true>},
@@ -1400,63 +1382,15 @@ static long long jobs_for_lanes(const slaq_handle* h, long long active) {
     return h->fit_cluster_jobs > 0 ? (long long)h->fit_cluster_jobs : active;
 }
 
-// Doubles of shared memory per warp: the parked sums, the window rows and one spare row.  It grows if the longest window
-// does not fit at 32 lanes.
-static int fit_slice(const slaq_handle* h, size_t bytes) {
-    return std::max((int)(bytes / sizeof(double)), kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32);
-}
 static int team_slice(const slaq_handle* h) { return kParked * 2 + ((h->max_hist + 31) / 32 + 1) * 32; }
 static size_t team_smem(const slaq_handle* h, int parts) {
     return sizeof(double) * ((size_t)h->max_hist + 2 * (size_t)parts * team_slice(h));
 }
-static int rows_at(int slice, int L) { return (slice - kParked * (64 / L)) / 32 - 1; }
 
-// The warps of a block and the fewest lanes a job gets, from the cluster's jobs and the longest window alone.  Fewer lanes are less
-// work - the solver's step and the reductions of a trial cost a warp the same whatever it carries - and longer chains of rows.  Fewer
-// warps have room for fewer lanes, and leave issue slots empty.  Costs in cycles per trial: a warp alone takes `chain` + `chain_row` per row, a
-// sub-partition issues `issue` + `issue_row` per row for each of its warps, of which a part counts `part` more; slots beyond what is
-// resident are another wave, of which `mixed` is hidden behind the one before.  Every window is taken for full, and a fifth of the jobs,
-// half the time, for new ones of a few points.  Fitted to the fits of 700 to 200,000 windows of 20 to 1,000 points at 8, 12 and 16 warps and
-// 2 to 32 lanes: full ones 2.4 % from the best choice on average, ragged ones 2.9 %, a fifth of them new 6.3 %.  Sixteen warps for
-// all with the lanes they have room for, the rule before, were 7.4, 9.6 and 11.2 % from it.
-struct FitPlan {
-    int kind, lanes;   // index into kFitWarps; least lanes
-    size_t slice_bytes;
-};
-static FitPlan fit_plan(const slaq_handle* h, long long active) {
-    constexpr struct {
-        double chain, chain_row, issue, issue_row, part, mixed;
-    } cost_of[3] = {{4600, 315, 1230, 95, 0.5, 0.55}, {3600, 220, 1250, 97, 0.9, 0.4}, {3300, 190, 1340, 106, 0.1, 0.4}};
-    const int Hmax = h->max_hist;
-    const double jobs = (double)std::max(1LL, jobs_for_lanes(h, active)), sub = 4.0 * h->sm_count;
-    const bool by_size = h->fit_slice_bytes == kDefaultFitSlice;
-    FitPlan best = {kTwelve, 32, by_size ? kFitSlices[kTwelve] : h->fit_slice_bytes};
-    double least = -1.0;
-    for (int L = 32; L >= 2; L >>= 1) {
-        for (int kind : {kTwelve, kEight, kSixteen}) {
-            const size_t bytes = by_size ? kFitSlices[kind] : h->fit_slice_bytes;
-            if (rows_at(fit_slice(h, bytes), L) * L < Hmax) continue;
-            if (kind != kTwelve && !by_size) continue;
-            if (kind == kSixteen && L > 2) continue;   // more lanes are always better off with more registers
-            const auto& c = cost_of[kind];
-            const double rows = (Hmax + L - 1) / L, chain = c.chain + c.chain_row * rows, each = c.issue + c.issue_row * rows;
-            const double resident = kFitWarps[kind] / 4;
-            auto wave = [&](double n) { return n > 0.02 ? std::max(chain, std::min(std::ceil(n), n + c.part) * each) : 0.0; };
-            auto cycles = [&](double n) {   // n slots per sub-partition
-                const double full = std::floor(n / resident);
-                const double stepped = full * wave(resident) + wave(n - full * resident);
-                return c.mixed * n * std::max(each, chain / resident) + (1.0 - c.mixed) * stepped;
-            };
-            const double slots = jobs * L / 32.0 / sub, cost = cycles(slots) + cycles(0.8 * slots);
-            if (least < 0.0 || cost <= least) best = {kind, L, bytes}, least = cost;
-        }
-    }
-    // Beyond a wave and a half more lanes only add work, although the longest windows then get more lanes than the others.
-    if (best.kind == kTwelve)
-        while (best.lanes > 2 && jobs * (best.lanes / 2) >= 1.5 * 32.0 * kFitWarps[kTwelve] * h->sm_count) best.lanes >>= 1;
-    return best;
+static FitPlan plan_of(const slaq_handle* h, long long active) {
+    return fit_plan(h->max_hist, jobs_for_lanes(h, active), h->sm_count, h->fit_slice_bytes);
 }
-int fit_least_lanes(const slaq_handle* h) { return fit_plan(h, h->n_active).lanes; }
+int fit_least_lanes(const slaq_handle* h) { return plan_of(h, h->n_active).lanes; }
 
 // Warps per family of a job's team; 0: no teams.  A question of the cluster's active jobs and the windows alone, which every shard
 // answers alike, whatever its capacity: several warps add in another order than one, and one in another than a part of one.  With a warp per sub-partition at most, a lane is left four rows of the longest
@@ -1526,26 +1460,10 @@ static FitChoice fit_choice(const slaq_handle* h, long long active) {
         c.kernel = (const void*)c.team;
         return c;
     }
-    // Length classes, longest first.  A warp's slice holds the parked sums of its jobs (kParked doubles per job and
-    // family), the window rows of 32 points and one spare row.  The class with L = 32, 16, .. lanes per job takes
-    // the windows that do not fit at L/2 lanes; the last one has the fewest lanes and takes the rest.
-    FitClasses& cls = c.cls;
-    const FitPlan plan = parts == 1 ? FitPlan{kEight, 32, kFitSlices[kEight]} : fit_plan(h, active);
+    const FitPlan plan = parts == 1 ? FitPlan{kEight, 32, kFitSlices[kEight]} : plan_of(h, active);
     c.warps = kFitWarps[plan.kind];
-    cls.slice = fit_slice(h, plan.slice_bytes);
-    const int L_min = plan.lanes;
-    int h_hi = Hmax;
-    for (int L = 32; L >= L_min && h_hi > 0; L >>= 1) {
-        const int h_lo = L > L_min ? std::max(rows_at(cls.slice, L / 2), 0) * (L / 2) : 0;
-        if (h_lo >= h_hi) continue;
-        cls.h_lo[cls.n] = h_lo;
-        cls.h_hi[cls.n] = h_hi;
-        cls.L[cls.n] = L;
-        ++cls.n;
-        h_hi = h_lo;
-    }
-    for (int k = cls.n; k < kMaxFitClasses; ++k) cls.h_lo[k] = cls.h_hi[k] = 0, cls.L[k] = 32;
-    c.fit = parts == 1 ? kFitAsTeam[warm] : kFitKernels[plan.kind][warm][cls.n == 1 ? __builtin_ctz((unsigned)cls.L[0]) : 0];
+    c.cls = fit_classes(Hmax, plan);
+    c.fit = parts == 1 ? kFitAsTeam[warm] : kFitKernels[plan.kind][warm][c.cls.n == 1 ? __builtin_ctz((unsigned)c.cls.L[0]) : 0];
     c.kernel = (const void*)c.fit;
     return c;
 }

@@ -11,7 +11,6 @@
 namespace slaq {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kParked = 12;                 // doubles per job and family kept in shared memory between sweeps
 
 __device__ __forceinline__ bool finite_d(double v) { return fabs(v) <= 1.7976931348623157e308; }
 

@@ -9,6 +9,7 @@
 
 #include "slaq.h"
 #include "slaq_bounds.cuh"
+#include "slaq_fit_plan.cuh"
 
 namespace slaq {
 
@@ -17,8 +18,6 @@ constexpr int kMaxCoresLimit = 1024;
 constexpr int kRadixBits = 11;
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kRadixPasses = 6;       // 11 + 11 + 11 + 11 + 11 + 9 bits, most significant first
-constexpr int kMaxFitClasses = 8;     // window-length classes of the fit (one launch each)
-constexpr size_t kDefaultFitSlice = 13824;
 constexpr int kFitQueueBase = 8;      // ticket[kFitQueueBase + c]: work queue head of class c
 constexpr int kTickets = 16;
 
