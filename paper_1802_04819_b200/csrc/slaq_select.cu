@@ -26,8 +26,8 @@
 // How much of a row is looked at.  Jobs get few cores on average, so of a large table only the first `depth` cores
 // of each row enter the histogram; their bin bounds the threshold from below, and only the rows whose last gain
 // still reaches that bound are continued (once, until they fall below it) before the interval is taken again.  Gains
-// behind a row's first gain below the bound are below it too and can never be handed out.  Of 60,000 rows and
-// more the bound comes from a sample of them, before any other is looked at (predict_to_bound).
+// behind a row's first gain below the bound are below it too and can never be handed out.  Of large tables
+// (select_bounded) the bound comes from a sample of the rows, before any other is looked at (predict_to_bound).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -35,6 +35,7 @@
 
 #include "slaq_gain_curve.cuh"
 #include "slaq_internal.cuh"
+#include "slaq_select_plan.cuh"
 
 namespace slaq {
 
@@ -725,10 +726,9 @@ __device__ __forceinline__ void predict_row(const SelectArgs& a, Shared& sh, boo
 // listed, those that need more than four gains from the front, and their gains make the histogram the interval is taken from.
 // Should the sample have misled (fewer gains than wanted at or above the bound), every row is predicted to its end: slow, and the same result.
 // Predicting the first 16 gains of every row and taking the bound from those instead continued rows for a bound far below the
-// threshold, since they hold too few of the gains of the rows that get many (launch for 1,000,000 rows of 128: 438 -> 204 us, first gains
+// threshold, since they hold too few of the gains of the rows that get many (launch for 1,000,000 rows of 128: 437 -> 201 us, first gains
 // 142 -> 60 of them, continued rows 151 -> 50, walk 106 -> 30).
 // Returns false after a barrier that was not reached.
-constexpr int kSampleLeast = 32, kSampleShare = 64;   // rows a block samples: at least, and one in so many
 constexpr int kFirstGains = 4;
 template <class Args>
 __device__ bool predict_to_bound(const Args& args, const SelectArgs& a, Shared& sh, CurveTile& tile, int j0, int j1, unsigned int& arrived,
@@ -812,9 +812,11 @@ __device__ bool predict_to_bound(const Args& args, const SelectArgs& a, Shared& 
                 store_alloc(a, j, active ? floor_cores : 0, active && floor_cores ? tile.v[tid] : 0.0, active);
                 *handed += active ? floor_cores : 0;
             } else if (state == 2) {
-                list[atomicAdd(&sh.narrow[0], 1u)] = j;
+                const int at = (int)atomicAdd(&sh.narrow[0], 1u);
+                if (index_ok(at, n, kErrJob, a.err_word)) list[at] = j;
             } else {
-                list[n - 1 - (int)atomicAdd(&sh.narrow[1], 1u)] = j;
+                const int at = n - 1 - (int)atomicAdd(&sh.narrow[1], 1u);
+                if (index_ok(at, n, kErrJob, a.err_word)) list[at] = j;
             }
         }
         __syncthreads();
@@ -826,7 +828,7 @@ __device__ bool predict_to_bound(const Args& args, const SelectArgs& a, Shared& 
         bool in;
         const int r = draw(*n_more, &in);
         if (__all_sync(kFull, !in)) break;
-        predict_row(a, sh, in, in ? list[r] : j0, kFirstGains, bound, kTopKey, bound, true, low);
+        predict_row(a, sh, in, in && index_ok(r, n, kErrJob, a.err_word) ? list[r] : j0, kFirstGains, bound, kTopKey, bound, true, low);
     }
     add_low(sh, low);
     flush_first(sh, a.gl->fine_more);
@@ -1037,7 +1039,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_kernel(const __grid_consta
     for (int base = 0; base < n_walk; base += kThreads) {   // uniform trip count: a warp finishes its long rows together
         const int at = base + slot;
         const bool in = at < n_walk;
-        const int j = !in ? j0 : !listed ? j0 + at : list[at < n_more ? at : j1 - j0 - 1 - (at - n_more)];
+        const int place = at < n_more ? at : j1 - j0 - 1 - (at - n_more);   // in the list: the longer ones from its front, the others from its end
+        const int j = !in ? j0 : !listed ? j0 + at : index_ok(place, j1 - j0, kErrJob, a.err_word) ? list[place] : j0;
         const bool active = in && (!a.count || a.count[j] > 0);
         const double* row = resident ? rows_sh + (size_t)(j - j0) * a.stride : a.gain + (size_t)j * a.cap;
         int s = 0, c = 0;
@@ -1361,11 +1364,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const __grid_
 // Rule for the rows' home.  Up to kResidentGains gains per block (two evaluations per thread) all of them are predicted
 // at once, kept in shared memory and walked there; the whole table is written as well.  Beyond that prediction is what
 // costs (910 us for 128 gains of a million jobs each), so rows start with four times the average number of
-// cores handed out, at least 16, and only rows that need more are continued.  From kBoundedRows rows on gains are predicted down to a bound
-// from a sample instead, whose barrier and long rows cost the smaller ones 3 to 6 us more than it gives (launch of 33,000 rows: 34 -> 37
-// us, of 100,000: 55 -> 47).
-constexpr int kResidentGains = 2048;
-constexpr int kBoundedRows = 60000;
+// cores handed out, at least 16, and only rows that need more are continued.  Large tables are predicted down to a bound from a
+// sample instead (select_bounded).
 constexpr int kKeepLast = 8192;
 constexpr int kSmallGains = 6144, kSmallRows = 256;   // one block up to here (see select_small_kernel)
 
@@ -1387,13 +1387,6 @@ int select_setup(int* blocks_per_sm) {
     return 0;
 }
 
-// Cores per row that enter the first histogram.
-static int select_depth(long long J, int cap, long long want, int sm_count) {
-    if (J * cap <= (long long)kResidentGains * sm_count) return cap;
-    const long long average = (want + J - 1) / J + 1;
-    return (int)std::min<long long>(cap, std::max<long long>(16, (4 * average + 15) / 16 * 16));
-}
-
 // The part of the arguments that depends on the sizes, the same for all handles of a launch (J: their rows in all).
 struct SelectPlan {
     int depth, W, rows, stride, keep_last, bounded;
@@ -1408,7 +1401,7 @@ static SelectPlan plan_select(long long J, int cap, long long want, bool curves,
     SelectPlan p;
     const long long gains = J * cap;
     p.depth = select_depth(J, cap, want, sm_count);
-    p.bounded = curves && p.depth < cap && J >= kBoundedRows;
+    p.bounded = curves && select_bounded(J, cap, want, sm_count, sm_count * blocks_per_sm);
     p.W = 1;
     long long grid;
     if (gains <= (long long)kResidentGains * sm_count) {
