@@ -274,7 +274,10 @@ __device__ __forceinline__ void sweep(const Lanes& S, int fam, int H, int k_all,
     // other, 7 + 4 + 2 + 1 exchanges instead of 13 in every step, and every sum ends in one lane.
     double chk, objective;
     if (S.L() == 2) {
-        // these bound the others: |x| <= 1, and sum |w u r x^k| <= sqrt(sum w u^2 . sum w r^2)
+        // Family I: sum w u^2 and sum w u^2 x^4 bound what lies between, and sum |w u r x^k| <= sqrt(sum w u^2 x^2k . sum w r^2).  Family II:
+        // sum w e^2 bounds its sums without x.  Those with x, which counts rows in cold fits and is counted in rows by the chains always, can be
+        // up to the square of a lane's rows (9,025 at eight warps) times as large.  Where they overflow and sum w e^2 does not, within four
+        // orders of the end of the range, the point stands, no step is found from it and the fit ends there; more lanes drop it.
         objective = v[12];
         chk = (v[0] + v[4]) + v[12];
     } else {
