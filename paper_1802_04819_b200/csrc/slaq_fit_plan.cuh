@@ -12,7 +12,8 @@ constexpr int kMaxFitClasses = 8;     // window-length classes of a launch
 constexpr size_t kSmemLimit = 226 * 1024;   // shared memory one block may use on sm_100, less the static part
 
 // Warps of the fit kernel's block and shared memory of each.  Fewer warps have larger slices, so that a job needs fewer lanes, and more
-// registers: 128 at sixteen warps, 147 to 168 at twelve, 168 to 192 at eight, where two rows overlap.
+// registers: 128 a thread at sixteen warps, 147 to 168 at twelve (of 168), 168 to 192 at eight (of 255), where two rows overlap.  Warm
+// starts spill at sixteen (104 bytes) and at twelve with several classes (200 bytes), cold fits nowhere.
 enum { kSixteen, kTwelve, kEight };
 constexpr int kFitWarps[3] = {16, 12, 8};
 constexpr size_t kDefaultFitSlice = 13824;
