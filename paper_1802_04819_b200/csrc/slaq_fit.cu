@@ -1414,9 +1414,7 @@ static cudaError_t launch_sort(slaq_handle* h, cudaStream_t st, int* launches) {
     const int J = h->max_jobs, Hmax = h->max_hist;
     const size_t bins = sizeof(int) * ((size_t)Hmax + 1);
     long long* const stamp = h->scratch.stamps;
-    const auto sorter = J <= kOneBlockSort ? (const void*)length_sort_kernel : (const void*)length_scatter_kernel;
-    if (2 * bins > 48 * 1024)
-        if (const cudaError_t no = cudaFuncSetAttribute(sorter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * bins))) return no;
+    static_assert(2 * sizeof(int) * (kMaxHistLimit + 1) + 32 * sizeof(int) <= 48 * 1024, "both sorts take what a block may use without asking");
     if (J <= kOneBlockSort) {
         *launches += 1;
         return launch_behind(length_sort_kernel, 1, 1024, 2 * bins, st, h->job.count, J, Hmax, h->scratch.start, h->scratch.order, stamp,
