@@ -1,36 +1,25 @@
-"""Clusters that take each of the fit kernel's block sizes, with windows at the edges of the lane classes, against the oracle; the plan is
-the library's own, compiled for the host."""
+"""Clusters that take each of the fit kernel's block sizes, with windows at the edges of the lane classes, against the oracle."""
 
 import numpy as np
 import pytest
 
-from fit_plan import fit_plan
 from gpu_common import R_ATOL, R_RTOL, compare_epoch, make_scheduler, oracle_epoch, oracle_spread, tolerance_widths
 from workloads import make_workload
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("jobs,longest,packed,plan", [
-    (600, 200, False, (8, 32, 1)),
-    (1500, 417, False, (8, 16, 1)),
-    (2500, 208, False, (12, 16, 1)),
-    (3000, 40, False, (8, 8, 1)),
-    (4000, 8, False, (8, 2, 1)),
-    (1000, 8, True, (8, 4, 1)),
-    (1200, 261, True, (12, 32, 1)),
-    (5000, 260, True, (12, 8, 1)),
-    (5000, 261, True, (12, 8, 1)),
-    (12000, 119, False, (12, 4, 1)),
-    (20000, 8, False, (12, 2, 1)),
-    (24000, 261, True, (12, 4, 2)),     # one point more than four lanes take
-    (35000, 20, False, (16, 2, 1)),
-    (45000, 200, False, (12, 2, 2)),    # two lanes take 118 points
+@pytest.mark.parametrize("jobs,longest,packed", [
+    (600, 200, False),        # eight warps, 32 lanes
+    (1500, 417, False),       # eight, 16 lanes, rows to the last
+    (2500, 208, False),       # eight, fewer lanes
+    (5000, 260, True),        # twelve, several lanes per job; longest window the slice takes at four lanes
+    (5000, 261, True),        # one more point than that
+    (12000, 119, False),      # twelve, two classes: 118 points fit at two lanes
+    (35000, 20, False),       # sixteen: one wave at two lanes
 ])
-def test_every_block_size_matches_the_oracle(oracle_mod, jobs, longest, packed, plan):
-    warps, least, classes, _ = fit_plan(longest, jobs)
-    assert (warps, least, len(classes)) == plan
-    edges = [h for h in (3, 4, 5, 31, 32, 33, 63, 64, 65, 82, 83, 117, 118, 119, 259, 260, longest - 1, longest) if h <= longest]
+def test_every_block_size_matches_the_oracle(oracle_mod, jobs, longest, packed):
+    edges = [h for h in (3, 4, 5, 31, 32, 33, 63, 64, 65, 82, 83, 117, 118, 119, longest - 1, longest) if h <= longest]
     lengths = np.resize(np.array(edges, dtype=np.int64), jobs)
     lengths[-3:] = longest
     wl = make_workload(2, hist_lengths=lengths)
@@ -47,39 +36,3 @@ def test_every_block_size_matches_the_oracle(oracle_mod, jobs, longest, packed, 
         spread = oracle_spread(oracle_mod, wl, j, cap)
         assert (np.abs(Rg[j] - Rc[j]) <= 4.0 * spread + R_RTOL * np.abs(Rc[j]) + R_ATOL).all(), j
     compare_epoch(alloc, pred, ref, wl.total_cores, cap, allow_unstable=misses.size, total_rtol=1e-7)
-
-
-EDGES = [4, 5, 31, 32, 33, 64, 117, 118, 119, 128, 259, 260, 261, 300, 512, 543, 544, 545, 700, 999, 1000]
-
-
-@pytest.mark.parametrize("warm", [0, 1])
-def test_the_edges_of_the_classes_that_a_large_cluster_has(oracle_mod, warm):
-    """Few jobs told that they are part of a large cluster: twelve warps, four classes.  Cold against the oracle; warm started against 32
-    lanes per job from the same curves."""
-    import paper_1802_04819_b200 as slaq
-    assert [(lanes, high) for lanes, _, high in fit_plan(1000, 100_000)[2]] == [(16, 1000), (8, 544), (4, 260), (2, 118)]
-    lengths = np.resize(np.array(EDGES, dtype=np.int64), 1260)
-    wl = make_workload(3, hist_lengths=lengths)
-    a = make_scheduler(wl, max_hist=1000)
-    a.set_param(slaq.binding.P_FIT_CLUSTER_JOBS, 100_000)
-    alloc, _ = a.schedule(wl.epoch_seconds, wl.total_cores)
-    pred, cap = a.get_predictions(), wl.max_cores_per_job
-    if not warm:
-        compare_epoch(alloc, pred, oracle_epoch(oracle_mod, wl), wl.total_cores, cap)
-        return
-    b = make_scheduler(wl, max_hist=1000)
-    b.set_param(slaq.binding.P_FIT_CLUSTER_JOBS, 600)
-    assert fit_plan(1000, 600)[1] == 32
-    b.schedule(wl.epoch_seconds, wl.total_cores)
-    b.set_fit_state(a.get_fit_state())
-    ids, next_loss = np.arange(wl.n_jobs, dtype=np.int32), 0.999 * wl.losses[wl.offsets[1:] - 1]
-    for s in (a, b):
-        s.set_param(slaq.binding.P_WARM_START, 1)
-        s.set_param(slaq.binding.P_LM_TRIALS, 5)
-        s.append_losses(ids, next_loss)
-    alloc_a, _ = a.schedule(wl.epoch_seconds, wl.total_cores)
-    alloc_b, _ = b.schedule(wl.epoch_seconds, wl.total_cores)
-    ref = b.get_predictions()
-    ref["alloc"] = alloc_b
-    # five trials continue unfinished iterations, whose end depends on rounding in single jobs: one in a thousand
-    compare_epoch(alloc_a, a.get_predictions(), ref, wl.total_cores, cap, allow_unstable=1, total_rtol=1e-7)
